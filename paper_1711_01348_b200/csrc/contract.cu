@@ -8,17 +8,15 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <climits>
 
-#include "contract.h"
-#include "program.h"
+#include "contract.cuh"
 
 namespace {
 
 constexpr int BK = TADC_BK;
 constexpr int KK_UNROLL = 8;          // summation indices per unrolled body of the multiply-add loop
 constexpr int STAGES = 2;
-constexpr int DEAD = INT_MIN / 2;      // guard part of a row or summation index that does not exist
+using namespace tadc;
 
 __device__ __forceinline__ void cp_async4(float *dst, const float *src, bool live)
 {
@@ -34,26 +32,6 @@ __device__ __forceinline__ void cp_async16(float *dst, const float *src, bool li
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
-
-struct Parts { int a, b, o, ga, gb; };
-
-// digits of a flattened index, last digit fastest, folded into the offset parts of the group
-__device__ __forceinline__ Parts decode(const TadcGroup &G, unsigned idx)
-{
-    Parts p{0, 0, 0, 0, 0};
-#pragma unroll
-    for (int d = TADC_MAX_DIGITS - 1; d >= 0; --d) {
-        if (d < G.n_digits) {
-            const unsigned e = (unsigned)G.ext[d];
-            const unsigned q = idx / e;
-            const int r = (int)(idx - q * e);
-            idx = q;
-            p.a += r * G.sA[d]; p.b += r * G.sB[d]; p.o += r * G.sO[d];
-            p.ga += r * G.gA[d]; p.gb += r * G.gB[d];
-        }
-    }
-    return p;
-}
 
 // One stage of one operand: BK x BR values into smem[kl * (BR + 4) + rl].  rows[rl] = (offset part, guard
 // part) of tile row rl, ktab[kl] the same for the stage's summation index kl.  CHECK = false is the path
@@ -137,35 +115,6 @@ __device__ __forceinline__ void gather(float *smem, const float *__restrict__ sr
         for (unsigned j = 0; j < PER; ++j) cp_async4(smem + kl * LD + rl0 + RSTEP * j, src + off[j], live[j]);
     }
     }
-}
-
-__device__ __forceinline__ float own_tanh(float x)
-{
-    const float ax = fabsf(x);
-    const float e = __expf(2.f * ax);
-    const float t = 1.f - __fdividef(2.f, e + 1.f);
-    const float x2 = x * x;
-    const float small = x * (1.f + x2 * (-0.33333334f + x2 * (0.13333334f + x2 * -0.05396825f)));
-    return ax < 0.25f ? small : copysignf(t, x);
-}
-
-// the steps every finished sum goes through before it is stored
-__device__ __forceinline__ float epilogue(const TadcProgram &P, const TadpPointers &ptrs, float v, unsigned off)
-{
-    for (int s = 0; s < P.n_epi; ++s) {
-        switch (P.epi_op[s]) {
-        case TE_NEG: v = -v; break;
-        case TE_EXP: v = __expf(v); break;
-        case TE_MULC: v *= P.epi_imm[s]; break;
-        case TE_ADDC: v += P.epi_imm[s]; break;
-        case TE_SQR: v *= v; break;
-        case TE_TANH: v = own_tanh(v); break;
-        case TE_MUL_LOAD: v *= __ldg(ptrs.in[P.epi_ptr[s]] + (unsigned)(P.epi_base[s] + (int)off)); break;
-        case TE_ADD_LOAD: v += __ldg(ptrs.in[P.epi_ptr[s]] + (unsigned)(P.epi_base[s] + (int)off)); break;
-        default: break;
-        }
-    }
-    return v;
 }
 
 template <int BM, int BN, int TM, int TN>
@@ -747,9 +696,12 @@ cudaError_t launch_shape(const TadcProgram &P, const TadpPointers &ptrs, cudaStr
 
 }  // namespace
 
+cudaError_t tad_launch_mma(const TadcProgram &P, const TadpPointers &ptrs, unsigned sms, cudaStream_t stream);
+
 cudaError_t tad_launch_contract(const TadcProgram &P, const TadpPointers &ptrs, unsigned sms, cudaStream_t stream)
 {
     if (P.M.extent <= 0 || P.N.extent <= 0 || P.Z.extent <= 0) return cudaSuccess;
+    if (P.shape == 7) return tad_launch_mma(P, ptrs, sms, stream);
     if (P.shape == 5) {
         const unsigned rows_per_block = P.modeA == TG_K ? 16u : 512u;
         dim3 grid(((unsigned)P.M.extent + rows_per_block - 1u) / rows_per_block, (unsigned)std::max(1, P.ksplit), 1u);

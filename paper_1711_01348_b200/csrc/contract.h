@@ -14,11 +14,14 @@
 
 #define TADC_MAX_DIGITS 4
 #define TADC_BK 32            // summation indices per shared-memory stage
+#define TADC_KS 64            // the same for the tensor-core kernel
 
 struct TadcGroup {             // flattened index group, last digit fastest
     int32_t n_digits;
     int32_t extent;            // product of ext[]
     int32_t ext[TADC_MAX_DIGITS];
+    uint32_t div_mul[TADC_MAX_DIGITS];     // n / ext[d] = (n * div_mul[d]) >> div_shift[d] for n < 2^31
+    int32_t div_shift[TADC_MAX_DIGITS];
     int32_t sA[TADC_MAX_DIGITS];   // element stride of every digit in operand A, operand B, the output
     int32_t sB[TADC_MAX_DIGITS];
     int32_t sO[TADC_MAX_DIGITS];
@@ -32,6 +35,9 @@ enum TadcGather : int {
     TG_K,          // lanes along the summation index, 4 bytes per copy
     TG_ROW16       // rows contiguous and 16-byte aligned: 16 bytes per copy along the row index
 };
+
+// the same for the tensor-core kernel (shape 7; see mma.cu): which index the lanes run along, or 32-byte vectors
+enum TadcMmaGather : int { TM_ROW = 0, TM_KVEC, TM_K, TM_RVEC };
 
 // steps applied to every finished sum before it is stored (in this order)
 enum TadcEpilogueOp : int { TE_END = 0, TE_NEG, TE_EXP, TE_MULC, TE_ADDC, TE_MUL_LOAD, TE_ADD_LOAD, TE_SQR, TE_TANH, TE_SIN, TE_COS };
@@ -50,7 +56,8 @@ struct alignas(16) TadcProgram {
     int32_t accumulate;            // 1: out += result
     int32_t out_vec4;              // 1: four consecutive n are four consecutive, 16-byte aligned output elements
     int32_t shape;                 // tiles: 0 = 128 x 128 (8 x 8 per thread), 1 = 128 x 32, 2 = 128 x 64, 3 = 128 x 36 (8 x 4 per thread);
-                                   // 4 = sums of rows (a warp per output), 5 = streamed narrow contraction, 6 = sums of columns (a thread per output)
+                                   // 4 = sums of rows (a warp per output), 5 = streamed narrow contraction, 6 = sums of columns (a thread per output),
+                                   // 7 = tensor-core tiles of 128 rows (mma.cu)
     float scale;
     int32_t n_epi;
     int32_t epi_op[TADC_MAX_EPI];

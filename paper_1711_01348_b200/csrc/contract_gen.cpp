@@ -42,9 +42,21 @@ bool fill_group(TadcGroup &G, std::vector<Digit> &ds, const AGuard *ga, const AG
         G.gA[d] = ga ? fit(ga->coef[ds[d].var]) : 0;
         G.gB[d] = gb ? fit(gb->coef[ds[d].var]) : 0;
         extent = mul_ck(extent, ds[d].ext);
+        const uint64_t e = (uint64_t)std::max<int64_t>(1, ds[d].ext);
+        int s = 0; while ((uint64_t(1) << s) < e) ++s;
+        G.div_mul[d] = (uint32_t)(((uint64_t(1) << (31 + s)) / e) + 1);
+        G.div_shift[d] = 31 + s;
     }
     G.extent = fit(extent);
     return true;
+}
+
+// tensor-core tiles (mma.cu) or multiply-add tiles (contract.cu): a x b outputs, k terms each.  A stage of the tensor-core
+// kernel costs the same however full it is, so a side below 8 or fewer than 16 terms would leave most of it empty; below
+// 2^20 multiply-adds either kernel is one short wave (a step of the 203 x 157 x 7 intro expression does not change).
+bool mma_pays(int64_t a, int64_t b, int64_t k)
+{
+    return std::max(a, b) >= 64 && std::min(a, b) >= 8 && k >= 16 && (double)a * (double)b * (double)k >= (double)(1 << 20);
 }
 
 }  // namespace
@@ -63,6 +75,28 @@ bool emit_program(const System &s0, float scale, int accumulate, bool allow_spli
     bool b_has_rows = false;                               // B reads some variable that is not summed
     for (int v = 0; v < nv; ++v) if (!s.vars[v].reduce && s.vars[v].ext > 1 && s.B.coef[v] != 0) b_has_rows = true;
     if (contiguous >= 0 && s.A.coef[contiguous] != 0 && s.B.coef[contiguous] == 0 && s.B.ptr >= 0 && b_has_rows) std::swap(s.A, s.B);
+    // large enough for the tensor-core tiles: the output's contiguous variable then indexes the rows (a warp's lanes hold
+    // consecutive rows and store them together), unless the other side is too narrow to be the tile's 128 rows
+    bool mma = false, turned = false;                       // turned: the operands traded places for the tile
+    {
+        auto side = [&](const AMap &x, const AMap &y) {            // outputs of the group only x indexes
+            int64_t n = 1;
+            for (int v = 0; v < nv; ++v) if (!s.vars[v].reduce && s.vars[v].ext > 1 && x.coef[v] != 0 && y.coef[v] == 0) n = mul_ck(n, s.vars[v].ext);
+            return n;
+        };
+        int64_t kext = 1, rest = 1;
+        for (int v = 0; v < nv; ++v) {
+            if (s.vars[v].reduce) kext = mul_ck(kext, s.vars[v].ext);
+            else if (s.vars[v].ext > 1 && s.A.coef[v] == 0 && s.B.coef[v] == 0) rest = mul_ck(rest, s.vars[v].ext);
+        }
+        if (s.B.ptr >= 0) {
+            int64_t a = side(s.A, s.B), b = side(s.B, s.A);
+            mma = mma_pays(a, b, kext) && rest == 1 && s.A.limit < (int64_t(1) << 30) && s.B.limit < (int64_t(1) << 30);   // (byte offsets of 32 bits)
+            const bool out_a = contiguous >= 0 && s.A.coef[contiguous] != 0 && s.B.coef[contiguous] == 0;
+            const bool out_b = contiguous >= 0 && s.B.coef[contiguous] != 0 && s.A.coef[contiguous] == 0;
+            if (mma && ((out_b && b >= 128) || (!out_a && b > a) || (out_a && a < 128 && b > a))) { std::swap(s.A, s.B); turned = true; }
+        }
+    }
     std::vector<Digit> dm, dn, dk, dz;
     for (int v = 0; v < nv; ++v) {
         if (s.vars[v].ext == 1) continue;                  // a single value: nothing to index
@@ -76,7 +110,7 @@ bool emit_program(const System &s0, float scale, int accumulate, bool allow_spli
     // fastest digit last: rows by their stride in the operand, columns by their stride in the output
     std::stable_sort(dm.begin(), dm.end(), [&](const Digit &x, const Digit &y) { return mag(x.sA) > mag(y.sA); });
     std::stable_sort(dn.begin(), dn.end(), [&](const Digit &x, const Digit &y) {
-        return mag(x.sO) != mag(y.sO) ? mag(x.sO) > mag(y.sO) : mag(x.sB) > mag(y.sB); });
+        return !mma && mag(x.sO) != mag(y.sO) ? mag(x.sO) > mag(y.sO) : mag(x.sB) > mag(y.sB); });
     std::stable_sort(dk.begin(), dk.end(), [&](const Digit &x, const Digit &y) {
         return std::min(mag(x.sA), mag(x.sB)) > std::min(mag(y.sA), mag(y.sB)); });
     // guards: at most one per operand; a guard belongs to an operand whose groups hold all its variables
@@ -137,7 +171,7 @@ bool emit_program(const System &s0, float scale, int accumulate, bool allow_spli
     const bool one_column = P.N.extent == 1 && P.Z.extent == 1 && P.K.n_digits <= 1 && !P.guardA && !P.guardB && P.M.extent >= 1024;
     const bool col_sums = one_column && P.M.n_digits == 1 && P.M.sA[0] == 1 && P.K.n_digits == 1 && std::llabs((int64_t)P.K.sA[0]) != 1;
     const bool row_sums = one_column && !col_sums;
-    if (!one_column && fill < (strict_fill ? 0.15 : 0.05)) return false;    // mostly empty tiles: the interpreter's schedules do better
+    if (!one_column && !mma && fill < (strict_fill ? 0.15 : 0.05)) return false;    // mostly empty tiles: the interpreter's schedules do better
     // gather modes: the one whose warp-wide copy touches fewer 128-byte lines (lanes along the row index:
     // 32 rows at one summation index; lanes along the summation index: 2 rows x 16 indices)
     auto mode_of = [&](const std::vector<Digit> &rows, bool second, const AGuard *gd, int64_t base) {
@@ -199,6 +233,46 @@ bool emit_program(const System &s0, float scale, int accumulate, bool allow_spli
             if (eff > best + 0.02) { best = eff; split = s; }
         }
     }
+    if (mma && !one_column) {
+        // ---- tensor-core tiles ----
+        P.shape = 7;
+        auto vectors = [&](const std::vector<Digit> &fast, const std::vector<Digit> &other, bool second, const AGuard *gd, int64_t base) {
+            // octets of the group are 32 consecutive, 16-byte aligned bytes: the run of consecutive elements along its
+            // fastest digits is a multiple of eight long and everything else moves by multiples of four
+            auto st = [&](const Digit &d) { return second ? d.sB : d.sA; };
+            int64_t run = 1;
+            int d = (int)fast.size() - 1;
+            for (; d >= 0 && st(fast[d]) == run; --d) { if (gd && gd->coef[fast[d].var]) return false; run *= fast[d].ext; }
+            if (run % 8 || base % 4) return false;
+            for (; d >= 0; --d) if (st(fast[d]) % 4) return false;
+            for (const std::vector<Digit> *g : {&other, (const std::vector<Digit> *)&dz}) for (const Digit &e : *g) if (st(e) % 4) return false;
+            return true;
+        };
+        auto mma_mode = [&](const std::vector<Digit> &rows, bool second, const AGuard *gd, int64_t base, int legacy) {
+            if (vectors(dk, rows, second, gd, base)) return (int)TM_KVEC;
+            if (second && vectors(rows, dk, second, gd, base)) return (int)TM_RVEC;
+            return legacy == TG_K ? (int)TM_K : (int)TM_ROW;
+        };
+        P.modeA = mma_mode(dm, false, ga, s.A.base, P.modeA);
+        P.modeB = mma_mode(dn, true, gb, s.B.base, P.modeB);
+        P.out_vec4 = 0;
+        const int64_t bn = P.N.extent <= 64 ? 64 : 128;
+        const int64_t tiles = ((P.M.extent + 127) / 128) * ((P.N.extent + bn - 1) / bn) * P.Z.extent;
+        const int64_t stages = (P.K.extent + TADC_KS - 1) / TADC_KS, cells = (int64_t)P.M.extent * P.N.extent * P.Z.extent;
+        // blocks run one per SM: the split with the least estimated time (us): stages of a block, its fixed part, the planes
+        split = 1;
+        double best = 0;
+        for (int64_t sp = 1; sp <= std::min<int64_t>(stages, 64); ++sp) {
+            if (sp > 1 && (!allow_split || sp * cells > (int64_t(1) << 24))) break;
+            const int64_t per = (stages + sp - 1) / sp, real = (stages + per - 1) / per;
+            const double waves = std::ceil((double)(tiles * real) / 148.0);
+            const double t = waves * (1.2 * (double)per + 2.5) + (real > 1 ? 4.0 + (double)(real + 1) * (double)cells * 4e-6 / 3.0 : 0.0);
+            if (sp == 1 || t < best * 0.97) { best = t; split = sp; }
+        }
+        const int64_t per = ((stages + split - 1) / split) * TADC_KS;
+        P.kchunk = fit(std::max<int64_t>(per, TADC_KS));
+        P.ksplit = fit(std::max<int64_t>(1, (P.K.extent + P.kchunk - 1) / P.kchunk));
+    }
     if (row_sums) { P.shape = 4; split = 1; }
     if (col_sums) {
         // a thread per row, blocks of 256 rows: the summation is split to fill the GPU
@@ -213,7 +287,7 @@ bool emit_program(const System &s0, float scale, int accumulate, bool allow_spli
     }
     // the streaming kernel for narrow contractions (see tad_skinny_kernel): one digit per group, B rows of consecutive,
     // 16-byte aligned elements, A consecutive along k (128-bit loads) or along m
-    if (!one_column && s.B.ptr >= 0 && !ga && !gb && P.Z.extent == 1 && P.N.extent >= 2 && P.N.extent <= 36 && P.M.n_digits == 1 &&
+    if (P.shape != 7 && !one_column && s.B.ptr >= 0 && !ga && !gb && P.Z.extent == 1 && P.N.extent >= 2 && P.N.extent <= 36 && P.M.n_digits == 1 &&
         P.K.n_digits == 1 && P.N.n_digits == 1 && P.N.sB[0] == 1 && P.M.extent >= 512 && P.K.extent >= 512) {
         const int64_t sBk = P.K.sB[0], sAk = P.K.sA[0], sAm = P.M.sA[0];
         const bool b_ok = sBk > 0 && sBk % 4 == 0 && s.B.base % 4 == 0 && (P.N.extent % 4 == 0 || sBk >= (P.N.extent + 3) / 4 * 4);
@@ -234,7 +308,7 @@ bool emit_program(const System &s0, float scale, int accumulate, bool allow_spli
             P.ksplit = fit((P.K.extent + per128 - 1) / per128);
         }
     }
-    if (P.shape != 5 && P.shape != 6) {
+    if (P.shape != 5 && P.shape != 6 && P.shape != 7) {
     split = std::max<int64_t>(1, split);
     const int64_t per = ((kstages + split - 1) / split) * TADC_BK;
     P.kchunk = fit(std::max<int64_t>(per, TADC_BK));
@@ -252,8 +326,8 @@ bool emit_program(const System &s0, float scale, int accumulate, bool allow_spli
         return t + "\n";
     };
     std::snprintf(line, sizeof line, "; contraction %d x %d x %d (batch %d): A=ptr %d mode %d guard %d, B=ptr %d mode %d guard %d, tile %s, ksplit %d x %d, vec4 %d, scale %g, accumulate %d\n",
-                  P.M.extent, P.N.extent, P.K.extent, P.Z.extent, P.ptrA, P.modeA, P.guardA, P.ptrB, P.modeB, P.guardB,
-                  P.shape == 6 ? "column sums" : P.shape == 5 ? "streamed" : P.shape == 4 ? "row sums" : P.shape == 1 ? "128x32" : P.shape == 3 ? "128x36" : P.shape == 2 ? "128x64" : "128x128", P.ksplit, P.kchunk, P.out_vec4, (double)P.scale, P.accumulate);
+                  turned ? P.N.extent : P.M.extent, turned ? P.M.extent : P.N.extent, P.K.extent, P.Z.extent, P.ptrA, P.modeA, P.guardA, P.ptrB, P.modeB, P.guardB,
+                  P.shape == 7 ? (P.N.extent <= 64 ? "tensor 128x64" : "tensor 128x128") : P.shape == 6 ? "column sums" : P.shape == 5 ? "streamed" : P.shape == 4 ? "row sums" : P.shape == 1 ? "128x32" : P.shape == 3 ? "128x36" : P.shape == 2 ? "128x64" : "128x128", P.ksplit, P.kchunk, P.out_vec4, (double)P.scale, P.accumulate);
     text += line;
     text += group_text("m", P.M) + group_text("n", P.N) + group_text("k", P.K) + group_text("z", P.Z);
     return true;

@@ -145,8 +145,13 @@ tad_status launch_contractions(const tad::Kernel &k, const TadpPointers &ptrs, c
         if (P.ksplit > 1 && !ptrs.part) { tad::set_error("internal: partial-sum buffer missing"); return TAD_ERR_WORKSPACE; }
         // 16-byte copies and stores need 16-byte aligned tensors: fall back to 4-byte accesses otherwise
         auto misaligned = [](const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) != 0; };
-        if (P.modeA == TG_ROW16 && misaligned(ptrs.in[P.ptrA])) P.modeA = TG_ROW;
-        if (P.ptrB >= 0 && P.modeB == TG_ROW16 && misaligned(ptrs.in[P.ptrB])) P.modeB = TG_ROW;
+        if (P.shape == 7) {
+            if (P.modeA == TM_KVEC && misaligned(ptrs.in[P.ptrA])) P.modeA = TM_K;
+            if (P.modeB == TM_KVEC && misaligned(ptrs.in[P.ptrB])) P.modeB = TM_K;
+            if (P.modeB == TM_RVEC && misaligned(ptrs.in[P.ptrB])) P.modeB = TM_ROW;
+        }
+        else if (P.modeA == TG_ROW16 && misaligned(ptrs.in[P.ptrA])) P.modeA = TG_ROW;
+        if (P.shape != 7 && P.ptrB >= 0 && P.modeB == TG_ROW16 && misaligned(ptrs.in[P.ptrB])) P.modeB = TG_ROW;
         if (P.out_vec4 && misaligned(ptrs.out)) P.out_vec4 = 0;
         // the streaming kernel copies B in 16-byte pieces
         if (P.shape == 5 && misaligned(ptrs.in[P.ptrB])) P.shape = 3;

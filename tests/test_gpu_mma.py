@@ -1,0 +1,79 @@
+"""Tensor-core contraction kernel: tile edges, every gather mode, splits, guards, non-finite operands.
+
+Tolerance per output, relative to the sum of |terms|: the products left out by the three-way bf16 split 2^-23, four
+truncated accumulator steps per stage of 64 summation indices (each below 2^-23 of a partial sum, the steps of the small
+products below one more together), one rounding 2^-24 per stage for the running sum and per plane: (8 + stages) 2^-23
+bounds them all."""
+import math
+
+import pytest
+import torch
+
+from workloads import configs as W
+
+pytestmark = pytest.mark.gpu
+
+from tests.gpu_util import GpuRun  # noqa: E402
+
+
+def _close(got, want, scale, n_terms, what):
+    tol = (8 + math.ceil(n_terms / 64)) * 2.0 ** -23 * scale + 1e-30
+    err = (torch.from_numpy(got).double() - want).abs()
+    assert bool((err <= tol).all()), f"{what}: worst {float((err / tol).max()):.2f} of the tolerance"
+
+
+# (rows, summed, columns): tile and stage edges, remainders of the 16-wide steps, a split summation, wide and narrow sides
+SIZES = [(128, 64, 128), (127, 63, 129), (129, 65, 127), (257, 17, 64), (64, 130, 257), (8, 2050, 300), (300, 333, 65),
+         (513, 16, 700), (160, 5000, 136)]
+
+
+@pytest.mark.parametrize("transposed", [False, True])
+@pytest.mark.parametrize("ni,nk,nj", SIZES)
+def test_matrix_products(ni, nk, nj, transposed):
+    e = W.ex_matmul_t(ni, nj, nk) if transposed else W.ex_matmul(ni, nk, nj)
+    args, df = W.make_inputs(e, ("normal", 0, 1), seed=ni + nk)
+    run = GpuRun(e, args, df)
+    f = run.forward()
+    dx, dy = run.backward()
+    x, y, d = args[0].double(), args[1].double(), df.double()
+    y = y.T if transposed else y                                # summed x columns
+    _close(f, x @ y, x.abs() @ y.abs(), nk, "forward")
+    _close(dx, d @ y.T, d.abs() @ y.T.abs(), nj, "dx")
+    want, scale = x.T @ d, x.T.abs() @ d.abs()
+    _close(dy, want.T if transposed else want, scale.T if transposed else scale, ni, "dy")
+
+
+@pytest.mark.parametrize("nb,nc,no,nt,nu", [(2, 64, 72, 130, 5), (3, 13, 65, 257, 3), (1, 20, 128, 64, 4)])
+def test_strided_convolution(nb, nc, no, nt, nu):
+    """Guards, several digits per group and strided stores (the residue classes of dx)."""
+    e = W.conv1d(nb, nc, no, nt, nu)
+    args, df = W.make_inputs(e, ("normal", 0, 1), seed=nt)
+    run = GpuRun(e, args, df)
+    f = run.forward()
+    dx, dw = run.backward()
+
+    def conv(x, w, d):
+        x.requires_grad_(True), w.requires_grad_(True)
+        out = torch.nn.functional.conv1d(x, w, stride=2)[:, :, :nt]
+        return (out.detach(),) + torch.autograd.grad(out, (x, w), d)
+    want = conv(args[0].double(), args[1].double(), df.double())
+    scale = conv(args[0].double().abs(), args[1].double().abs(), df.double().abs())
+    for got, w, s, n, what in zip((f, dx, dw), want, scale, (nc * nu, no * nu, nb * nt), ("forward", "dx", "dw")):
+        _close(got, w, s, n, what)
+
+
+def test_non_finite_operands():
+    """Infinities and NaNs of the operands, and values beyond the bf16 range, give what the definition gives."""
+    e = W.ex_matmul(130, 70, 140)
+    args, df = W.make_inputs(e, ("normal", 0, 1), seed=3)
+    x, y = args
+    y[y.abs() < 1e-3] = 0.5
+    x[3, 5], x[40, 69], x[129, 0], x[77, 7] = math.inf, -math.inf, math.nan, 3.4028234e38
+    y[7] = 0.25
+    f = torch.from_numpy(GpuRun(e, args, df).forward())
+    assert torch.equal(f[3], math.inf * torch.sign(y[5]))
+    assert torch.equal(f[40], -math.inf * torch.sign(y[69]))
+    assert bool(f[129].isnan().all())
+    want = x.double() @ y.double()
+    rows = [r for r in range(130) if r not in (3, 40, 129)]
+    assert bool(((f.double() - want)[rows].abs() <= 1e-5 * (x.double().abs() @ y.double().abs())[rows]).all())
