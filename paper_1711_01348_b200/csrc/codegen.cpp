@@ -720,6 +720,227 @@ bool try_elementwise(Gen &g, Kernel &k, const Emitter &em, const std::vector<Tad
     return true;
 }
 
+// temporaries: shared values and values hoisted out of the loop that consumes them; returns their number
+int assign_temporaries(Gen &g, int root, int scale)
+{
+    std::vector<bool> hoisted(g.inst.size(), false);
+    auto effective_level = [&](int i) { return i == root ? g.kappa : g.inst[i].zlevel; };
+    for (int i = 0; i < (int)g.inst.size(); ++i) {
+        const Inst &in = g.inst[i];
+        if (!in.uses) continue;
+        for (int c : {in.a, in.b}) {
+            if (c < 0 || g.inst[c].op == I_CONST) continue;
+            const Inst &ch = g.inst[c];
+            if (in.op == I_SUM) { if (ch.home_sum != i) hoisted[c] = true; }   // a sum's body is consumed inside its loop
+            else if (ch.home_sum != in.home_sum) hoisted[c] = true;
+            else if (ch.home_sum < 0 && ch.zlevel != effective_level(i)) hoisted[c] = true;
+        }
+    }
+    int n_temps = 0;
+    for (int i = 0; i < (int)g.inst.size(); ++i) {
+        Inst &in = g.inst[i];
+        in.temp = -1;
+        if (!in.uses || in.op == I_CONST || i == root || i == scale) continue;
+        if (in.uses > 1 || hoisted[i]) {
+            if (n_temps >= TADP_NUM_TEMPS + TADP_MAX_SPILL) throw Unsupported("too many temporaries");
+            in.temp = n_temps++;
+        }
+    }
+    return n_temps;
+}
+
+// A kernel without guards whose loops have fixed ranges and whose whole index space is small becomes a point program
+// (point.h): the same stack program with one handler per operation, the terms of an output spread over lanes.
+// Up to 2^22 points the kernel was faster than every vector shape of the interpreter in every part measured (us, interpreter
+// -> points): intro 64 x 64 x 5 db 110 -> 12, 203 x 157 x 7 db 366 -> 12, da 23 -> 12, forward 26 -> 19; 700 x 700 x 8
+// (2^21.9) forward 44 -> 31, db 136 -> 41; all elementary functions over 200003 outputs: forward 79 -> 36, dv 131 -> 80.
+// Plain element-wise programs (no sums, no temporaries) have the element-wise kernel, which is as fast from 2^16 outputs on.
+constexpr double POINT_SPACE = double(1 << 22), POINT_PLAIN = double(1 << 16);
+
+bool try_points(Gen &g, Kernel &k, int root, int scale, bool allow_split, const std::vector<std::vector<TadpRow>> &lower,
+                const std::vector<std::vector<TadpRow>> &upper, const std::vector<TadpRow> &guards)
+{
+    if (g.p.opt.debug_bounds || root < 0 || !guards.empty()) return false;
+    TadpProgram &prog = k.prog;
+    const int nv = (int)g.vars.size();
+    std::vector<int64_t> lo(nv, 0), ext(nv, 1);
+    std::vector<int> zv;                                     // variables flattened into the term index
+    for (int v = 0; v < g.n_outer; ++v) { lo[v] = prog.outer_lo[v]; ext[v] = std::max(1, prog.outer_ext[v]); if (prog.outer_ext[v] < 1) return false; }
+    for (int l = 0; l < g.kappa; ++l) {
+        int64_t a = INT64_MIN, b = INT64_MAX;
+        for (const std::vector<TadpRow> *rows : {&lower[l], &upper[l]})
+            for (const TadpRow &r : *rows) {
+                for (int v = 0; v < TADP_MAX_VARS; ++v) if (r.coef[v]) return false;
+                if (rows == &lower[l]) a = std::max(a, ceil_div(r.c0, r.den)); else b = std::min(b, floor_div(r.c0, r.den));
+            }
+        if (a == INT64_MIN || b == INT64_MAX || b < a) return false;
+        const int v = g.n_outer + g.zorder[l];
+        lo[v] = a; ext[v] = b - a + 1;
+        zv.push_back(v);
+    }
+    // ---- the program: once per output, per term, on the sum ----
+    g.unroll_var = -1;
+    const int n_temps = assign_temporaries(g, root, scale);
+    Emitter em(g);
+    int body = 0, tail = 0;
+    em.temps_of_level(0);
+    body = (int)em.code.size();
+    for (int l = 0; l < g.kappa; ++l) em.temps_of_level(l + 1);
+    // a term that is a sum with a constant range: its summands are terms
+    int top = root;
+    while (g.inst[top].op == I_SUM && g.inst[top].temp < 0 && (int)zv.size() < TADQ_MAX_VARS) {
+        const Inst &in = g.inst[top];
+        if (in.hi < in.lo) return false;
+        lo[in.var] = in.lo; ext[in.var] = in.hi - in.lo + 1;
+        zv.push_back(in.var);
+        em.temps_of_sum(top);
+        top = in.a;
+    }
+    if (g.inst[top].op == I_MUL && g.inst[top].temp < 0) { em.expr(g.inst[top].a); em.expr(g.inst[top].b); em.emit(P_MACC, 0, 0, 0, -2); }
+    else { em.expr(top); em.emit(P_ACC, 0, 0, 0, -1); }
+    tail = (int)em.code.size();
+    if (scale >= 0) { em.expr(scale); em.emit(P_SCALE, 0, 0, 0, -1); }
+    const int n = (int)em.code.size();
+    if (em.depth != 0 || n > TADQ_MAX_STEPS || (int)g.loads.size() > TADQ_MAX_LOADS || g.n_outer + (int)zv.size() > TADQ_MAX_VARS) return false;
+    if (em.max_depth + n_temps > TADQ_MAX_SLOTS) return false;
+    // ---- the size of the index space, sums inside the term included ----
+    std::vector<int> sv;
+    double points = 1, terms = 1, inner = 1;
+    for (const TadpLoop &L : em.loops) {
+        if (std::find(sv.begin(), sv.end(), L.var) != sv.end()) return false;
+        sv.push_back(L.var);
+        lo[L.var] = L.const_lo; ext[L.var] = std::max<int64_t>(1, (int64_t)L.const_hi - L.const_lo + 1);
+        inner *= (double)ext[L.var];
+    }
+    if (sv.size() > TADQ_MAX_SUMS) return false;
+    for (int v = 0; v < g.n_outer; ++v) points *= (double)ext[v];
+    for (int v : zv) terms *= (double)ext[v];
+    if (points * terms * inner > POINT_SPACE) return false;
+    // plain element-wise programs have a kernel of their own, which a few thousand outputs do not fill
+    if (g.kappa == 0 && zv.empty() && sv.empty() && n_temps == 0 && points > POINT_PLAIN) return false;
+    // every offset the kernel can form must lie inside its tensor
+    auto inside = [&](const int32_t *coef, int n_coef, int64_t base, int64_t limit_) {
+        int64_t mn = base, mx = base;
+        for (int v = 0; v < n_coef; ++v) {
+            if (!coef[v]) continue;
+            const int64_t a = coef[v] * lo[v], b = coef[v] * (lo[v] + ext[v] - 1);
+            mn += std::min(a, b); mx += std::max(a, b);
+        }
+        return mn >= 0 && mx < limit_;
+    };
+    for (const TadpLoad &L : g.loads) if (!inside(L.coef, nv, L.base, L.limit)) return false;
+    if (!inside(prog.out_coef, g.n_outer, prog.out_base, prog.out_limit)) return false;
+    // ---- lanes: along the variable that makes the largest tensor consecutive, else along the output's own ----
+    const TadpLoad *big = nullptr;
+    for (const TadpLoad &L : g.loads) if (!big || L.limit > big->limit) big = &L;
+    std::vector<int> ov;
+    for (int v = 0; v < g.n_outer; ++v) ov.push_back(v);
+    auto fastest_last = [&](std::vector<int> &vs, auto &&better) {
+        if (vs.empty()) return;
+        size_t at = 0;
+        for (size_t i = 1; i < vs.size(); ++i) if (better(vs[i], vs[at])) at = i;
+        std::rotate(vs.begin() + at, vs.begin() + at + 1, vs.end());
+    };
+    auto unit_of_big = [&](int v) { return big && std::abs(big->coef[v]) == 1 && ext[v] > 1; };
+    auto out_step = [&](int v) { return prog.out_coef[v] ? std::abs(prog.out_coef[v]) : INT32_MAX; };
+    fastest_last(ov, [&](int a, int b) { return unit_of_big(a) != unit_of_big(b) ? unit_of_big(a) : out_step(a) < out_step(b); });
+    fastest_last(zv, [&](int a, int b) { return unit_of_big(a) != unit_of_big(b) ? unit_of_big(a) : ext[a] > ext[b]; });
+    TadqProgram Q{};
+    Q.n_out = (int32_t)ov.size(); Q.n_z = (int32_t)zv.size();
+    Q.points = to_i32((int64_t)points); Q.terms = to_i32((int64_t)terms);
+    std::vector<int> at(nv, -1);                              // variable -> position in the program
+    int pos = 0;
+    for (const std::vector<int> *vs : {&ov, &zv})
+        for (int v : *vs) {
+            at[v] = pos;
+            Q.lo[pos] = to_i32(lo[v]); Q.ext[pos] = to_i32(ext[v]);
+            const uint64_t d = (uint64_t)ext[v];
+            int sh = 0; while ((uint64_t(1) << sh) < d) ++sh;
+            Q.div_mul[pos] = (uint32_t)(((uint64_t(1) << (31 + sh)) / d) + 1); Q.div_shift[pos] = 31 + sh;
+            if (v < g.n_outer) Q.out_coef[pos] = prog.out_coef[v];
+            ++pos;
+        }
+    for (size_t i = 0; i < g.loads.size(); ++i) {
+        const TadpLoad &L = g.loads[i];
+        Q.loads[i].ptr = L.ptr; Q.loads[i].base = L.base;
+        for (int v = 0; v < nv; ++v) {
+            if (!L.coef[v]) continue;
+            const auto it = std::find(sv.begin(), sv.end(), v);
+            if (it != sv.end()) Q.loads[i].scoef[it - sv.begin()] = L.coef[v];
+            else if (at[v] >= 0) Q.loads[i].coef[at[v]] = L.coef[v];
+            else return false;
+        }
+    }
+    Q.n_sums = (int32_t)sv.size();
+    for (size_t i = 0; i < sv.size(); ++i) { Q.s_lo[i] = to_i32(lo[sv[i]]); Q.s_hi[i] = to_i32(lo[sv[i]] + ext[sv[i]] - 1); }
+    for (const TadpLoop &L : em.loops) if (L.const_hi < L.const_lo) return false;
+    auto slot = [&](int s) { return (uint8_t)(s >= 0 ? s : TADQ_NONE); };
+    auto temp = [&](int t) { return (uint8_t)(em.max_depth + t); };
+    for (int w = 0; w < n; ++w) {
+        const TadpInsn &in = em.code[w];
+        const int d = em.depth_at[w];                         // values on the stack before this word
+        TadqStep st{};
+        st.imm = in.imm; st.s = TADQ_NONE;
+        switch (in.handler >> 3) {
+        case P_CONST: st.op = Q_CONST; st.s = slot(d - 1); break;
+        case P_ZERO: st.op = Q_CONST; st.imm = 0; st.s = slot(d - 1); break;
+        case P_LOAD: st.op = Q_LOAD; st.a = in.a; st.s = slot(d - 1); break;
+        case P_LDT: st.op = Q_SLOT; st.a = temp(in.a); st.s = slot(d - 1); break;
+        case P_NEG: st.op = Q_NEG; break;
+        case P_SQR: st.op = Q_SQR; break;
+        case P_CUBE: st.op = Q_CUBE; break;
+        case P_MULC: st.op = Q_MULC; break;
+        case P_ADDC: st.op = Q_ADDC; break;
+        case P_LDADD: st.op = Q_LDADD; st.a = in.a; break;
+        case P_LDMUL: st.op = Q_LDMUL; st.a = in.a; break;
+        case P_LDADDSQ: st.op = Q_LDADDSQ; st.a = in.a; break;
+        case P_FN: st.op = Q_FN; st.b = in.b; break;
+        case P_ADD: case P_SUMADD: st.op = Q_ADD; st.s = slot(d - 2); break;
+        case P_SUB: st.op = Q_SUB; st.s = slot(d - 2); break;
+        case P_MUL: st.op = Q_MUL; st.s = slot(d - 2); break;
+        case P_DIV: st.op = Q_DIV; st.s = slot(d - 2); break;
+        case P_FMAT: st.op = Q_FMA; st.s = slot(d - 2); st.a = temp(in.a); break;
+        case P_FMA: st.op = Q_FMA; st.s = slot(d - 3); st.a = slot(d - 2); break;
+        case P_STT: st.op = Q_STORE; st.a = temp(in.a); st.s = slot(d - 2); break;
+        case P_ACC: if (d != 1) return false; st.op = Q_ACC; break;
+        case P_MACC: if (d != 2) return false; st.op = Q_MACC; st.s = slot(0); break;
+        case P_SCALE: if (d != 1) return false; st.op = Q_SCALE; break;
+        case P_SLOOP: st.op = Q_LOOP; st.a = (uint8_t)(std::find(sv.begin(), sv.end(), em.loops[in.a].var) - sv.begin()); break;
+        case P_SUMEND: st.op = Q_SUMNEXT; st.s = slot(d - 2); st.a = (uint8_t)(std::find(sv.begin(), sv.end(), em.loops[in.a].var) - sv.begin()); break;
+        case P_SEND: st.op = Q_NEXT; st.a = (uint8_t)(std::find(sv.begin(), sv.end(), em.loops[in.a].var) - sv.begin()); break;
+        default: return false;
+        }
+        Q.steps[w] = st;
+    }
+    Q.body = body; Q.tail = tail; Q.n_steps = n;
+    Q.n_slots = std::max(1, em.max_depth + n_temps);
+    Q.out_base = prog.out_base; Q.accumulate = prog.accumulate;
+    // ---- schedule: lanes per output until the GPU has a few warps per scheduler, shares where even that is too few blocks ----
+    Q.lt = 1; Q.zsplit = 1; Q.along_terms = 0; Q.unroll = 1;
+    const bool sums = g.kappa >= 1 || Q.n_z > 0;
+    if (sums) {
+        Q.along_terms = !zv.empty() && unit_of_big(zv.back()) && !(!ov.empty() && unit_of_big(ov.back())) ? 1 : 0;
+        Q.unroll = terms >= 4 ? 4 : 1;
+        if (Q.along_terms) while (Q.lt < 32 && Q.lt < terms) Q.lt *= 2;
+        while (Q.lt < 256 && points * Q.lt < 148.0 * 512.0 && Q.lt * Q.unroll < terms) Q.lt *= 2;
+        if (Q.lt == 1 && terms == 1) Q.lt = 2;                // (a single term still goes through the summing path)
+        int64_t cells = 1;
+        for (int v = g.n_outer - 1; v >= 0; --v) { prog.part_coef[v] = to_i32(cells); if (at[v] >= 0) Q.part_coef[at[v]] = to_i32(cells); cells = mul_ck(cells, ext[v]); }
+        const double blocks = std::ceil(points * Q.lt / 256.0), batches = terms / ((double)Q.lt * Q.unroll);
+        if (allow_split && g.kappa >= 1 && blocks < 148 && batches >= 8 && cells <= (1 << 20))
+            Q.zsplit = (int32_t)std::max(1.0, std::min({128.0, std::floor(296.0 / blocks), std::floor(batches / 4)}));
+        Q.part_limit = to_i32(cells);
+    } else if (points >= 131072) Q.unroll = 4;
+    prog.zsplit = Q.zsplit; prog.part_limit = Q.part_limit; prog.n_outer = g.n_outer; prog.write_only_live = 0;
+    k.point = {Q};
+    k.vec = 0; k.vec_u = 0;
+    char line[200];
+    std::snprintf(line, sizeof line, "; point program: %d outputs x %d terms, %d steps, %d slots, %d points per thread, %d lanes per output%s, %d shares\n", Q.points,
+                  Q.terms, Q.n_steps, Q.n_slots, Q.unroll, Q.lt, Q.along_terms ? " (consecutive)" : "", Q.zsplit);
+    k.listing = line + em.listing();
+    return true;
+}
+
 // shared tail: choose temps, emit, fill the program
 void emit_kernel(Gen &g, Kernel &k, int root, const std::vector<std::vector<TadpRow>> &lower,
                  const std::vector<std::vector<TadpRow>> &upper, const std::vector<TadpRow> &guards, bool allow_split = false,
@@ -767,6 +988,11 @@ void emit_kernel(Gen &g, Kernel &k, int root, const std::vector<std::vector<Tadp
     if (may_factor && try_factoring(g, k, root, scale, allow_split, lower, upper, guards)) return;
     // sums of products of index expressions (most derivative terms once the functions are tabulated)
     if (try_line(g, k, root, scale, allow_split, lower, upper, guards)) return;
+    // small index spaces
+    try {
+        if (try_points(g, k, root, scale, allow_split, lower, upper, guards)) return;
+    } catch (const Unsupported &) {                           // too deep or too many temporaries for it
+    }
     // a short loop whose range shifts from lane to lane will be walked relative to every element's own
     // start, which needs the elements of a thread to lie along the lane variable only
     bool relative_candidate = false;
@@ -786,30 +1012,7 @@ void emit_kernel(Gen &g, Kernel &k, int root, const std::vector<std::vector<Tadp
                 for (int x = 0; x < (int)g.vars.size(); ++x) if (r.coef[x]) lane_bound_vars |= 1u << x;
     }
     choose_element_variable(g, !relative_candidate, lane_bound_vars);
-    // temporaries: shared values and values hoisted out of the loop that consumes them
-    std::vector<bool> hoisted(g.inst.size(), false);
-    auto effective_level = [&](int i) { return i == root ? g.kappa : g.inst[i].zlevel; };
-    for (int i = 0; i < (int)g.inst.size(); ++i) {
-        const Inst &in = g.inst[i];
-        if (!in.uses) continue;
-        for (int c : {in.a, in.b}) {
-            if (c < 0 || g.inst[c].op == I_CONST) continue;
-            const Inst &ch = g.inst[c];
-            if (in.op == I_SUM) { if (ch.home_sum != i) hoisted[c] = true; }   // a sum's body is consumed inside its loop
-            else if (ch.home_sum != in.home_sum) hoisted[c] = true;
-            else if (ch.home_sum < 0 && ch.zlevel != effective_level(i)) hoisted[c] = true;
-        }
-    }
-    int n_temps = 0;
-    for (int i = 0; i < (int)g.inst.size(); ++i) {
-        Inst &in = g.inst[i];
-        in.temp = -1;
-        if (!in.uses || in.op == I_CONST || i == root || i == scale) continue;
-        if (in.uses > 1 || hoisted[i]) {
-            if (n_temps >= TADP_NUM_TEMPS + TADP_MAX_SPILL) throw Unsupported("too many temporaries");
-            in.temp = n_temps++;
-        }
-    }
+    const int n_temps = assign_temporaries(g, root, scale);
     Emitter em(g);
     em.temps_of_level(0);
     std::vector<int> zbegin(g.kappa);

@@ -11,6 +11,7 @@
 #include "contract.h"
 #include "ew.h"
 #include "line.h"
+#include "point.h"
 
 namespace tad {
 
@@ -73,6 +74,7 @@ struct Kernel {
     std::vector<TadcProgram> contract;   // non-empty: the kernel is a contraction, run by the tile kernel (one launch per
                                          // program) instead of the interpreter
     std::vector<TadeProgram> ew;         // non-empty: a kernel without loops, run by the element-wise kernel
+    std::vector<TadqProgram> point;      // non-empty: a general term over a small index space, run by the point kernel
     std::vector<TadlProgram> line;       // non-empty: sums of products of index expressions, run by the line-sum kernel
     // Expression optimisation: tensors in the auxiliary area of the workspace and the kernels that fill them
     // (launched in this order before the kernel itself, each writing the tensor out_aux)

@@ -22,6 +22,7 @@ TAD_VM_SHAPES(TAD_DECLARE_VM)
 bool tad_launch_vm_16_1_rich(const TadpProgram &prog, const TadpPointers &ptrs, bool debug, unsigned items, unsigned sms, cudaStream_t stream);
 cudaError_t tad_launch_contract(const TadcProgram &P, const TadpPointers &ptrs, unsigned sms, cudaStream_t stream);
 cudaError_t tad_launch_ew(const TadeProgram &P, const TadpPointers &ptrs, unsigned sms, cudaStream_t stream);
+cudaError_t tad_launch_points(const TadqProgram &P, const TadpPointers &ptrs, cudaStream_t stream);
 cudaError_t tad_launch_line(const TadlProgram &P, const TadpPointers &ptrs, unsigned sms, cudaStream_t stream);
 
 namespace {
@@ -191,6 +192,11 @@ bool reads_slot(const tad::Kernel &k, int slot)
         for (int i = 0; i < k.ew[0].n_loads; ++i) if (k.ew[0].loads[i].ptr == slot) return true;
         return false;
     }
+    if (!k.point.empty()) {
+        for (const TadqStep *st = k.point[0].steps; st < k.point[0].steps + k.point[0].n_steps; ++st)
+            if ((st->op == Q_LOAD || st->op == Q_LDADD || st->op == Q_LDMUL || st->op == Q_LDADDSQ) && k.point[0].loads[st->a].ptr == slot) return true;
+        return false;
+    }
     if (!k.line.empty()) {
         for (int i = 0; i < k.line[0].n_loads; ++i) if (k.line[0].loads[i].ptr == slot) return true;
         for (int i = 0; i < k.line[0].n_scale; ++i) if (k.line[0].scale[i].ptr == slot) return true;
@@ -259,17 +265,17 @@ tad_status launch(const tad::Kernel &k, TadpPointers ptrs, bool debug, cudaStrea
         if (e != cudaSuccess) { tad::set_error(std::string("element-wise launch failed: ") + cudaGetErrorString(e)); return TAD_ERR_CUDA; }
         return TAD_OK;
     }
-    if (!k.line.empty()) {
-        const TadlProgram &L = k.line[0];
-        if (L.zsplit > 1 && !ptrs.part) { tad::set_error("internal: partial-sum buffer missing"); return TAD_ERR_WORKSPACE; }
-        cudaError_t e = tad_launch_line(L, ptrs, (unsigned)sm_count(), stream);
-        if (e == cudaSuccess && L.zsplit > 1) {
+    if (!k.line.empty() || !k.point.empty()) {
+        const int shares = k.line.empty() ? k.point[0].zsplit : k.line[0].zsplit;
+        if (shares > 1 && !ptrs.part) { tad::set_error("internal: partial-sum buffer missing"); return TAD_ERR_WORKSPACE; }
+        cudaError_t e = k.line.empty() ? tad_launch_points(k.point[0], ptrs, stream) : tad_launch_line(k.line[0], ptrs, (unsigned)sm_count(), stream);
+        if (e == cudaSuccess && shares > 1) {
             const unsigned n = (unsigned)k.prog.part_limit;
             const unsigned rblocks = std::min((n + 31u) / 32u, (unsigned)sm_count() * 8u);
             launch_reduce_partials(k.prog, ptrs, rblocks, stream);
             e = cudaGetLastError();
         }
-        if (e != cudaSuccess) { tad::set_error(std::string("line-sum launch failed: ") + cudaGetErrorString(e)); return TAD_ERR_CUDA; }
+        if (e != cudaSuccess) { tad::set_error(std::string("line-sum or point launch failed: ") + cudaGetErrorString(e)); return TAD_ERR_CUDA; }
         return TAD_OK;
     }
     const int zsplit = k.prog.zsplit > 1 ? k.prog.zsplit : 1;
