@@ -16,7 +16,7 @@ CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libtad.so")
 SOURCES = ["intalg.cpp", "plan.cpp", "codegen.cpp", "contract_gen.cpp", "factor.cpp", "line_gen.cpp", "print.cpp", "api.cpp", "runtime.cu", "contract.cu", "mma.cu", "ew.cu", "line.cu", "point.cu"]
-HEADERS = ["intalg.h", "plan.h", "gen.h", "program.h", "contract.h", "contract.cuh", "ew.h", "line.h", "point.h", "vm.cuh", "vm_shapes.h", "vm_inst.cu",
+HEADERS = ["intalg.h", "plan.h", "gen.h", "program.h", "contract.h", "contract.cuh", "launch.h", "ew.h", "line.h", "point.h", "vm.cuh", "vm_shapes.h", "vm_inst.cu",
            os.path.join("..", "..", "include", "tad.h")]
 ARCH = ["-gencode", "arch=compute_100a,code=sm_100a"]
 

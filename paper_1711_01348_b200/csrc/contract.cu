@@ -9,6 +9,7 @@
 
 #include <algorithm>
 
+#include "launch.h"
 #include "contract.cuh"
 
 namespace {
@@ -130,6 +131,7 @@ template <int BM, int BN, int TM, int TN>
 __global__ void __launch_bounds__(Cfg<BM, BN, TM, TN>::NT, (TM * TN >= 64 ? 2 : Cfg<BM, BN, TM, TN>::NT <= 160 ? 4 : 3))
 tad_contract_kernel(const __grid_constant__ TadcProgram P, const __grid_constant__ TadpPointers ptrs, const unsigned tiles_m, const unsigned tiles_n)
 {
+    tad_wait_previous();
     using C = Cfg<BM, BN, TM, TN>;
     constexpr int NT = C::NT, LDA = C::LDA, LDB = C::LDB;
     constexpr int GM = TM / 4, GN = TN / 4;           // groups of four rows / columns per thread
@@ -383,6 +385,7 @@ tad_contract_kernel(const __grid_constant__ TadcProgram P, const __grid_constant
 __global__ void __launch_bounds__(256)
 tad_contract_reduce(const __grid_constant__ TadcProgram P, const __grid_constant__ TadpPointers ptrs)
 {
+    tad_wait_previous();
     const unsigned Mext = (unsigned)P.M.extent, Next = (unsigned)P.N.extent;
     const unsigned per_z = Mext * Next;
     const unsigned cells = per_z * (unsigned)P.Z.extent;
@@ -407,6 +410,7 @@ tad_contract_reduce(const __grid_constant__ TadcProgram P, const __grid_constant
 __global__ void __launch_bounds__(256)
 tad_rowsum_kernel(const __grid_constant__ TadcProgram P, const __grid_constant__ TadpPointers ptrs)
 {
+    tad_wait_previous();
     const unsigned lane = threadIdx.x & 31u;
     const unsigned warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, n_warps = (gridDim.x * blockDim.x) >> 5;
     const float *__restrict__ A = ptrs.in[P.ptrA];
@@ -484,6 +488,7 @@ constexpr int SK_KC = 128;         // summation indices per stage of B
 __global__ void __launch_bounds__(256, 2)
 tad_skinny_kernel(const __grid_constant__ TadcProgram P, const __grid_constant__ TadpPointers ptrs)
 {
+    tad_wait_previous();
     __shared__ __align__(16) float bs[2][SK_KC * SK_COLS];
     const unsigned tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
     const float *__restrict__ A = ptrs.in[P.ptrA];
@@ -639,6 +644,7 @@ tad_skinny_kernel(const __grid_constant__ TadcProgram P, const __grid_constant__
 __global__ void __launch_bounds__(256)
 tad_colsum_kernel(const __grid_constant__ TadcProgram P, const __grid_constant__ TadpPointers ptrs)
 {
+    tad_wait_previous();
     const unsigned m = blockIdx.x * 256u + threadIdx.x;
     const unsigned Mext = (unsigned)P.M.extent, K = (unsigned)P.K.extent;
     if (m >= Mext) return;
@@ -690,7 +696,7 @@ cudaError_t launch_shape(const TadcProgram &P, const TadpPointers &ptrs, cudaStr
     }
     const unsigned tiles_m = ((unsigned)P.M.extent + BM - 1) / BM, tiles_n = ((unsigned)P.N.extent + BN - 1) / BN;
     dim3 grid(tiles_m * tiles_n, (unsigned)std::max(1, P.ksplit), (unsigned)P.Z.extent);
-    kern<<<grid, C::NT, C::SMEM, stream>>>(P, ptrs, tiles_m, tiles_n);
+    tad_launch(kern, grid, C::NT, C::SMEM, stream, P, ptrs, tiles_m, tiles_n);
     return cudaGetLastError();
 }
 
@@ -705,23 +711,23 @@ cudaError_t tad_launch_contract(const TadcProgram &P, const TadpPointers &ptrs, 
     if (P.shape == 5) {
         const unsigned rows_per_block = P.modeA == TG_K ? 16u : 512u;
         dim3 grid(((unsigned)P.M.extent + rows_per_block - 1u) / rows_per_block, (unsigned)std::max(1, P.ksplit), 1u);
-        tad_skinny_kernel<<<grid, 256, 0, stream>>>(P, ptrs);
+        tad_launch(tad_skinny_kernel, grid, 256, 0, stream, P, ptrs);
         cudaError_t e = cudaGetLastError();
         if (e == cudaSuccess && P.ksplit > 1) {
             const unsigned long long cells = (unsigned long long)P.M.extent * P.N.extent;
             const unsigned blocks = (unsigned)std::min<unsigned long long>((cells + 255) / 256, (unsigned long long)sms * 8);
-            tad_contract_reduce<<<blocks, 256, 0, stream>>>(P, ptrs);
+            tad_launch(tad_contract_reduce, blocks, 256, 0, stream, P, ptrs);
             e = cudaGetLastError();
         }
         return e;
     }
     if (P.shape == 6) {
         dim3 grid(((unsigned)P.M.extent + 255u) / 256u, (unsigned)std::max(1, P.ksplit), 1u);
-        tad_colsum_kernel<<<grid, 256, 0, stream>>>(P, ptrs);
+        tad_launch(tad_colsum_kernel, grid, 256, 0, stream, P, ptrs);
         cudaError_t e = cudaGetLastError();
         if (e == cudaSuccess && P.ksplit > 1) {
             const unsigned blocks = (unsigned)std::min<unsigned long long>(((unsigned long long)P.M.extent + 255) / 256, (unsigned long long)sms * 8);
-            tad_contract_reduce<<<blocks, 256, 0, stream>>>(P, ptrs);
+            tad_launch(tad_contract_reduce, blocks, 256, 0, stream, P, ptrs);
             e = cudaGetLastError();
         }
         return e;
@@ -729,7 +735,7 @@ cudaError_t tad_launch_contract(const TadcProgram &P, const TadpPointers &ptrs, 
     if (P.shape == 4) {
         const unsigned warps = (unsigned)P.M.extent;
         const unsigned blocks = std::min((warps + 7u) / 8u, sms * 16u);
-        tad_rowsum_kernel<<<blocks, 256, 0, stream>>>(P, ptrs);
+        tad_launch(tad_rowsum_kernel, blocks, 256, 0, stream, P, ptrs);
         return cudaGetLastError();
     }
     cudaError_t e = P.shape == 1 ? launch_shape<128, 32, 8, 4>(P, ptrs, stream)
@@ -739,7 +745,7 @@ cudaError_t tad_launch_contract(const TadcProgram &P, const TadpPointers &ptrs, 
     if (P.ksplit > 1) {
         const unsigned long long cells = (unsigned long long)P.M.extent * P.N.extent * P.Z.extent;
         const unsigned blocks = (unsigned)std::min<unsigned long long>((cells + 255) / 256, (unsigned long long)sms * 8);
-        tad_contract_reduce<<<blocks, 256, 0, stream>>>(P, ptrs);
+        tad_launch(tad_contract_reduce, blocks, 256, 0, stream, P, ptrs);
         e = cudaGetLastError();
     }
     return e;

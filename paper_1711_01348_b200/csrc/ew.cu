@@ -12,6 +12,7 @@
 
 #include <algorithm>
 
+#include "launch.h"
 #include "ew.h"
 #include "vm.cuh"
 
@@ -27,6 +28,7 @@ __global__ void __launch_bounds__(256)
 tad_ew_kernel(const __grid_constant__ TadeProgram P, const __grid_constant__ TadpPointers ptrs, const unsigned n_items,
               const unsigned cols, const unsigned lane_blocks, const unsigned n_rows)
 {
+    tad_wait_previous();
     const unsigned tid = threadIdx.x;
     const unsigned rows_per_block = 256u / cols;
     const unsigned tc = tid % cols, tr = tid / cols;
@@ -183,6 +185,7 @@ __global__ void __launch_bounds__(256, 3)
 tad_prod_kernel(const __grid_constant__ TadeProgram P, const __grid_constant__ ProdPlan Q, const __grid_constant__ TadpPointers ptrs,
                 const unsigned n_items, const unsigned cols, const unsigned lane_blocks, const unsigned n_runs, const unsigned runs_per_line)
 {
+    tad_wait_previous();
     const unsigned tid = threadIdx.x;
     const unsigned rows_per_block = 256u / cols;
     const unsigned tc = tid % cols, tr = tid / cols;
@@ -425,7 +428,7 @@ cudaError_t tad_launch_ew(const TadeProgram &P, const TadpPointers &ptrs, unsign
         const unsigned long long its = ((runs + per_block - 1) / per_block) * lblocks;
         if (its >= (1ull << 32) || runs >= (1ull << 31)) return cudaErrorInvalidValue;
         const unsigned g = (unsigned)std::min<unsigned long long>(its, (unsigned long long)sms * 32ull);
-#define TAD_PROD_LAUNCH(V, MM) tad_prod_kernel<V, MM><<<g, 256, 0, stream>>>(P, Q, ptrs, (unsigned)its, pc, lblocks, (unsigned)runs, (unsigned)per_line)
+#define TAD_PROD_LAUNCH(V, MM) tad_launch(tad_prod_kernel<V, MM>, g, 256, 0, stream, P, Q, ptrs, (unsigned)its, pc, lblocks, (unsigned)runs, (unsigned)per_line)
         switch ((Q.vec ? 4 : 0) + Q.n_moving) {
         case 0: TAD_PROD_LAUNCH(false, 0); break;
         case 1: TAD_PROD_LAUNCH(false, 1); break;
@@ -447,6 +450,6 @@ cudaError_t tad_launch_ew(const TadeProgram &P, const TadpPointers &ptrs, unsign
     const unsigned long long items = row_blocks * lane_blocks;
     if (items >= (1ull << 32) || rows >= (1ull << 31)) return cudaErrorInvalidValue;
     const unsigned grid = (unsigned)std::min<unsigned long long>(items, (unsigned long long)sms * 16ull);
-    tad_ew_kernel<<<grid, 256, 0, stream>>>(P, ptrs, (unsigned)items, cols, lane_blocks, (unsigned)rows);
+    tad_launch(tad_ew_kernel, grid, 256, 0, stream, P, ptrs, (unsigned)items, cols, lane_blocks, (unsigned)rows);
     return cudaGetLastError();
 }

@@ -5,6 +5,7 @@
 #include <algorithm>
 #include <climits>
 
+#include "launch.h"
 #include "line.h"
 
 namespace {
@@ -79,6 +80,7 @@ __global__ void __launch_bounds__(256)
 tad_line_kernel(const __grid_constant__ TadlProgram P, const __grid_constant__ TadpPointers ptrs, const unsigned n_items,
                 const unsigned cols, const unsigned lane_blocks, const unsigned n_rows, const int unroll)
 {
+    tad_wait_previous();
     const unsigned tid = threadIdx.x, lane = tid & 31u;
     const bool by_warp = P.mode == 1;
     const int lane_var = P.lane_var;
@@ -218,7 +220,7 @@ cudaError_t tad_launch_line(const TadlProgram &P, const TadpPointers &ptrs, unsi
     if (items >= (1ull << 31) || rows >= (1ull << 31)) return cudaErrorInvalidValue;
     const unsigned gx = (unsigned)std::min<unsigned long long>(items, (unsigned long long)sms * 32ull);
     dim3 grid(gx, (unsigned)std::max(1, P.zsplit), 1u);
-    if (P.stream) tad_line_kernel<true><<<grid, 256, 0, stream>>>(P, ptrs, (unsigned)items, cols, lane_blocks, (unsigned)rows, P.unroll);
-    else tad_line_kernel<false><<<grid, 256, 0, stream>>>(P, ptrs, (unsigned)items, cols, lane_blocks, (unsigned)rows, P.unroll);
+    if (P.stream) tad_launch(tad_line_kernel<true>, grid, 256, 0, stream, P, ptrs, (unsigned)items, cols, lane_blocks, (unsigned)rows, P.unroll);
+    else tad_launch(tad_line_kernel<false>, grid, 256, 0, stream, P, ptrs, (unsigned)items, cols, lane_blocks, (unsigned)rows, P.unroll);
     return cudaGetLastError();
 }

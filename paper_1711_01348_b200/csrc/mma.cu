@@ -28,6 +28,7 @@
 
 #include <algorithm>
 
+#include "launch.h"
 #include "contract.cuh"
 
 namespace {
@@ -197,6 +198,7 @@ template <int BN, int MA, int MB>
 __global__ void __launch_bounds__(NT, 1)
 tad_mma_kernel(const __grid_constant__ TadcProgram P, const __grid_constant__ TadpPointers ptrs, const unsigned tiles_n)
 {
+    tad_wait_previous();
     using C = MmaCfg<BN, MA, MB>;
     constexpr bool TS = C::TS;
     constexpr int COLS = C::COLS;
@@ -477,6 +479,7 @@ tad_mma_kernel(const __grid_constant__ TadcProgram P, const __grid_constant__ Ta
 __global__ void __launch_bounds__(256)
 tad_mma_reduce(const __grid_constant__ TadcProgram P, const __grid_constant__ TadpPointers ptrs)
 {
+    tad_wait_previous();
     const unsigned Mext = (unsigned)P.M.extent, Next = (unsigned)P.N.extent;
     const unsigned per_z = Mext * Next;
     const unsigned planes = (unsigned)P.ksplit;
@@ -512,7 +515,7 @@ cudaError_t launch_mma(const TadcProgram &P, const TadpPointers &ptrs, cudaStrea
     }
     const unsigned tiles_m = ((unsigned)P.M.extent + BM - 1) / BM, tiles_n = ((unsigned)P.N.extent + BN - 1) / BN;
     dim3 grid(tiles_m * tiles_n, (unsigned)std::max(1, P.ksplit), (unsigned)P.Z.extent);
-    kern<<<grid, NT, C::SMEM, stream>>>(P, ptrs, tiles_n);
+    tad_launch(kern, grid, NT, C::SMEM, stream, P, ptrs, tiles_n);
     return cudaGetLastError();
 }
 
@@ -530,7 +533,7 @@ cudaError_t tad_launch_mma(const TadcProgram &P, const TadpPointers &ptrs, unsig
     if (e == cudaSuccess && P.ksplit > 1) {
         const unsigned long long cells = (unsigned long long)P.M.extent * P.N.extent;
         const unsigned blocks = (unsigned)std::min<unsigned long long>((cells + 255) / 256, (unsigned long long)sms * 8);
-        tad_mma_reduce<<<blocks, 256, 0, stream>>>(P, ptrs);
+        tad_launch(tad_mma_reduce, blocks, 256, 0, stream, P, ptrs);
         e = cudaGetLastError();
     }
     return e;

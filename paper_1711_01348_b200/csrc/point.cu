@@ -9,6 +9,7 @@
 
 #include <algorithm>
 
+#include "launch.h"
 #include "point.h"
 #include "vm.cuh"
 
@@ -135,6 +136,7 @@ template <int U>
 __global__ void __launch_bounds__(NT)
 tad_point_kernel(const __grid_constant__ TadqProgram P, const __grid_constant__ TadpPointers ptrs)
 {
+    tad_wait_previous();
     extern __shared__ __align__(16) float sm[];
     const int tid = (int)threadIdx.x;
     int var[MV][U];
@@ -229,7 +231,7 @@ cudaError_t launch_points(const TadqProgram &P, const TadpPointers &ptrs, cudaSt
             if (dev >= 0 && dev < 64) attr_set[dev] = true;
         }
     }
-    tad_point_kernel<U><<<grid, NT, smem, stream>>>(P, ptrs);
+    tad_launch(tad_point_kernel<U>, grid, NT, smem, stream, P, ptrs);
     return cudaGetLastError();
 }
 

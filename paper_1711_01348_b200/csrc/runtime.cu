@@ -8,9 +8,12 @@
 #include <new>
 #include <string>
 
+#include "launch.h"
 #include "plan.h"
 #include "program.h"
 #include "vm_shapes.h"
+
+thread_local bool tad_launch_plain = false;
 
 namespace tad {
 void set_error(const std::string &m);
@@ -38,6 +41,7 @@ template <int REDUCE_WARPS>
 __global__ void __launch_bounds__(REDUCE_WARPS * 32)
 tad_reduce_partials(const __grid_constant__ TadpProgram P, float *out, const float *part)
 {
+    tad_wait_previous();
     __shared__ float sub[REDUCE_WARPS][32];
     const unsigned n = (unsigned)P.part_limit;
     const int planes = P.zsplit;
@@ -71,8 +75,8 @@ tad_reduce_partials(const __grid_constant__ TadpProgram P, float *out, const flo
 
 void launch_reduce_partials(const TadpProgram &P, const TadpPointers &ptrs, unsigned blocks, cudaStream_t stream)
 {
-    if (P.zsplit > 128) tad_reduce_partials<32><<<blocks, 32 * 32, 0, stream>>>(P, ptrs.out, ptrs.part);
-    else tad_reduce_partials<8><<<blocks, 8 * 32, 0, stream>>>(P, ptrs.out, ptrs.part);
+    if (P.zsplit > 128) tad_launch(tad_reduce_partials<32>, blocks, 32 * 32, 0, stream, P, ptrs.out, ptrs.part);
+    else tad_launch(tad_reduce_partials<8>, blocks, 8 * 32, 0, stream, P, ptrs.out, ptrs.part);
 }
 
 // Sixteen independent multiply-add chains per thread, operands in registers only: the rate at which this GPU
@@ -95,6 +99,7 @@ tad_fma_rate_kernel(float *sink, int iters, float m)
 
 __global__ void tad_fill_zero(float *out, unsigned n)
 {
+    tad_wait_previous();
     const unsigned stride = gridDim.x * blockDim.x;
     for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) out[i] = 0.f;
 }
@@ -253,7 +258,9 @@ tad_status launch(const tad::Kernel &k, TadpPointers ptrs, bool debug, cudaStrea
                 }
                 beside.push_back(k.aux[pk.out_aux].slot);
             }
+            tad_launch_plain = !on_side && !beside.empty();
             const tad_status st = launch(pk, pp, debug, on_side ? side->s : stream, nullptr, on_side ? nullptr : side);
+            tad_launch_plain = false;
             if (st != TAD_OK) return st;
         }
         if (!join()) { tad::set_error("event record / wait failed"); return TAD_ERR_CUDA; }
@@ -314,7 +321,7 @@ tad_status launch(const tad::Kernel &k, TadpPointers ptrs, bool debug, cudaStrea
 tad_status zero_fill(float *out, int64_t n, cudaStream_t stream)
 {
     const unsigned blocks = (unsigned)std::min<int64_t>((n + 255) / 256, (int64_t)sm_count() * 16);
-    tad_fill_zero<<<blocks, 256, 0, stream>>>(out, (unsigned)n);
+    tad_launch(tad_fill_zero, blocks, 256, 0, stream, out, (unsigned)n);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) { tad::set_error(std::string("zero fill launch failed: ") + cudaGetErrorString(e)); return TAD_ERR_CUDA; }
     return TAD_OK;

@@ -3,6 +3,7 @@
 
 #include <algorithm>
 
+#include "launch.h"
 #include "vm.cuh"
 
 #ifndef TAD_TA
@@ -20,6 +21,7 @@ template <int TA, int UB, bool DEBUG, bool REL>
 __global__ void __launch_bounds__(VmCfg<TA, UB>::WARPS * 32, (TA * UB >= 32 ? 3 : 2))
 tad_vm_kernel(const __grid_constant__ TadpProgram P, const __grid_constant__ TadpPointers ptrs, unsigned n_items)
 {
+    tad_wait_previous();
     constexpr int E = TA * UB;
     const unsigned lane = threadIdx.x & 31u;
     const unsigned warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -192,11 +194,11 @@ bool TAD_LAUNCH_NAME(TAD_TA, TAD_UB)(const TadpProgram &prog, const TadpPointers
     // one warp per work item, grid-stride; at most 128 warps' worth of blocks per SM
     const unsigned blocks = std::min((items + WPB - 1) / WPB, sms * (128u / WPB));
     if (debug) {
-        if constexpr (TA <= 4 && UB == 1) tad_vm_kernel<TA, UB, true, true><<<blocks, WPB * 32, 0, stream>>>(prog, ptrs, items);
+        if constexpr (TA <= 4 && UB == 1) tad_launch(tad_vm_kernel<TA, UB, true, true>, blocks, WPB * 32, 0, stream, prog, ptrs, items);
         else return false;
     } else if (prog.rel_var >= 0) {
-        if constexpr (UB == 1) tad_vm_kernel<TA, UB, false, true><<<blocks, WPB * 32, 0, stream>>>(prog, ptrs, items);
+        if constexpr (UB == 1) tad_launch(tad_vm_kernel<TA, UB, false, true>, blocks, WPB * 32, 0, stream, prog, ptrs, items);
         else return false;
-    } else tad_vm_kernel<TA, UB, false, false><<<blocks, WPB * 32, 0, stream>>>(prog, ptrs, items);
+    } else tad_launch(tad_vm_kernel<TA, UB, false, false>, blocks, WPB * 32, 0, stream, prog, ptrs, items);
     return true;
 }
