@@ -236,21 +236,34 @@ bool emit_program(const System &s0, float scale, int accumulate, bool allow_spli
     if (mma && !one_column) {
         // ---- tensor-core tiles ----
         P.shape = 7;
-        auto vectors = [&](const std::vector<Digit> &fast, const std::vector<Digit> &other, bool second, const AGuard *gd, int64_t base) {
+        auto vectors = [&](const std::vector<Digit> &fast, const std::vector<Digit> &other, bool second, const AGuard *gd, int64_t base, bool along_rows = false) {
             // octets of the group are 32 consecutive, 16-byte aligned bytes: the run of consecutive elements along its
             // fastest digits is a multiple of eight long and everything else moves by multiples of four
             auto st = [&](const Digit &d) { return second ? d.sB : d.sA; };
             int64_t run = 1;
             int d = (int)fast.size() - 1;
             for (; d >= 0 && st(fast[d]) == run; --d) { if (gd && gd->coef[fast[d].var]) return false; run *= fast[d].ext; }
-            if (run % 8 || base % 4) return false;
+            if (base % 4) return false;
+            // (a last octet that is cut short is read whole and masked, where its row reaches that far)
+            if (run % 8) {
+                if (along_rows || fast.size() != 1 || d >= 0) return false;
+                int64_t pitch = 0, last = base;
+                for (const std::vector<Digit> *g : {&other, (const std::vector<Digit> *)&dz})
+                    for (const Digit &e : *g) {
+                        if (st(e) <= 0) return false;
+                        pitch = pitch ? std::min<int64_t>(pitch, st(e)) : st(e);
+                        last += st(e) * (e.ext - 1);
+                    }
+                const int64_t whole = (run + 7) / 8 * 8;
+                if (pitch < whole || last + whole > (second ? s.B.limit : s.A.limit)) return false;
+            }
             for (; d >= 0; --d) if (st(fast[d]) % 4) return false;
             for (const std::vector<Digit> *g : {&other, (const std::vector<Digit> *)&dz}) for (const Digit &e : *g) if (st(e) % 4) return false;
             return true;
         };
         auto mma_mode = [&](const std::vector<Digit> &rows, bool second, const AGuard *gd, int64_t base, int legacy) {
             if (vectors(dk, rows, second, gd, base)) return (int)TM_KVEC;
-            if (second && vectors(rows, dk, second, gd, base)) return (int)TM_RVEC;
+            if (second && vectors(rows, dk, second, gd, base, true)) return (int)TM_RVEC;
             return legacy == TG_K ? (int)TM_K : (int)TM_ROW;
         };
         P.modeA = mma_mode(dm, false, ga, s.A.base, P.modeA);

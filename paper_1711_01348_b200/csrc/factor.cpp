@@ -664,8 +664,10 @@ static bool factor_kernel(Gen &g, Kernel &k, int root, int scale, bool allow_spl
             int64_t kext = 1;
             for (int v = 0; v < TADP_MAX_VARS; ++v) if (G.kmask & (1u << v)) kext = mul_ck(kext, F.vext[v]);
             fusion.cols = kext + (int64_t)S.size() - 1;
-            fusion.a_tensor = F.new_tensor(F.vars_of(fusion.mmask), fusion.cols);
-            fusion.b_tensor = F.new_tensor(F.vars_of(fusion.nmask), fusion.cols);
+            // (rows of whole 32-byte pieces: the contraction reads them as vectors)
+            const int64_t padded = (fusion.cols + 7) / 8 * 8;
+            fusion.a_tensor = F.new_tensor(F.vars_of(fusion.mmask), padded);
+            fusion.b_tensor = F.new_tensor(F.vars_of(fusion.nmask), padded);
             int64_t col = kext;
             for (size_t mi = 0; mi < S.size(); ++mi) {
                 Mono ma, mb; ma.c = S[mi].c; mb.c = 1;

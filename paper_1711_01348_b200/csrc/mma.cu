@@ -27,6 +27,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "launch.h"
 #include "contract.cuh"
@@ -108,13 +109,13 @@ __device__ __forceinline__ unsigned long long make_desc(unsigned addr, unsigned 
 //   TM_RVEC  t = row, contiguous and aligned: two 128-bit loads                                  -> MN-major
 // (the row operand of the TM_ROW mode goes to tensor memory: a thread then takes the row of its own lane and the
 // sixteen summation indices of MMA step warp / 4)
-template <int MODE, int R, bool TMEM>
+template <int MODE, int R, bool TMEM, int THREADS = NCW * 32>
 struct Unit {
     static constexpr bool KMAJOR = MODE == TM_ROW || MODE == TM_KVEC, VEC = MODE == TM_KVEC || MODE == TM_RVEC;
     int l, t0, dst;
     __device__ __forceinline__ Unit(int tid, int i)
     {
-        const int u = tid + i * NCW * 32;
+        const int u = tid + i * THREADS;
         int o;
         if (TMEM) { l = tid % BM; o = (tid / BM) * 2 + i; }
         else if (MODE == TM_ROW) { l = u % R; o = u / R; }
@@ -132,11 +133,11 @@ __device__ __forceinline__ float ldf(const float *__restrict__ src, unsigned byt
 }
 
 // rows: offsets and guards of the tile's rows; kt: offsets and guards of the stage's summation indices (KS each)
-template <int MODE, int R, bool TMEM, bool CHECK>
+template <int MODE, int R, bool TMEM, bool CHECK, int THREADS = NCW * 32>
 __device__ __forceinline__ void load_unit(float (&v)[8], const float *__restrict__ src, const int tid, const int i, const unsigned *row, const int *rowg,
                                           const unsigned *kt, const int *ktg, const unsigned gext)
 {
-    using U = Unit<MODE, R, TMEM>;
+    using U = Unit<MODE, R, TMEM, THREADS>;
     const U u(tid, i);
     const unsigned base = U::KMAJOR ? row[u.l] : kt[u.l];
     const unsigned *tab = (U::KMAJOR ? kt : row) + u.t0;
@@ -165,6 +166,17 @@ __device__ __forceinline__ void load_unit(float (&v)[8], const float *__restrict
             if ((unsigned)(gbase + g[j]) < gext) v[j] = ldf(src, base + t[j]);
         }
     }
+}
+
+// Summation indices past the end of the range (left of them remain from the stage's first on) count as zeros.  They are
+// loaded like all others - their table entries repeat the first index, rows past the edge of the matrix repeat the first
+// row, whose offset has the alignment that vector loads need - and masked when they are used: a test at the load would
+// wait for every unit's data in turn.
+template <class U>
+__device__ __forceinline__ void mask_unit(float (&v)[8], const U &u, const int left)
+{
+#pragma unroll
+    for (int j = 0; j < 8; ++j) if ((U::KMAJOR ? u.t0 + j : u.l) >= left) v[j] = 0.f;
 }
 
 // eight values -> three times eight bf16 (packed in pairs)
@@ -247,16 +259,14 @@ tad_mma_kernel(const __grid_constant__ TadcProgram P, const __grid_constant__ Ta
         if (warp < KT) fill_ktab(warp, lane);
         for (int r = tid; r < BM; r += NCW * 32) {
             const unsigned m = tile_m * BM + r;
-            Parts p{0, 0, 0, 0, 0};
-            if (m < Mext) p = decode(P.M, m);
-            rowA[r] = m < Mext ? (unsigned)(P.baseA + z.a + p.a) * 4u : 0u; rowgA[r] = m < Mext ? P.guardA_c0 + z.ga + p.ga : DEAD; outM[r] = p.o;
+            const Parts p = decode(P.M, m < Mext ? m : 0u);
+            rowA[r] = (unsigned)(P.baseA + z.a + p.a) * 4u; rowgA[r] = m < Mext ? P.guardA_c0 + z.ga + p.ga : DEAD; outM[r] = p.o;
         }
         for (int r = tid - BM; r < BN; r += NCW * 32) {
             if (r < 0) continue;
             const unsigned n = tile_n * BN + r;
-            Parts p{0, 0, 0, 0, 0};
-            if (n < Next) p = decode(P.N, n);
-            rowB[r] = n < Next ? (unsigned)(P.baseB + z.b + p.b) * 4u : 0u; rowgB[r] = n < Next ? P.guardB_c0 + z.gb + p.gb : DEAD; outN[r] = p.o;
+            const Parts p = decode(P.N, n < Next ? n : 0u);
+            rowB[r] = (unsigned)(P.baseB + z.b + p.b) * 4u; rowgB[r] = n < Next ? P.guardB_c0 + z.gb + p.gb : DEAD; outN[r] = p.o;
         }
     }
     fence_before();
@@ -322,7 +332,6 @@ tad_mma_kernel(const __grid_constant__ TadcProgram P, const __grid_constant__ Ta
         const int quad = warp & 3, col0 = (warp >> 2) * COLS;
         const float *__restrict__ A = ptrs.in[P.ptrA];
         const float *__restrict__ B = ptrs.in[P.ptrB];
-        const bool edgeA = P.guardA || (tile_m + 1) * BM > Mext, edgeB = P.guardB || (tile_n + 1) * BN > Next;
         const unsigned gextA = (unsigned)P.guardA_ext, gextB = (unsigned)P.guardB_ext;
         float va[C::UA][8], vb[C::UB][8];
         auto load = [&](float (&v)[8], int i, int s, bool second, bool check) {
@@ -353,19 +362,26 @@ tad_mma_kernel(const __grid_constant__ TadcProgram P, const __grid_constant__ Ta
             fence_before();
         };
 #pragma unroll
-        for (int i = 0; i < C::UA; ++i) load(va[i], i, 0, false, edgeA || kend - kbeg < KS);
+        for (int i = 0; i < C::UA; ++i) load(va[i], i, 0, false, P.guardA != 0);
 #pragma unroll
-        for (int i = 0; i < C::UB; ++i) load(vb[i], i, 0, true, edgeB || kend - kbeg < KS);
+        for (int i = 0; i < C::UB; ++i) load(vb[i], i, 0, true, P.guardB != 0);
         for (int s = 0; s < n_stages && ok; ++s) {
             unsigned char *st = stages + (s & 1) * C::STAGE;
-            const bool more = s + 1 < n_stages, tail = kend - kbeg - (unsigned)s * KS < 2 * KS;      // the next stage is a partial one
+            const bool more = s + 1 < n_stages;
+            const int left = (int)min((unsigned)KS, kend - kbeg - (unsigned)s * KS);
             if (more && s + 1 >= KT) ok = mbar_wait(bar_tab + 8 * ((s + 1) % KT), ((s + 1) / KT - 1) & 1, &failed);
             if (!ok) break;
+            if (left < KS) {
+#pragma unroll
+                for (int i = 0; i < C::UA; ++i) mask_unit(va[i], Unit<MA, BM, TS>(tid, i), left);
+#pragma unroll
+                for (int i = 0; i < C::UB; ++i) mask_unit(vb[i], Unit<MB, BN, false>(tid, i), left);
+            }
             unsigned p1[4], p2[4], p3[4];
 #pragma unroll
             for (int i = 0; i < C::UA; ++i) {
                 split_unit(va[i], p1, p2, p3);
-                if (more) load(va[i], i, s + 1, false, edgeA || tail);
+                if (more) load(va[i], i, s + 1, false, P.guardA != 0);
                 const Unit<MA, BM, TS> u(tid, i);
                 if (TS) {
                     const unsigned at = tmem + ((unsigned)(quad * 32) << 16) + TMEM_A + (s & 1) * 96 + u.t0 / 2;
@@ -380,7 +396,7 @@ tad_mma_kernel(const __grid_constant__ TadcProgram P, const __grid_constant__ Ta
 #pragma unroll
             for (int i = 0; i < C::UB; ++i) {
                 split_unit(vb[i], p1, p2, p3);
-                if (more) load(vb[i], i, s + 1, true, edgeB || tail);
+                if (more) load(vb[i], i, s + 1, true, P.guardB != 0);
                 const Unit<MB, BN, false> u(tid, i);
                 *reinterpret_cast<uint4 *>(st + u.dst) = make_uint4(p1[0], p1[1], p1[2], p1[3]);
                 *reinterpret_cast<uint4 *>(st + C::PART_B + u.dst) = make_uint4(p2[0], p2[1], p2[2], p2[3]);
@@ -474,6 +490,320 @@ tad_mma_kernel(const __grid_constant__ TadcProgram P, const __grid_constant__ Ta
     }
 }
 
+// ---------------------------------------------------------------------------------------------------------
+// Contractions of one stage (up to 64 summation indices): forward passes and staged adjoints of expressions whose sum
+// was pushed inside, where the work is the epilogue and the traffic of the outputs.  With a block per tile, gather,
+// split, MMA and epilogue of a tile ran one after another (8192 x 8192 x 34: 220 us for 268 MB of output).  Here a block
+// walks a run of tiles with the row tile fastest and its warps work on different tiles at a time:
+//   warps 16-22  gather and split the row operand of the next tile (and the column operand where the column tile changes)
+//   warp 23      issues the MMAs of the current one into one of two accumulators
+//   warps 0-15   read the accumulator of the tile before (32 rows x 32 columns each), apply the epilogue and store; the
+//                values of a tensor that the epilogue reads are loaded while the MMAs still run
+// ---------------------------------------------------------------------------------------------------------
+constexpr int SE = 16, SC = 7, SNT = (SE + SC + 1) * 32;    // epilogue and gather warps; six warps per scheduler leave 80 registers each
+
+struct ShortCfg {
+    static constexpr int PART = BM * KS * 2, OPERAND = 3 * PART;
+    static constexpr int TABLES = 2 * BM * 8 + 2 * BM * 8 + 4 * KS * 4 + SE * 64 * 4;    // row tables of both operands (twice), k tables, output columns
+    static constexpr size_t SMEM = 1024 + 4 * size_t(OPERAND) + TABLES;
+};
+
+template <int MA, int MB>
+__global__ void __launch_bounds__(SNT, 1)
+tad_mma_short_kernel(const __grid_constant__ TadcProgram P, const __grid_constant__ TadpPointers ptrs, const unsigned tiles_m, const unsigned tiles_n, const unsigned n_items)
+{
+    tad_wait_previous();
+    using C = ShortCfg;
+    extern __shared__ unsigned char smem_raw[];
+    __shared__ unsigned long long bars[6];
+    __shared__ unsigned tmem_base_s;
+    __shared__ volatile int failed;
+    const unsigned smem0 = (smem_u32(smem_raw) + 1023u) & ~1023u;
+    unsigned char *bufs = smem_raw + (smem0 - smem_u32(smem_raw));                     // A0, A1, B0, B1
+    unsigned *rowoff = reinterpret_cast<unsigned *>(bufs + 4 * C::OPERAND);            // [operand][buffer][row], then the guards likewise
+    int *rowgrd = reinterpret_cast<int *>(rowoff + 4 * BM);
+    int *ktab = rowgrd + 4 * BM;                                                       // offsets A, guards A, offsets B, guards B
+    int *outN = ktab + 4 * KS;                                                         // per epilogue warp: output offsets of its 32 columns, twice
+    const unsigned bar_full = smem_u32(&bars[0]), bar_done = smem_u32(&bars[2]), bar_free = smem_u32(&bars[4]);
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+    const unsigned Mext = (unsigned)P.M.extent, Next = (unsigned)P.N.extent, K = (unsigned)P.K.extent;
+    const unsigned per = n_items / gridDim.x, extra = n_items % gridDim.x;
+    const unsigned first = blockIdx.x * per + min(blockIdx.x, extra);
+    const unsigned strip0 = first / tiles_m, row0 = first - strip0 * tiles_m;          // strip: column tile and batch index
+    const int n_tiles = (int)(per + (blockIdx.x < extra ? 1u : 0u));
+    const int kpad = (int)((K + 15u) & ~15u);
+    if (warp == SE + SC) {
+        if (lane == 0) {
+            failed = 0;
+            for (int i = 0; i < 2; ++i) { mbar_init(bar_full + 8 * i, SC); mbar_init(bar_done + 8 * i, 1); mbar_init(bar_free + 8 * i, SE); }
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        }
+        __syncwarp();
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 256;" ::"r"(smem_u32(&tmem_base_s)) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    } else if (tid < KS) {
+        Parts p{0, 0, 0, DEAD, DEAD};
+        if ((unsigned)tid < K) p = decode(P.K, tid);
+        ktab[tid] = p.a * 4; ktab[KS + tid] = p.ga; ktab[2 * KS + tid] = p.b * 4; ktab[3 * KS + tid] = p.gb;
+    }
+    fence_before();
+    __syncthreads();
+    fence_after();
+    const unsigned tmem = __shfl_sync(0xffffffffu, tmem_base_s, 0);
+    bool ok = true;
+    if (warp == SE + SC) {
+        // ---- MMA warp ----
+        constexpr bool a_k = MA == TM_ROW || MA == TM_KVEC, b_k = MB == TM_ROW || MB == TM_KVEC;
+        constexpr unsigned stepA = a_k ? 32u : 16u * 128u, stepB = b_k ? 32u : 16u * 128u;
+        constexpr unsigned lboA = a_k ? 16u : KS * 128u, lboB = b_k ? 16u : KS * 128u;
+        constexpr int PA[6] = {2, 1, 0, 1, 0, 0}, PB[6] = {0, 1, 2, 0, 1, 0};      // small products first
+        unsigned strip = strip0, tile_m = row0;
+        int q = 0, t = 0;
+        for (; t < n_tiles && ok; ++t) {
+            if (t > 0 && ++tile_m == tiles_m) { tile_m = 0; ++strip; ++q; }
+            ok = mbar_wait(bar_full + 8 * (t & 1), (t >> 1) & 1, &failed);
+            if (ok && t >= 2) ok = mbar_wait(bar_free + 8 * (t & 1), ((t - 2) >> 1) & 1, &failed);
+            fence_after();
+            if (!ok) break;
+            const unsigned n_pad = min((unsigned)BM, (Next - (strip % tiles_n) * BM + 15u) / 16u * 16u);
+            const unsigned idesc = (1u << 4) | (1u << 7) | (1u << 10) | (a_k ? 0u : 1u << 15) | (b_k ? 0u : 1u << 16) | ((n_pad >> 3) << 17) | ((BM >> 4) << 24);
+            const unsigned long long da = make_desc(smem0 + (t & 1) * C::OPERAND, lboA, 1024u), db = make_desc(smem0 + (2 + (q & 1)) * C::OPERAND, lboB, 1024u);
+            const int steps = kpad / 16;
+#pragma unroll
+            for (int pr = 0; pr < 6; ++pr)
+#pragma unroll
+                for (int kk = 0; kk < KS / 16; ++kk) {
+                    if (kk >= steps) continue;
+                    mma_ss(tmem + (t & 1) * BM, da + ((PA[pr] * C::PART + kk * stepA) >> 4), db + ((PB[pr] * C::PART + kk * stepB) >> 4), idesc, pr + kk > 0);
+                }
+            mma_commit(bar_done + 8 * (t & 1));
+        }
+        // MMAs of a block that gave up still read its shared memory: wait for them (again with a limit)
+        if (!ok)
+            for (int s = max(0, t - 2); s < t; ++s)
+                for (int i = 0; i < WAIT_LIMIT; ++i) {
+                    unsigned done;
+                    asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }" : "=r"(done) : "r"(bar_done + 8 * (s & 1)), "r"((s >> 1) & 1) : "memory");
+                    if (__all_sync(0xffffffffu, done)) break;
+                }
+    } else if (warp >= SE) {
+        // ---- gathering warps ----
+        const int ct = tid - SE * 32;
+        constexpr int CT = SC * 32, UNITS = BM * KS / 8, UN = (UNITS + CT - 1) / CT;
+        unsigned tile_m = row0, strip = strip0, tile_n = 0;
+        int q = -1;
+        Parts z{0, 0, 0, 0, 0};
+        auto gather = [&](auto mode, const float *__restrict__ src, const unsigned *row, const int *rowg, const int *kt, bool check, unsigned gext, unsigned char *dst) {
+            constexpr int MODE = decltype(mode)::value;
+            using U = Unit<MODE, BM, false, CT>;
+            const unsigned *kto = reinterpret_cast<const unsigned *>(kt);
+            float v[UN][8];
+#pragma unroll
+            for (int i = 0; i < UN; ++i) {
+                const U u(ct, i);
+                if (ct + i * CT >= UNITS || (U::KMAJOR ? u.t0 : u.l) >= kpad) continue;
+                if (check) load_unit<MODE, BM, false, true, CT>(v[i], src, ct, i, row, rowg, kto, kt + KS, gext);
+                else load_unit<MODE, BM, false, false, CT>(v[i], src, ct, i, row, rowg, kto, kt + KS, gext);
+            }
+#pragma unroll
+            for (int i = 0; i < UN; ++i) {
+                const U u(ct, i);
+                if (ct + i * CT >= UNITS || (U::KMAJOR ? u.t0 : u.l) >= kpad) continue;
+                unsigned p1[4], p2[4], p3[4];
+                if (kpad != (int)K) mask_unit(v[i], u, (int)K);
+                split_unit(v[i], p1, p2, p3);
+                *reinterpret_cast<uint4 *>(dst + u.dst) = make_uint4(p1[0], p1[1], p1[2], p1[3]);
+                *reinterpret_cast<uint4 *>(dst + C::PART + u.dst) = make_uint4(p2[0], p2[1], p2[2], p2[3]);
+                *reinterpret_cast<uint4 *>(dst + 2 * C::PART + u.dst) = make_uint4(p3[0], p3[1], p3[2], p3[3]);
+            }
+        };
+        for (int t = 0; t < n_tiles && ok; ++t) {
+            // the MMAs of tile t - 2 are done: its row buffer, and every column buffer but the last two, are free
+            if (t >= 2) ok = mbar_wait(bar_done + 8 * (t & 1), ((t - 2) >> 1) & 1, &failed);
+            if (!ok) break;
+            const bool fresh = t == 0 || ++tile_m == tiles_m;
+            if (fresh) {
+                if (t > 0) { tile_m = 0; ++strip; }
+                ++q;
+                tile_n = strip % tiles_n;
+                z = decode(P.Z, strip / tiles_n);
+            }
+            for (int r = ct; r < (fresh ? 2 : 1) * BM; r += CT) {
+                if (r < BM) {
+                    const unsigned m = tile_m * BM + r;
+                    const Parts p = decode(P.M, m < Mext ? m : 0u);
+                    rowoff[(t & 1) * BM + r] = (unsigned)(P.baseA + z.a + p.a) * 4u;
+                    rowgrd[(t & 1) * BM + r] = m < Mext ? P.guardA_c0 + z.ga + p.ga : DEAD;
+                } else {
+                    const unsigned n = tile_n * BM + (r - BM);
+                    const Parts p = decode(P.N, n < Next ? n : 0u);
+                    rowoff[(2 + (q & 1)) * BM + r - BM] = (unsigned)(P.baseB + z.b + p.b) * 4u;
+                    rowgrd[(2 + (q & 1)) * BM + r - BM] = n < Next ? P.guardB_c0 + z.gb + p.gb : DEAD;
+                }
+            }
+            // (a warp that is here has read the tables of the tile before: the tables alternate, one barrier per tile is enough)
+            asm volatile("bar.sync 1, %0;" ::"n"(CT) : "memory");
+            if (fresh)
+                gather(std::integral_constant<int, MB>{}, ptrs.in[P.ptrB], rowoff + (2 + (q & 1)) * BM, rowgrd + (2 + (q & 1)) * BM, ktab + 2 * KS,
+                       P.guardB != 0, (unsigned)P.guardB_ext, bufs + (2 + (q & 1)) * C::OPERAND);
+            gather(std::integral_constant<int, MA>{}, ptrs.in[P.ptrA], rowoff + (t & 1) * BM, rowgrd + (t & 1) * BM, ktab,
+                   P.guardA || (tile_m + 1) * BM > Mext, (unsigned)P.guardA_ext, bufs + (t & 1) * C::OPERAND);
+            fence_async();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar_full + 8 * (t & 1));
+        }
+    } else {
+        // ---- epilogue warps: 32 rows x 32 columns of a tile each ----
+        const int quad = warp & 3, col0 = (warp >> 2) * 32;
+        int *cols = outN + warp * 64;                          // output offsets of this warp's columns, of an even and an odd column tile
+        int pre = -1;                                          // the epilogue step whose tensor is loaded ahead
+        for (int e = P.n_epi - 1; e >= 0; --e) if (P.epi_op[e] == TE_MUL_LOAD || P.epi_op[e] == TE_ADD_LOAD) pre = e;
+        // A tile is two pieces of 16 columns.  The values that the epilogue reads for a piece are loaded a piece ahead (the
+        // ones of a tile's first piece while its MMAs still run); one copy of the code serves both pieces.
+        unsigned tile_m = row0, strip = strip0, n0 = 0;
+        int ncol = 0, ob = 0;                                  // columns of this warp, the same for all its lanes; the row's output offset
+        bool row = false;
+        int zo = 0;
+        float w[16], wn[16];
+#pragma unroll
+        for (int j = 0; j < 16; ++j) { w[j] = 0.f; wn[j] = 0.f; }
+        const float *__restrict__ src0 = pre >= 0 ? ptrs.in[P.epi_ptr[pre]] + (ptrdiff_t)P.epi_base[pre] : nullptr;
+        const bool pre_mul = pre >= 0 && P.epi_op[pre] == TE_MUL_LOAD;
+        auto begin_tile = [&](int t) {
+            if (t == 0 || ++tile_m == tiles_m) {
+                if (t > 0) { tile_m = 0; ++strip; }
+                n0 = (strip % tiles_n) * BM + col0;
+                zo = P.baseO + decode(P.Z, strip / tiles_n).o;
+                ncol = n0 < Next ? (int)min(32u, Next - n0) : 0;
+                __syncwarp();
+                cols[(strip & 1u) * 32 + lane] = n0 + lane < Next ? decode(P.N, n0 + lane).o : 0;
+                __syncwarp();
+            }
+            const unsigned m = tile_m * BM + quad * 32 + lane;
+            row = m < Mext;
+            ob = zo + decode(P.M, row ? m : 0u).o;
+        };
+        auto load_ahead = [&](int h) {
+            if (pre < 0 || !row) return;
+            const int *cs = cols + (strip & 1u) * 32;
+            if (ncol >= h + 16) {
+#pragma unroll
+                for (int j = 0; j < 16; ++j) wn[j] = __ldg(src0 + (ob + cs[h + j]));
+            } else if (ncol > h) {
+#pragma unroll
+                for (int j = 0; j < 16; ++j) wn[j] = __ldg(src0 + (ob + cs[h + j < ncol ? h + j : h]));
+            }
+        };
+        if (n_tiles > 0) { begin_tile(0); load_ahead(0); }
+#pragma unroll 1
+        for (int it = 0; it < 2 * n_tiles; ++it) {
+            const int t = it >> 1, h = (it & 1) * 16, live = ncol - h;
+            if (h == 0) {
+                ok = ok && mbar_wait(bar_done + 8 * (t & 1), (t >> 1) & 1, &failed);
+                fence_after();
+            }
+            float v[16];
+            if (ok) {
+                unsigned r[16];
+                tmem_ld16(tmem + ((unsigned)(quad * 32) << 16) + (t & 1) * BM + col0 + h, r);
+                tmem_wait_ld();
+#pragma unroll
+                for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
+            }
+            if (h != 0) {
+                fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar_free + 8 * (t & 1));
+            }
+#pragma unroll
+            for (int j = 0; j < 16; ++j) w[j] = wn[j];
+            // one multiply-add per value finds the non-finite ones (columns past the end hold leftovers of another kernel)
+            float test = 0.f;
+            if (live < 16) {
+#pragma unroll
+                for (int j = 0; j < 16; ++j) if (j >= live) v[j] = 0.f;
+            }
+#pragma unroll
+            for (int j = 0; j < 16; ++j) test = fmaf(v[j], 0.f, test);
+            const bool redo = __any_sync(0xffffffffu, (row && test != 0.f) || !ok);
+            const int off0 = ob;
+            const bool row_now = row;
+            const unsigned m_tile = tile_m, s_now = strip;
+            const int *co = cols + (s_now & 1u) * 32 + h;
+            if (h == 0) load_ahead(16);
+            else if (t + 1 < n_tiles) { __syncwarp(); begin_tile(t + 1); load_ahead(0); }
+            if (!redo) {
+                if (P.scale != 1.f) {
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) v[j] *= P.scale;
+                }
+#define TAD_EPI_ALL(expr) _Pragma("unroll") for (int j = 0; j < 16; ++j) { float &x = v[j]; expr; }
+                for (int e = 0; e < P.n_epi; ++e) {
+                    const float imm = P.epi_imm[e];
+                    switch (P.epi_op[e]) {
+                    case TE_NEG: TAD_EPI_ALL(x = -x) break;
+                    case TE_EXP: TAD_EPI_ALL(x = __expf(x)) break;
+                    case TE_MULC: TAD_EPI_ALL(x *= imm) break;
+                    case TE_ADDC: TAD_EPI_ALL(x += imm) break;
+                    case TE_SQR: TAD_EPI_ALL(x *= x) break;
+                    case TE_TANH: TAD_EPI_ALL(x = own_tanh(x)) break;
+                    case TE_MUL_LOAD: case TE_ADD_LOAD: {
+                        const bool mul = P.epi_op[e] == TE_MUL_LOAD;
+                        if (e == pre) { if (pre_mul) { TAD_EPI_ALL(x *= w[j]) } else { TAD_EPI_ALL(x += w[j]) } }
+                        else if (row_now) {
+                            const float *__restrict__ src = ptrs.in[P.epi_ptr[e]];
+                            const int sb = P.epi_base[e];
+                            TAD_EPI_ALL(if (j < live) { const float y = __ldg(src + (unsigned)(sb + off0 + co[j])); x = mul ? x * y : x + y; })
+                        }
+                        break;
+                    }
+                    default: break;
+                    }
+                }
+#undef TAD_EPI_ALL
+                float *__restrict__ out = ptrs.out;
+                if (row_now && P.accumulate) {
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) if (j < live) out[(unsigned)(off0 + co[j])] += v[j];
+                } else if (row_now && live >= 16) {
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) out[(unsigned)(off0 + co[j])] = v[j];
+                } else if (row_now) {
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) if (j < live) out[(unsigned)(off0 + co[j])] = v[j];
+                }
+            } else if (row_now) {
+                // non-finite sums: this piece once more, with fp32 multiply-adds from the operands themselves
+                const char *pa = reinterpret_cast<const char *>(ptrs.in[P.ptrA]), *pb = reinterpret_cast<const char *>(ptrs.in[P.ptrB]);
+                const Parts z_now = decode(P.Z, s_now / tiles_n), pm_now = decode(P.M, m_tile * BM + quad * 32 + lane);
+#pragma unroll 1
+                for (int j = 0; j < min(live, 16); ++j) {
+                    const Parts pn = decode(P.N, (s_now % tiles_n) * BM + col0 + h + j);
+                    float sum = 0.f;
+#pragma unroll 1
+                    for (unsigned k = 0; k < K; ++k) {
+                        const Parts p = decode(P.K, k);
+                        const bool la = !P.guardA || (unsigned)(P.guardA_c0 + z_now.ga + pm_now.ga + p.ga) < (unsigned)P.guardA_ext;
+                        const bool lb = !P.guardB || (unsigned)(P.guardB_c0 + z_now.gb + pn.gb + p.gb) < (unsigned)P.guardB_ext;
+                        const float x = la ? __ldg(reinterpret_cast<const float *>(pa + (unsigned)(P.baseA + z_now.a + pm_now.a + p.a) * 4u)) : 0.f;
+                        const float y = lb ? __ldg(reinterpret_cast<const float *>(pb + (unsigned)(P.baseB + z_now.b + pn.b + p.b) * 4u)) : 0.f;
+                        sum = fmaf(x, y, sum);
+                    }
+                    const unsigned off = (unsigned)(off0 + pn.o);
+                    const float v1 = epilogue(P, ptrs, sum * P.scale, off);
+                    ptrs.out[off] = P.accumulate ? ptrs.out[off] + v1 : v1;
+                }
+            }
+        }
+    }
+    fence_before();
+    __syncthreads();
+    if (warp == SE + SC) {
+        fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" ::"r"(tmem) : "memory");
+    }
+}
+
 // Adds the planes of a split summation, plane 0 first: planes are [column][row], a thread per output, consecutive
 // threads on consecutive rows.
 __global__ void __launch_bounds__(256)
@@ -511,6 +841,11 @@ cudaError_t launch_mma(const TadcProgram &P, const TadpPointers &ptrs, cudaStrea
     if (dev < 0 || dev >= 64 || !attr_set[dev]) {
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::SMEM);
         if (e != cudaSuccess) return e;
+        // the warpgroups' register shares must fit into what the block is launched with
+        cudaFuncAttributes at;
+        e = cudaFuncGetAttributes(&at, kern);
+        if (e != cudaSuccess) return e;
+        if (at.numRegs * NT < NCW * 32 * REG_CONV + 128 * REG_MMA) return cudaErrorInvalidConfiguration;
         if (dev >= 0 && dev < 64) attr_set[dev] = true;
     }
     const unsigned tiles_m = ((unsigned)P.M.extent + BM - 1) / BM, tiles_n = ((unsigned)P.N.extent + BN - 1) / BN;
@@ -519,13 +854,36 @@ cudaError_t launch_mma(const TadcProgram &P, const TadpPointers &ptrs, cudaStrea
     return cudaGetLastError();
 }
 
+template <int MA, int MB>
+cudaError_t launch_short(const TadcProgram &P, const TadpPointers &ptrs, unsigned sms, cudaStream_t stream)
+{
+    static bool attr_set[64] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    auto kern = tad_mma_short_kernel<MA, MB>;
+    if (dev < 0 || dev >= 64 || !attr_set[dev]) {
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ShortCfg::SMEM);
+        if (e != cudaSuccess) return e;
+        if (dev >= 0 && dev < 64) attr_set[dev] = true;
+    }
+    const unsigned tiles_m = ((unsigned)P.M.extent + BM - 1) / BM, tiles_n = ((unsigned)P.N.extent + BM - 1) / BM;
+    const unsigned long long items = (unsigned long long)tiles_m * tiles_n * (unsigned)P.Z.extent;
+    if (items >= (1ull << 31)) return cudaErrorInvalidValue;
+    return tad_launch(kern, (unsigned)std::min<unsigned long long>(items, sms), SNT, ShortCfg::SMEM, stream, P, ptrs, tiles_m, tiles_n, (unsigned)items);
+}
+
 }  // namespace
 
 cudaError_t tad_launch_mma(const TadcProgram &P, const TadpPointers &ptrs, unsigned sms, cudaStream_t stream)
 {
     cudaError_t e = cudaErrorInvalidValue;
+    // the pipelined kernel from four tiles per SM on (8192 x 8192 x 34 forward 220 -> 148 us, staged adjoint 280 -> 181 us);
+    // with one or two tiles a block has nothing to overlap (1301 x 2477 x 23: 18 us as blocks of one tile, 23 us here)
+    const unsigned long long tiles = (unsigned long long)((P.M.extent + BM - 1) / BM) * (unsigned)((P.N.extent + BM - 1) / BM) * (unsigned)P.Z.extent;
+    const bool short_pays = P.K.extent <= KS && P.ksplit <= 1 && P.N.extent > 64 && tiles >= 4ull * sms;
 #define TAD_MMA_CASE(MA, MB)                                                                                              \
-    case MA * 4 + MB: e = P.N.extent <= 64 ? launch_mma<64, MA, MB>(P, ptrs, stream) : launch_mma<128, MA, MB>(P, ptrs, stream); break;
+    case MA * 4 + MB: e = short_pays ? launch_short<MA, MB>(P, ptrs, sms, stream) : P.N.extent <= 64 ? launch_mma<64, MA, MB>(P, ptrs, stream) : launch_mma<128, MA, MB>(P, ptrs, stream); break;
 #define TAD_MMA_ROW(MA) TAD_MMA_CASE(MA, TM_ROW) TAD_MMA_CASE(MA, TM_KVEC) TAD_MMA_CASE(MA, TM_K) TAD_MMA_CASE(MA, TM_RVEC)
     switch (P.modeA * 4 + P.modeB) { TAD_MMA_ROW(TM_ROW) TAD_MMA_ROW(TM_KVEC) TAD_MMA_ROW(TM_K) default: break; }
 #undef TAD_MMA_ROW

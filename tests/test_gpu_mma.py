@@ -43,6 +43,13 @@ def test_matrix_products(ni, nk, nj, transposed):
     _close(dy, want.T if transposed else want, scale.T if transposed else scale, ni, "dy")
 
 
+@pytest.mark.parametrize("ni,nk,nj", [(3077, 34, 3201), (3200, 64, 3072), (200, 17, 38000)])
+def test_one_stage_contractions(ni, nk, nj):
+    """At most 64 terms and enough tiles for the pipelined kernel: ragged edges in both directions, full and cut stages."""
+    test_matrix_products(ni, nk, nj, False)
+    test_matrix_products(ni, nk, nj, True)
+
+
 @pytest.mark.parametrize("nb,nc,no,nt,nu", [(2, 64, 72, 130, 5), (3, 13, 65, 257, 3), (1, 20, 128, 64, 4)])
 def test_strided_convolution(nb, nc, no, nt, nu):
     """Guards, several digits per group and strided stores (the residue classes of dx)."""
@@ -62,17 +69,18 @@ def test_strided_convolution(nb, nc, no, nt, nu):
         _close(got, w, s, n, what)
 
 
-def test_non_finite_operands():
+@pytest.mark.parametrize("nk,nj", [(70, 140), (33, 76000)])
+def test_non_finite_operands(nk, nj):
     """Infinities and NaNs of the operands, and values beyond the bf16 range, give what the definition gives."""
-    e = W.ex_matmul(130, 70, 140)
+    e = W.ex_matmul(130, nk, nj)
     args, df = W.make_inputs(e, ("normal", 0, 1), seed=3)
     x, y = args
     y[y.abs() < 1e-3] = 0.5
-    x[3, 5], x[40, 69], x[129, 0], x[77, 7] = math.inf, -math.inf, math.nan, 3.4028234e38
+    x[3, 5], x[40, nk - 1], x[129, 0], x[77, 7] = math.inf, -math.inf, math.nan, 3.4028234e38
     y[7] = 0.25
     f = torch.from_numpy(GpuRun(e, args, df).forward())
     assert torch.equal(f[3], math.inf * torch.sign(y[5]))
-    assert torch.equal(f[40], -math.inf * torch.sign(y[69]))
+    assert torch.equal(f[40], -math.inf * torch.sign(y[nk - 1]))
     assert bool(f[129].isnan().all())
     want = x.double() @ y.double()
     rows = [r for r in range(130) if r not in (3, 40, 129)]
