@@ -30,9 +30,12 @@ struct alignas(16) TadlProgram {
     int32_t zsplit;                        // > 1: grid.y shares, each writing a plane of partial sums; share = s0 * n_share[1] + s1
     int32_t n_share[2], chunk_shift[2], zbox_lo[2];
     // the box of loop l is cut into pieces of 2^chunk_shift values counted from zbox_lo; share s_l of an output walks the
-    // s_l-th piece counted from the one its range starts in (cut to the range), so that neighbouring outputs stay in step
+    // s_l-th piece counted from the one its range starts in (cut to the range).  In mode 0 the lanes of a row walk the union
+    // of their ranges together and share s_l also takes every n_share[l]-th piece behind its first
     int32_t part_limit, part_coef[TADP_MAX_VARS];
+    int32_t lane_stride, lane_skew;        // mode 0: lane l of a row owns output s l + r of the lane variable and runs the inner loop at z = u + t l:
+                                           // at one u the warp's reads of load 0 are then consecutive whatever its index map
     int32_t stream;                        // load 0 is consecutive along the lanes: read with evict-first loads
-    int32_t unroll;                        // terms a thread keeps in flight: 2, 4 or 8
+    int32_t unroll;                        // mode 1: terms a thread keeps in flight: 2, 4 or 8
     int32_t live_plane;                    // share 0 also writes plane zsplit: 1 where the guards hold (outputs of masked gradients that exist)
 };

@@ -218,7 +218,32 @@ bool try_line(Gen &g, Kernel &k, int root, int scale, bool allow_split, const st
     // a masked gradient's box also holds positions that are no elements (their offsets may fall on real ones): the
     // reduction writes only where the guards held
     P.unroll = 4;
-    P.stream = (P.mode == 1 ? std::abs(P.loads[0].cz[l_in]) == 1 : std::abs(P.loads[0].coef[P.lane_var]) == 1) ? 1 : 0;
+    // lanes whose reads of load 0 are consecutive: along the lane variable as it is, or every s-th output of it with the
+    // inner loop shifted by t per lane, where  s coef + t step = +-1
+    P.lane_stride = 1; P.lane_skew = 0;
+    bool unit = P.mode == 1 ? std::abs(B.cz[l_in]) == 1 : std::abs(B.coef[lane]) == 1;
+    if (P.mode == 0 && !unit && B.cz[l_in] != 0 && B.coef[lane] != 0)
+        for (int s = 1; s <= 8 && !unit && prog.outer_ext[lane] / s >= 32; ++s)
+            for (int64_t want : {1, -1}) {
+                const int64_t rest = want - (int64_t)s * B.coef[lane];
+                if (unit || rest % B.cz[l_in] || std::llabs(rest / B.cz[l_in]) > 8) continue;
+                unit = true; P.lane_stride = s; P.lane_skew = (int32_t)(rest / B.cz[l_in]);
+            }
+    P.stream = unit ? 1 : 0;
+    // pieces per thread: as many as leave the GPU two rounds of resident warps, the set-up of an output and its plane of
+    // partial sums being paid once for all of them (every n-th piece goes to the same thread: outputs with short ranges
+    // give every share the same work)
+    const int pieces = P.zsplit;
+    if (P.mode == 0) {
+        double warps = outputs / 32.0 * P.zsplit;
+        for (int l : {l_in, 0})
+            while (P.n_share[l] > 1 && warps >= 2.0 * 148 * 48) {
+                const int less = (P.n_share[l] + 1) / 2;
+                warps *= (double)less / P.n_share[l];
+                P.n_share[l] = less;
+            }
+        P.zsplit = P.n_share[0] * P.n_share[1];
+    }
     P.live_plane = (P.zsplit > 1 && prog.write_only_live) ? 1 : 0;
     if (P.zsplit <= 1) prog.write_only_live = 0;
     k.line = {P};
@@ -226,8 +251,8 @@ bool try_line(Gen &g, Kernel &k, int root, int scale, bool allow_split, const st
     prog.zsplit = P.zsplit; prog.part_limit = P.part_limit; prog.n_outer = g.n_outer;
     for (int v = 0; v < g.n_outer; ++v) prog.part_coef[v] = P.part_coef[v];
     char line[256];
-    std::snprintf(line, sizeof line, "; line sums: %d loads x %d loops, outer factor of %d loads, %s, lanes along variable %d, %d shares, %d guards\n",
-                  P.n_loads, P.n_loops, P.n_scale, P.mode == 1 ? "a warp per output" : "a thread per output", P.lane_var, P.zsplit, P.n_guards);
+    std::snprintf(line, sizeof line, "; line sums: %d loads x %d loops, outer factor of %d loads, %s, lanes along variable %d, %d shares, %d guards, %d planes, lane stride %d skew %d\n",
+                  P.n_loads, P.n_loops, P.n_scale, P.mode == 1 ? "a warp per output" : "a thread per output", P.lane_var, pieces, P.n_guards, P.zsplit, P.lane_stride, P.lane_skew);
     k.listing = line;
     for (int i = 0; i < P.n_loads; ++i) {
         std::snprintf(line, sizeof line, ";   load %d ptr=%d base=%d coef=[%d %d %d %d] step=[%d %d]%s\n", i, P.loads[i].ptr, P.loads[i].base, P.loads[i].coef[0],
