@@ -331,7 +331,7 @@ tad_status zero_fill(float *out, int64_t n, cudaStream_t stream)
 
 // streams and events of tad_step_host, owned by a plan
 struct HostStep {
-    static constexpr int N_EVENTS = 4 + TADP_MAX_PTRS;
+    static constexpr int N_EVENTS = 5 + TADP_MAX_PTRS;
     cudaStream_t in = nullptr, out = nullptr;
     cudaEvent_t ev[N_EVENTS] = {};
     void release()
@@ -544,6 +544,34 @@ tad_status tad_backward(const tad_plan *plan, const float *const *args, const fl
     return TAD_OK;
 }
 
+// Elements of an argument that lie on one line  base + step i, 0 <= i < n,  and are the only ones that the expression reads
+// (a diagonal, a strided vector), when they are few enough that a copy of single elements beats a copy of the tensor:
+// 2048 elements of a 2048 x 2048 matrix 12 us instead of 308 us over PCIe, 8192 of 8192 x 8192 68 us instead of 4.8 ms.
+static bool read_line(const tad_plan *plan, int arg, int64_t &base, int64_t &step, int64_t &n)
+{
+    bool found = false;
+    for (const tad::AccessPlan &ap : plan->access) {
+        if (ap.arg != arg || !ap.used) continue;
+        int64_t b = 0, st = 1, s = 0, len = 1;
+        std::vector<int64_t> coef(ap.n, 0);
+        for (int r = ap.rank - 1; r >= 0; --r) {
+            b += st * ap.off[r];
+            for (int c = 0; c < ap.n; ++c) coef[c] += st * ap.A(r, c);
+            st *= plan->arg_shape[arg][r];
+        }
+        for (int c = 0; c < ap.n; ++c) {
+            if (coef[c] == 0) continue;
+            if (ap.box_hi[c] == ap.box_lo[c]) { b += coef[c] * ap.box_lo[c]; continue; }
+            if (s) return false;
+            s = std::abs(coef[c]); len = ap.box_hi[c] - ap.box_lo[c] + 1;
+            b += coef[c] * (coef[c] > 0 ? ap.box_lo[c] : ap.box_hi[c]);
+        }
+        if (!s || (found && (b != base || s != step || len != n))) return false;
+        base = b; step = s; n = len; found = true;
+    }
+    return found && step >= 64 && n >= 2 && step * 4 < (int64_t(1) << 31);
+}
+
 size_t tad_staging_bytes(const tad_plan *plan)
 {
     if (!plan) return 0;
@@ -594,19 +622,33 @@ tad_status tad_step_host(const tad_plan *plan, const float *const *h_args, const
         cudaEvent_t event() { return used < HostStep::N_EVENTS ? hs->ev[used++] : nullptr; }
     } side{static_cast<HostStep *>(plan->host_step)};
     side.in = side.hs->in; side.out = side.hs->out;
-    cudaEvent_t ev_start = side.event(), ev_args = side.event(), ev_df = side.event(), ev_f = side.event();
-    if (!ev_start || !ev_args || !ev_df || !ev_f) { tad::set_error("event creation failed"); return TAD_ERR_CUDA; }
+    cudaEvent_t ev_start = side.event(), ev_args = side.event(), ev_df = side.event(), ev_f = side.event(), ev_zero = side.event();
+    if (!ev_start || !ev_args || !ev_df || !ev_f || !ev_zero) { tad::set_error("event creation failed"); return TAD_ERR_CUDA; }
     // whatever the caller queued on its stream comes first
     if (!check(cudaEventRecord(ev_start, stream), "event record") || !check(cudaStreamWaitEvent(side.in, ev_start, 0), "stream wait") ||
         !check(cudaStreamWaitEvent(side.out, ev_start, 0), "stream wait")) return TAD_ERR_CUDA;
     cur = static_cast<char *>(staging) + pad(tad_workspace_bytes(plan));
+    bool line_of[TADP_MAX_PTRS] = {}, zeros_ahead = false;
     for (int a = 0; a < plan->n_args; ++a) {
         const size_t bytes = size_t(plan->arg_elems[a]) * 4;
         float *dx = reinterpret_cast<float *>(cur); cur += pad(bytes);
         float *dg = reinterpret_cast<float *>(cur); cur += pad(bytes);
         if (!h_args[a]) { tad::set_error("NULL host argument"); return TAD_ERR_INVALID_ARG; }
-        if (!check(cudaMemcpyAsync(dx, h_args[a], bytes, cudaMemcpyHostToDevice, side.in), "copy of an argument")) return TAD_ERR_CUDA;
+        int64_t base, step, n;
+        const bool line = read_line(plan, a, base, step, n);
+        const cudaError_t ce = line ? cudaMemcpy2DAsync(dx + base, size_t(step) * 4, h_args[a] + base, size_t(step) * 4, 4, size_t(n), cudaMemcpyHostToDevice, side.in)
+                                    : cudaMemcpyAsync(dx, h_args[a], bytes, cudaMemcpyHostToDevice, side.in);
+        if (!check(ce, "copy of an argument")) return TAD_ERR_CUDA;
         d_args[a] = dx; d_dargs[a] = h_dargs[a] ? dg : nullptr;
+        // a gradient that is zero off the line: its zeros come down while the inputs go up, the line itself at the end
+        line_of[a] = line && h_dargs[a] && plan->arg_zero_fill[a];
+        if (line_of[a]) {
+            const tad_status zs = zero_fill(dg, plan->arg_elems[a], side.out);
+            if (zs != TAD_OK) return zs;
+            if (!check(cudaEventRecord(ev_zero, side.out), "event record") ||
+                !check(cudaMemcpyAsync(h_dargs[a], dg, bytes, cudaMemcpyDeviceToHost, side.out), "copy of a gradient")) return TAD_ERR_CUDA;
+            zeros_ahead = true;
+        }
     }
     if (!check(cudaEventRecord(ev_args, side.in), "event record")) return TAD_ERR_CUDA;
     if (!check(cudaMemcpyAsync(d_df, h_df, fbytes, cudaMemcpyHostToDevice, side.in), "copy of df")) return TAD_ERR_CUDA;
@@ -624,6 +666,8 @@ tad_status tad_step_host(const tad_plan *plan, const float *const *h_args, const
     }
     if (plan->opt.saved_forward) d_args[plan->n_args] = d_f;      // the backward pass reads f
     if (!check(cudaStreamWaitEvent(stream, ev_df, 0), "stream wait")) return TAD_ERR_CUDA;
+    // (the kernels write the line after its zeros are there; the copy of the zeros may still run, the line follows it)
+    if (zeros_ahead && !check(cudaStreamWaitEvent(stream, ev_zero, 0), "stream wait")) return TAD_ERR_CUDA;
     if (plan->opt.debug_bounds && !check(cudaMemsetAsync(ws, 0, 256, stream), "clearing the debug word")) return TAD_ERR_CUDA;
     bool need_stage = false;
     for (int a = 0; a < plan->n_args; ++a)
@@ -637,6 +681,12 @@ tad_status tad_step_host(const tad_plan *plan, const float *const *h_args, const
     int order[TADP_MAX_PTRS];
     for (int a = 0; a < plan->n_args; ++a) order[a] = a;
     std::stable_sort(order, order + plan->n_args, [&](int x, int y) { return plan->arg_elems[x] > plan->arg_elems[y]; });
+    auto copy_gradient = [&](int a) {
+        int64_t base, step, n;
+        if (line_of[a] && read_line(plan, a, base, step, n))
+            return cudaMemcpy2DAsync(h_dargs[a] + base, size_t(step) * 4, d_dargs[a] + base, size_t(step) * 4, 4, size_t(n), cudaMemcpyDeviceToHost, side.out);
+        return cudaMemcpyAsync(h_dargs[a], d_dargs[a], size_t(plan->arg_elems[a]) * 4, cudaMemcpyDeviceToHost, side.out);
+    };
     for (int oi = 0; oi < plan->n_args; ++oi) {
         const int a = order[oi];
         if (!d_dargs[a]) continue;
@@ -645,8 +695,7 @@ tad_status tad_step_host(const tad_plan *plan, const float *const *h_args, const
         cudaEvent_t ev_g = side.event();
         if (!ev_g) { tad::set_error("event creation failed"); return TAD_ERR_CUDA; }
         if (!check(cudaEventRecord(ev_g, stream), "event record") || !check(cudaStreamWaitEvent(side.out, ev_g, 0), "stream wait") ||
-            !check(cudaMemcpyAsync(h_dargs[a], d_dargs[a], size_t(plan->arg_elems[a]) * 4, cudaMemcpyDeviceToHost, side.out), "copy of a gradient"))
-            return TAD_ERR_CUDA;
+            !check(copy_gradient(a), "copy of a gradient")) return TAD_ERR_CUDA;
     }
     if (!check(cudaStreamSynchronize(stream), "stream synchronise") || !check(cudaStreamSynchronize(side.out), "stream synchronise") ||
         !check(cudaStreamSynchronize(side.in), "stream synchronise")) return TAD_ERR_CUDA;
