@@ -48,6 +48,7 @@ tad_status tad_compile(const tad_expr *expr, const tad_options *opt, tad_plan **
         p->backward.reserve(p->access.size());
         for (int q = 0; q < (int)p->access.size(); ++q)
             if (p->access[q].used) generate_backward(*p, q);
+        share_auxiliaries(*p);
     });
     if (st != TAD_OK) { delete p; return st; }
     *out = p;

@@ -755,7 +755,7 @@ int assign_temporaries(Gen &g, int root, int scale)
 // -> points): intro 64 x 64 x 5 db 110 -> 12, 203 x 157 x 7 db 366 -> 12, da 23 -> 12, forward 26 -> 19; 700 x 700 x 8
 // (2^21.9) forward 44 -> 31, db 136 -> 41; all elementary functions over 200003 outputs: forward 79 -> 36, dv 131 -> 80.
 // Plain element-wise programs (no sums, no temporaries) have the element-wise kernel, which is as fast from 2^16 outputs on.
-constexpr double POINT_SPACE = double(1 << 22), POINT_PLAIN = double(1 << 16);
+constexpr double POINT_SPACE = double(1 << 22), POINT_PLAIN = double(1 << 16), POINT_CHAIN = 148.0 * 512;
 
 bool try_points(Gen &g, Kernel &k, int root, int scale, bool allow_split, const std::vector<std::vector<TadpRow>> &lower,
                 const std::vector<std::vector<TadpRow>> &upper, const std::vector<TadpRow> &guards)
@@ -783,12 +783,39 @@ bool try_points(Gen &g, Kernel &k, int root, int scale, bool allow_split, const 
     const int n_temps = assign_temporaries(g, root, scale);
     Emitter em(g);
     int body = 0, tail = 0;
-    em.temps_of_level(0);
+    // An element-wise kernel around one sum, with too few outputs to fill the GPU by themselves: the summands become terms
+    // and what is computed from the sum runs behind it (exp(-sum ...) of 64 x 64 outputs 13 -> 6 us).
+    int inner_sum = -1;
+    std::vector<char> on_sum(g.inst.size(), 0);
+    if (g.kappa == 0 && g.inst[root].op != I_SUM && scale < 0) {
+        int n_outer_sums = 0;
+        for (int i = 0; i < (int)g.inst.size(); ++i) if (g.inst[i].uses && g.inst[i].op == I_SUM && g.inst[i].home_sum < 0) { ++n_outer_sums; inner_sum = i; }
+        double outs = 1;
+        for (int v = 0; v < g.n_outer; ++v) outs *= (double)ext[v];
+        if (n_outer_sums != 1 || outs > POINT_CHAIN || g.inst[inner_sum].hi - g.inst[inner_sum].lo < 3) inner_sum = -1;
+    }
+    if (inner_sum >= 0) {
+        on_sum[inner_sum] = 1;
+        for (int i = inner_sum + 1; i < (int)g.inst.size(); ++i)
+            if (g.inst[i].uses) for (int c : {g.inst[i].a, g.inst[i].b}) if (c >= 0 && on_sum[c]) on_sum[i] = 1;
+        if (!on_sum[root]) return false;
+    }
+    auto outer_temps = [&](bool behind) {
+        for (int i = 0; i < (int)g.inst.size(); ++i) {
+            const Inst &in = g.inst[i];
+            if (in.temp < 0 || !in.uses || in.home_sum >= 0 || in.zlevel != 0 || i == inner_sum || (on_sum[i] != 0) != behind) continue;
+            em.body(i);
+            em.emit(P_STT, in.temp, 0, 0, -1);
+        }
+    };
+    const int sum_temp = inner_sum < 0 ? -1 : g.inst[inner_sum].temp >= 0 ? g.inst[inner_sum].temp : n_temps;
+    const int all_temps = n_temps + (sum_temp == n_temps ? 1 : 0);
+    outer_temps(false);
     body = (int)em.code.size();
     for (int l = 0; l < g.kappa; ++l) em.temps_of_level(l + 1);
     // a term that is a sum with a constant range: its summands are terms
-    int top = root;
-    while (g.inst[top].op == I_SUM && g.inst[top].temp < 0 && (int)zv.size() < TADQ_MAX_VARS) {
+    int top = inner_sum >= 0 ? inner_sum : root;
+    while (g.inst[top].op == I_SUM && (g.inst[top].temp < 0 || top == inner_sum) && (int)zv.size() < TADQ_MAX_VARS) {
         const Inst &in = g.inst[top];
         if (in.hi < in.lo) return false;
         lo[in.var] = in.lo; ext[in.var] = in.hi - in.lo + 1;
@@ -799,10 +826,18 @@ bool try_points(Gen &g, Kernel &k, int root, int scale, bool allow_split, const 
     if (g.inst[top].op == I_MUL && g.inst[top].temp < 0) { em.expr(g.inst[top].a); em.expr(g.inst[top].b); em.emit(P_MACC, 0, 0, 0, -2); }
     else { em.expr(top); em.emit(P_ACC, 0, 0, 0, -1); }
     tail = (int)em.code.size();
+    if (inner_sum >= 0) {
+        const int own = g.inst[inner_sum].temp;
+        g.inst[inner_sum].temp = sum_temp;
+        outer_temps(true);
+        em.expr(root);
+        em.emit(P_ACC, 0, 0, 0, -1);
+        g.inst[inner_sum].temp = own;
+    }
     if (scale >= 0) { em.expr(scale); em.emit(P_SCALE, 0, 0, 0, -1); }
     const int n = (int)em.code.size();
     if (em.depth != 0 || n > TADQ_MAX_STEPS || (int)g.loads.size() > TADQ_MAX_LOADS || g.n_outer + (int)zv.size() > TADQ_MAX_VARS) return false;
-    if (em.max_depth + n_temps > TADQ_MAX_SLOTS) return false;
+    if (em.max_depth + all_temps > TADQ_MAX_SLOTS) return false;
     // ---- the size of the index space, sums inside the term included ----
     std::vector<int> sv;
     double points = 1, terms = 1, inner = 1;
@@ -913,14 +948,15 @@ bool try_points(Gen &g, Kernel &k, int root, int scale, bool allow_split, const 
         Q.steps[w] = st;
     }
     Q.body = body; Q.tail = tail; Q.n_steps = n;
-    Q.n_slots = std::max(1, em.max_depth + n_temps);
+    Q.n_slots = std::max(1, em.max_depth + all_temps);
+    Q.value_slot = inner_sum >= 0 ? em.max_depth + sum_temp : -1;
     Q.out_base = prog.out_base; Q.accumulate = prog.accumulate;
     // ---- schedule: lanes per output until the GPU has a few warps per scheduler, shares where even that is too few blocks ----
     Q.lt = 1; Q.zsplit = 1; Q.along_terms = 0; Q.unroll = 1;
     const bool sums = g.kappa >= 1 || Q.n_z > 0;
     if (sums) {
         Q.along_terms = !zv.empty() && unit_of_big(zv.back()) && !(!ov.empty() && unit_of_big(ov.back())) ? 1 : 0;
-        Q.unroll = terms >= 4 ? 4 : 1;
+        Q.unroll = terms >= 4 && inner_sum < 0 ? 4 : 1;
         if (Q.along_terms) while (Q.lt < 32 && Q.lt < terms) Q.lt *= 2;
         while (Q.lt < 256 && points * Q.lt < 148.0 * 512.0 && Q.lt * Q.unroll < terms) Q.lt *= 2;
         if (Q.lt == 1 && terms == 1) Q.lt = 2;                // (a single term still goes through the summing path)
@@ -928,7 +964,7 @@ bool try_points(Gen &g, Kernel &k, int root, int scale, bool allow_split, const 
         for (int v = g.n_outer - 1; v >= 0; --v) { prog.part_coef[v] = to_i32(cells); if (at[v] >= 0) Q.part_coef[at[v]] = to_i32(cells); cells = mul_ck(cells, ext[v]); }
         const double blocks = std::ceil(points * Q.lt / 256.0), batches = terms / ((double)Q.lt * Q.unroll);
         if (allow_split && g.kappa >= 1 && blocks < 148 && batches >= 8 && cells <= (1 << 20))
-            Q.zsplit = (int32_t)std::max(1.0, std::min({128.0, std::floor(296.0 / blocks), std::floor(batches / 4)}));
+            Q.zsplit = (int32_t)std::max(1.0, std::min({128.0, std::floor(148.0 * 5 / blocks), std::floor(batches / 1.5)}));
         Q.part_limit = to_i32(cells);
     } else if (points >= 131072) Q.unroll = 4;
     prog.zsplit = Q.zsplit; prog.part_limit = Q.part_limit; prog.n_outer = g.n_outer; prog.write_only_live = 0;
@@ -1608,6 +1644,69 @@ void generate_backward(tad_plan &p, int q)
     finish_stats(g, k, true, p.arg_elems[ap.arg], terms, zero_fill && first_of_arg);
     account(p, k);
     if (zero_fill && first_of_arg) k.stats.n_launches += 1;
+}
+
+// ---------------------------------------------------------------------------------------
+namespace {
+
+template <class T> bool same_bytes(const std::vector<T> &a, const std::vector<T> &b)
+{
+    return a.size() == b.size() && (a.empty() || !std::memcmp(a.data(), b.data(), a.size() * sizeof(T)));
+}
+
+// reads nothing but arguments, df, staged adjoints and the saved forward output
+bool reads_inputs_only(const tad_plan &p, const Kernel &k)
+{
+    const int slot0 = p.n_args + 1 + (int)p.stages.size();
+    auto input = [&](int slot) { return slot < slot0 || (p.opt.saved_forward && slot == TADP_F_SLOT); };
+    if (!k.pre.empty() || !k.aux.empty()) return false;
+    if (!k.contract.empty()) {
+        for (const TadcProgram &c : k.contract) if (!input(c.ptrA) || !input(c.ptrB) || c.n_epi) return false;
+        return true;
+    }
+    if (!k.ew.empty()) { for (int i = 0; i < k.ew[0].n_loads; ++i) if (!input(k.ew[0].loads[i].ptr)) return false; return true; }
+    if (!k.point.empty()) { for (const TadqLoad &L : k.point[0].loads) if (!input(L.ptr)) return false; return true; }
+    if (!k.line.empty()) {
+        for (int i = 0; i < k.line[0].n_loads; ++i) if (!input(k.line[0].loads[i].ptr)) return false;
+        for (int i = 0; i < k.line[0].n_scale; ++i) if (!input(k.line[0].scale[i].ptr)) return false;
+        return true;
+    }
+    for (int i = 0; i < k.prog.n_loads; ++i) if (!input(k.prog.loads[i].ptr)) return false;
+    return true;
+}
+
+bool same_kernel(const Kernel &a, const Kernel &b)
+{
+    if (a.vec != b.vec || a.vec_u != b.vec_u || a.rich != b.rich) return false;
+    if (!same_bytes(a.contract, b.contract) || !same_bytes(a.ew, b.ew) || !same_bytes(a.point, b.point) || !same_bytes(a.line, b.line)) return false;
+    return !a.contract.empty() || !a.ew.empty() || !std::memcmp(&a.prog, &b.prog, sizeof a.prog);
+}
+
+}  // namespace
+
+void share_auxiliaries(tad_plan &p)
+{
+    struct Member { Kernel *owner, *pre; };
+    std::vector<std::vector<Member>> groups;
+    for (Kernel &k : p.backward)
+        for (Kernel &pk : k.pre) {
+            int writers = 0;
+            for (const Kernel &o : k.pre) writers += o.out_aux == pk.out_aux;
+            if (writers != 1 || !reads_inputs_only(p, pk)) continue;
+            bool placed = false;
+            for (auto &g : groups)
+                if (!placed && g[0].owner != &k && g.back().owner != &k && same_kernel(*g[0].pre, pk) &&
+                    g[0].owner->aux[g[0].pre->out_aux].bytes == k.aux[pk.out_aux].bytes) { g.push_back({&k, &pk}); placed = true; }
+            if (!placed) groups.push_back({{&k, &pk}});
+        }
+    size_t cursor = (p.aux_bytes + 255) & ~size_t(255);
+    for (auto &g : groups) {
+        if (g.size() < 2) continue;
+        for (Member &m : g) { m.pre->shared = p.n_shared; m.owner->aux[m.pre->out_aux].offset = cursor; }
+        cursor += (g[0].owner->aux[g[0].pre->out_aux].bytes + 255) & ~size_t(255);
+        ++p.n_shared;
+    }
+    if (p.n_shared) p.aux_bytes = cursor;
 }
 
 }  // namespace tad

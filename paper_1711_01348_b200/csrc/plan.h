@@ -83,6 +83,8 @@ struct Kernel {
     size_t aux_bytes = 0;
     std::vector<Kernel> pre;
     int out_aux = -1;
+    int shared = -1;           // an auxiliary kernel whose result other gradients need too: its number in the plan (its tensor then
+                               // lies behind the kernels' own areas)
     KernelStats stats;
     std::string listing;
 };
@@ -112,7 +114,8 @@ struct tad_plan {
     std::vector<std::vector<int>> arg_kernels;  // per argument: indices into backward, launch order
     std::vector<bool> arg_zero_fill;            // the gradient is cleared before its kernels add into it
     size_t partial_bytes = 0;                   // workspace for the partial sums of split summations (largest kernel)
-    size_t aux_bytes = 0;                       // workspace for auxiliary tensors (largest kernel)
+    size_t aux_bytes = 0;                       // workspace for auxiliary tensors (largest kernel, then the shared ones)
+    int n_shared = 0;                           // auxiliary kernels that several gradients have in common
     mutable void *side = nullptr;               // second stream and its events (independent memory-bound passes run beside a contraction)
     mutable void *host_step = nullptr;          // streams and events of tad_step_host, created by its first call
 };
@@ -133,6 +136,9 @@ size_t enumerate_access(const tad_plan &p, int q, const int64_t *beta, std::vect
 void generate_forward(tad_plan &p);
 void generate_stages(tad_plan &p);
 void generate_backward(tad_plan &p, int q);
+// auxiliary tensors that several gradients compute alike (row sums of the staged adjoint, function tables) get one place
+// each, so that one backward call computes them once
+void share_auxiliaries(tad_plan &p);
 
 // print.cpp: the expression (which = -1) or the derivative through index expression `which` in the notation of Sec. 6
 std::string print_expression(const tad_plan &p, int which, const char *const *arg_names, const char *const *idx_names);

@@ -154,6 +154,19 @@ tad_point_kernel(const __grid_constant__ TadqProgram P, const __grid_constant__ 
     const unsigned lt = (unsigned)P.lt, lo_n = NT / lt;
     const unsigned tl = P.along_terms ? tid % lt : tid / lo_n, ol = P.along_terms ? tid / lt : tid % lo_n;
     const unsigned per = (terms + gridDim.y - 1u) / gridDim.y, t0 = blockIdx.y * per, t1 = min(terms, t0 + per);
+    // fixed-order tree over the term lanes of an output
+    float *red = sm + P.n_slots * NT * U;
+    auto total = [&]() {
+        float sum = acc.v[0];
+#pragma unroll
+        for (int u = 1; u < U; ++u) sum += acc.v[u];
+        red[ol * lt + tl] = sum;
+        __syncthreads();
+        for (unsigned h = lt / 2; h >= 1; h /= 2) {
+            if (tl < h) red[ol * lt + tl] += red[ol * lt + tl + h];
+            __syncthreads();
+        }
+    };
     unsigned live = 0;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
@@ -179,7 +192,18 @@ tad_point_kernel(const __grid_constant__ TadqProgram P, const __grid_constant__ 
             }
             pc = P.body; end = P.tail;
             t += lt * U;
-        } else { pc = P.tail; phase = 3u; }
+        } else {
+            pc = P.tail; phase = 3u;
+            if (P.value_slot >= 0) {
+                // the sum of the output, known to all of its lanes, is a value of the tail
+                total();
+                Vals<U> s;
+#pragma unroll
+                for (int u = 0; u < U; ++u) { s.v[u] = red[ol * lt]; acc.v[u] = 0.f; }
+                slot_put<U>(sm, P.value_slot, s);
+                mask = live;
+            }
+        }
         run_steps<U>(P, ptrs, sm, pc, end, var, mask, X, acc);
     }
     if (!sums) {
@@ -192,20 +216,9 @@ tad_point_kernel(const __grid_constant__ TadqProgram P, const __grid_constant__ 
         }
         return;
     }
-    float sum = acc.v[0];
-#pragma unroll
-    for (int u = 1; u < U; ++u) sum += acc.v[u];
-    // fixed-order tree over the term lanes of an output
-    __syncthreads();
-    float *red = sm;
-    red[ol * lt + tl] = sum;
-    __syncthreads();
-    for (unsigned h = lt / 2; h >= 1; h /= 2) {
-        if (tl < h) red[ol * lt + tl] += red[ol * lt + tl + h];
-        __syncthreads();
-    }
+    if (P.value_slot < 0) total();
     if (tl != 0 || !live) return;
-    sum = red[ol * lt];
+    const float sum = P.value_slot < 0 ? red[ol * lt] : acc.v[0];
     int o = P.out_base; unsigned cell = 0;
 #pragma unroll
     for (int d = 0; d < MV; ++d) { o += P.out_coef[d] * var[d][0]; if (d < P.n_out) cell += (unsigned)(P.part_coef[d] * (var[d][0] - P.lo[d])); }
@@ -217,7 +230,7 @@ template <int U>
 cudaError_t launch_points(const TadqProgram &P, const TadpPointers &ptrs, cudaStream_t stream)
 {
     const bool sums = P.terms > 1 || P.lt > 1;
-    const size_t smem = (size_t)std::max(1, P.n_slots) * NT * U * 4;
+    const size_t smem = ((size_t)P.n_slots * U + 1) * NT * 4;
     const unsigned per = sums ? (unsigned)(NT / P.lt) : (unsigned)NT * U;
     dim3 grid(((unsigned)P.points + per - 1u) / per, (unsigned)std::max(1, P.zsplit), 1u);
     if (smem > 48 * 1024) {
@@ -226,7 +239,7 @@ cudaError_t launch_points(const TadqProgram &P, const TadpPointers &ptrs, cudaSt
         cudaError_t e = cudaGetDevice(&dev);
         if (e != cudaSuccess) return e;
         if (dev < 0 || dev >= 64 || !attr_set[dev]) {
-            e = cudaFuncSetAttribute(tad_point_kernel<U>, cudaFuncAttributeMaxDynamicSharedMemorySize, TADQ_MAX_SLOTS * NT * U * 4);
+            e = cudaFuncSetAttribute(tad_point_kernel<U>, cudaFuncAttributeMaxDynamicSharedMemorySize, (TADQ_MAX_SLOTS * U + 1) * NT * 4);
             if (e != cudaSuccess) return e;
             if (dev >= 0 && dev < 64) attr_set[dev] = true;
         }

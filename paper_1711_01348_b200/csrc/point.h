@@ -45,6 +45,7 @@ struct alignas(16) TadqProgram {
     int32_t s_lo[TADQ_MAX_SUMS], s_hi[TADQ_MAX_SUMS];
     int32_t body, tail, n_steps;           // steps [0, body) once per output, [body, tail) per term, [tail, n_steps) on the sum
     int32_t n_slots, n_sums;
+    int32_t value_slot;                    // >= 0: the finished sum goes to this slot and the tail computes the output from it
     int32_t out_base, out_coef[TADQ_MAX_VARS], accumulate;
     int32_t unroll;                        // points of a thread in flight: 1 or 4
     int32_t lt, along_terms;               // term lanes per output in a block of 256 threads; lanes run along the terms

@@ -219,8 +219,9 @@ bool streams_only(const tad::Kernel &k)
 }
 
 // pending: an event the kernel that writes the output must wait for (the zero fill of its tensor on the second stream)
+// done: shared auxiliary tensors that this call of the library has computed already
 tad_status launch(const tad::Kernel &k, TadpPointers ptrs, bool debug, cudaStream_t stream, char *aux_base = nullptr,
-                  Side *side = nullptr, cudaEvent_t pending = nullptr)
+                  Side *side = nullptr, cudaEvent_t pending = nullptr, std::vector<char> *done = nullptr)
 {
     if (!k.aux.empty()) {
         // auxiliary tensors of this kernel, then the kernels that fill them, in order
@@ -246,6 +247,10 @@ tad_status launch(const tad::Kernel &k, TadpPointers ptrs, bool debug, cudaStrea
         }
         for (int i : order) {
             const tad::Kernel &pk = k.pre[i];
+            if (done && pk.shared >= 0) {
+                if ((*done)[pk.shared]) continue;
+                (*done)[pk.shared] = 1;
+            }
             TadpPointers pp = ptrs;
             pp.out = reinterpret_cast<float *>(aux_base + k.aux[pk.out_aux].offset);
             const bool on_side = use_side && streams_only(pk);
@@ -488,8 +493,8 @@ tad_status tad_backward_stage(const tad_plan *plan, const float *const *args, co
     return TAD_OK;
 }
 
-tad_status tad_backward_arg(const tad_plan *plan, const float *const *args, const float *df,
-                            int32_t arg, float *darg, void *workspace, size_t workspace_bytes, void *cuda_stream)
+static tad_status backward_arg(const tad_plan *plan, const float *const *args, const float *df, int32_t arg, float *darg,
+                               void *workspace, size_t workspace_bytes, void *cuda_stream, std::vector<char> *done)
 {
     if (!plan || !df || !darg || (plan->n_args && !args)) { tad::set_error("NULL argument"); return TAD_ERR_INVALID_ARG; }
     if (arg < 0 || arg >= plan->n_args) { tad::set_error("no such argument"); return TAD_ERR_INVALID_ARG; }
@@ -517,11 +522,17 @@ tad_status tad_backward_arg(const tad_plan *plan, const float *const *args, cons
     ptrs.out = darg;
     for (int ki : plan->arg_kernels[arg]) {
         tad_status st = launch(plan->backward[ki], ptrs, plan->opt.debug_bounds != 0, stream,
-                               workspace ? static_cast<char *>(workspace) + aux_offset(plan) : nullptr, side, pending);
+                               workspace ? static_cast<char *>(workspace) + aux_offset(plan) : nullptr, side, pending, done);
         pending = nullptr;
         if (st != TAD_OK) return st;
     }
     return TAD_OK;
+}
+
+tad_status tad_backward_arg(const tad_plan *plan, const float *const *args, const float *df,
+                            int32_t arg, float *darg, void *workspace, size_t workspace_bytes, void *cuda_stream)
+{
+    return backward_arg(plan, args, df, arg, darg, workspace, workspace_bytes, cuda_stream, nullptr);
 }
 
 tad_status tad_backward(const tad_plan *plan, const float *const *args, const float *df,
@@ -536,9 +547,10 @@ tad_status tad_backward(const tad_plan *plan, const float *const *args, const fl
         tad_status st = tad_backward_stage(plan, args, df, workspace, workspace_bytes, cuda_stream);
         if (st != TAD_OK) return st;
     }
+    std::vector<char> done(plan->n_shared, 0);
     for (int a = 0; a < plan->n_args; ++a) {
         if (!dargs[a]) continue;
-        tad_status st = tad_backward_arg(plan, args, df, a, dargs[a], workspace, workspace_bytes, cuda_stream);
+        tad_status st = backward_arg(plan, args, df, a, dargs[a], workspace, workspace_bytes, cuda_stream, &done);
         if (st != TAD_OK) return st;
     }
     return TAD_OK;
@@ -687,10 +699,11 @@ tad_status tad_step_host(const tad_plan *plan, const float *const *h_args, const
             return cudaMemcpy2DAsync(h_dargs[a] + base, size_t(step) * 4, d_dargs[a] + base, size_t(step) * 4, 4, size_t(n), cudaMemcpyDeviceToHost, side.out);
         return cudaMemcpyAsync(h_dargs[a], d_dargs[a], size_t(plan->arg_elems[a]) * 4, cudaMemcpyDeviceToHost, side.out);
     };
+    std::vector<char> done(plan->n_shared, 0);
     for (int oi = 0; oi < plan->n_args; ++oi) {
         const int a = order[oi];
         if (!d_dargs[a]) continue;
-        st = tad_backward_arg(plan, d_args, d_df, a, d_dargs[a], ws, tad_workspace_bytes(plan), stream);
+        st = backward_arg(plan, d_args, d_df, a, d_dargs[a], ws, tad_workspace_bytes(plan), stream, &done);
         if (st != TAD_OK) return st;
         cudaEvent_t ev_g = side.event();
         if (!ev_g) { tad::set_error("event creation failed"); return TAD_ERR_CUDA; }

@@ -32,6 +32,10 @@ CASES = {
     "shares": lambda: W.ex_all_ops(60001),
     "four_points": lambda: W.ex_all_ops(131073),
     "shared_sum": lambda: _shared_sum(37, 53, 6),
+    # the sum as terms and a tail behind it: values before, inside and behind the sum, at few and at many outputs
+    "tail_behind_sum": lambda: _shared_sum(3, 7, 45),
+    "tail_many_outputs": lambda: _shared_sum(151, 400, 4),
+    "tail_all_functions": lambda: W.intro(40, 31, 33),
 }
 
 
