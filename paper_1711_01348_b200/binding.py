@@ -180,10 +180,7 @@ class Plan:
     # ---- device entry points (pointers are integers, e.g. torch.Tensor.data_ptr()) ----
     @staticmethod
     def _ptr_array(ptrs: Sequence[Optional[int]]):
-        arr = (C.c_void_p * max(1, len(ptrs)))()
-        for i, p in enumerate(ptrs):
-            arr[i] = p if p else None
-        return arr
+        return (C.c_void_p * max(1, len(ptrs)))(*[p or None for p in ptrs])
 
     def workspace_bytes(self) -> int:
         return int(lib.tad_workspace_bytes(self._h))

@@ -755,10 +755,10 @@ int assign_temporaries(Gen &g, int root, int scale)
 // -> points): intro 64 x 64 x 5 db 110 -> 12, 203 x 157 x 7 db 366 -> 12, da 23 -> 12, forward 26 -> 19; 700 x 700 x 8
 // (2^21.9) forward 44 -> 31, db 136 -> 41; all elementary functions over 200003 outputs: forward 79 -> 36, dv 131 -> 80.
 // Plain element-wise programs (no sums, no temporaries) have the element-wise kernel, which is as fast from 2^16 outputs on.
-constexpr double POINT_SPACE = double(1 << 22), POINT_PLAIN = double(1 << 16), POINT_CHAIN = 148.0 * 512;
+constexpr double POINT_SPACE = double(1 << 22), POINT_PLAIN = double(1 << 16), POINT_CHAIN = 148.0 * 512, POINT_AHEAD = double(1 << 17);
 
 bool try_points(Gen &g, Kernel &k, int root, int scale, bool allow_split, const std::vector<std::vector<TadpRow>> &lower,
-                const std::vector<std::vector<TadpRow>> &upper, const std::vector<TadpRow> &guards)
+                const std::vector<std::vector<TadpRow>> &upper, const std::vector<TadpRow> &guards, double limit = POINT_SPACE)
 {
     if (g.p.opt.debug_bounds || root < 0 || !guards.empty()) return false;
     TadpProgram &prog = k.prog;
@@ -850,7 +850,7 @@ bool try_points(Gen &g, Kernel &k, int root, int scale, bool allow_split, const 
     if (sv.size() > TADQ_MAX_SUMS) return false;
     for (int v = 0; v < g.n_outer; ++v) points *= (double)ext[v];
     for (int v : zv) terms *= (double)ext[v];
-    if (points * terms * inner > POINT_SPACE) return false;
+    if (points * terms * inner > limit) return false;
     // plain element-wise programs have a kernel of their own, which a few thousand outputs do not fill
     if (g.kappa == 0 && zv.empty() && sv.empty() && n_temps == 0 && points > POINT_PLAIN) return false;
     // every offset the kernel can form must lie inside its tensor
@@ -1022,6 +1022,13 @@ void emit_kernel(Gen &g, Kernel &k, int root, const std::vector<std::vector<Tadp
     if (try_contraction(g, k, root, scale, allow_split, lower, upper, guards)) return;
     // sums that can be pushed inside the term (Sec. 6's missing clean-up step): auxiliary kernels + a smaller kernel
     if (may_factor && try_factoring(g, k, root, scale, allow_split, lower, upper, guards)) return;
+    // short sums ahead of a kernel: as point programs they share a launch with the others
+    if (!may_factor && g.kappa == 0 && g.inst[root].op == I_SUM) {
+        try {
+            if (try_points(g, k, root, scale, allow_split, lower, upper, guards, POINT_AHEAD)) return;
+        } catch (const Unsupported &) {
+        }
+    }
     // sums of products of index expressions (most derivative terms once the functions are tabulated)
     if (try_line(g, k, root, scale, allow_split, lower, upper, guards)) return;
     // small index spaces
@@ -1323,9 +1330,26 @@ void emit_plain_kernel(Gen &g, Kernel &k, int root, const std::vector<std::vecto
     emit_kernel(g, k, root, lower, upper, guards, allow_split, false);
 }
 
+// Auxiliary kernels that are all point programs run as few launches: a batch ends where a kernel reads what one of the
+// batch writes.  (Forward pass of the intro expression at 1301 x 2477 x 21: six launches of 4 us before the contraction.)
+static void batch_auxiliaries(Kernel &k)
+{
+    if (k.pre.size() < 2) return;
+    for (const Kernel &pk : k.pre) if (pk.point.empty() || pk.point[0].zsplit > 1 || !pk.pre.empty()) return;
+    int batch = 0, first = 0;
+    for (int i = 0; i < (int)k.pre.size(); ++i) {
+        bool reads = i - first >= TADQ_BATCH;
+        for (int j = first; j < i; ++j)
+            for (const TadqLoad &L : k.pre[i].point[0].loads) reads = reads || (L.ptr && L.ptr == k.aux[k.pre[j].out_aux].slot);
+        if (reads) { ++batch; first = i; }
+        k.pre[i].batch = batch;
+    }
+}
+
 // workspace needs and launches of a kernel with its auxiliary kernels
 static void account(tad_plan &p, Kernel &k)
 {
+    batch_auxiliaries(k);
     std::function<void(const Kernel &)> walk = [&](const Kernel &x) {
         if (x.ew.empty() && x.contract.empty() && x.prog.zsplit > 1)   // (line-sum kernels keep their shares in prog too)
             p.partial_bytes = std::max(p.partial_bytes, (size_t(x.prog.zsplit) + 1) * size_t(x.prog.part_limit) * 4);
@@ -1341,7 +1365,8 @@ static void account(tad_plan &p, Kernel &k)
         if (!x.ew.empty()) n = 1;
         else if (x.contract.empty()) n = 1 + (x.prog.zsplit > 1 ? 1 + (x.prog.write_only_live && x.line.empty() ? 1 : 0) : 0);
         for (const TadcProgram &cp : x.contract) n += 1 + (cp.ksplit > 1 ? 1 : 0);
-        for (const Kernel &y : x.pre) n += launches(y);
+        for (size_t i = 0; i < x.pre.size(); ++i)
+            if (x.pre[i].batch < 0 || i == 0 || x.pre[i].batch != x.pre[i - 1].batch) n += launches(x.pre[i]);
         return n;
     };
     k.stats.n_launches = launches(k);

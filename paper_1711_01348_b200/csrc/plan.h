@@ -83,6 +83,7 @@ struct Kernel {
     size_t aux_bytes = 0;
     std::vector<Kernel> pre;
     int out_aux = -1;
+    int batch = -1;            // an auxiliary kernel that runs in one launch with the others of the same number
     int shared = -1;           // an auxiliary kernel whose result other gradients need too: its number in the plan (its tensor then
                                // lies behind the kernels' own areas)
     KernelStats stats;

@@ -132,12 +132,10 @@ __device__ __forceinline__ void decode(const TadqProgram &P, const int first, co
     }
 }
 
+// block bx of the program; its share number by of n_shares
 template <int U>
-__global__ void __launch_bounds__(NT)
-tad_point_kernel(const __grid_constant__ TadqProgram P, const __grid_constant__ TadpPointers ptrs)
+__device__ __forceinline__ void run_block(const TadqProgram &P, const TadpPointers &ptrs, float *out, float *sm, const unsigned bx, const unsigned by, const unsigned n_shares)
 {
-    tad_wait_previous();
-    extern __shared__ __align__(16) float sm[];
     const int tid = (int)threadIdx.x;
     int var[MV][U];
 #pragma unroll
@@ -153,7 +151,7 @@ tad_point_kernel(const __grid_constant__ TadqProgram P, const __grid_constant__ 
     const bool sums = terms > 1 || P.lt > 1;
     const unsigned lt = (unsigned)P.lt, lo_n = NT / lt;
     const unsigned tl = P.along_terms ? tid % lt : tid / lo_n, ol = P.along_terms ? tid / lt : tid % lo_n;
-    const unsigned per = (terms + gridDim.y - 1u) / gridDim.y, t0 = blockIdx.y * per, t1 = min(terms, t0 + per);
+    const unsigned per = (terms + n_shares - 1u) / n_shares, t0 = by * per, t1 = min(terms, t0 + per);
     // fixed-order tree over the term lanes of an output
     float *red = sm + P.n_slots * NT * U;
     auto total = [&]() {
@@ -170,7 +168,7 @@ tad_point_kernel(const __grid_constant__ TadqProgram P, const __grid_constant__ 
     unsigned live = 0;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-        const unsigned q = sums ? blockIdx.x * lo_n + ol : (blockIdx.x * U + u) * NT + tid;
+        const unsigned q = sums ? bx * lo_n + ol : (bx * U + u) * NT + tid;
         if (q < points) live |= 1u << u;
         decode<U>(P, 0, P.n_out, min(q, points - 1u), var, u);
         decode<U>(P, P.n_out, P.n_z, 0u, var, u);
@@ -212,7 +210,7 @@ tad_point_kernel(const __grid_constant__ TadqProgram P, const __grid_constant__ 
             int o = P.out_base;
 #pragma unroll
             for (int d = 0; d < MV; ++d) o += P.out_coef[d] * var[d][u];
-            if (live & (1u << u)) ptrs.out[(unsigned)o] = P.accumulate ? ptrs.out[(unsigned)o] + acc.v[u] : acc.v[u];
+            if (live & (1u << u)) out[(unsigned)o] = P.accumulate ? out[(unsigned)o] + acc.v[u] : acc.v[u];
         }
         return;
     }
@@ -222,30 +220,72 @@ tad_point_kernel(const __grid_constant__ TadqProgram P, const __grid_constant__ 
     int o = P.out_base; unsigned cell = 0;
 #pragma unroll
     for (int d = 0; d < MV; ++d) { o += P.out_coef[d] * var[d][0]; if (d < P.n_out) cell += (unsigned)(P.part_coef[d] * (var[d][0] - P.lo[d])); }
-    if (P.zsplit > 1) ptrs.part[(size_t)blockIdx.y * (unsigned)P.part_limit + cell] = sum;
-    else ptrs.out[(unsigned)o] = P.accumulate ? ptrs.out[(unsigned)o] + sum : sum;
+    if (P.zsplit > 1) ptrs.part[(size_t)by * (unsigned)P.part_limit + cell] = sum;
+    else out[(unsigned)o] = P.accumulate ? out[(unsigned)o] + sum : sum;
+}
+
+template <int U>
+__global__ void __launch_bounds__(NT)
+tad_point_kernel(const __grid_constant__ TadqProgram P, const __grid_constant__ TadpPointers ptrs)
+{
+    tad_wait_previous();
+    extern __shared__ __align__(16) float sm[];
+    run_block<U>(P, ptrs, ptrs.out, sm, blockIdx.x, blockIdx.y, gridDim.y);
+}
+
+template <int U>
+__global__ void __launch_bounds__(NT)
+tad_point_batch_kernel(const __grid_constant__ TadqBatch B, const __grid_constant__ TadpPointers ptrs)
+{
+    tad_wait_previous();
+    extern __shared__ __align__(16) float sm[];
+    int i = 0;
+    while (i + 1 < B.n && blockIdx.x >= B.first[i + 1]) ++i;
+    run_block<U>(B.p[i], ptrs, B.out[i], sm, blockIdx.x - B.first[i], 0u, 1u);
+}
+
+template <int U>
+unsigned blocks_of(const TadqProgram &P)
+{
+    const unsigned per = P.terms > 1 || P.lt > 1 ? (unsigned)(NT / P.lt) : (unsigned)NT * U;
+    return ((unsigned)P.points + per - 1u) / per;
+}
+
+template <int U>
+size_t smem_of(const TadqProgram &P) { return ((size_t)P.n_slots * U + 1) * NT * 4; }
+
+template <int U, class K>
+cudaError_t allow_smem(K kernel, size_t smem)
+{
+    if (smem <= 48 * 1024) return cudaSuccess;
+    static bool attr_set[64] = {};                             // (one per kernel type: the batch and the single kernel differ in K)
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= 64 || !attr_set[dev]) {
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (TADQ_MAX_SLOTS * U + 1) * NT * 4);
+        if (e != cudaSuccess) return e;
+        if (dev >= 0 && dev < 64) attr_set[dev] = true;
+    }
+    return cudaSuccess;
+}
+
+template <int U>
+cudaError_t launch_batch(TadqBatch &B, const TadpPointers &ptrs, cudaStream_t stream)
+{
+    size_t smem = 0;
+    B.first[0] = 0;
+    for (int i = 0; i < B.n; ++i) { B.first[i + 1] = B.first[i] + blocks_of<U>(B.p[i]); smem = std::max(smem, smem_of<U>(B.p[i])); }
+    const cudaError_t e = allow_smem<U>(tad_point_batch_kernel<U>, smem);
+    return e != cudaSuccess ? e : tad_launch(tad_point_batch_kernel<U>, B.first[B.n], NT, smem, stream, B, ptrs);
 }
 
 template <int U>
 cudaError_t launch_points(const TadqProgram &P, const TadpPointers &ptrs, cudaStream_t stream)
 {
-    const bool sums = P.terms > 1 || P.lt > 1;
-    const size_t smem = ((size_t)P.n_slots * U + 1) * NT * 4;
-    const unsigned per = sums ? (unsigned)(NT / P.lt) : (unsigned)NT * U;
-    dim3 grid(((unsigned)P.points + per - 1u) / per, (unsigned)std::max(1, P.zsplit), 1u);
-    if (smem > 48 * 1024) {
-        static bool attr_set[64] = {};
-        int dev = 0;
-        cudaError_t e = cudaGetDevice(&dev);
-        if (e != cudaSuccess) return e;
-        if (dev < 0 || dev >= 64 || !attr_set[dev]) {
-            e = cudaFuncSetAttribute(tad_point_kernel<U>, cudaFuncAttributeMaxDynamicSharedMemorySize, (TADQ_MAX_SLOTS * U + 1) * NT * 4);
-            if (e != cudaSuccess) return e;
-            if (dev >= 0 && dev < 64) attr_set[dev] = true;
-        }
-    }
-    tad_launch(tad_point_kernel<U>, grid, NT, smem, stream, P, ptrs);
-    return cudaGetLastError();
+    const size_t smem = smem_of<U>(P);
+    const cudaError_t e = allow_smem<U>(tad_point_kernel<U>, smem);
+    return e != cudaSuccess ? e : tad_launch(tad_point_kernel<U>, dim3(blocks_of<U>(P), (unsigned)std::max(1, P.zsplit)), NT, smem, stream, P, ptrs);
 }
 
 }  // namespace
@@ -254,4 +294,15 @@ cudaError_t tad_launch_points(const TadqProgram &P, const TadpPointers &ptrs, cu
 {
     if (P.points <= 0) return cudaSuccess;
     return P.unroll == 4 ? launch_points<4>(P, ptrs, stream) : launch_points<1>(P, ptrs, stream);
+}
+
+// n programs (at most TADQ_BATCH, none split into shares) that write out[i]
+cudaError_t tad_launch_point_batch(const TadqProgram *const *progs, float *const *out, int n, const TadpPointers &ptrs, cudaStream_t stream)
+{
+    TadqBatch B;
+    B.n = n;
+    bool four = false;
+    for (int i = 0; i < n; ++i) { B.p[i] = *progs[i]; B.out[i] = out[i]; four = four || progs[i]->unroll == 4; }
+    for (int i = n; i < TADQ_BATCH; ++i) { B.p[i] = *progs[0]; B.out[i] = nullptr; B.first[i + 1] = 0; }
+    return four ? launch_batch<4>(B, ptrs, stream) : launch_batch<1>(B, ptrs, stream);
 }

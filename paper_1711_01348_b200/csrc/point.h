@@ -9,7 +9,7 @@
 
 #include "program.h"
 
-#define TADQ_MAX_STEPS 112
+#define TADQ_MAX_STEPS 96
 #define TADQ_MAX_LOADS 12
 #define TADQ_MAX_VARS 4        // output variables and flattened loop variables
 #define TADQ_MAX_SUMS 4        // bound sums inside the term
@@ -52,4 +52,13 @@ struct alignas(16) TadqProgram {
     int32_t zsplit, part_limit, part_coef[TADQ_MAX_VARS];      // > 1: grid.y shares of the terms, a plane of partial sums each
     TadqLoad loads[TADQ_MAX_LOADS];
     TadqStep steps[TADQ_MAX_STEPS];
+};
+
+// Programs that do not read each other's results run as one launch, each on a range of its blocks.
+#define TADQ_BATCH 6
+struct alignas(16) TadqBatch {
+    int32_t n;
+    uint32_t first[TADQ_BATCH + 1];        // first block of every program
+    float *out[TADQ_BATCH];
+    TadqProgram p[TADQ_BATCH];
 };

@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cstdio>
 #include <mutex>
 #include <new>
@@ -26,6 +27,7 @@ bool tad_launch_vm_16_1_rich(const TadpProgram &prog, const TadpPointers &ptrs, 
 cudaError_t tad_launch_contract(const TadcProgram &P, const TadpPointers &ptrs, unsigned sms, cudaStream_t stream);
 cudaError_t tad_launch_ew(const TadeProgram &P, const TadpPointers &ptrs, unsigned sms, cudaStream_t stream);
 cudaError_t tad_launch_points(const TadqProgram &P, const TadpPointers &ptrs, cudaStream_t stream);
+cudaError_t tad_launch_point_batch(const TadqProgram *const *progs, float *const *out, int n, const TadpPointers &ptrs, cudaStream_t stream);
 cudaError_t tad_launch_line(const TadlProgram &P, const TadpPointers &ptrs, unsigned sms, cudaStream_t stream);
 
 namespace {
@@ -104,11 +106,24 @@ __global__ void tad_fill_zero(float *out, unsigned n)
     for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) out[i] = 0.f;
 }
 
+// up to four tensors in one launch (a step of small gradients is a handful of launches)
+struct FillMany { float *out[4]; unsigned n[4]; int count; };
+__global__ void tad_fill_zero_many(const __grid_constant__ FillMany F)
+{
+    tad_wait_previous();
+    const unsigned stride = gridDim.x * blockDim.x;
+    for (int k = 0; k < F.count; ++k)
+        for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < F.n[k]; i += stride) F.out[k][i] = 0.f;
+}
+
 int sm_count()
 {
+    static std::atomic<int> known[64];                        // per device, asked for once (every launch uses it)
     int dev = 0, n = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 148;
+    if (dev >= 0 && dev < 64 && (n = known[dev].load(std::memory_order_relaxed)) > 0) return n;
     if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) return 148;
+    if (dev >= 0 && dev < 64) known[dev].store(n, std::memory_order_relaxed);
     return n;
 }
 
@@ -219,6 +234,31 @@ bool streams_only(const tad::Kernel &k)
 }
 
 // pending: an event the kernel that writes the output must wait for (the zero fill of its tensor on the second stream)
+// point programs that wait to be launched together: none reads what another of them writes
+struct PointBatch {
+    const TadqProgram *prog[TADQ_BATCH];
+    float *out[TADQ_BATCH];
+    int n = 0;
+    TadpPointers ptrs{};
+    tad_status flush(cudaStream_t stream)
+    {
+        if (n == 0) return TAD_OK;
+        cudaError_t e;
+        if (n == 1) { ptrs.out = out[0]; e = tad_launch_points(*prog[0], ptrs, stream); }
+        else e = tad_launch_point_batch(prog, out, n, ptrs, stream);
+        n = 0;
+        if (e != cudaSuccess) { tad::set_error(std::string("point launch failed: ") + cudaGetErrorString(e)); return TAD_ERR_CUDA; }
+        return TAD_OK;
+    }
+    tad_status add(const TadqProgram &P, const TadpPointers &p, float *o, cudaStream_t stream)
+    {
+        if (P.points <= 0) return TAD_OK;
+        if (n == TADQ_BATCH) { const tad_status st = flush(stream); if (st != TAD_OK) return st; }
+        ptrs = p; prog[n] = &P; out[n] = o; ++n;
+        return TAD_OK;
+    }
+};
+
 // done: shared auxiliary tensors that this call of the library has computed already
 tad_status launch(const tad::Kernel &k, TadpPointers ptrs, bool debug, cudaStream_t stream, char *aux_base = nullptr,
                   Side *side = nullptr, cudaEvent_t pending = nullptr, std::vector<char> *done = nullptr)
@@ -245,6 +285,8 @@ tad_status launch(const tad::Kernel &k, TadpPointers ptrs, bool debug, cudaStrea
             while (at > 0 && !reads_slot(k.pre[i], k.aux[k.pre[order[at - 1]].out_aux].slot)) --at;
             order.insert(order.begin() + at, i);
         }
+        PointBatch batch;
+        int in_batch = -1;
         for (int i : order) {
             const tad::Kernel &pk = k.pre[i];
             if (done && pk.shared >= 0) {
@@ -253,6 +295,13 @@ tad_status launch(const tad::Kernel &k, TadpPointers ptrs, bool debug, cudaStrea
             }
             TadpPointers pp = ptrs;
             pp.out = reinterpret_cast<float *>(aux_base + k.aux[pk.out_aux].offset);
+            if (pk.batch >= 0) {
+                tad_status st = pk.batch != in_batch ? batch.flush(stream) : TAD_OK;
+                in_batch = pk.batch;
+                if (st == TAD_OK) st = batch.add(pk.point[0], ptrs, pp.out, stream);
+                if (st != TAD_OK) return st;
+                continue;
+            }
             const bool on_side = use_side && streams_only(pk);
             bool wait = false;
             for (int slot : beside) wait = wait || reads_slot(pk, slot);
@@ -268,6 +317,8 @@ tad_status launch(const tad::Kernel &k, TadpPointers ptrs, bool debug, cudaStrea
             tad_launch_plain = false;
             if (st != TAD_OK) return st;
         }
+        const tad_status fs = batch.flush(stream);
+        if (fs != TAD_OK) return fs;
         if (!join()) { tad::set_error("event record / wait failed"); return TAD_ERR_CUDA; }
     }
     if (pending && cudaStreamWaitEvent(stream, pending, 0) != cudaSuccess) { tad::set_error("event wait failed"); return TAD_ERR_CUDA; }
@@ -494,7 +545,8 @@ tad_status tad_backward_stage(const tad_plan *plan, const float *const *args, co
 }
 
 static tad_status backward_arg(const tad_plan *plan, const float *const *args, const float *df, int32_t arg, float *darg,
-                               void *workspace, size_t workspace_bytes, void *cuda_stream, std::vector<char> *done)
+                               void *workspace, size_t workspace_bytes, void *cuda_stream, std::vector<char> *done,
+                               PointBatch *later = nullptr, bool filled = false)
 {
     if (!plan || !df || !darg || (plan->n_args && !args)) { tad::set_error("NULL argument"); return TAD_ERR_INVALID_ARG; }
     if (arg < 0 || arg >= plan->n_args) { tad::set_error("no such argument"); return TAD_ERR_INVALID_ARG; }
@@ -504,7 +556,7 @@ static tad_status backward_arg(const tad_plan *plan, const float *const *args, c
     if (!fill_inputs(plan, args, df, workspace, ptrs)) return TAD_ERR_INVALID_ARG;
     Side *side = side_of(plan);
     cudaEvent_t pending = nullptr;
-    if (plan->arg_kernels[arg].empty() || plan->arg_zero_fill[arg]) {
+    if (!filled && (plan->arg_kernels[arg].empty() || plan->arg_zero_fill[arg])) {
         // the fill of a gradient whose first kernel prepares auxiliary tensors runs beside that preparation
         const bool beside = side && !plan->arg_kernels[arg].empty() && !plan->backward[plan->arg_kernels[arg][0]].pre.empty();
         if (beside) {
@@ -520,6 +572,11 @@ static tad_status backward_arg(const tad_plan *plan, const float *const *args, c
         }
     }
     ptrs.out = darg;
+    // a gradient that is one point program reads inputs and staged adjoints only: it may share a launch with others
+    if (later && plan->arg_kernels[arg].size() == 1) {
+        const tad::Kernel &k = plan->backward[plan->arg_kernels[arg][0]];
+        if (!k.point.empty() && k.point[0].zsplit <= 1 && k.pre.empty()) return later->add(k.point[0], ptrs, darg, stream);
+    }
     for (int ki : plan->arg_kernels[arg]) {
         tad_status st = launch(plan->backward[ki], ptrs, plan->opt.debug_bounds != 0, stream,
                                workspace ? static_cast<char *>(workspace) + aux_offset(plan) : nullptr, side, pending, done);
@@ -548,12 +605,30 @@ tad_status tad_backward(const tad_plan *plan, const float *const *args, const fl
         if (st != TAD_OK) return st;
     }
     std::vector<char> done(plan->n_shared, 0);
+    // gradients to be cleared that have no preparation to run beside: in one launch
+    FillMany fill{};
+    bool filled[TADP_MAX_PTRS] = {};
+    unsigned longest = 0;
+    for (int a = 0; a < plan->n_args && fill.count < 4; ++a) {
+        const bool clears = plan->arg_kernels[a].empty() || plan->arg_zero_fill[a];
+        if (!dargs[a] || !clears || (!plan->arg_kernels[a].empty() && !plan->backward[plan->arg_kernels[a][0]].pre.empty())) continue;
+        fill.out[fill.count] = dargs[a]; fill.n[fill.count] = (unsigned)plan->arg_elems[a]; ++fill.count;
+        filled[a] = true;
+        longest = std::max(longest, (unsigned)plan->arg_elems[a]);
+    }
+    if (fill.count == 1) { fill.count = 0; for (bool &f : filled) f = false; }
+    if (fill.count) {
+        const unsigned blocks = std::min((longest + 255u) / 256u, (unsigned)sm_count() * 16u);
+        const cudaError_t e = tad_launch(tad_fill_zero_many, std::max(1u, blocks), 256, 0, (cudaStream_t)cuda_stream, fill);
+        if (e != cudaSuccess) { tad::set_error(std::string("zero fill launch failed: ") + cudaGetErrorString(e)); return TAD_ERR_CUDA; }
+    }
+    PointBatch later;
     for (int a = 0; a < plan->n_args; ++a) {
         if (!dargs[a]) continue;
-        tad_status st = backward_arg(plan, args, df, a, dargs[a], workspace, workspace_bytes, cuda_stream, &done);
+        tad_status st = backward_arg(plan, args, df, a, dargs[a], workspace, workspace_bytes, cuda_stream, &done, &later, filled[a]);
         if (st != TAD_OK) return st;
     }
-    return TAD_OK;
+    return later.flush((cudaStream_t)cuda_stream);
 }
 
 // Elements of an argument that lie on one line  base + step i, 0 <= i < n,  and are the only ones that the expression reads
