@@ -151,7 +151,9 @@ void tad_destroy(tad_plan *plan);
  * workspace must be 256-byte aligned.  It holds the staged adjoints, the partial sums of
  * summations that are split over several thread blocks, the auxiliary tensors of the
  * expression optimisation (sums pushed inside the term: small pre-evaluated tensors and
- * contraction results, Sec. 6's clean-up step), and the debug word of a debug_bounds plan.
+ * contraction results, Sec. 6's clean-up step), the debug word of a debug_bounds plan and, last,
+ * an operand of a large contraction laid out for the tensor cores; a smaller workspace that
+ * holds all but that one is accepted, and the contraction reads the operand as it is.
  * One workspace serves both calls; calls that share it must not overlap on the device. */
 size_t tad_workspace_bytes(const tad_plan *plan);
 
@@ -161,8 +163,8 @@ size_t tad_workspace_bytes(const tad_plan *plan);
  *   args       host array of n_args DEVICE pointers (read-only inputs), none NULL
  *   f          DEVICE pointer, prod(out_shape) floats, fully overwritten
  *   workspace  DEVICE pointer, tad_workspace_bytes() bytes, 256-byte aligned, caller-owned.  Only plans
- *              whose forward pass uses auxiliary tensors or a split summation read it; for every other
- *              plan NULL / 0 is accepted.  TAD_ERR_WORKSPACE when it is needed and missing or too small.
+ *              whose forward pass uses auxiliary tensors or a split summation need it; every other
+ *              plan accepts NULL / 0 (a large contraction is faster with it).  TAD_ERR_WORKSPACE when it is needed and missing or too small.
  */
 tad_status tad_forward(const tad_plan *plan, const float *const *args, float *f,
                        void *workspace, size_t workspace_bytes, void *cuda_stream);
@@ -212,7 +214,7 @@ tad_status tad_backward_arg(const tad_plan *plan, const float *const *args, cons
  *
  * The scratch is a fixed array of TAD_NOALLOC_SCRATCH_BYTES inside the library image; every
  * GPU that loads the library holds that much memory until the process exits.  A plan whose
- * tad_workspace_bytes() is larger is rejected with TAD_ERR_WORKSPACE and a message; nothing
+ * workspace (without an operand laid out for the tensor cores) is larger is rejected with TAD_ERR_WORKSPACE and a message; nothing
  * is launched in that case.  The call allocates nothing (no cudaMalloc / cudaFree, no
  * allocating library routine); inputs and outputs are still the caller's buffers, with the
  * same meaning as in tad_backward.

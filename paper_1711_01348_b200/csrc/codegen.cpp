@@ -1353,9 +1353,11 @@ static void account(tad_plan &p, Kernel &k)
     std::function<void(const Kernel &)> walk = [&](const Kernel &x) {
         if (x.ew.empty() && x.contract.empty() && x.prog.zsplit > 1)   // (line-sum kernels keep their shares in prog too)
             p.partial_bytes = std::max(p.partial_bytes, (size_t(x.prog.zsplit) + 1) * size_t(x.prog.part_limit) * 4);
-        for (const TadcProgram &cp : x.contract)
+        for (const TadcProgram &cp : x.contract) {
             if (cp.ksplit > 1)
                 p.partial_bytes = std::max(p.partial_bytes, size_t(cp.ksplit) * size_t(cp.M.extent) * size_t(cp.N.extent) * size_t(cp.Z.extent) * 4);
+            if (cp.image) p.image_bytes = std::max(p.image_bytes, image_bytes(cp));
+        }
         for (const Kernel &y : x.pre) walk(y);
     };
     walk(k);
@@ -1364,7 +1366,7 @@ static void account(tad_plan &p, Kernel &k)
         int n = 0;
         if (!x.ew.empty()) n = 1;
         else if (x.contract.empty()) n = 1 + (x.prog.zsplit > 1 ? 1 + (x.prog.write_only_live && x.line.empty() ? 1 : 0) : 0);
-        for (const TadcProgram &cp : x.contract) n += 1 + (cp.ksplit > 1 ? 1 : 0);
+        for (const TadcProgram &cp : x.contract) n += 1 + (cp.ksplit > 1 ? 1 : 0) + cp.image;
         for (size_t i = 0; i < x.pre.size(); ++i)
             if (x.pre[i].batch < 0 || i == 0 || x.pre[i].batch != x.pre[i - 1].batch) n += launches(x.pre[i]);
         return n;

@@ -37,7 +37,9 @@ enum TadcGather : int {
 };
 
 // the same for the tensor-core kernel (shape 7; see mma.cu): which index the lanes run along, or 32-byte vectors
-enum TadcMmaGather : int { TM_ROW = 0, TM_KVEC, TM_K, TM_RVEC };
+constexpr int TADC_IMAGE_COLS = 128;    // columns of a tile whose operand is split ahead
+
+enum TadcMmaGather : int { TM_ROW = 0, TM_KVEC, TM_K, TM_RVEC, TM_IMAGE };     // TM_IMAGE: column operand split ahead (see image)
 
 // steps applied to every finished sum before it is stored (in this order)
 enum TadcEpilogueOp : int { TE_END = 0, TE_NEG, TE_EXP, TE_MULC, TE_ADDC, TE_MUL_LOAD, TE_ADD_LOAD, TE_SQR, TE_TANH, TE_SIN, TE_COS };
@@ -58,6 +60,8 @@ struct alignas(16) TadcProgram {
     int32_t shape;                 // tiles: 0 = 128 x 128 (8 x 8 per thread), 1 = 128 x 32, 2 = 128 x 64, 3 = 128 x 36 (8 x 4 per thread);
                                    // 4 = sums of rows (a warp per output), 5 = streamed narrow contraction, 6 = sums of columns (a thread per output),
                                    // 7 = tensor-core tiles of 128 rows (mma.cu)
+    int32_t image;                 // shape 7: 1 = a kernel of its own splits the column operand into the tiles' shared-memory images
+                                   // (image_bytes() of the workspace; without that much the operand is gathered as usual)
     float scale;
     int32_t n_epi;
     int32_t epi_op[TADC_MAX_EPI];

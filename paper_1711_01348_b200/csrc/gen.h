@@ -335,6 +335,13 @@ struct System {
 
 // builds one contraction program from a system whose loops all have fixed ranges; an operand with ptr < 0 is
 // a tensor of ones (a plain summation of the other operand).  strict_fill: refuse mostly empty tiles
+// bytes of the column operand's image (contract.h: image): three bf16 parts of every tile and stage
+inline size_t image_bytes(const TadcProgram &P)
+{
+    const size_t tiles = (size_t(P.N.extent) + TADC_IMAGE_COLS - 1) / TADC_IMAGE_COLS, stages = (size_t(P.K.extent) + TADC_KS - 1) / TADC_KS;
+    return tiles * stages * size_t(P.Z.extent) * (3 * TADC_IMAGE_COLS * TADC_KS * 2);
+}
+
 bool emit_program(const System &s, float scale, int accumulate, bool allow_split, bool strict_fill, TadcProgram &P, std::string &text);
 
 // contract_gen.cpp: recognises a kernel whose term is a product of two index expressions summed over

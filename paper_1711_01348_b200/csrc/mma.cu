@@ -197,10 +197,10 @@ __device__ __forceinline__ void split_unit(const float (&v)[8], unsigned (&p1)[4
 
 template <int BN, int MA, int MB>
 struct MmaCfg {
-    static constexpr bool TS = MA == TM_ROW;
+    static constexpr bool TS = MA == TM_ROW, IMAGE = MB == TM_IMAGE;
     static constexpr int PART_A = BM * KS * 2, PART_B = BN * KS * 2;                 // bytes of one bf16 part of a stage
     static constexpr int STAGE = (TS ? 0 : 3 * PART_A) + 3 * PART_B;
-    static constexpr int UA = BM * KS / 8 / (NCW * 32), UB = BN * KS / 8 / (NCW * 32);   // units per thread
+    static constexpr int UA = BM * KS / 8 / (NCW * 32), UB = IMAGE ? 0 : BN * KS / 8 / (NCW * 32);   // units per thread
     static constexpr int COLS = BN * 32 / (NCW * 8);                                  // accumulator columns per thread
     static constexpr int TABLES = (BM + BN) * 12 + KT * KS * 16;                      // row offsets, guards, output offsets; k tables
     static constexpr size_t SMEM = 1024 + 2 * size_t(STAGE) + TABLES;
@@ -210,12 +210,11 @@ template <int BN, int MA, int MB>
 __global__ void __launch_bounds__(NT, 1)
 tad_mma_kernel(const __grid_constant__ TadcProgram P, const __grid_constant__ TadpPointers ptrs, const unsigned tiles_n)
 {
-    tad_wait_previous();
     using C = MmaCfg<BN, MA, MB>;
     constexpr bool TS = C::TS;
     constexpr int COLS = C::COLS;
     extern __shared__ unsigned char smem_raw[];
-    __shared__ unsigned long long bars[4 + KT];
+    __shared__ unsigned long long bars[6 + KT];
     __shared__ unsigned tmem_base_s;
     __shared__ volatile int failed;
     const unsigned smem0 = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -223,7 +222,7 @@ tad_mma_kernel(const __grid_constant__ TadcProgram P, const __grid_constant__ Ta
     unsigned *rowA = reinterpret_cast<unsigned *>(stages + 2 * C::STAGE), *rowB = rowA + BM;          // bytes
     int *rowgA = reinterpret_cast<int *>(rowB + BN), *rowgB = rowgA + BM, *outM = rowgB + BN, *outN = outM + BM;
     int *ktab = outN + BN;                                   // per ring slot: offsets A, guards A, offsets B, guards B (KS each)
-    const unsigned bar_full = smem_u32(&bars[0]), bar_done = smem_u32(&bars[2]), bar_tab = smem_u32(&bars[4]);
+    const unsigned bar_full = smem_u32(&bars[0]), bar_done = smem_u32(&bars[2]), bar_tab = smem_u32(&bars[6]), bar_copy = smem_u32(&bars[4]);
 
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const unsigned tile_n = blockIdx.x % tiles_n, tile_m = blockIdx.x / tiles_n;
@@ -249,6 +248,7 @@ tad_mma_kernel(const __grid_constant__ TadcProgram P, const __grid_constant__ Ta
             failed = 0;
             mbar_init(bar_full, NCW); mbar_init(bar_full + 8, NCW);
             mbar_init(bar_done, 1); mbar_init(bar_done + 8, 1);
+            mbar_init(bar_copy, 1); mbar_init(bar_copy + 8, 1);
             for (int i = 0; i < KT; ++i) mbar_init(bar_tab + 8 * i, 1);
             asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         }
@@ -272,6 +272,7 @@ tad_mma_kernel(const __grid_constant__ TadcProgram P, const __grid_constant__ Ta
     fence_before();
     __syncthreads();
     fence_after();
+    tad_wait_previous();                                     // (nothing above reads memory)
     const unsigned tmem = __shfl_sync(0xffffffffu, tmem_base_s, 0);
     constexpr unsigned TMEM_A = 2 * BN;                      // columns of the row operand's stages (TS): 3 x 32 each
     bool ok = true;
@@ -280,7 +281,7 @@ tad_mma_kernel(const __grid_constant__ TadcProgram P, const __grid_constant__ Ta
         // ---- MMA warp ----
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REG_MMA));
         const int n_stages_mma = warp == NCW ? n_stages : 0;
-        constexpr bool a_k = MA == TM_ROW || MA == TM_KVEC, b_k = MB == TM_ROW || MB == TM_KVEC;
+        constexpr bool a_k = MA == TM_ROW || MA == TM_KVEC, b_k = MB == TM_ROW || MB == TM_KVEC || MB == TM_IMAGE;
         const unsigned n_pad = min((unsigned)BN, (Next - tile_n * BN + 15u) / 16u * 16u);
         const unsigned idesc = (1u << 4) | (1u << 7) | (1u << 10) | (a_k ? 0u : 1u << 15) | (b_k ? 0u : 1u << 16) | ((n_pad >> 3) << 17) | ((BM >> 4) << 24);
         // K-major: eight rows of 128 bytes per repeat; MN-major: blocks of 64 rows, eight summation indices per repeat
@@ -289,6 +290,7 @@ tad_mma_kernel(const __grid_constant__ TadcProgram P, const __grid_constant__ Ta
         int issued = 0;
         for (int s = 0; s < n_stages_mma && ok; ++s) {
             ok = mbar_wait(bar_full + 8 * (s & 1), (s >> 1) & 1, &failed);
+            if (C::IMAGE) ok = ok && mbar_wait(bar_copy + 8 * (s & 1), (s >> 1) & 1, &failed);
             fence_after();
             if (!ok) break;
             const unsigned sm = smem0 + (s & 1) * C::STAGE;
@@ -333,23 +335,44 @@ tad_mma_kernel(const __grid_constant__ TadcProgram P, const __grid_constant__ Ta
         const float *__restrict__ A = ptrs.in[P.ptrA];
         const float *__restrict__ B = ptrs.in[P.ptrB];
         const unsigned gextA = (unsigned)P.guardA_ext, gextB = (unsigned)P.guardB_ext;
-        float va[C::UA][8], vb[C::UB][8];
+        float va[C::UA][8], vb[C::UB > 0 ? C::UB : 1][8];
         auto load = [&](float (&v)[8], int i, int s, bool second, bool check) {
             const unsigned *t = reinterpret_cast<const unsigned *>(ktab + (s % KT) * 4 * KS) + (second ? 2 * KS : 0);
             const int *tg = reinterpret_cast<const int *>(t + KS);
+            if constexpr (C::IMAGE) second = false;
             if (!second) {
                 if (check) load_unit<MA, BM, TS, true>(v, A, tid, i, rowA, rowgA, t, tg, gextA);
                 else load_unit<MA, BM, TS, false>(v, A, tid, i, rowA, rowgA, t, tg, gextA);
             } else {
-                if (check) load_unit<MB, BN, false, true>(v, B, tid, i, rowB, rowgB, t, tg, gextB);
-                else load_unit<MB, BN, false, false>(v, B, tid, i, rowB, rowgB, t, tg, gextB);
+                constexpr int MODE_B = C::IMAGE ? (int)TM_ROW : MB;
+                if (check) load_unit<MODE_B, BN, false, true>(v, B, tid, i, rowB, rowgB, t, tg, gextB);
+                else load_unit<MODE_B, BN, false, false>(v, B, tid, i, rowB, rowgB, t, tg, gextB);
             }
         };
+        // the column operand's image of stage s, as one bulk copy behind the row operand's buffer (its MMAs of stage s - 2 are done)
+        int copies = 0;
+        auto copy_image = [&](int s) {
+            if (!C::IMAGE || warp != 0 || s >= n_stages) return;
+            ++copies;
+            if (lane == 0) {
+                const size_t total = ((size_t)P.K.extent + KS - 1) / KS;
+                const unsigned char *from = ptrs.image +
+                                   (((size_t)zb * tiles_n + tile_n) * total + kbeg / KS + s) * (3 * C::PART_B);
+                const unsigned to = smem0 + (s & 1) * C::STAGE + (TS ? 0 : 3 * C::PART_A), bar = bar_copy + 8 * (s & 1);
+                asm volatile("fence.proxy.async.global;" ::: "memory");   // (the image is another kernel's plain stores)
+                asm volatile("{ .reg .b64 t; mbarrier.arrive.expect_tx.shared::cta.b64 t, [%0], %1; }" ::"r"(bar), "r"(3 * C::PART_B) : "memory");
+                asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(to), "l"(from), "r"(3 * C::PART_B), "r"(bar) : "memory");
+            }
+            __syncwarp();
+        };
+        copy_image(0);
+        copy_image(1);
         // adds the finished stage s to the registers
         auto collect = [&](int s) {
             ok = ok && mbar_wait(bar_done + 8 * (s & 1), (s >> 1) & 1, &failed);
             fence_after();
             if (!ok) return;
+            copy_image(s + 2);
             const unsigned at = tmem + ((unsigned)(quad * 32) << 16) + (s & 1) * BN + col0;
 #pragma unroll
             for (int c = 0; c < COLS; c += 16) {
@@ -375,7 +398,7 @@ tad_mma_kernel(const __grid_constant__ TadcProgram P, const __grid_constant__ Ta
 #pragma unroll
                 for (int i = 0; i < C::UA; ++i) mask_unit(va[i], Unit<MA, BM, TS>(tid, i), left);
 #pragma unroll
-                for (int i = 0; i < C::UB; ++i) mask_unit(vb[i], Unit<MB, BN, false>(tid, i), left);
+                for (int i = 0; i < C::UB; ++i) mask_unit(vb[i], Unit<C::IMAGE ? (int)TM_ROW : MB, BN, false>(tid, i), left);
             }
             unsigned p1[4], p2[4], p3[4];
 #pragma unroll
@@ -397,7 +420,7 @@ tad_mma_kernel(const __grid_constant__ TadcProgram P, const __grid_constant__ Ta
             for (int i = 0; i < C::UB; ++i) {
                 split_unit(vb[i], p1, p2, p3);
                 if (more) load(vb[i], i, s + 1, true, P.guardB != 0);
-                const Unit<MB, BN, false> u(tid, i);
+                const Unit<C::IMAGE ? (int)TM_ROW : MB, BN, false> u(tid, i);
                 *reinterpret_cast<uint4 *>(st + u.dst) = make_uint4(p1[0], p1[1], p1[2], p1[3]);
                 *reinterpret_cast<uint4 *>(st + C::PART_B + u.dst) = make_uint4(p2[0], p2[1], p2[2], p2[3]);
                 *reinterpret_cast<uint4 *>(st + 2 * C::PART_B + u.dst) = make_uint4(p3[0], p3[1], p3[2], p3[3]);
@@ -409,6 +432,14 @@ tad_mma_kernel(const __grid_constant__ TadcProgram P, const __grid_constant__ Ta
             if (s > 0) collect(s - 1);
         }
         if (n_stages > 0) collect(n_stages - 1);
+        // copies of a block that gave up still write its shared memory: wait for them (again with a limit)
+        if (!ok)
+            for (int s = max(0, copies - 2); s < copies; ++s)
+                for (int i = 0; i < WAIT_LIMIT; ++i) {
+                    unsigned there;
+                    asm volatile("{ .reg .pred p; mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }" : "=r"(there) : "r"(bar_copy + 8 * (s & 1)), "r"((s >> 1) & 1) : "memory");
+                    if (__all_sync(0xffffffffu, there)) break;
+                }
         // ---- outputs: a thread holds COLS columns of its row; consecutive lanes are consecutive rows ----
         const unsigned rl = (unsigned)(quad * 32 + lane), m = tile_m * BM + rl, n0 = tile_n * BN + col0;
         const int live = m < Mext && n0 < Next ? (int)min((unsigned)COLS, Next - n0) : 0;
@@ -829,6 +860,66 @@ tad_mma_reduce(const __grid_constant__ TadcProgram P, const __grid_constant__ Ta
     }
 }
 
+// Splits the column operand into the images of its tiles: a block per stage, 32 columns and batch index reads 32 x 64
+// elements (lanes along the index that is consecutive; eight loads a thread, all in flight), and writes the three bf16 parts
+// of every column in the K-major, 128-byte swizzled order of the MMA's shared memory.  A block per whole tile and stage took
+// 21 us at any size (a serial chain of table, loads and stores in 20 to 40 blocks); pieces of 32 columns take about 5.
+constexpr int IC = 32, IMAGE_BN = TADC_IMAGE_COLS;     // columns of a block, of a tile
+
+__global__ void __launch_bounds__(256)
+tad_mma_image_kernel(const __grid_constant__ TadcProgram P, const __grid_constant__ TadpPointers ptrs)
+{
+    constexpr int BN = IMAGE_BN, LD = KS + 1, PART = BN * KS * 2;
+    __shared__ float tile[IC * LD];
+    __shared__ unsigned rows[IC], kt[KS];
+    __shared__ int rowg[IC], ktg[KS];
+    const int tid = threadIdx.x;
+    const unsigned stage = blockIdx.x, n0 = blockIdx.y * IC, zb = blockIdx.z, Next = (unsigned)P.N.extent, K = (unsigned)P.K.extent;
+    if (tid < IC + KS) {
+        if (tid < IC) {
+            const Parts z = decode(P.Z, zb);
+            const unsigned n = n0 + tid;
+            const Parts p = decode(P.N, n < Next ? n : 0u);
+            rows[tid] = (unsigned)(P.baseB + z.b + p.b); rowg[tid] = n < Next ? P.guardB_c0 + z.gb + p.gb : DEAD;
+        } else {
+            const unsigned k = stage * KS + (tid - IC);
+            const Parts p = decode(P.K, k < K ? k : 0u);
+            kt[tid - IC] = (unsigned)p.b; ktg[tid - IC] = k < K ? p.gb : DEAD;
+        }
+    }
+    __syncthreads();
+    tad_wait_previous();
+    const float *__restrict__ B = ptrs.in[P.ptrB];
+    const bool along_rows = P.modeB == TM_ROW || P.modeB == TM_RVEC;
+    constexpr int UNITS = IC * KS / 256;
+    float v[UNITS];
+#pragma unroll
+    for (int i = 0; i < UNITS; ++i) {
+        const int e = tid + i * 256, r = along_rows ? e % IC : e / KS, k = along_rows ? e / IC : e % KS;
+        // (columns past the edge, indices past the end and guarded elements are zeros; a program without a guard has extent 1)
+        v[i] = (unsigned)(rowg[r] + ktg[k]) < (unsigned)P.guardB_ext ? __ldg(B + (rows[r] + kt[k])) : 0.f;
+    }
+#pragma unroll
+    for (int i = 0; i < UNITS; ++i) {
+        const int e = tid + i * 256, r = along_rows ? e % IC : e / KS, k = along_rows ? e / IC : e % KS;
+        tile[r * LD + k] = v[i];
+    }
+    __syncthreads();
+    const unsigned tiles = (Next + BN - 1) / BN, stages = (K + KS - 1) / KS, tile_n = n0 / BN;
+    unsigned char *dst = ptrs.image + (((size_t)zb * tiles + tile_n) * stages + stage) * (3 * PART);
+    const int lc = tid / (KS / 8), l = n0 % BN + lc, o = tid % (KS / 8);
+    unsigned p1[4], p2[4], p3[4];
+    float u[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) u[j] = tile[lc * LD + o * 8 + j];
+    split_unit(u, p1, p2, p3);
+    unsigned char *at = dst + l * 128 + ((o ^ (l & 7)) << 4);
+    *reinterpret_cast<uint4 *>(at) = make_uint4(p1[0], p1[1], p1[2], p1[3]);
+    *reinterpret_cast<uint4 *>(at + PART) = make_uint4(p2[0], p2[1], p2[2], p2[3]);
+    *reinterpret_cast<uint4 *>(at + 2 * PART) = make_uint4(p3[0], p3[1], p3[2], p3[3]);
+}
+static_assert(IC * KS / 8 == 256, "one unit a thread");
+
 template <int BN, int MA, int MB>
 cudaError_t launch_mma(const TadcProgram &P, const TadpPointers &ptrs, cudaStream_t stream)
 {
@@ -884,6 +975,16 @@ cudaError_t tad_launch_mma(const TadcProgram &P, const TadpPointers &ptrs, unsig
     const bool short_pays = P.K.extent <= KS && P.ksplit <= 1 && P.N.extent > 64 && tiles >= 4ull * sms;
 #define TAD_MMA_CASE(MA, MB)                                                                                              \
     case MA * 4 + MB: e = short_pays ? launch_short<MA, MB>(P, ptrs, sms, stream) : P.N.extent <= 64 ? launch_mma<64, MA, MB>(P, ptrs, stream) : launch_mma<128, MA, MB>(P, ptrs, stream); break;
+    if (P.image && !short_pays) {
+        const dim3 grid((unsigned)(P.K.extent + KS - 1) / KS, (unsigned)(P.N.extent + IMAGE_BN - 1) / IMAGE_BN * (IMAGE_BN / IC), (unsigned)P.Z.extent);
+        e = tad_launch(tad_mma_image_kernel, grid, 256, 0, stream, P, ptrs);
+        if (e != cudaSuccess) return e;
+        switch (P.modeA) {
+        case TM_ROW: e = launch_mma<IMAGE_BN, TM_ROW, TM_IMAGE>(P, ptrs, stream); break;
+        case TM_KVEC: e = launch_mma<IMAGE_BN, TM_KVEC, TM_IMAGE>(P, ptrs, stream); break;
+        default: e = launch_mma<IMAGE_BN, TM_K, TM_IMAGE>(P, ptrs, stream); break;
+        }
+    } else
 #define TAD_MMA_ROW(MA) TAD_MMA_CASE(MA, TM_ROW) TAD_MMA_CASE(MA, TM_KVEC) TAD_MMA_CASE(MA, TM_K) TAD_MMA_CASE(MA, TM_RVEC)
     switch (P.modeA * 4 + P.modeB) { TAD_MMA_ROW(TM_ROW) TAD_MMA_ROW(TM_KVEC) TAD_MMA_ROW(TM_K) default: break; }
 #undef TAD_MMA_ROW

@@ -163,6 +163,7 @@ tad_status launch_contractions(const tad::Kernel &k, const TadpPointers &ptrs, c
     bool forked = false;
     for (size_t i = 0; i < k.contract.size(); ++i) {
         TadcProgram P = k.contract[i];
+        if (!ptrs.image) P.image = 0;
         if (P.ksplit > 1 && !ptrs.part) { tad::set_error("internal: partial-sum buffer missing"); return TAD_ERR_WORKSPACE; }
         // 16-byte copies and stores need 16-byte aligned tensors: fall back to 4-byte accesses otherwise
         auto misaligned = [](const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) != 0; };
@@ -416,10 +417,19 @@ size_t stage_offset(const tad_plan *plan, int s)
     return (plan->opt.debug_bounds ? 256 : 0) + size_t(s) * pad256(size_t(plan->out_elems) * 4);
 }
 
-// workspace layout: ... [planes of partial sums][auxiliary tensors]
+// workspace layout: ... [planes of partial sums][auxiliary tensors][image of a column operand]
 size_t aux_offset(const tad_plan *plan)
 {
     return stage_offset(plan, (int)plan->stages.size()) + pad256(plan->partial_bytes);
+}
+
+// what a plan cannot do without; contractions whose operand image does not fit behind it gather as usual
+size_t required_bytes(const tad_plan *plan) { return aux_offset(plan) + pad256(plan->aux_bytes); }
+
+unsigned char *image_of(const tad_plan *plan, void *workspace, size_t workspace_bytes)
+{
+    return workspace && plan->image_bytes && workspace_bytes >= tad_workspace_bytes(plan) && (reinterpret_cast<uintptr_t>(workspace) & 255u) == 0
+        ? static_cast<unsigned char *>(workspace) + required_bytes(plan) : nullptr;
 }
 
 // some kernel of the forward pass divides a summation among blocks (planes of partial sums in the workspace)
@@ -432,7 +442,7 @@ bool forward_splits(const tad::Kernel &k)
 
 bool check_workspace(const tad_plan *plan, void *workspace, size_t workspace_bytes)
 {
-    const size_t need = tad_workspace_bytes(plan);
+    const size_t need = required_bytes(plan);
     if (need && (!workspace || workspace_bytes < need || (reinterpret_cast<uintptr_t>(workspace) & 255u))) {
         tad::set_error("workspace missing, smaller than tad_workspace_bytes() or not 256-byte aligned");
         return false;
@@ -440,8 +450,9 @@ bool check_workspace(const tad_plan *plan, void *workspace, size_t workspace_byt
     return true;
 }
 
-bool fill_inputs(const tad_plan *plan, const float *const *args, const float *df, void *workspace, TadpPointers &ptrs)
+bool fill_inputs(const tad_plan *plan, const float *const *args, const float *df, void *workspace, size_t workspace_bytes, TadpPointers &ptrs)
 {
+    ptrs.image = image_of(plan, workspace, workspace_bytes);
     for (int a = 0; a < plan->n_args; ++a) {
         if (!args[a]) { tad::set_error("NULL argument tensor"); return false; }
         ptrs.in[a] = args[a];
@@ -503,7 +514,7 @@ extern "C" {
 size_t tad_workspace_bytes(const tad_plan *plan)
 {
     if (!plan) return 0;
-    return aux_offset(plan) + pad256(plan->aux_bytes);
+    return required_bytes(plan) + pad256(plan->image_bytes);
 }
 
 tad_status tad_forward(const tad_plan *plan, const float *const *args, float *f,
@@ -520,6 +531,7 @@ tad_status tad_forward(const tad_plan *plan, const float *const *args, float *f,
     ptrs.out = f;
     ptrs.debug = nullptr;
     char *aux_base = nullptr;
+    ptrs.image = image_of(plan, workspace, workspace_bytes);
     if (needs_ws) {
         ptrs.part = plan->partial_bytes
             ? reinterpret_cast<float *>(static_cast<char *>(workspace) + stage_offset(plan, (int)plan->stages.size())) : nullptr;
@@ -534,7 +546,7 @@ tad_status tad_backward_stage(const tad_plan *plan, const float *const *args, co
     if (!plan || !df || (plan->n_args && !args)) { tad::set_error("NULL argument"); return TAD_ERR_INVALID_ARG; }
     if (!check_workspace(plan, workspace, workspace_bytes)) return TAD_ERR_WORKSPACE;
     TadpPointers ptrs{};
-    if (!fill_inputs(plan, args, df, workspace, ptrs)) return TAD_ERR_INVALID_ARG;
+    if (!fill_inputs(plan, args, df, workspace, workspace_bytes, ptrs)) return TAD_ERR_INVALID_ARG;
     for (int s = 0; s < (int)plan->stages.size(); ++s) {
         ptrs.out = reinterpret_cast<float *>(static_cast<char *>(workspace) + stage_offset(plan, s));
         tad_status st = launch(plan->stages[s], ptrs, plan->opt.debug_bounds != 0, (cudaStream_t)cuda_stream,
@@ -553,7 +565,7 @@ static tad_status backward_arg(const tad_plan *plan, const float *const *args, c
     if (!check_workspace(plan, workspace, workspace_bytes)) return TAD_ERR_WORKSPACE;
     cudaStream_t stream = (cudaStream_t)cuda_stream;
     TadpPointers ptrs{};
-    if (!fill_inputs(plan, args, df, workspace, ptrs)) return TAD_ERR_INVALID_ARG;
+    if (!fill_inputs(plan, args, df, workspace, workspace_bytes, ptrs)) return TAD_ERR_INVALID_ARG;
     Side *side = side_of(plan);
     cudaEvent_t pending = nullptr;
     if (!filled && (plan->arg_kernels[arg].empty() || plan->arg_zero_fill[arg])) {
@@ -794,7 +806,7 @@ tad_status tad_backward_noalloc(const tad_plan *plan, const float *const *args, 
                                 float *const *dargs, void *cuda_stream)
 {
     if (!plan) { tad::set_error("NULL plan"); return TAD_ERR_INVALID_ARG; }
-    const size_t need = tad_workspace_bytes(plan);
+    const size_t need = required_bytes(plan);
     if (need > TAD_NOALLOC_SCRATCH_BYTES) {
         char msg[160];
         snprintf(msg, sizeof msg, "this plan needs %zu bytes of scratch, tad_backward_noalloc holds at most %zu; "

@@ -9,6 +9,7 @@ import math
 import pytest
 import torch
 
+from paper_1711_01348_b200 import Plan
 from workloads import configs as W
 
 pytestmark = pytest.mark.gpu
@@ -67,6 +68,37 @@ def test_strided_convolution(nb, nc, no, nt, nu):
     scale = conv(args[0].double().abs(), args[1].double().abs(), df.double().abs())
     for got, w, s, n, what in zip((f, dx, dw), want, scale, (nc * nu, no * nu, nb * nt), ("forward", "dx", "dw")):
         _close(got, w, s, n, what)
+
+
+# (rows, summed, columns): every gather order of the operand that is split ahead, ragged tiles and stages, with and without a split
+@pytest.mark.parametrize("ni,nk,nj", [(700, 5003, 501), (5003, 501, 700), (640, 200, 13001)])
+def test_columns_split_ahead(ni, nk, nj):
+    for e in (W.ex_matmul(ni, nk, nj), W.ex_matmul_t(ni, nj, nk)):
+        assert any("columns split ahead" in Plan(e).disassemble(w) for w in (-1, 0, 1))
+    test_matrix_products(ni, nk, nj, False)
+    test_matrix_products(ni, nk, nj, True)
+
+
+@pytest.mark.parametrize("nb,nc,no,nt,nu", [(1, 3000, 512, 500, 3), (16, 96, 160, 1100, 5)])
+def test_convolution_split_ahead(nb, nc, no, nt, nu):
+    """A guarded operand split ahead, and one whose rows are windows."""
+    assert "columns split ahead" in Plan(W.conv1d(nb, nc, no, nt, nu)).disassemble(-1)
+    test_strided_convolution(nb, nc, no, nt, nu)
+
+
+def test_split_ahead_without_room():
+    """A workspace that holds all but the split operand gives the same result, as does a forward call without any."""
+    e = W.conv1d(16, 96, 160, 1100, 5)
+    args, df = W.make_inputs(e, ("normal", 0, 1), seed=5)
+    run = GpuRun(e, args, df)
+    f, grads = run.forward(), run.backward()
+    run.plan.forward([a.data_ptr() for a in run.args], run.f.data_ptr(), torch.cuda.current_stream().cuda_stream)
+    run.ws = run.ws[:-1]
+    again = run.backward()
+    scale = torch.nn.functional.conv1d(args[0].double().abs(), args[1].double().abs(), stride=2)[:, :, :1100]
+    _close(run.f.cpu().numpy(), torch.from_numpy(f).double(), scale, 480, "forward")
+    for a, b in zip(again, grads):
+        assert float(abs(a - b).max()) <= 1e-5 * float(abs(b).max())
 
 
 @pytest.mark.parametrize("nk,nj", [(70, 140), (33, 76000)])
