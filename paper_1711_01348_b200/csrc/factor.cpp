@@ -25,7 +25,10 @@ namespace {
 
 constexpr double SMALL_SPACE = double(1 << 24);     // index spaces up to this size are summed by an interpreter kernel
 constexpr double MIN_SPACE = double(1 << 15);       // kernels with a smaller index space stay as they are
-constexpr double MIN_GAIN = 6.0;                    // a contraction must shrink its index space at least this much
+// A contraction must shrink its index space at least this much.  The least that is measured to pay: the intro expression at
+// 8192 x 8192 with sums of 3, 4 and 5 terms takes 642, 722 and 812 us forward as written and 122 with the sums pushed inside
+// (backward 1707, 1880, 2078 against 640).
+constexpr double MIN_GAIN = 3.0;
 constexpr size_t MAX_MONOS = 16;
 constexpr size_t MAX_DEGREE = 6;
 
