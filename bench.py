@@ -244,6 +244,23 @@ def time_workload(key, opts, dev, distributed, replicas, rows=0, saved_forward=F
             "ms_per_step": total_ms / steps, "n_stages": n_stages, "steps": steps}
 
 
+def line_elements(expr, p):
+    """Elements of argument p if the expression reads one strided line of it (a diagonal), else 0: tad_step_host copies
+    only those up, and behind the gradient's zeros only those down."""
+    accs = [a for a in expr.accesses if a.arg == p]
+    if len(accs) != 1:
+        return 0
+    step = [0] * expr.n_idx
+    stride = 1
+    for row, extent in zip(reversed(accs[0].A), reversed(expr.arg_shapes[p])):
+        step = [s + stride * r for s, r in zip(step, row)]
+        stride *= extent
+    moving = [v for v, s in enumerate(step) if s]
+    if len(moving) != 1 or moving[0] >= len(expr.out_shape) or abs(step[moving[0]]) < 64:
+        return 0
+    return expr.out_shape[moving[0]]
+
+
 def part_records(run, peaks, fp32_clock_tflops, fp32_measured_tflops):
     """Per part: time, algorithmic work (the expression as written, counted by the plan), the roof that binds
     it and the achieved fraction against three denominators: `frac` (measured HBM copy bandwidth / FP32 peak
@@ -321,8 +338,9 @@ def run_ours(opts):
         torch.cuda.synchronize()
         e2e_s = (time.perf_counter() - t0) / e2e_steps
         e2e_s = replicas.max_over_ranks(e2e_s, distributed, dev)
-        h2d = sum(a.numel() * 4 for a in args) + df.numel() * 4
-        d2h = h_f.numel() * 4 + sum(d.numel() * 4 for d in h_dargs)
+        lines = [line_elements(expr, p) for p in range(len(args))]
+        h2d = sum(4 * (n or a.numel()) for a, n in zip(args, lines)) + df.numel() * 4
+        d2h = h_f.numel() * 4 + sum(4 * (d.numel() + n) for d, n in zip(h_dargs, lines))
         e2e = {"value": world * elements_per_step(expr) / e2e_s, "unit": UNIT,
                "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h, "ms_per_step": 1e3 * e2e_s}
         del staging, h_args, h_df, h_f, h_dargs

@@ -58,7 +58,7 @@ struct alignas(16) TadcProgram {
     int32_t accumulate;            // 1: out += result
     int32_t out_vec4;              // 1: four consecutive n are four consecutive, 16-byte aligned output elements
     int32_t shape;                 // tiles: 0 = 128 x 128 (8 x 8 per thread), 1 = 128 x 32, 2 = 128 x 64, 3 = 128 x 36 (8 x 4 per thread);
-                                   // 4 = sums of rows (a warp per output), 5 = streamed narrow contraction, 6 = sums of columns (a thread per output),
+                                   // 4 = sums of rows (a warp per output), 6 = sums of columns (a thread per output),
                                    // 7 = tensor-core tiles of 128 rows (mma.cu)
     int32_t image;                 // shape 7: 1 = a kernel of its own splits the column operand into the tiles' shared-memory images
                                    // (image_bytes() of the workspace; without that much the operand is gathered as usual)

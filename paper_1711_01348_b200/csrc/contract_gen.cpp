@@ -53,11 +53,13 @@ bool fill_group(TadcGroup &G, std::vector<Digit> &ds, const AGuard *ga, const AG
 }
 
 // tensor-core tiles (mma.cu) or multiply-add tiles (contract.cu): a x b outputs, k terms each.  A stage of the tensor-core
-// kernel costs the same however full it is, so a side below 8 or fewer than 16 terms would leave most of it empty; below
-// 2^20 multiply-adds either kernel is one short wave (a step of the 203 x 157 x 7 intro expression does not change).
+// kernel costs the same however full it is, so fewer than 16 terms would leave most of it empty; below 2^20 multiply-adds
+// either kernel is one short wave (a step of the 203 x 157 x 7 intro expression does not change).  A narrow side pays all
+// the same, because the wide operand is what takes the time and sixteen columns are the smallest MMA: 4000 x 3000 summed,
+// 2 columns 183 us in multiply-add tiles, 28 here; 5 columns 50 / 28; 8192 x 8192 summed, 5 columns 180 / 121.
 bool mma_pays(int64_t a, int64_t b, int64_t k)
 {
-    return std::max(a, b) >= 64 && std::min(a, b) >= 8 && k >= 16 && (double)a * (double)b * (double)k >= (double)(1 << 20);
+    return std::max(a, b) >= 64 && std::min(a, b) >= 2 && k >= 16 && (double)a * (double)b * (double)k >= (double)(1 << 20);
 }
 
 }  // namespace
@@ -305,37 +307,13 @@ bool emit_program(const System &s0, float scale, int accumulate, bool allow_spli
         P.kchunk = fit(std::max<int64_t>(per, 1));
         P.ksplit = fit((P.K.extent + P.kchunk - 1) / P.kchunk);
     }
-    // the streaming kernel for narrow contractions (see tad_skinny_kernel): one digit per group, B rows of consecutive,
-    // 16-byte aligned elements, A consecutive along k (128-bit loads) or along m
-    if (P.shape != 7 && !one_column && s.B.ptr >= 0 && !ga && !gb && P.Z.extent == 1 && P.N.extent >= 2 && P.N.extent <= 36 && P.M.n_digits == 1 &&
-        P.K.n_digits == 1 && P.N.n_digits == 1 && P.N.sB[0] == 1 && P.M.extent >= 512 && P.K.extent >= 512) {
-        const int64_t sBk = P.K.sB[0], sAk = P.K.sA[0], sAm = P.M.sA[0];
-        const bool b_ok = sBk > 0 && sBk % 4 == 0 && s.B.base % 4 == 0 && (P.N.extent % 4 == 0 || sBk >= (P.N.extent + 3) / 4 * 4);
-        // (A along k is left to the tiles: with the lanes along k every lane reads its own rows of B from shared
-        // memory, which that memory cannot deliver at the rate of the multiply-adds; the kernel keeps the path)
-        const bool along_k = false && sAk == 1;
-        const bool along_m = sAm == 1;
-        if (b_ok && (along_k || along_m)) {
-            P.shape = 5;
-            P.modeA = along_k ? TG_K : TG_ROW;
-            const int64_t row_blocks = along_k ? (P.M.extent + 15) / 16 : (P.M.extent + 511) / 512;
-            split = 1;
-            if (allow_split && row_blocks < 222) split = std::max<int64_t>(1, std::min<int64_t>(296 / row_blocks, P.K.extent / 512));
-            const int64_t cells = (int64_t)P.M.extent * P.N.extent;
-            while (split > 1 && split * cells > (int64_t(1) << 25)) --split;
-            const int64_t per128 = ((P.K.extent + split - 1) / split + 127) / 128 * 128;
-            P.kchunk = fit(per128);
-            P.ksplit = fit((P.K.extent + per128 - 1) / per128);
-        }
-    }
-    if (P.shape != 5 && P.shape != 6 && P.shape != 7) {
+    if (P.shape != 6 && P.shape != 7) {
     split = std::max<int64_t>(1, split);
     const int64_t per = ((kstages + split - 1) / split) * TADC_BK;
     P.kchunk = fit(std::max<int64_t>(per, TADC_BK));
     P.ksplit = fit(std::max<int64_t>(1, (P.K.extent + P.kchunk - 1) / P.kchunk));
     if (P.ksplit <= 1) { P.ksplit = 1; P.kchunk = fit(std::max<int64_t>(kstages, 1) * TADC_BK); }
     }
-    if (P.shape == 5 && P.ksplit <= 1) { P.ksplit = 1; P.kchunk = fit((P.K.extent + 127) / 128 * 128); }
     char line[320];
     auto group_text = [&](const char *name, const TadcGroup &G) {
         std::string t = std::string("  ") + name + ":";
@@ -347,7 +325,7 @@ bool emit_program(const System &s0, float scale, int accumulate, bool allow_spli
     };
     std::snprintf(line, sizeof line, "; contraction %d x %d x %d (batch %d): A=ptr %d mode %d guard %d, B=ptr %d mode %d guard %d, tile %s, ksplit %d x %d, vec4 %d, scale %g, accumulate %d\n",
                   turned ? P.N.extent : P.M.extent, turned ? P.M.extent : P.N.extent, P.K.extent, P.Z.extent, P.ptrA, P.modeA, P.guardA, P.ptrB, P.modeB, P.guardB,
-                  P.shape == 7 ? (P.N.extent <= 64 ? "tensor 128x64" : "tensor 128x128") : P.shape == 6 ? "column sums" : P.shape == 5 ? "streamed" : P.shape == 4 ? "row sums" : P.shape == 1 ? "128x32" : P.shape == 3 ? "128x36" : P.shape == 2 ? "128x64" : "128x128", P.ksplit, P.kchunk, P.out_vec4, (double)P.scale, P.accumulate);
+                  P.shape == 7 ? (P.N.extent <= 64 ? "tensor 128x64" : "tensor 128x128") : P.shape == 6 ? "column sums" : P.shape == 4 ? "row sums" : P.shape == 1 ? "128x32" : P.shape == 3 ? "128x36" : P.shape == 2 ? "128x64" : "128x128", P.ksplit, P.kchunk, P.out_vec4, (double)P.scale, P.accumulate);
     if (P.image) std::snprintf(line + std::strlen(line) - 1, sizeof line - std::strlen(line), ", columns split ahead\n");
     text += line;
     text += group_text("m", P.M) + group_text("n", P.N) + group_text("k", P.K) + group_text("z", P.Z);

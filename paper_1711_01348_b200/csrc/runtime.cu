@@ -176,7 +176,6 @@ tad_status launch_contractions(const tad::Kernel &k, const TadpPointers &ptrs, c
         if (P.shape != 7 && P.ptrB >= 0 && P.modeB == TG_ROW16 && misaligned(ptrs.in[P.ptrB])) P.modeB = TG_ROW;
         if (P.out_vec4 && misaligned(ptrs.out)) P.out_vec4 = 0;
         // the streaming kernel copies B in 16-byte pieces
-        if (P.shape == 5 && misaligned(ptrs.in[P.ptrB])) P.shape = 3;
         // single-column passes beside the tile kernel: no planes of partial sums, outputs of their own
         const bool beside = side && k.contract.size() > 1 && i > 0 && P.ksplit == 1 && !P.accumulate && (P.shape == 4 || P.shape == 6);
         cudaStream_t on = stream;
@@ -436,7 +435,8 @@ unsigned char *image_of(const tad_plan *plan, void *workspace, size_t workspace_
 bool forward_splits(const tad::Kernel &k)
 {
     for (const TadcProgram &cp : k.contract) if (cp.ksplit > 1) return true;
-    for (const tad::Kernel &pk : k.pre) if (forward_splits(pk) || (pk.contract.empty() && pk.prog.zsplit > 1)) return true;
+    if (k.ew.empty() && k.contract.empty() && k.prog.zsplit > 1) return true;
+    for (const tad::Kernel &pk : k.pre) if (forward_splits(pk)) return true;
     return false;
 }
 

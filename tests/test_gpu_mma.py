@@ -44,6 +44,13 @@ def test_matrix_products(ni, nk, nj, transposed):
     _close(dy, want.T if transposed else want, scale.T if transposed else scale, ni, "dy")
 
 
+@pytest.mark.parametrize("ni,nk,nj", [(600, 900, 2), (5, 1300, 700), (7, 4001, 130), (3000, 400, 3)])
+def test_narrow_products(ni, nk, nj):
+    """A side of a few rows or columns, as an output and as the summed side of the gradients."""
+    test_matrix_products(ni, nk, nj, False)
+    test_matrix_products(ni, nk, nj, True)
+
+
 @pytest.mark.parametrize("ni,nk,nj", [(3077, 34, 3201), (3200, 64, 3072), (200, 17, 38000)])
 def test_one_stage_contractions(ni, nk, nj):
     """At most 64 terms and enough tiles for the pipelined kernel: ragged edges in both directions, full and cut stages."""
