@@ -23,10 +23,11 @@ namespace tad {
 
 namespace {
 
-// Index spaces up to this size are summed by one kernel of their own instead of being split into a contraction.  The intro
-// expression with a line at 2^24 / here, forward and all gradients in us: 1000 x 1500 x 6 56 + 475 / 22 + 158, 1000 x 1000 x 16
-// 116 + 595 / 19 + 148, 4000 x 128 x 20 65 + 550 / 36 + 134; at 2^20 the launches begin to weigh (600 x 600 x 5 88 -> 119).
-constexpr double SMALL_SPACE = double(1 << 22);
+// Index spaces up to this size are summed by one kernel of their own, as written.  Smaller ones are faster as contractions too
+// (the intro expression with a line at 2^24 / 2^22, forward and all gradients in us: 1000 x 1500 x 6 56 + 475 / 22 + 158,
+// 1000 x 1000 x 16 116 + 595 / 19 + 148), but a sum of squares (a + b)^2 with a near -b loses digits when it is expanded
+// (a about 10, b about -10: 1.6 times the tolerance of 1e-4; about 30: 12 times), so the line stays where the size demands it.
+constexpr double SMALL_SPACE = double(1 << 24);
 constexpr double MIN_SPACE = double(1 << 15);       // kernels with a smaller index space stay as they are
 // A contraction must shrink its index space at least this much.  The least that is measured to pay: the intro expression at
 // 8192 x 8192 with sums of 3, 4 and 5 terms takes 642, 722 and 812 us forward as written and 122 with the sums pushed inside

@@ -1,0 +1,34 @@
+"""Sums whose summands cancel.  In (a + b)^2 c with a near -b the expanded form c a^2 + 2 c a b + c b^2 loses the digits that
+the term as written keeps, so an expression of moderate size, or with a short sum, is evaluated as written: within the
+tolerance of every parity test, whose scale is the sum of |terms| of the expression as written."""
+import pytest
+
+from oracle.oracle import max_threads
+from paper_1711_01348_b200 import Plan
+from workloads import configs as W
+
+# index spaces of up to 2^24 elements
+MODERATE = [(1000, 1500, 6), (1000, 1000, 16), (4000, 128, 20)]
+
+
+def _offset_inputs(e):
+    args, df = W.make_inputs(e, ("uniform", -0.5, 0.5), seed=9)
+    args[0] += 30.0
+    args[1] -= 30.0
+    return args, df
+
+
+@pytest.mark.parametrize("ni,nj,nk", MODERATE)
+def test_evaluated_as_written(ni, nj, nk):
+    plan = Plan(W.intro(ni, nj, nk))
+    for which in [-1] + [-2 - s for s in range(plan.num_stages())]:
+        assert "; factored" not in plan.disassemble(which)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("ni,nj,nk", MODERATE)
+def test_cancelling_summands(ni, nj, nk):
+    from tests.gpu_util import check_against_oracle
+    e = W.intro(ni, nj, nk)
+    args, df = _offset_inputs(e)
+    check_against_oracle(e, args, df, nthreads=max_threads())
