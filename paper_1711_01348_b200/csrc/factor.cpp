@@ -29,10 +29,10 @@ namespace {
 // (a about 10, b about -10: 1.6 times the tolerance of 1e-4; about 30: 12 times), so the line stays where the size demands it.
 constexpr double SMALL_SPACE = double(1 << 24);
 constexpr double MIN_SPACE = double(1 << 15);       // kernels with a smaller index space stay as they are
-// A contraction must shrink its index space at least this much.  The least that is measured to pay: the intro expression at
-// 8192 x 8192 with sums of 3, 4 and 5 terms takes 642, 722 and 812 us forward as written and 122 with the sums pushed inside
-// (backward 1707, 1880, 2078 against 640).
-constexpr double MIN_GAIN = 3.0;
+// A contraction must shrink its index space at least this much.  Sums of 3 to 5 terms would be faster as contractions as well
+// (the intro expression at 8192 x 8192: 642, 722 and 812 us forward as written, 122 with the sums pushed inside; backward 1707,
+// 1880 and 2078 against 640), but lose digits where their summands cancel, as above.
+constexpr double MIN_GAIN = 6.0;
 constexpr size_t MAX_MONOS = 16;
 constexpr size_t MAX_DEGREE = 6;
 

@@ -9,6 +9,8 @@ from workloads import configs as W
 
 # index spaces of up to 2^24 elements
 MODERATE = [(1000, 1500, 6), (1000, 1000, 16), (4000, 128, 20)]
+# larger ones with sums of a few terms
+SHORT = [(2500, 2400, 3), (2500, 2400, 5)]
 
 
 def _offset_inputs(e):
@@ -18,7 +20,7 @@ def _offset_inputs(e):
     return args, df
 
 
-@pytest.mark.parametrize("ni,nj,nk", MODERATE)
+@pytest.mark.parametrize("ni,nj,nk", MODERATE + SHORT)
 def test_evaluated_as_written(ni, nj, nk):
     plan = Plan(W.intro(ni, nj, nk))
     for which in [-1] + [-2 - s for s in range(plan.num_stages())]:
@@ -26,9 +28,10 @@ def test_evaluated_as_written(ni, nj, nk):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("ni,nj,nk", MODERATE)
-def test_cancelling_summands(ni, nj, nk):
+@pytest.mark.parametrize("ni,nj,nk", MODERATE + SHORT)
+@pytest.mark.parametrize("offset", [True, False])
+def test_cancelling_summands(ni, nj, nk, offset):
     from tests.gpu_util import check_against_oracle
     e = W.intro(ni, nj, nk)
-    args, df = _offset_inputs(e)
+    args, df = _offset_inputs(e) if offset else W.make_inputs(e, ("uniform", -0.5, 0.5), seed=nk)
     check_against_oracle(e, args, df, nthreads=max_threads())

@@ -14,7 +14,7 @@ from workloads import configs as W
 
 pytestmark = pytest.mark.gpu
 
-from tests.gpu_util import GpuRun, assert_close  # noqa: E402
+from tests.gpu_util import GpuRun  # noqa: E402
 
 
 def _close(got, want, scale, n_terms, what):
@@ -124,36 +124,3 @@ def test_non_finite_operands(nk, nj):
     want = x.double() @ y.double()
     rows = [r for r in range(130) if r not in (3, 40, 129)]
     assert bool(((f.double() - want)[rows].abs() <= 1e-5 * (x.double().abs() @ y.double().abs())[rows]).all())
-
-
-@pytest.mark.parametrize("nk", [3, 5])
-def test_short_sums_pushed_inside(nk):
-    """Sums of a few terms, expanded into a contraction with an epilogue; the tolerance of every gradient test (1e-4 of the
-    sum of |terms|, those of the expanded form)."""
-    n, m = 2500, 2400
-    e = W.intro(n, m, nk)
-    assert "; contraction" in Plan(e).disassemble(-1)
-    args, df = W.make_inputs(e, ("uniform", -0.5, 0.5), seed=nk)
-    run = GpuRun(e, args, df)
-    f, grads = run.forward(), run.backward()
-    a, b, c, d = (x.double().requires_grad_(True) for x in args)
-
-    def value(a, b, c, d):
-        ci = torch.diagonal(c)[:, None]
-        cubes = sum(d[k:k + n] ** 3 for k in range(nk))[:, None]
-        return torch.exp(-((a * a).sum(1)[:, None] * ci + 2 * ci * (a @ b.T) + ci * (b * b).sum(1) + cubes))
-    want = value(a, b, c, d)
-    exact = torch.autograd.grad(want, (a, b, c, d), df.double())
-    assert_close(f, want.detach().numpy(), want.detach().numpy(), "forward")
-    with torch.no_grad():
-        g = df.double().abs() * want
-        ci = torch.diagonal(c).abs()
-        rows, cols = g.sum(1), g.sum(0)
-        sa = 2 * ci[:, None] * (a.abs() * rows[:, None] + g @ b.abs())
-        sb = 2 * ((g * ci[:, None]).T @ a.abs() + b.abs() * (g * ci[:, None]).sum(0)[:, None])
-        sc = torch.diag((a * a).sum(1) * rows + 2 * (a.abs() * (g @ b.abs())).sum(1) + g @ (b * b).sum(1))
-        sd = torch.zeros_like(d)
-        for k in range(nk):
-            sd[k:k + n] += 3 * d[k:k + n] ** 2 * rows
-    for got, x, s, what in zip(grads, exact, (sa, sb, sc, sd), "abcd"):
-        assert_close(got, x.numpy(), s.numpy(), "d" + what)
