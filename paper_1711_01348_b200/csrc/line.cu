@@ -75,10 +75,12 @@ __device__ __forceinline__ float walk(const float *const (&src)[4], const int (&
     return total;
 }
 
-template <bool STREAM>
+// A warp or a thread per output (modes 1 and 0): every one walks its own range from its own start.  The rule that chooses
+// between this and the lanes in step is in_step_pays() of line_gen.cpp.
+template <bool STREAM, bool BY_WARP>
 __global__ void __launch_bounds__(256)
-tad_line_warp_kernel(const __grid_constant__ TadlProgram P, const __grid_constant__ TadpPointers ptrs, const unsigned n_items,
-                     const unsigned n_rows, const int unroll)
+tad_line_walk_kernel(const __grid_constant__ TadlProgram P, const __grid_constant__ TadpPointers ptrs, const unsigned n_items,
+                     const unsigned cols, const unsigned lane_blocks, const unsigned n_rows, const int unroll)
 {
     tad_wait_previous();
     const unsigned tid = threadIdx.x, lane = tid & 31u;
@@ -92,9 +94,15 @@ tad_line_warp_kernel(const __grid_constant__ TadlProgram P, const __grid_constan
     const float *const srcs[4] = {src0, src1, src2, src3};
     const int sq[4] = {P.loads[0].sq, P.loads[1].sq, P.loads[2].sq, P.loads[3].sq};
     for (unsigned item = blockIdx.x; item < n_items; item += gridDim.x) {
-        const unsigned w = item * 8u + (tid >> 5);                // the output of this warp
-        const unsigned row = w / (unsigned)P.outer_ext[lane_var], lane0 = w - row * (unsigned)P.outer_ext[lane_var];
-        if (row >= n_rows) continue;
+        unsigned row, lane0;                                      // the output of this warp or thread
+        if (BY_WARP) {
+            const unsigned w = item * 8u + (tid >> 5);
+            row = w / (unsigned)P.outer_ext[lane_var]; lane0 = w - row * (unsigned)P.outer_ext[lane_var];
+        } else {
+            const unsigned rows_per_block = 256u / cols, lb = item % lane_blocks, rb = item / lane_blocks;
+            row = rb * rows_per_block + tid / cols; lane0 = lb * cols + tid % cols;
+        }
+        if (row >= n_rows || lane0 >= (unsigned)P.outer_ext[lane_var]) continue;
         int var[V];
         unsigned rem = row;
 #pragma unroll
@@ -129,8 +137,8 @@ tad_line_warp_kernel(const __grid_constant__ TadlProgram P, const __grid_constan
                 lo0 = max(lo0, a); hi0 = min(hi0, a + (1 << P.chunk_shift[0]) - 1);
             }
             const bool two = P.n_loops == 2;
-            constexpr int step_in = 32;
-            const int first_in = (int)lane;
+            constexpr int step_in = BY_WARP ? 32 : 1;
+            const int first_in = BY_WARP ? (int)lane : 0;
             // the innermost loop advances every offset by its own step
             const int l_in = two ? 1 : 0;
             const int d0 = P.loads[0].cz[l_in] * step_in, d1 = P.loads[1].cz[l_in] * step_in;
@@ -151,6 +159,7 @@ tad_line_warp_kernel(const __grid_constant__ TadlProgram P, const __grid_constan
                 int o[4] = {o0, o1, o2, o3};
                 const int d[4] = {d0, d1, d2, d3};
                 float part;
+// (chosen at run time: with a constant 4 the compiler orders the loads so that the sums of 4096 rows of 4096 take 60 us instead of 37)
 #define TAD_WALK(NL) (unroll == 2 ? walk<NL, 2, STREAM>(srcs, sq, o, d, zs, hi, step_in) : unroll == 4 ? walk<NL, 4, STREAM>(srcs, sq, o, d, zs, hi, step_in) : walk<NL, 8, STREAM>(srcs, sq, o, d, zs, hi, step_in))
                 if (n_loads == 1) part = TAD_WALK(1);
                 else if (n_loads == 2) part = TAD_WALK(2);
@@ -160,9 +169,11 @@ tad_line_warp_kernel(const __grid_constant__ TadlProgram P, const __grid_constan
                 acc += part;
             }
         }
+        if (BY_WARP) {
 #pragma unroll
-        for (int d = 16; d >= 1; d >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, d);
-        if (lane != 0) continue;
+            for (int d = 16; d >= 1; d >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, d);
+            if (lane != 0) continue;
+        }
         // the factor outside the sums
         float sc = P.cscale * P.cterm;
         for (int q = 0; q < P.n_scale; ++q) {
@@ -188,7 +199,7 @@ tad_line_warp_kernel(const __grid_constant__ TadlProgram P, const __grid_constan
     }
 }
 
-// A thread per output (mode 0).  The lanes of a row walk the union of their ranges in step, U terms in flight, so that
+// A thread per output in step (mode 2).  The lanes of a row walk the union of their ranges in step, U terms in flight, so that
 // load 0 is read in full lines whatever the ranges are; a batch outside some lane's range runs with a test per term.
 // (Every lane walking its own range from its own start read 16 pieces of different rows per load where the bounds move
 // with the lane, and paid the set-up of an output - divisions, guards - for every share of 64 terms: sums over
@@ -367,7 +378,7 @@ cudaError_t tad_launch_line(const TadlProgram &P, const TadpPointers &ptrs, unsi
     if (P.mode == 1) items = (rows * lane_ext + 7) / 8;                 // eight warps, eight outputs per block
     else {
         const unsigned along = (lane_ext + (unsigned)P.lane_stride - 1u) / (unsigned)P.lane_stride;
-        rows *= (unsigned)P.lane_stride;
+        rows *= (unsigned)P.lane_stride;                                // (1 but for lanes in step)
         while (cols < 256u && cols < along) cols *= 2u;
         lane_blocks = (along + cols - 1u) / cols;
         items = ((rows + 256u / cols - 1) / (256u / cols)) * lane_blocks;
@@ -375,9 +386,11 @@ cudaError_t tad_launch_line(const TadlProgram &P, const TadpPointers &ptrs, unsi
     if (items >= (1ull << 31) || rows >= (1ull << 31)) return cudaErrorInvalidValue;
     const unsigned gx = (unsigned)std::min<unsigned long long>(items, (unsigned long long)sms * 32ull);
     dim3 grid(gx, (unsigned)std::max(1, P.zsplit), 1u);
-    if (P.mode == 1)
-        return P.stream ? tad_launch(tad_line_warp_kernel<true>, grid, 256, 0, stream, P, ptrs, (unsigned)items, (unsigned)rows, P.unroll)
-                        : tad_launch(tad_line_warp_kernel<false>, grid, 256, 0, stream, P, ptrs, (unsigned)items, (unsigned)rows, P.unroll);
+    if (P.mode != 2) {
+        const auto walk_kernel = P.mode == 1 ? (P.stream ? tad_line_walk_kernel<true, true> : tad_line_walk_kernel<false, true>)
+                                             : (P.stream ? tad_line_walk_kernel<true, false> : tad_line_walk_kernel<false, false>);
+        return tad_launch(walk_kernel, grid, 256, 0, stream, P, ptrs, (unsigned)items, cols, lane_blocks, (unsigned)rows, P.unroll);
+    }
     switch (P.n_loads) {
     case 1: return launch_rows<1>(P, ptrs, grid, (unsigned)items, cols, lane_blocks, (unsigned)rows, stream);
     case 2: return launch_rows<2>(P, ptrs, grid, (unsigned)items, cols, lane_blocks, (unsigned)rows, stream);

@@ -14,6 +14,102 @@
 
 namespace tad {
 
+namespace {
+
+// what the lanes of a warp walk: mean values over 64 warps spread over the outputs
+struct Walks {
+    double live;      // share of the positions that are elements with terms
+    double runs;      // runs of the inner loop (united over the lanes)
+    double own;       // terms of a run: of the lane with the most
+    double joint;     // ... and of the union of the lanes' ranges
+};
+
+Walks sample_walks(const TadlProgram &P)
+{
+    auto floor_div = [](int64_t a, int64_t b) { int64_t q = a / b; return (a % b != 0 && a < 0) ? q - 1 : q; };
+    auto row_num = [&](const TadlRow &R, const int64_t *var, int64_t z0) {
+        int64_t n = R.c0 + (int64_t)R.cz * z0;
+        for (int v = 0; v < P.n_outer; ++v) n += R.coef[v] * var[v];
+        return n;
+    };
+    auto range = [&](int l, const int64_t *var, int64_t z0, int64_t &lo, int64_t &hi) {
+        lo = INT64_MIN; hi = INT64_MAX;
+        for (int r = 0; r < P.n_lower[l]; ++r) lo = std::max(lo, -floor_div(-row_num(P.lower[l][r], var, z0), P.lower[l][r].den));
+        for (int r = 0; r < P.n_upper[l]; ++r) hi = std::min(hi, floor_div(row_num(P.upper[l][r], var, z0), P.upper[l][r].den));
+    };
+    constexpr int WARPS = 64;
+    const int in = P.n_loops - 1;
+    const int64_t along = (P.outer_ext[P.lane_var] + P.lane_stride - 1) / P.lane_stride;
+    int64_t rows = P.lane_stride;
+    for (int v = 0; v < P.n_outer; ++v) if (v != P.lane_var) rows *= std::max(1, P.outer_ext[v]);
+    const int64_t groups = (along + 31) / 32, total = rows * groups;
+    Walks w{0, 0, 0, 0};
+    if (total <= 0) return w;
+    double lanes = 0, with_terms = 0, alive = 0;
+    for (int i = 0; i < WARPS; ++i) {
+        const int64_t at = (int64_t)(((double)i + 0.5) / WARPS * (double)total) % total;
+        const int64_t row = at / groups, l0 = at % groups * 32;
+        int64_t var[32][TADP_MAX_VARS] = {}, first = INT64_MAX, last = INT64_MIN;
+        bool live[32] = {};
+        int64_t lo0[32], hi0[32];
+        for (int l = 0; l < 32 && l0 + l < along; ++l) {
+            int64_t rem = row;
+            const int64_t r = rem % P.lane_stride; rem /= P.lane_stride;
+            for (int v = P.n_outer - 1; v >= 0; --v) {
+                const int64_t e = std::max(1, P.outer_ext[v]);
+                if (v == P.lane_var) { var[l][v] = P.outer_lo[v] + P.lane_stride * (l0 + l) + r; continue; }
+                var[l][v] = P.outer_lo[v] + rem % e; rem /= e;
+            }
+            if (var[l][P.lane_var] >= P.outer_lo[P.lane_var] + (int64_t)P.outer_ext[P.lane_var]) continue;
+            lanes += 1;
+            bool ok = true;
+            for (int g = 0; g < P.n_guards; ++g) ok = ok && row_num(P.guards[g], var[l], 0) <= 0;
+            if (!ok) continue;
+            range(0, var[l], 0, lo0[l], hi0[l]);
+            if (lo0[l] > hi0[l]) continue;
+            live[l] = true; with_terms += 1;
+            first = std::min(first, lo0[l]); last = std::max(last, hi0[l]);
+        }
+        if (first > last) continue;
+        const double runs = in ? (double)(last - first + 1) : 1.0;
+        const int64_t z0 = first + (last - first) * (2 * (i % 4) + 1) / 8;
+        int64_t own = 0, a = INT64_MAX, b = INT64_MIN;
+        for (int l = 0; l < 32; ++l) {
+            if (!live[l]) continue;
+            int64_t lo = lo0[l], hi = hi0[l];
+            if (in) { if (z0 < lo0[l] || z0 > hi0[l]) continue; range(1, var[l], z0, lo, hi); }
+            if (lo > hi) continue;
+            const int64_t skew = P.lane_skew * (l0 + l);
+            own = std::max(own, hi - lo + 1); a = std::min(a, lo - skew); b = std::max(b, hi - skew);
+        }
+        alive += 1; w.runs += runs;
+        w.own += (double)own; w.joint += a > b ? 0.0 : (double)(b - a + 1);
+    }
+    w.live = lanes > 0 ? with_terms / lanes : 0;
+    if (alive > 0) { w.runs /= alive; w.own /= alive; w.joint /= alive; }
+    return w;
+}
+
+// Lanes in step or every thread by itself?  In step, load 0 is read in full lines and four times as many terms are in flight,
+// but every run pays for the union of the ranges, rounded up to batches of sixteen, and a thread needs more registers.
+// Measured over 371 kernels of random expressions, lattices and the benchmark's workloads, in step / by itself in us:
+//   one loop   x[2i + 3j] of 4096^2 terms 36 / 81, 512^3 terms 164 / 265, 9000 outputs of 60 terms 8 / 20;
+//              but 443821 outputs of 21 terms 40 / 33, 2050560 of 22 60 / 39, 953400 of 45 45 / 36, 235873 of 2 16 / 9,
+//              28 million positions of which few are elements 306 / 145
+//   two loops  512 x 512 terms for 512 outputs 126 / 268, 400 x 47 for 3425 66 / 88;
+//              but 371 x 5 for 66660 outputs 663 / 313, 159 x 3 for 54760 175 / 102, and, with load 0 in pieces either way,
+//              144 x 59 for 5879 85 / 47
+bool in_step_pays(const Walks &w, int n_loops, double longest, double outputs, int pieces, bool unit)
+{
+    if (w.joint > 2 * w.own) return false;
+    if (n_loops == 1) return longest >= (outputs <= 131072 ? 12 : 64);
+    const double threads = outputs * pieces * w.live;            // with terms
+    if (w.live < 1.0 / 64 || (!unit && threads >= 262144)) return false;
+    return w.own >= (threads <= 65536 ? 20 : 40);
+}
+
+}  // namespace
+
 bool try_line(Gen &g, Kernel &k, int root, int scale, bool allow_split, const std::vector<std::vector<TadpRow>> &lower_in,
               const std::vector<std::vector<TadpRow>> &upper_in, const std::vector<TadpRow> &guards)
 {
@@ -215,35 +311,48 @@ bool try_line(Gen &g, Kernel &k, int root, int scale, bool allow_split, const st
         }
         P.zsplit = P.n_share[0] * P.n_share[1];
     }
-    // a masked gradient's box also holds positions that are no elements (their offsets may fall on real ones): the
-    // reduction writes only where the guards held
-    P.unroll = 4;
-    // lanes whose reads of load 0 are consecutive: along the lane variable as it is, or every s-th output of it with the
-    // inner loop shifted by t per lane, where  s coef + t step = +-1
+    // lanes whose reads of load 0 are consecutive: along the lane variable as it is, or (in step) every s-th output of it with
+    // the inner loop shifted by t per lane, where  s coef + t step = +-1
     P.lane_stride = 1; P.lane_skew = 0;
     bool unit = P.mode == 1 ? std::abs(B.cz[l_in]) == 1 : std::abs(B.coef[lane]) == 1;
-    if (P.mode == 0 && !unit && B.cz[l_in] != 0 && B.coef[lane] != 0)
-        for (int s = 1; s <= 8 && !unit && prog.outer_ext[lane] / s >= 32; ++s)
-            for (int64_t want : {1, -1}) {
-                const int64_t rest = want - (int64_t)s * B.coef[lane];
-                if (unit || rest % B.cz[l_in] || std::llabs(rest / B.cz[l_in]) > 8) continue;
-                unit = true; P.lane_stride = s; P.lane_skew = (int32_t)(rest / B.cz[l_in]);
-            }
-    P.stream = unit ? 1 : 0;
-    // pieces per thread: as many as leave the GPU two rounds of resident warps, the set-up of an output and its plane of
-    // partial sums being paid once for all of them (every n-th piece goes to the same thread: outputs with short ranges
-    // give every share the same work)
     const int pieces = P.zsplit;
     if (P.mode == 0) {
-        double warps = outputs / 32.0 * P.zsplit;
-        for (int l : {l_in, 0})
-            while (P.n_share[l] > 1 && warps >= 2.0 * 148 * 48) {
-                const int less = (P.n_share[l] + 1) / 2;
-                warps *= (double)less / P.n_share[l];
-                P.n_share[l] = less;
-            }
-        P.zsplit = P.n_share[0] * P.n_share[1];
+        TadlProgram Q = P;
+        bool unit_in_step = unit;
+        if (!unit && B.cz[l_in] != 0 && B.coef[lane] != 0)
+            for (int s = 1; s <= 8 && !unit_in_step && prog.outer_ext[lane] / s >= 32; ++s)
+                for (int64_t want : {1, -1}) {
+                    const int64_t rest = want - (int64_t)s * B.coef[lane];
+                    if (unit_in_step || rest % B.cz[l_in] || std::llabs(rest / B.cz[l_in]) > 8) continue;
+                    unit_in_step = true; Q.lane_stride = s; Q.lane_skew = (int32_t)(rest / B.cz[l_in]);
+                }
+        const Walks w = sample_walks(Q);
+        if (in_step_pays(w, n_loops, ext_in, outputs, pieces, unit_in_step)) {
+            Q.mode = 2;
+            unit = unit_in_step;
+            // pieces per thread: as many as leave the GPU two rounds of resident warps, the set-up of an output and its plane of
+            // partial sums being paid once for all of them (every n-th piece goes to the same thread: outputs with short ranges
+            // give every share the same work).  Where most positions are no elements some warps per SM must have terms all the
+            // same (34 of 138790 positions with terms, 17 shares cut to 3: 7.5 -> 180 ms).
+            double warps = outputs / 32.0 * Q.zsplit;
+            for (int l : {l_in, 0})
+                while (Q.n_share[l] > 1 && warps >= 2.0 * 148 * 48 && warps * w.live >= 148.0 * 4) {
+                    const int less = (Q.n_share[l] + 1) / 2;
+                    warps *= (double)less / Q.n_share[l];
+                    Q.n_share[l] = less;
+                }
+            Q.zsplit = Q.n_share[0] * Q.n_share[1];
+            P = Q;
+        } else if (pieces > 1 && outputs / 32.0 * w.live >= 148.0 * 48) {
+            // enough outputs with terms to fill the GPU by themselves: planes would only cost their traffic (13 x 4 terms for
+            // 388752 outputs in two shares 70 us, unsplit 26; 28 x 4 for 235216 in 14 shares 130 us, unsplit 71)
+            P.n_share[0] = P.n_share[1] = 1; P.zsplit = 1;
+        }
     }
+    P.stream = unit ? 1 : 0;
+    P.unroll = 4;
+    // a masked gradient's box also holds positions that are no elements (their offsets may fall on real ones): the
+    // reduction writes only where the guards held
     P.live_plane = (P.zsplit > 1 && prog.write_only_live) ? 1 : 0;
     if (P.zsplit <= 1) prog.write_only_live = 0;
     k.line = {P};
@@ -252,7 +361,7 @@ bool try_line(Gen &g, Kernel &k, int root, int scale, bool allow_split, const st
     for (int v = 0; v < g.n_outer; ++v) prog.part_coef[v] = P.part_coef[v];
     char line[256];
     std::snprintf(line, sizeof line, "; line sums: %d loads x %d loops, outer factor of %d loads, %s, lanes along variable %d, %d shares, %d guards, %d planes, lane stride %d skew %d\n",
-                  P.n_loads, P.n_loops, P.n_scale, P.mode == 1 ? "a warp per output" : "a thread per output", P.lane_var, pieces, P.n_guards, P.zsplit, P.lane_stride, P.lane_skew);
+                  P.n_loads, P.n_loops, P.n_scale, P.mode == 1 ? "a warp per output" : P.mode == 2 ? "a thread per output in step" : "a thread per output", P.lane_var, pieces, P.n_guards, P.zsplit, P.lane_stride, P.lane_skew);
     k.listing = line;
     for (int i = 0; i < P.n_loads; ++i) {
         std::snprintf(line, sizeof line, ";   load %d ptr=%d base=%d coef=[%d %d %d %d] step=[%d %d]%s\n", i, P.loads[i].ptr, P.loads[i].base, P.loads[i].coef[0],

@@ -19,6 +19,21 @@ def _strided(n, m, a, c, extra):
     return b.done()
 
 
+def _few_elements(n, nj, nk):
+    """f_i = sum_jk x_{j+k} y_{i+j} with x as long as the output: nj + nk - 1 elements of its gradient have terms."""
+    b = Builder("few_elements", [n], 2, ["x", "y"], [[n], [n + nj]])
+    p = b.bin("mul", b.load("x", [[0, 1, 1]]), b.load("y", [[1, 1, 0]]))
+    b.sum(1, 0, nj - 1, b.sum(2, 0, nk - 1, p))
+    return b.done()
+
+
+def _short_runs(n, m, k):
+    """f_ij = sum_k x_{i+k} w_{j+k}: the gradient of x walks m runs of at most k terms."""
+    b = Builder("short_runs", [n, m], 1, ["x", "w"], [[n + k - 1], [m + k - 1]])
+    b.sum(2, 0, k - 1, b.bin("mul", b.load("x", [[1, 0, 1]]), b.load("w", [[0, 1, 1]])))
+    return b.done()
+
+
 CASES = {
     "bounds_move_with_the_lane": lambda: W.shifted(777),
     "short_rows": lambda: W.nonunimodular(21),
@@ -29,6 +44,8 @@ CASES = {
     "no_unit_lanes": lambda: _strided(90, 80, 11, 13, True),
     "one_lane_wide": lambda: _strided(1500, 1, 1, 1, True),
     "many_pieces": lambda: _strided(9, 40000, 1, 1, True),
+    "few_elements": lambda: _few_elements(30001, 6, 29),
+    "short_runs": lambda: _short_runs(1500, 90, 3),
 }
 
 
