@@ -33,6 +33,9 @@ constexpr double MIN_SPACE = double(1 << 15);       // kernels with a smaller in
 // (the intro expression at 8192 x 8192: 642, 722 and 812 us forward as written, 122 with the sums pushed inside; backward 1707,
 // 1880 and 2078 against 640), but lose digits where their summands cancel, as above.
 constexpr double MIN_GAIN = 6.0;
+// A sum over one product is only reordered, sum_z c X Y(z) = c X sum_z Y(z), and its terms stay what they were: it follows lower
+// lines (random contraction of 1.3e7 terms 147 -> 9 us forward, 110 -> 17 us backward; 440 -> 160 and 131 -> 39 us for others).
+constexpr double SMALL_PRODUCT = double(1 << 22), MIN_GAIN_PRODUCT = 3.0;
 constexpr size_t MAX_MONOS = 16;
 constexpr size_t MAX_DEGREE = 6;
 
@@ -216,6 +219,13 @@ struct Factorizer {
         return tensor_load(t, 0);
     }
 
+    // the sum being solved: is it over one product, and its lines
+    bool one_product = false;
+    double small_space = SMALL_SPACE, min_gain = MIN_GAIN;
+    // an auxiliary kernel over two or more variables is neither split nor spread over lanes beyond one block: few outputs with
+    // many terms each stay in the kernel they belong to, which is (one output of 562 x 595 terms: 141 ms here, 0.5 ms there)
+    bool serial(uint32_t outs, uint32_t sums) const { return vars_of(sums).size() >= 2 && space(outs) < 4096 && space(outs | sums) > 4096 * space(outs); }
+
     // sum over kmask of  a_inst * product(b_atoms): a request in the group of (a_inst, kmask)
     int request(int a_inst, uint32_t kmask, const std::vector<int> &b_atoms)
     {
@@ -251,9 +261,10 @@ struct Factorizer {
         for (int v = 0; v < TADP_MAX_VARS; ++v) if ((emask & (1u << v)) && !(live & (1u << v))) mult *= (double)vext[v];
         while (live) {
             const uint32_t d_all = deps_of(red);
-            if (space(d_all) <= SMALL_SPACE) {
+            if (space(d_all) <= small_space) {
                 // everything that is left is small: one interpreter kernel; factors over its output variables join it
                 const uint32_t d_out = d_all & ~live;
+                if (one_product && serial(d_out, live)) return -1;
                 Mono body; body.atoms = red;
                 std::vector<int> keep;
                 for (int a : pre) { if ((w.inst[a].deps & ~d_out) == 0 && w.inst[a].deps) body.atoms.push_back(a); else keep.push_back(a); }
@@ -278,9 +289,10 @@ struct Factorizer {
                 const double cost = space(deps_of(sv)), outsp = space(deps_of(sv) & ~kv);
                 if (best < 0 || cost < best_cost || (cost == best_cost && outsp < best_out)) { best = v; best_cost = cost; best_out = outsp; best_k = kv; best_s = sv; }
             }
-            if (best < 0 || best_cost / best_out < MIN_GAIN) return -1;
+            if (best < 0 || best_cost / best_out < min_gain) return -1;
             int t_inst = -1;
-            if (best_cost <= SMALL_SPACE) {
+            if (best_cost <= small_space) {
+                if (one_product && serial(deps_of(best_s) & ~best_k, best_k)) return -1;
                 Mono body; body.atoms = best_s;
                 t_inst = small_sum(deps_of(best_s) & ~best_k, best_k, Poly{body});
             } else {
@@ -291,7 +303,7 @@ struct Factorizer {
                 std::vector<int> rest;
                 bool taken = false;
                 for (int a : best_s) { if (a == big && !taken) { taken = true; continue; } rest.push_back(a); }
-                if (!rest.empty() && space(deps_of(rest)) > SMALL_SPACE && !(rest.size() == 1 && is_plain_load(rest[0]))) return -1;
+                if (!rest.empty() && space(deps_of(rest)) > small_space && !(rest.size() == 1 && is_plain_load(rest[0]))) return -1;
                 // the streamed operand must bring enough rows of its own to fill tiles (variables that the second
                 // operand reads too only number independent contractions)
                 if (space(w.inst[big].deps & ~best_k & ~deps_of(rest)) < 64) return -1;
@@ -322,12 +334,15 @@ struct Factorizer {
         Poly P;
         if (!expand(body, P) || P.empty()) return -1;
         if (space(w.inst[body].deps | emask) < MIN_SPACE) return -1;
+        one_product = P.size() == 1;
+        small_space = one_product ? SMALL_PRODUCT : SMALL_SPACE;
+        min_gain = one_product ? MIN_GAIN_PRODUCT : MIN_GAIN;
         // monomials whose whole index space is small are summed together by one interpreter kernel per output set
         std::map<uint32_t, Poly> small;
         Poly rest;
         for (const Mono &m : P) {
             const uint32_t d = deps_of(m.atoms);
-            if (space(d | emask) <= SMALL_SPACE && (d & emask)) small[d & ~emask].push_back(m);
+            if (space(d | emask) <= small_space && (d & emask)) small[d & ~emask].push_back(m);
             else rest.push_back(m);
         }
         // nothing but small monomials: the sum is cheap as it is
