@@ -779,6 +779,12 @@ bool try_points(Gen &g, Kernel &k, int root, int scale, bool allow_split, const 
         zv.push_back(v);
     }
     // ---- the program: once per output, per term, on the sum ----
+    bool unrolled_sum = false;                               // would the interpreter keep several summands of a sum in flight?
+    {
+        Gen other = g;
+        choose_element_variable(other, true, 0u);
+        unrolled_sum = other.unroll_var >= 0 && other.vars[other.unroll_var].kind == 2;
+    }
     g.unroll_var = -1;
     const int n_temps = assign_temporaries(g, root, scale);
     Emitter em(g);
@@ -851,6 +857,12 @@ bool try_points(Gen &g, Kernel &k, int root, int scale, bool allow_split, const 
     for (int v = 0; v < g.n_outer; ++v) points *= (double)ext[v];
     for (int v : zv) terms *= (double)ext[v];
     if (points * terms * inner > limit) return false;
+    // Few threads, each in a long serial chain of sums: the interpreter is faster where it keeps several summands of the inner sum
+    // in flight and there is nothing to spread over lanes or blocks here (us, points -> interpreter: 2998 outputs of 3 x 31
+    // summands 64 -> 36, 15755 of 2 x 30 108 -> 57, 2647 of 2 x 16 63 -> 48), or next to nothing (one output of 2818 terms with
+    // 10 x 29 summands 1415 -> 299, with eleven blocks of points 680).  With terms to spread it loses (274 outputs of 115 terms
+    // with 30 summands 2183, here 301), and behind three kernel coordinates (2299 terms with 180 summands 694, here 333).
+    if (unrolled_sum && inner_sum < 0 && inner >= 16 && points * terms < 148.0 * 256 && (terms == 1 || (points <= 4 && g.kappa <= 2))) return false;
     // plain element-wise programs have a kernel of their own, which a few thousand outputs do not fill
     if (g.kappa == 0 && zv.empty() && sv.empty() && n_temps == 0 && points > POINT_PLAIN) return false;
     // every offset the kernel can form must lie inside its tensor
@@ -956,15 +968,22 @@ bool try_points(Gen &g, Kernel &k, int root, int scale, bool allow_split, const 
     const bool sums = g.kappa >= 1 || Q.n_z > 0;
     if (sums) {
         Q.along_terms = !zv.empty() && unit_of_big(zv.back()) && !(!ov.empty() && unit_of_big(ov.back())) ? 1 : 0;
-        Q.unroll = terms >= 4 && inner_sum < 0 ? 4 : 1;
+        // (many short sums: a thread to each leaves no lane idle, and its neighbours' lines are in the L1 cache; a forward pass
+        // with 277440 sums of 12 terms 154 us with 16 lanes and four points each, most of them masked off, 34 this way)
+        if (terms < 32 && points >= 148.0 * 512.0) Q.along_terms = 0;
+        // A term with long sums inside is work enough for a thread by itself where four of them to a thread would leave the GPU
+        // idle, and its terms are spread over blocks as far as they go (one output of 2299 terms with 180 summands each:
+        // one block 520 us, nine blocks 333 us; of 2643 terms with 176: 274 -> 259).
+        const bool deep = inner >= 8 && points * terms < 4 * 148.0 * 128;
+        Q.unroll = terms >= 4 && inner_sum < 0 && !deep ? 4 : 1;
         if (Q.along_terms) while (Q.lt < 32 && Q.lt < terms) Q.lt *= 2;
         while (Q.lt < 256 && points * Q.lt < 148.0 * 512.0 && Q.lt * Q.unroll < terms) Q.lt *= 2;
         if (Q.lt == 1 && terms == 1) Q.lt = 2;                // (a single term still goes through the summing path)
         int64_t cells = 1;
         for (int v = g.n_outer - 1; v >= 0; --v) { prog.part_coef[v] = to_i32(cells); if (at[v] >= 0) Q.part_coef[at[v]] = to_i32(cells); cells = mul_ck(cells, ext[v]); }
         const double blocks = std::ceil(points * Q.lt / 256.0), batches = terms / ((double)Q.lt * Q.unroll);
-        if (allow_split && g.kappa >= 1 && blocks < 148 && batches >= 8 && cells <= (1 << 20))
-            Q.zsplit = (int32_t)std::max(1.0, std::min({128.0, std::floor(148.0 * 5 / blocks), std::floor(batches / 1.5)}));
+        if (allow_split && g.kappa >= 1 && blocks < 148 && batches * (deep ? inner : 1.0) >= 8 && cells <= (1 << 20))
+            Q.zsplit = (int32_t)std::max(1.0, std::min({128.0, std::floor(148.0 * 5 / blocks), std::floor(deep ? batches : batches / 1.5)}));
         Q.part_limit = to_i32(cells);
     } else if (points >= 131072) Q.unroll = 4;
     prog.zsplit = Q.zsplit; prog.part_limit = Q.part_limit; prog.n_outer = g.n_outer; prog.write_only_live = 0;
