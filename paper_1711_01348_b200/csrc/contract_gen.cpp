@@ -16,6 +16,7 @@
 // class becomes a contraction of its own; the remaining constant bounds of z turn into a guard
 // that reads operand elements outside them as zero.
 #include <algorithm>
+#include <cmath>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -94,7 +95,8 @@ bool emit_program(const System &s0, float scale, int accumulate, bool allow_spli
         }
         if (s.B.ptr >= 0) {
             int64_t a = side(s.A, s.B), b = side(s.B, s.A);
-            mma = mma_pays(a, b, kext) && rest == 1 && s.A.limit < (int64_t(1) << 30) && s.B.limit < (int64_t(1) << 30);   // (byte offsets of 32 bits)
+            // (a smaller constant would leave the normal numbers when the kernel multiplies it by 2^-48)
+            mma = mma_pays(a, b, kext) && std::fabs(scale) >= 0x1p-70f && rest == 1 && s.A.limit < (int64_t(1) << 30) && s.B.limit < (int64_t(1) << 30);   // (byte offsets of 32 bits)
             const bool out_a = contiguous >= 0 && s.A.coef[contiguous] != 0 && s.B.coef[contiguous] == 0;
             const bool out_b = contiguous >= 0 && s.B.coef[contiguous] != 0 && s.A.coef[contiguous] == 0;
             if (mma && ((out_b && b >= 128) || (!out_a && b > a) || (out_a && a < 128 && b > a))) { std::swap(s.A, s.B); turned = true; }

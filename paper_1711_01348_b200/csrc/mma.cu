@@ -1,16 +1,19 @@
 // Tensor-core kernel for contraction programs (contract.h), fp32 in and fp32 out.
 //
-// Every fp32 operand element is split exactly into three bf16 values, x = x1 + x2 + x3 (8 + 8 + 8 significant
-// bits, each part the rounded remainder of the ones before it), and a product is the sum of six bf16 products,
+// Every fp32 operand element is multiplied by 2^24 and split exactly into three bf16 values, 2^24 x = x1 + x2 + x3 (8 + 8 + 8
+// significant bits, each part the rounded remainder of the ones before it), and a product is the sum of six bf16 products,
 //     a b = a1 b1 + (a1 b2 + a2 b1) + (a1 b3 + a2 b2 + a3 b1).
+// The factor keeps the parts of the smallest operands out of the subnormal numbers: bf16 ends where fp32 ends, so the third
+// part of an |x| below 2^-109 would lose bits, then the second (relative error 2e-6 at 2^-115, 5e-4 at 1e-37); with it every
+// fp32 value below 2^104 is split exactly, and the sums are multiplied by 2^-48, which is exact.
 // What is left out, a2 b3 + a3 b2 + a3 b3, is at most 2^-23 |a b| and about 2^-26 |a b| in the mean square, below
 // the rounding of the additions.  bf16 products are exact in the fp32 accumulator; the accumulator itself
 // truncates, so a sum stays in it for one stage of 64 summation indices only (small products first, then four
 // steps of a1 b1) and the stages are added up in fp32 registers with round-to-nearest.  Measured against float64
 // (2-norm, normal operands): 0.8e-7 at 64 terms, 1.2e-7 at 1100, 1.3e-7 at 2048; chains of fp32 multiply-adds
-// gave 4.2e-7 at 1100.  Outputs of a warp whose sums come out non-finite or huge (an operand beyond the bf16
-// range, an infinity times a zero part) are evaluated again with fp32 multiply-adds from the operands
-// themselves, so infinities and NaNs are those of the definition.
+// gave 4.2e-7 at 1100.  Outputs of a warp whose sums come out non-finite (an infinity times a zero part, an operand of
+// 2^104 or more, a sum of 2^80 or more) are evaluated again with fp32 multiply-adds from the operands themselves, so
+// infinities and NaNs are those of the definition.
 //
 // One block per SM.  Warps 0-15 gather the operands of a stage through the offset tables (global -> registers, a
 // whole stage ahead), split them and write them to shared memory in the 128-byte swizzled layout of the MMA
@@ -109,20 +112,28 @@ __device__ __forceinline__ unsigned long long make_desc(unsigned addr, unsigned 
 //   TM_RVEC  t = row, contiguous and aligned: two 128-bit loads                                  -> MN-major
 // (the row operand of the TM_ROW mode goes to tensor memory: a thread then takes the row of its own lane and the
 // sixteen summation indices of MMA step warp / 4)
-template <int MODE, int R, bool TMEM, int THREADS = NCW * 32>
+template <int MODE, int R, bool TMEM>
 struct Unit {
     static constexpr bool KMAJOR = MODE == TM_ROW || MODE == TM_KVEC, VEC = MODE == TM_KVEC || MODE == TM_RVEC;
     int l, t0, dst;
     __device__ __forceinline__ Unit(int tid, int i)
     {
-        const int u = tid + i * THREADS;
-        int o;
-        if (TMEM) { l = tid % BM; o = (tid / BM) * 2 + i; }
-        else if (MODE == TM_ROW) { l = u % R; o = u / R; }
-        else if (MODE == TM_KVEC) { o = u % (KS / 8); l = u / (KS / 8); }
-        else if (MODE == TM_K) { l = u % KS; o = u / KS; }
-        else { l = (u / 8) % KS; o = (u / (8 * KS)) * 8 + u % 8; }
-        t0 = o * 8;
+        if (TMEM) place(tid % BM, (tid / BM) * 2 + i);
+        else at(tid + i * NCW * 32, KS / 8);
+    }
+    // the u-th unit of a stage of n_o octets of summation indices
+    struct Among { int n_o; };
+    __device__ __forceinline__ Unit(int u, Among a) { at(u, a.n_o); }
+    __device__ __forceinline__ void at(int u, int n_o)
+    {
+        if (MODE == TM_ROW) place(u % R, u / R);
+        else if (MODE == TM_KVEC) { const int q = n_o == KS / 8 ? u / (KS / 8) : (u * (65536 / n_o + 1)) >> 16; place(q, u - q * n_o); }   // (u < 1024)
+        else if (MODE == TM_K) place(u % KS, u / KS);
+        else place((u / 8) % KS, (u / (8 * KS)) * 8 + u % 8);
+    }
+    __device__ __forceinline__ void place(int lane_at, int o)
+    {
+        l = lane_at; t0 = o * 8;
         dst = (KMAJOR ? 0 : (o >> 3) * (KS * 128)) + l * 128 + (((o & 7) ^ (l & 7)) << 4);
     }
 };
@@ -133,12 +144,10 @@ __device__ __forceinline__ float ldf(const float *__restrict__ src, unsigned byt
 }
 
 // rows: offsets and guards of the tile's rows; kt: offsets and guards of the stage's summation indices (KS each)
-template <int MODE, int R, bool TMEM, bool CHECK, int THREADS = NCW * 32>
-__device__ __forceinline__ void load_unit(float (&v)[8], const float *__restrict__ src, const int tid, const int i, const unsigned *row, const int *rowg,
+template <bool CHECK, class U>
+__device__ __forceinline__ void load_unit(float (&v)[8], const float *__restrict__ src, const U &u, const unsigned *row, const int *rowg,
                                           const unsigned *kt, const int *ktg, const unsigned gext)
 {
-    using U = Unit<MODE, R, TMEM, THREADS>;
-    const U u(tid, i);
     const unsigned base = U::KMAJOR ? row[u.l] : kt[u.l];
     const unsigned *tab = (U::KMAJOR ? kt : row) + u.t0;
     const int gbase = CHECK ? (U::KMAJOR ? rowg[u.l] : ktg[u.l]) : 0;
@@ -179,19 +188,42 @@ __device__ __forceinline__ void mask_unit(float (&v)[8], const U &u, const int l
     for (int j = 0; j < 8; ++j) if ((U::KMAJOR ? u.t0 + j : u.l) >= left) v[j] = 0.f;
 }
 
-// eight values -> three times eight bf16 (packed in pairs)
+constexpr float SPLIT_SCALE = 0x1p24f, SUM_SCALE = 0x1p-48f;      // of an operand, of a sum of products
+
+// two fp32 operations per instruction
+__device__ __forceinline__ float2 mul2(float2 a, float2 b)
+{
+    float2 r;
+    asm("{ .reg .b64 x, y, z; mov.b64 x, {%2, %3}; mov.b64 y, {%4, %5}; mul.rn.f32x2 z, x, y; mov.b64 {%0, %1}, z; }" : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return r;
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
+{
+    float2 r;
+    asm("{ .reg .b64 x, y, w, z; mov.b64 x, {%2, %3}; mov.b64 y, {%4, %5}; mov.b64 w, {%6, %7}; fma.rn.f32x2 z, x, y, w; mov.b64 {%0, %1}, z; }"
+        : "=f"(r.x), "=f"(r.y) : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+    return r;
+}
+
+// eight values times 2^24 -> three times eight bf16 (packed in pairs).  PAIRS: with two operations per instruction, which takes
+// the scaling out of the tile kernel's time (4096 x 2048 x 4096 353 -> 346 us); the one-stage kernel, whose few gathering warps
+// have no registers to spare for aligned pairs, is slower with it (8192 x 64 x 8192 153 -> 166 us).
+template <bool PAIRS>
 __device__ __forceinline__ void split_unit(const float (&v)[8], unsigned (&p1)[4], unsigned (&p2)[4], unsigned (&p3)[4])
 {
+    const float2 up = make_float2(SPLIT_SCALE, SPLIT_SCALE), minus = make_float2(-1.f, -1.f);
+    auto less = [&](float2 x, unsigned h) {                    // what two rounded parts leave
+        const float2 q = make_float2(__uint_as_float(h << 16), __uint_as_float(h & 0xffff0000u));
+        return PAIRS ? fma2(q, minus, x) : make_float2(x.x - q.x, x.y - q.y);
+    };
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-        const float x = v[2 * j], y = v[2 * j + 1];
-        unsigned h, m, l;
-        asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(h) : "f"(y), "f"(x));
-        const float rx = x - __uint_as_float(h << 16), ry = y - __uint_as_float(h & 0xffff0000u);
-        asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(m) : "f"(ry), "f"(rx));
-        const float sx = rx - __uint_as_float(m << 16), sy = ry - __uint_as_float(m & 0xffff0000u);
-        asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(l) : "f"(sy), "f"(sx));
-        p1[j] = h; p2[j] = m; p3[j] = l;
+        const float2 w = make_float2(v[2 * j], v[2 * j + 1]), x = PAIRS ? mul2(w, up) : make_float2(w.x * SPLIT_SCALE, w.y * SPLIT_SCALE);
+        asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(p1[j]) : "f"(x.y), "f"(x.x));
+        const float2 r = less(x, p1[j]);
+        asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(p2[j]) : "f"(r.y), "f"(r.x));
+        const float2 t = less(r, p2[j]);
+        asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(p3[j]) : "f"(t.y), "f"(t.x));
     }
 }
 
@@ -341,12 +373,13 @@ tad_mma_kernel(const __grid_constant__ TadcProgram P, const __grid_constant__ Ta
             const int *tg = reinterpret_cast<const int *>(t + KS);
             if constexpr (C::IMAGE) second = false;
             if (!second) {
-                if (check) load_unit<MA, BM, TS, true>(v, A, tid, i, rowA, rowgA, t, tg, gextA);
-                else load_unit<MA, BM, TS, false>(v, A, tid, i, rowA, rowgA, t, tg, gextA);
+                const Unit<MA, BM, TS> u(tid, i);
+                if (check) load_unit<true>(v, A, u, rowA, rowgA, t, tg, gextA);
+                else load_unit<false>(v, A, u, rowA, rowgA, t, tg, gextA);
             } else {
-                constexpr int MODE_B = C::IMAGE ? (int)TM_ROW : MB;
-                if (check) load_unit<MODE_B, BN, false, true>(v, B, tid, i, rowB, rowgB, t, tg, gextB);
-                else load_unit<MODE_B, BN, false, false>(v, B, tid, i, rowB, rowgB, t, tg, gextB);
+                const Unit<C::IMAGE ? (int)TM_ROW : MB, BN, false> u(tid, i);
+                if (check) load_unit<true>(v, B, u, rowB, rowgB, t, tg, gextB);
+                else load_unit<false>(v, B, u, rowB, rowgB, t, tg, gextB);
             }
         };
         // the column operand's image of stage s, as one bulk copy behind the row operand's buffer (its MMAs of stage s - 2 are done)
@@ -403,7 +436,7 @@ tad_mma_kernel(const __grid_constant__ TadcProgram P, const __grid_constant__ Ta
             unsigned p1[4], p2[4], p3[4];
 #pragma unroll
             for (int i = 0; i < C::UA; ++i) {
-                split_unit(va[i], p1, p2, p3);
+                split_unit<true>(va[i], p1, p2, p3);
                 if (more) load(va[i], i, s + 1, false, P.guardA != 0);
                 const Unit<MA, BM, TS> u(tid, i);
                 if (TS) {
@@ -418,7 +451,7 @@ tad_mma_kernel(const __grid_constant__ TadcProgram P, const __grid_constant__ Ta
             st += TS ? 0 : 3 * C::PART_A;
 #pragma unroll
             for (int i = 0; i < C::UB; ++i) {
-                split_unit(vb[i], p1, p2, p3);
+                split_unit<true>(vb[i], p1, p2, p3);
                 if (more) load(vb[i], i, s + 1, true, P.guardB != 0);
                 const Unit<C::IMAGE ? (int)TM_ROW : MB, BN, false> u(tid, i);
                 *reinterpret_cast<uint4 *>(st + u.dst) = make_uint4(p1[0], p1[1], p1[2], p1[3]);
@@ -472,6 +505,8 @@ tad_mma_kernel(const __grid_constant__ TadcProgram P, const __grid_constant__ Ta
                 }
             }
         } else if (live) {
+#pragma unroll
+            for (int j = 0; j < COLS; ++j) acc[j] *= SUM_SCALE;
             if (P.ksplit > 1) {
                 // plane of this share: columns outermost, so that the lanes write consecutive elements
                 float *dst = ptrs.part + ((size_t)zb * (unsigned)P.ksplit + ks) * Next * Mext + (size_t)n0 * Mext + m;
@@ -626,23 +661,25 @@ tad_mma_short_kernel(const __grid_constant__ TadcProgram P, const __grid_constan
         Parts z{0, 0, 0, 0, 0};
         auto gather = [&](auto mode, const float *__restrict__ src, const unsigned *row, const int *rowg, const int *kt, bool check, unsigned gext, unsigned char *dst) {
             constexpr int MODE = decltype(mode)::value;
-            using U = Unit<MODE, BM, false, CT>;
+            using U = Unit<MODE, BM, false>;
             const unsigned *kto = reinterpret_cast<const unsigned *>(kt);
+            // vectors along the summation index: the octets past its end are no units (34 indices: four rounds of units instead of five)
+            const int n_o = MODE == TM_KVEC ? kpad / 8 : KS / 8, units = MODE == TM_KVEC ? BM * n_o : UNITS;
             float v[UN][8];
 #pragma unroll
             for (int i = 0; i < UN; ++i) {
-                const U u(ct, i);
-                if (ct + i * CT >= UNITS || (U::KMAJOR ? u.t0 : u.l) >= kpad) continue;
-                if (check) load_unit<MODE, BM, false, true, CT>(v[i], src, ct, i, row, rowg, kto, kt + KS, gext);
-                else load_unit<MODE, BM, false, false, CT>(v[i], src, ct, i, row, rowg, kto, kt + KS, gext);
+                const U u(ct + i * CT, typename U::Among{n_o});
+                if (ct + i * CT >= units || (U::KMAJOR ? u.t0 : u.l) >= kpad) continue;
+                if (check) load_unit<true>(v[i], src, u, row, rowg, kto, kt + KS, gext);
+                else load_unit<false>(v[i], src, u, row, rowg, kto, kt + KS, gext);
             }
 #pragma unroll
             for (int i = 0; i < UN; ++i) {
-                const U u(ct, i);
-                if (ct + i * CT >= UNITS || (U::KMAJOR ? u.t0 : u.l) >= kpad) continue;
+                const U u(ct + i * CT, typename U::Among{n_o});
+                if (ct + i * CT >= units || (U::KMAJOR ? u.t0 : u.l) >= kpad) continue;
                 unsigned p1[4], p2[4], p3[4];
                 if (kpad != (int)K) mask_unit(v[i], u, (int)K);
-                split_unit(v[i], p1, p2, p3);
+                split_unit<false>(v[i], p1, p2, p3);
                 *reinterpret_cast<uint4 *>(dst + u.dst) = make_uint4(p1[0], p1[1], p1[2], p1[3]);
                 *reinterpret_cast<uint4 *>(dst + C::PART + u.dst) = make_uint4(p2[0], p2[1], p2[2], p2[3]);
                 *reinterpret_cast<uint4 *>(dst + 2 * C::PART + u.dst) = make_uint4(p3[0], p3[1], p3[2], p3[3]);
@@ -700,6 +737,7 @@ tad_mma_short_kernel(const __grid_constant__ TadcProgram P, const __grid_constan
         for (int j = 0; j < 16; ++j) { w[j] = 0.f; wn[j] = 0.f; }
         const float *__restrict__ src0 = pre >= 0 ? ptrs.in[P.epi_ptr[pre]] + (ptrdiff_t)P.epi_base[pre] : nullptr;
         const bool pre_mul = pre >= 0 && P.epi_op[pre] == TE_MUL_LOAD;
+        const float scale = P.scale * SUM_SCALE;               // (exact: the host keeps smaller constants away from this kernel)
         auto begin_tile = [&](int t) {
             if (t == 0 || ++tile_m == tiles_m) {
                 if (t > 0) { tile_m = 0; ++strip; }
@@ -764,10 +802,8 @@ tad_mma_short_kernel(const __grid_constant__ TadcProgram P, const __grid_constan
             if (h == 0) load_ahead(16);
             else if (t + 1 < n_tiles) { __syncwarp(); begin_tile(t + 1); load_ahead(0); }
             if (!redo) {
-                if (P.scale != 1.f) {
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) v[j] *= P.scale;
-                }
+                for (int j = 0; j < 16; ++j) v[j] *= scale;
 #define TAD_EPI_ALL(expr) _Pragma("unroll") for (int j = 0; j < 16; ++j) { float &x = v[j]; expr; }
                 for (int e = 0; e < P.n_epi; ++e) {
                     const float imm = P.epi_imm[e];
@@ -912,7 +948,7 @@ tad_mma_image_kernel(const __grid_constant__ TadcProgram P, const __grid_constan
     float u[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) u[j] = tile[lc * LD + o * 8 + j];
-    split_unit(u, p1, p2, p3);
+    split_unit<false>(u, p1, p2, p3);
     unsigned char *at = dst + l * 128 + ((o ^ (l & 7)) << 4);
     *reinterpret_cast<uint4 *>(at) = make_uint4(p1[0], p1[1], p1[2], p1[3]);
     *reinterpret_cast<uint4 *>(at + PART) = make_uint4(p2[0], p2[1], p2[2], p2[3]);

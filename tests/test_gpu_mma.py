@@ -18,7 +18,7 @@ from tests.gpu_util import GpuRun  # noqa: E402
 
 
 def _close(got, want, scale, n_terms, what):
-    tol = (8 + math.ceil(n_terms / 64)) * 2.0 ** -23 * scale + 1e-30
+    tol = (8 + math.ceil(n_terms / 64)) * 2.0 ** -23 * scale + 1e-45
     err = (torch.from_numpy(got).double() - want).abs()
     assert bool((err <= tol).all()), f"{what}: worst {float((err / tol).max()):.2f} of the tolerance"
 
@@ -41,6 +41,29 @@ def test_matrix_products(ni, nk, nj, transposed):
     _close(f, x @ y, x.abs() @ y.abs(), nk, "forward")
     _close(dx, d @ y.T, d.abs() @ y.T.abs(), nj, "dx")
     want, scale = x.T @ d, x.T.abs() @ d.abs()
+    _close(dy, want.T if transposed else want, scale.T if transposed else scale, ni, "dy")
+
+
+# every gather order, a split sum, a column operand split ahead, the one-stage kernel
+@pytest.mark.parametrize("ni,nk,nj", [(129, 65, 127), (300, 333, 65), (160, 5000, 136), (640, 200, 13001), (3077, 34, 3201)])
+@pytest.mark.parametrize("transposed", [False, True])
+@pytest.mark.parametrize("small,large", [(1e-37, 1e30), (1e-33, 1e-3), (1e-40, 1e33), (1e-5, 1e25)])
+def test_operands_of_all_magnitudes(ni, nk, nj, transposed, small, large):
+    """Operands whose second and third bf16 parts would be subnormal, subnormal ones, and large ones that are not split: the
+    products are ordinary numbers and no less exact than others."""
+    e = W.ex_matmul_t(ni, nj, nk) if transposed else W.ex_matmul(ni, nk, nj)
+    args, df = W.make_inputs(e, ("normal", 0, 1), seed=nk)
+    args[0] *= small
+    args[1] *= large
+    run = GpuRun(e, args, df)
+    f = run.forward()
+    dx, dy = run.backward()
+    x, y, d = args[0].double(), args[1].double(), df.double()
+    y = y.T if transposed else y
+    subnormal = 2.0 ** -126                                     # (results may be subnormal themselves: a unit of 2^-149 per term)
+    _close(f, x @ y, x.abs() @ y.abs() + nk * subnormal, nk, "forward")
+    _close(dx, d @ y.T, d.abs() @ y.T.abs(), nj, "dx")
+    want, scale = x.T @ d, x.T.abs() @ d.abs() + ni * subnormal
     _close(dy, want.T if transposed else want, scale.T if transposed else scale, ni, "dy")
 
 
