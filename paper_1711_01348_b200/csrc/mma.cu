@@ -96,6 +96,15 @@ __device__ __forceinline__ void tmem_st4(unsigned addr, const unsigned (&r)[4])
 }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
+// named barrier of some warps of a block (THREADS threads): the answer, the same for all, is whether x holds in any of them
+template <int THREADS>
+__device__ __forceinline__ bool any_of_warps(bool x)
+{
+    unsigned r;
+    asm volatile("{ .reg .pred p, q; setp.ne.u32 p, %1, 0; barrier.cta.red.or.pred q, 1, %2, p; selp.u32 %0, 1, 0, q; }" : "=r"(r) : "r"((unsigned)x), "n"(THREADS) : "memory");
+    return r != 0;
+}
+
 // shared-memory matrix descriptor, 128-byte swizzle: leading / stride byte offsets in units of 16 bytes
 __device__ __forceinline__ unsigned long long make_desc(unsigned addr, unsigned lbo, unsigned sbo)
 {
@@ -688,7 +697,6 @@ tad_mma_short_kernel(const __grid_constant__ TadcProgram P, const __grid_constan
         for (int t = 0; t < n_tiles && ok; ++t) {
             // the MMAs of tile t - 2 are done: its row buffer, and every column buffer but the last two, are free
             if (t >= 2) ok = mbar_wait(bar_done + 8 * (t & 1), ((t - 2) >> 1) & 1, &failed);
-            if (!ok) break;
             const bool fresh = t == 0 || ++tile_m == tiles_m;
             if (fresh) {
                 if (t > 0) { tile_m = 0; ++strip; }
@@ -709,8 +717,10 @@ tad_mma_short_kernel(const __grid_constant__ TadcProgram P, const __grid_constan
                     rowgrd[(2 + (q & 1)) * BM + r - BM] = n < Next ? P.guardB_c0 + z.gb + p.gb : DEAD;
                 }
             }
-            // (a warp that is here has read the tables of the tile before: the tables alternate, one barrier per tile is enough)
-            asm volatile("bar.sync 1, %0;" ::"n"(CT) : "memory");
+            // (a warp that is here has read the tables of the tile before: the tables alternate, one barrier per tile is enough.)
+            // Every warp comes here whatever its wait said, and all leave together if one ran out: a warp that left on its own
+            // would leave the others in this barrier for ever, and a wait can end either way when the MMAs finish at its limit.
+            if (any_of_warps<CT>(!ok)) { ok = false; break; }
             if (fresh)
                 gather(std::integral_constant<int, MB>{}, ptrs.in[P.ptrB], rowoff + (2 + (q & 1)) * BM, rowgrd + (2 + (q & 1)) * BM, ktab + 2 * KS,
                        P.guardB != 0, (unsigned)P.guardB_ext, bufs + (2 + (q & 1)) * C::OPERAND);
