@@ -11,9 +11,9 @@
 // truncates, so a sum stays in it for one stage of 64 summation indices only (small products first, then four
 // steps of a1 b1) and the stages are added up in fp32 registers with round-to-nearest.  Measured against float64
 // (2-norm, normal operands): 0.8e-7 at 64 terms, 1.2e-7 at 1100, 1.3e-7 at 2048; chains of fp32 multiply-adds
-// gave 4.2e-7 at 1100.  Outputs of a warp whose sums come out non-finite (an infinity times a zero part, an operand of
-// 2^104 or more, a sum of 2^80 or more) are evaluated again with fp32 multiply-adds from the operands themselves, so
-// infinities and NaNs are those of the definition.
+// gave 4.2e-7 at 1100.  Where sums come out non-finite (an infinity times a zero part, an operand of 2^104 or more, a sum of
+// 2^80 or more) the tile is evaluated again with fp32 multiply-adds from the operands themselves, so infinities and NaNs are
+// those of the definition.
 //
 // One block per SM.  Warps 0-15 gather the operands of a stage through the offset tables (global -> registers, a
 // whole stage ahead), split them and write them to shared memory in the 128-byte swizzled layout of the MMA
@@ -488,32 +488,8 @@ tad_mma_kernel(const __grid_constant__ TadcProgram P, const __grid_constant__ Ta
         bool odd = !ok;
 #pragma unroll
         for (int j = 0; j < COLS; ++j) odd = odd || (j < live && !(fabsf(acc[j]) <= 3.0e38f));
-        if (__any_sync(0xffffffffu, odd)) {
-            // the warp's outputs once more, with fp32 multiply-adds from the operands themselves
-            const float *__restrict__ A = ptrs.in[P.ptrA];
-            const float *__restrict__ B = ptrs.in[P.ptrB];
-#pragma unroll 1
-            for (int j = 0; j < live; ++j) {
-                const char *pa = reinterpret_cast<const char *>(A), *pb = reinterpret_cast<const char *>(B);
-                const unsigned ra = rowA[rl], rb = rowB[col0 + j];
-                const int ga = rowgA[rl], gb = rowgB[col0 + j];
-                float sum = 0.f;
-#pragma unroll 1
-                for (unsigned k = kbeg; k < kend; ++k) {
-                    const Parts p = decode(P.K, k);
-                    const bool la = !P.guardA || (unsigned)(ga + p.ga) < (unsigned)P.guardA_ext, lb = !P.guardB || (unsigned)(gb + p.gb) < (unsigned)P.guardB_ext;
-                    const float x = la ? __ldg(reinterpret_cast<const float *>(pa + (ra + (unsigned)p.a * 4u))) : 0.f;
-                    const float y = lb ? __ldg(reinterpret_cast<const float *>(pb + (rb + (unsigned)p.b * 4u))) : 0.f;
-                    sum = fmaf(x, y, sum);
-                }
-                if (P.ksplit > 1) ptrs.part[((size_t)zb * (unsigned)P.ksplit + ks) * Next * Mext + (size_t)(n0 + j) * Mext + m] = sum;
-                else {
-                    const unsigned off = (unsigned)(P.baseO + z.o + outM[rl] + outN[col0 + j]);
-                    const float v = epilogue(P, ptrs, sum * P.scale, off);
-                    ptrs.out[off] = P.accumulate ? ptrs.out[off] + v : v;
-                }
-            }
-        } else if (live) {
+        odd = __any_sync(0xffffffffu, odd);
+        if (!odd && live) {
 #pragma unroll
             for (int j = 0; j < COLS; ++j) acc[j] *= SUM_SCALE;
             if (P.ksplit > 1) {
@@ -556,6 +532,96 @@ tad_mma_kernel(const __grid_constant__ TadcProgram P, const __grid_constant__ Ta
                 }
             }
         }
+        // Warps with an infinite or NaN sum: their outputs once more, by the whole block, with fp32 multiply-adds from the operands
+        // themselves, 32 summation indices at a time through shared memory (the stages' place: every MMA and copy into it has been
+        // waited for).  Outputs with a NaN among their operands are NaN, and where that is all of them no sum is formed.
+        // Strided convolution 64 x 256 x 2048 with 1280 terms, NaN operands / one infinity / infinities: 1.6 / 0.5 / 6.6 ms; every output from its
+        // own terms 103 / 7.4 / 103 ms, the multiply-add tiles of contract.cu 1.93 ms whatever the values.
+        if (any_of_warps<NCW * 32>(odd)) {
+            constexpr int RK = 32, LA = BM + 4, LB = BN + 4, PER = BM * RK / (NCW * 32), PART = 16;
+            static_assert((LA + LB) * RK * 4 + 4 * RK * 4 + (BM + BN) * 4 <= 2 * C::STAGE, "room for the operands");
+            float *ta = reinterpret_cast<float *>(stages), *tb = ta + RK * LA;
+            int *rt = reinterpret_cast<int *>(tb + RK * LB);                        // offsets A, guards A, offsets B, guards B
+            int *nans = rt + 4 * RK;                                                // rows of A, columns of B that hold a NaN
+            constexpr bool a_rows = MA == TM_ROW;
+            const bool b_rows = P.modeB == TM_ROW || P.modeB == TM_RVEC;
+            for (int r = tid; r < BM + BN; r += NCW * 32) nans[r] = 0;
+            // indices k0 .. k0 + 31 of one operand (rows, its first guard part, its tables), zero where there is none; returns which are NaN
+            auto stage = [&](const float *src, bool rows, auto size, int ld, float *dst, int *flags, const unsigned *row, const int *rowg, const int *t, unsigned gext) {
+                constexpr int n = decltype(size)::value;
+                float x[PER];                                  // (all loads are under way before the first is stored)
+#pragma unroll
+                for (int i = 0; i < PER; ++i) {
+                    const int e = tid + i * NCW * 32, r = (rows ? e % n : e / RK) % n, k = (rows ? e / n : e) % RK;
+                    x[i] = 0.f;
+                    if (e < n * RK && (unsigned)(rowg[r] + t[RK + k]) < gext) x[i] = ldf(src, row[r] + (unsigned)t[k]);
+                }
+#pragma unroll
+                for (int i = 0; i < PER; ++i) {
+                    const int e = tid + i * NCW * 32, r = rows ? e % n : e / RK, k = rows ? e / n : e % RK;
+                    if (e >= n * RK) continue;
+                    dst[k * ld + r] = x[i];
+                    if (x[i] != x[i]) flags[r] = 1;
+                }
+            };
+            // pass -1 looks for NaNs, pass q forms the sums of the q-th sixteen columns of every warp
+#pragma unroll 1
+            for (int pass = -1; pass < COLS / PART; ++pass) {
+                float sum[PART];
+#pragma unroll
+                for (int j = 0; j < PART; ++j) sum[j] = 0.f;
+#pragma unroll 1
+                for (unsigned k0 = kbeg; k0 < kend; k0 += RK) {
+                    any_of_warps<NCW * 32>(false);             // (the block is done with the indices before)
+                    if (tid < RK) {
+                        Parts p{0, 0, 0, DEAD, DEAD};
+                        if (k0 + tid < kend) p = decode(P.K, k0 + tid);
+                        rt[tid] = p.a * 4; rt[RK + tid] = p.ga; rt[2 * RK + tid] = p.b * 4; rt[3 * RK + tid] = p.gb;
+                    }
+                    any_of_warps<NCW * 32>(false);
+                    stage(ptrs.in[P.ptrA], a_rows, std::integral_constant<int, BM>{}, LA, ta, nans, rowA, rowgA, rt, (unsigned)P.guardA_ext);     // (extent 1 without a guard)
+                    stage(ptrs.in[P.ptrB], b_rows, std::integral_constant<int, BN>{}, LB, tb, nans + BM, rowB, rowgB, rt + 2 * RK, (unsigned)P.guardB_ext);
+                    if (pass < 0) continue;
+                    any_of_warps<NCW * 32>(false);
+                    const int kn = (int)min((unsigned)RK, kend - k0);
+                    if (!odd) continue;
+#pragma unroll 4
+                    for (int k = 0; k < kn; ++k) {
+                        const float x = ta[k * LA + rl];
+                        const float4 *y = reinterpret_cast<const float4 *>(tb + k * LB + col0 + pass * PART);
+#pragma unroll
+                        for (int c = 0; c < PART / 4; ++c) {
+                            const float4 q = y[c];
+                            sum[4 * c] = fmaf(x, q.x, sum[4 * c]); sum[4 * c + 1] = fmaf(x, q.y, sum[4 * c + 1]);
+                            sum[4 * c + 2] = fmaf(x, q.z, sum[4 * c + 2]); sum[4 * c + 3] = fmaf(x, q.w, sum[4 * c + 3]);
+                        }
+                    }
+                }
+                bool left = false;                             // some output to be summed
+                if (pass < 0) {
+                    any_of_warps<NCW * 32>(false);
+                    if (odd && !nans[rl]) for (int j = 0; j < live; ++j) left = left || !nans[BM + col0 + j];
+                    left = any_of_warps<NCW * 32>(left);
+                    if (left) continue;
+                }
+                // (no output to be summed: one turn stores the NaNs of all columns)
+#pragma unroll 1
+                for (int c = pass < 0 ? 0 : pass * PART; odd && c < (pass < 0 ? COLS : (pass + 1) * PART); c += PART) {
+#pragma unroll
+                    for (int j = 0; j < PART; ++j) {
+                        if (c + j >= live) continue;
+                        const float v = nans[rl] || nans[BM + col0 + c + j] ? __int_as_float(0x7fffffff) : sum[j];
+                        if (P.ksplit > 1) ptrs.part[((size_t)zb * (unsigned)P.ksplit + ks) * Next * Mext + (size_t)(n0 + c + j) * Mext + m] = v;
+                        else {
+                            const unsigned off = (unsigned)(P.baseO + z.o + outM[rl] + outN[col0 + c + j]);
+                            const float r = epilogue(P, ptrs, v * P.scale, off);
+                            ptrs.out[off] = P.accumulate ? ptrs.out[off] + r : r;
+                        }
+                    }
+                }
+                if (pass < 0) break;
+            }
+        }
         fence_before();
     }
     __syncthreads();
@@ -579,7 +645,8 @@ constexpr int SE = 16, SC = 7, SNT = (SE + SC + 1) * 32;    // epilogue and gath
 
 struct ShortCfg {
     static constexpr int PART = BM * KS * 2, OPERAND = 3 * PART;
-    static constexpr int TABLES = 2 * BM * 8 + 2 * BM * 8 + 4 * KS * 4 + SE * 64 * 4;    // row tables of both operands (twice), k tables, output columns
+    static constexpr int MAX_TILES = 1024;      // of a block: the marks of its pieces must fit
+    static constexpr int TABLES = 2 * BM * 8 + 2 * BM * 8 + 4 * KS * 4 + SE * 64 * 4 + SE * MAX_TILES / 4;    // row tables of both operands (twice), k tables, output columns, marks
     static constexpr size_t SMEM = 1024 + 4 * size_t(OPERAND) + TABLES;
 };
 
@@ -599,6 +666,7 @@ tad_mma_short_kernel(const __grid_constant__ TadcProgram P, const __grid_constan
     int *rowgrd = reinterpret_cast<int *>(rowoff + 4 * BM);
     int *ktab = rowgrd + 4 * BM;                                                       // offsets A, guards A, offsets B, guards B
     int *outN = ktab + 4 * KS;                                                         // per epilogue warp: output offsets of its 32 columns, twice
+    unsigned *marks = reinterpret_cast<unsigned *>(outN + SE * 64) + (threadIdx.x >> 5) * (ShortCfg::MAX_TILES / 16);   // per epilogue warp: two pieces of every tile
     const unsigned bar_full = smem_u32(&bars[0]), bar_done = smem_u32(&bars[2]), bar_free = smem_u32(&bars[4]);
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const unsigned Mext = (unsigned)P.M.extent, Next = (unsigned)P.N.extent, K = (unsigned)P.K.extent;
@@ -734,6 +802,8 @@ tad_mma_short_kernel(const __grid_constant__ TadcProgram P, const __grid_constan
         // ---- epilogue warps: 32 rows x 32 columns of a tile each ----
         const int quad = warp & 3, col0 = (warp >> 2) * 32;
         int *cols = outN + warp * 64;                          // output offsets of this warp's columns, of an even and an odd column tile
+        for (int i = lane; i < (n_tiles + 15) / 16; i += 32) marks[i] = 0;
+        __syncwarp();
         int pre = -1;                                          // the epilogue step whose tensor is loaded ahead
         for (int e = P.n_epi - 1; e >= 0; --e) if (P.epi_op[e] == TE_MUL_LOAD || P.epi_op[e] == TE_ADD_LOAD) pre = e;
         // A tile is two pieces of 16 columns.  The values that the epilogue reads for a piece are loaded a piece ahead (the
@@ -849,25 +919,82 @@ tad_mma_short_kernel(const __grid_constant__ TadcProgram P, const __grid_constan
 #pragma unroll
                     for (int j = 0; j < 16; ++j) if (j < live) out[(unsigned)(off0 + co[j])] = v[j];
                 }
-            } else if (row_now) {
-                // non-finite sums: this piece once more, with fp32 multiply-adds from the operands themselves
-                const char *pa = reinterpret_cast<const char *>(ptrs.in[P.ptrA]), *pb = reinterpret_cast<const char *>(ptrs.in[P.ptrB]);
-                const Parts z_now = decode(P.Z, s_now / tiles_n), pm_now = decode(P.M, m_tile * BM + quad * 32 + lane);
+            } else if (lane == 0) marks[t >> 4] |= 1u << ((t & 15) * 2 + (it & 1));
+        }
+        // Pieces with non-finite sums, once more behind the loop (inside it the code costs the loop its registers: 225 -> 255 us at
+        // 8192 x 8192 x 34 with a tensor in the epilogue): fp32 multiply-adds from the operands themselves, sixteen columns at a
+        // time.  Outputs with a NaN among their operands are NaN, and where that is all of them no sum is formed.
+        // 8192 x 64 x 8192 with NaN operands / one infinity / infinities: 0.8 / 0.8 / 2.3 ms; with a decoded index and dependent loads for
+        // every term 18.8 / 8.0 / 18.8 ms, the multiply-add tiles of contract.cu 0.25 ms whatever the values.
+        __syncwarp();
+        const char *pa = reinterpret_cast<const char *>(ptrs.in[P.ptrA]), *pb = reinterpret_cast<const char *>(ptrs.in[P.ptrB]);
+        const unsigned gextA = (unsigned)P.guardA_ext, gextB = (unsigned)P.guardB_ext;         // (1 without a guard: the sum of the parts is then 0)
+        // which of 32 rows (columns; one per lane) hold a NaN: the lanes run along the summation index
+        auto holds_nan = [&](const char *src, unsigned off, int grd, const int *kt, unsigned gext) {
+            unsigned mask = 0;
+#pragma unroll 8
+            for (int r = 0; r < 32; ++r) {
+                const unsigned ro = __shfl_sync(0xffffffffu, off, r);
+                const int rg = __shfl_sync(0xffffffffu, grd, r);
+                bool nan = false;
+#pragma unroll
+                for (int k = 0; k < KS; k += 32) {
+                    float x = 0.f;
+                    if ((unsigned)(rg + kt[KS + k + lane]) < gext) x = __ldg(reinterpret_cast<const float *>(src + (ro + (unsigned)kt[k + lane])));
+                    nan = nan || x != x;
+                }
+                if (__any_sync(0xffffffffu, nan)) mask |= 1u << r;
+            }
+            return mask;
+        };
+        unsigned strip_of = 0xffffffffu, rb = 0, nan_col = 0, z_of = 0;
+        int gb = 0, on = 0;
+        Parts zp{0, 0, 0, 0, 0};
 #pragma unroll 1
-                for (int j = 0; j < min(live, 16); ++j) {
-                    const Parts pn = decode(P.N, (s_now % tiles_n) * BM + col0 + h + j);
-                    float sum = 0.f;
+        for (int t = 0; t < n_tiles; ++t) {
+            const unsigned pieces = (marks[t >> 4] >> ((t & 15) * 2)) & 3u;
+            if (!pieces) continue;
+            const unsigned at = first + (unsigned)t, s_at = at / tiles_m, c0 = (s_at % tiles_n) * BM + col0;
+            if (s_at != strip_of) {
+                strip_of = s_at;
+                z_of = s_at / tiles_n;
+                zp = decode(P.Z, z_of);
+                const Parts pn = decode(P.N, c0 + lane < Next ? c0 + lane : 0u);
+                rb = (unsigned)(P.baseB + zp.b + pn.b) * 4u;
+                gb = c0 + lane < Next ? P.guardB_c0 + zp.gb + pn.gb : DEAD;
+                on = pn.o;
+                nan_col = holds_nan(pb, rb, gb, ktab + 2 * KS, gextB);
+            }
+            const unsigned m = (at - s_at * tiles_m) * BM + quad * 32 + lane;
+            const bool live_row = m < Mext;
+            const Parts pm = decode(P.M, live_row ? m : 0u);
+            const unsigned ra = (unsigned)(P.baseA + zp.a + pm.a) * 4u;
+            const int ga = live_row ? P.guardA_c0 + zp.ga + pm.ga : DEAD, o_row = P.baseO + zp.o + pm.o;
+            const bool nan_row = (holds_nan(pa, ra, ga, ktab, gextA) >> lane) & 1u;
+            const bool some = __any_sync(0xffffffffu, live_row && !nan_row);
 #pragma unroll 1
+            for (int h = 0; h < 32; h += 16) {
+                const int n = min(16, (int)min(32u, Next > c0 ? Next - c0 : 0u) - h);
+                if (!((pieces >> (h / 16)) & 1u) || n <= 0) continue;
+                float sum[16];
+#pragma unroll
+                for (int j = 0; j < 16; ++j) sum[j] = 0.f;
+                if (some && ((~nan_col >> h) & ((1u << n) - 1u))) {
+#pragma unroll 2
                     for (unsigned k = 0; k < K; ++k) {
-                        const Parts p = decode(P.K, k);
-                        const bool la = !P.guardA || (unsigned)(P.guardA_c0 + z_now.ga + pm_now.ga + p.ga) < (unsigned)P.guardA_ext;
-                        const bool lb = !P.guardB || (unsigned)(P.guardB_c0 + z_now.gb + pn.gb + p.gb) < (unsigned)P.guardB_ext;
-                        const float x = la ? __ldg(reinterpret_cast<const float *>(pa + (unsigned)(P.baseA + z_now.a + pm_now.a + p.a) * 4u)) : 0.f;
-                        const float y = lb ? __ldg(reinterpret_cast<const float *>(pb + (unsigned)(P.baseB + z_now.b + pn.b + p.b) * 4u)) : 0.f;
-                        sum = fmaf(x, y, sum);
+                        const float x = (unsigned)(ga + ktab[KS + k]) < gextA ? __ldg(reinterpret_cast<const float *>(pa + (ra + (unsigned)ktab[k]))) : 0.f;
+                        // (lane j loads the value of column j)
+                        const float y = (unsigned)(gb + ktab[3 * KS + k]) < gextB ? __ldg(reinterpret_cast<const float *>(pb + (rb + (unsigned)ktab[2 * KS + k]))) : 0.f;
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) sum[j] = fmaf(x, __shfl_sync(0xffffffffu, y, h + j), sum[j]);
                     }
-                    const unsigned off = (unsigned)(off0 + pn.o);
-                    const float v1 = epilogue(P, ptrs, sum * P.scale, off);
+                }
+#pragma unroll
+                for (int j = 0; j < 16; ++j) {
+                    const unsigned off = (unsigned)(o_row + __shfl_sync(0xffffffffu, on, h + j));
+                    if (!live_row || j >= n) continue;
+                    const float v0 = nan_row || ((nan_col >> (h + j)) & 1u) ? __int_as_float(0x7fffffff) : sum[j];
+                    const float v1 = epilogue(P, ptrs, v0 * P.scale, off);
                     ptrs.out[off] = P.accumulate ? ptrs.out[off] + v1 : v1;
                 }
             }
@@ -1018,7 +1145,7 @@ cudaError_t tad_launch_mma(const TadcProgram &P, const TadpPointers &ptrs, unsig
     // the pipelined kernel from four tiles per SM on (8192 x 8192 x 34 forward 220 -> 148 us, staged adjoint 280 -> 181 us);
     // with one or two tiles a block has nothing to overlap (1301 x 2477 x 23: 18 us as blocks of one tile, 23 us here)
     const unsigned long long tiles = (unsigned long long)((P.M.extent + BM - 1) / BM) * (unsigned)((P.N.extent + BM - 1) / BM) * (unsigned)P.Z.extent;
-    const bool short_pays = P.K.extent <= KS && P.ksplit <= 1 && P.N.extent > 64 && tiles >= 4ull * sms;
+    const bool short_pays = P.K.extent <= KS && P.ksplit <= 1 && P.N.extent > 64 && tiles >= 4ull * sms && tiles <= (unsigned long long)ShortCfg::MAX_TILES * sms;
 #define TAD_MMA_CASE(MA, MB)                                                                                              \
     case MA * 4 + MB: e = short_pays ? launch_short<MA, MB>(P, ptrs, sms, stream) : P.N.extent <= 64 ? launch_mma<64, MA, MB>(P, ptrs, stream) : launch_mma<128, MA, MB>(P, ptrs, stream); break;
     if (P.image && !short_pays) {

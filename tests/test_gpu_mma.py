@@ -131,6 +131,51 @@ def test_split_ahead_without_room():
         assert float(abs(a - b).max()) <= 1e-5 * float(abs(b).max())
 
 
+# a ragged tile, several stages and shares, a column operand split ahead, the one-stage kernel
+@pytest.mark.parametrize("ni,nk,nj", [(130, 70, 140), (160, 5000, 136), (700, 5003, 501), (3077, 34, 3201)])
+@pytest.mark.parametrize("transposed", [False, True])
+def test_nan_rows_and_infinities(ni, nk, nj, transposed):
+    """NaNs reach the outputs that read them and no others; sums with an infinity among other values, of either sign and of both."""
+    e = W.ex_matmul_t(ni, nj, nk) if transposed else W.ex_matmul(ni, nk, nj)
+    args, df = W.make_inputs(e, ("normal", 0, 1), seed=ni)
+    x, y = args
+    yt = y.T if transposed else y                               # summed x columns (a view)
+    yt[yt.abs() < 1e-3] = 0.5
+    x[3, nk // 2], x[ni - 1, 0], yt[nk - 1, nj - 2] = math.nan, math.nan, math.nan
+    x[5, 7], x[6, 3], x[6, 9], x[ni // 2, nk - 2] = math.inf, math.inf, -math.inf, -math.inf
+    yt[11, 17] = -math.inf
+    f = torch.from_numpy(GpuRun(e, args, df).forward()).double()
+    want = x.double() @ yt.double()
+    assert torch.equal(f.isnan(), want.isnan())
+    infinite = want.isinf()
+    assert torch.equal(f[infinite], want[infinite])
+    finite = want.isfinite()
+    scale = x.double().abs() @ yt.double().abs()
+    assert bool(((f - want).abs()[finite] <= 1e-5 * scale[finite]).all())
+
+
+@pytest.mark.parametrize("ni,nk,nj", [(2000, 700, 1900), (8192, 64, 8192)])
+def test_non_finite_operands_do_not_stall(ni, nk, nj):
+    """An operand full of NaNs, as a diverged run has it, or one infinity: a small multiple of the time of ordinary values."""
+    e = W.ex_matmul(ni, nk, nj)
+    args, df = W.make_inputs(e, ("normal", 0, 1), seed=1)
+
+    def time(value, full):
+        run = GpuRun(e, args, df)
+        run.args[0].fill_(value) if full else run.args[0].view(-1)[77:78].fill_(value)
+        start, stop = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        run.forward()
+        start.record()
+        run.forward()
+        stop.record()
+        torch.cuda.synchronize()
+        return start.elapsed_time(stop)
+    ordinary = min(time(1.0, False) for _ in range(3))
+    # (the copy of the result to the host is in all of them; NaNs took 20 to 100 times as long when every output was summed by itself)
+    assert time(math.nan, True) <= 4 * ordinary
+    assert time(math.inf, False) <= 8 * ordinary
+
+
 @pytest.mark.parametrize("nk,nj", [(70, 140), (33, 76000)])
 def test_non_finite_operands(nk, nj):
     """Infinities and NaNs of the operands, and values beyond the bf16 range, give what the definition gives."""
