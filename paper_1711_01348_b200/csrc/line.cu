@@ -143,6 +143,7 @@ tad_line_walk_kernel(const __grid_constant__ TadlProgram P, const __grid_constan
             const int l_in = two ? 1 : 0;
             const int d0 = P.loads[0].cz[l_in] * step_in, d1 = P.loads[1].cz[l_in] * step_in;
             const int d2 = P.loads[2].cz[l_in] * step_in, d3 = P.loads[3].cz[l_in] * step_in;
+            float group = 0.f;                                // (runs are added up sixteen at a time, the groups behind them)
             for (int z0 = lo0; z0 <= (two ? hi0 : lo0); ++z0) {
                 int lo = lo0, hi = hi0;
                 int o0 = b0, o1 = b1, o2 = b2, o3 = b3;
@@ -166,8 +167,10 @@ tad_line_walk_kernel(const __grid_constant__ TadlProgram P, const __grid_constan
                 else if (n_loads == 3) part = TAD_WALK(3);
                 else part = TAD_WALK(4);
 #undef TAD_WALK
-                acc += part;
+                group += part;
+                if (((z0 - lo0) & 15) == 15) { acc += group; group = 0.f; }
             }
+            acc += group;
         }
         if (BY_WARP) {
 #pragma unroll
@@ -254,7 +257,7 @@ tad_line_kernel(const __grid_constant__ TadlProgram P, const __grid_constant__ T
 #pragma unroll
             for (int v = 0; v < V; ++v) base[i] += P.loads[i].coef[v] * var[v];
         }
-        float acc[4] = {0.f, 0.f, 0.f, 0.f};
+        float total = 0.f;
         // outer loop: its range is united over the warp
         int lo0 = 0, hi0 = 0, z_first = 0, z_last = 0, z_step = 1, z_run = 1;
         if (two) {
@@ -282,6 +285,9 @@ tad_line_kernel(const __grid_constant__ TadlProgram P, const __grid_constant__ T
             if (P.n_share[l_in] > 1) { run = 1 << P.chunk_shift[l_in]; step = run * P.n_share[l_in]; first += share_in * run; }
             for (int ps = first; ps <= u_hi; ps += step) {
                 const int pe = min(u_hi, ps + run - 1);
+                // (a piece has accumulators of its own, its sum is added to the ones before: no longer chains of additions than in
+                // pieces that are planes of their own)
+                float acc[4] = {0.f, 0.f, 0.f, 0.f};
                 int o[NL];
 #pragma unroll
                 for (int i = 0; i < NL; ++i) o[i] = base[i] + (two ? P.loads[i].cz[0] * z0 : 0) + d[i] * ps;
@@ -326,6 +332,7 @@ tad_line_kernel(const __grid_constant__ TadlProgram P, const __grid_constant__ T
 #pragma unroll
                     for (int i = 0; i < NL; ++i) o[i] += U * d[i];
                 }
+                total += (acc[0] + acc[1]) + (acc[2] + acc[3]);
             }
         }
         if (!exists) continue;
@@ -337,7 +344,7 @@ tad_line_kernel(const __grid_constant__ TadlProgram P, const __grid_constant__ T
             for (int v = 0; v < V; ++v) o += P.scale[q].coef[v] * var[v];
             if (live) sc *= __ldg(ptrs.in[P.scale[q].ptr] + (unsigned)o);
         }
-        const float result = live ? ((acc[0] + acc[1]) + (acc[2] + acc[3])) * sc : 0.f;
+        const float result = live ? total * sc : 0.f;
         if (P.zsplit > 1) {
             unsigned cell = 0;
 #pragma unroll
