@@ -163,8 +163,9 @@ size_t tad_workspace_bytes(const tad_plan *plan);
  *   args       host array of n_args DEVICE pointers (read-only inputs), none NULL
  *   f          DEVICE pointer, prod(out_shape) floats, fully overwritten
  *   workspace  DEVICE pointer, tad_workspace_bytes() bytes, 256-byte aligned, caller-owned.  Only plans
- *              whose forward pass uses auxiliary tensors or a split summation need it; every other
- *              plan accepts NULL / 0 (a large contraction is faster with it).  TAD_ERR_WORKSPACE when it is needed and missing or too small.
+ *              whose forward pass uses auxiliary tensors or a split summation other than a contraction's need
+ *              it; every other plan accepts NULL / 0 (a contraction is faster with it).  TAD_ERR_WORKSPACE when it
+ *              is needed and missing or too small.
  */
 tad_status tad_forward(const tad_plan *plan, const float *const *args, float *f,
                        void *workspace, size_t workspace_bytes, void *cuda_stream);
@@ -214,7 +215,8 @@ tad_status tad_backward_arg(const tad_plan *plan, const float *const *args, cons
  *
  * The scratch is a fixed array of TAD_NOALLOC_SCRATCH_BYTES inside the library image; every
  * GPU that loads the library holds that much memory until the process exits.  A plan whose
- * workspace (without an operand laid out for the tensor cores) is larger is rejected with TAD_ERR_WORKSPACE and a message; nothing
+ * workspace is larger even without what a contraction can do without (an operand laid out for the
+ * tensor cores, planes of a split sum) is rejected with TAD_ERR_WORKSPACE and a message; nothing
  * is launched in that case.  The call allocates nothing (no cudaMalloc / cudaFree, no
  * allocating library routine); inputs and outputs are still the caller's buffers, with the
  * same meaning as in tad_backward.

@@ -1371,7 +1371,7 @@ static void account(tad_plan &p, Kernel &k)
     batch_auxiliaries(k);
     std::function<void(const Kernel &)> walk = [&](const Kernel &x) {
         if (x.ew.empty() && x.contract.empty() && x.prog.zsplit > 1)   // (line-sum kernels keep their shares in prog too)
-            p.partial_bytes = std::max(p.partial_bytes, (size_t(x.prog.zsplit) + 1) * size_t(x.prog.part_limit) * 4);
+            p.partial_least = std::max(p.partial_least, (size_t(x.prog.zsplit) + 1) * size_t(x.prog.part_limit) * 4);
         for (const TadcProgram &cp : x.contract) {
             if (cp.ksplit > 1)
                 p.partial_bytes = std::max(p.partial_bytes, size_t(cp.ksplit) * size_t(cp.M.extent) * size_t(cp.N.extent) * size_t(cp.Z.extent) * 4);
@@ -1380,6 +1380,7 @@ static void account(tad_plan &p, Kernel &k)
         for (const Kernel &y : x.pre) walk(y);
     };
     walk(k);
+    p.partial_bytes = std::max(p.partial_bytes, p.partial_least);
     p.aux_bytes = std::max(p.aux_bytes, k.aux_bytes);
     std::function<int(const Kernel &)> launches = [&](const Kernel &x) {
         int n = 0;

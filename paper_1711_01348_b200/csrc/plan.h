@@ -116,6 +116,7 @@ struct tad_plan {
     std::vector<bool> arg_zero_fill;            // the gradient is cleared before its kernels add into it
     size_t image_bytes = 0;                     // workspace for a contraction's column operand split ahead (largest; optional)
     size_t partial_bytes = 0;                   // workspace for the partial sums of split summations (largest kernel)
+    size_t partial_least = 0;                   // ... of the summations that cannot do without (a contraction can run in fewer shares)
     size_t aux_bytes = 0;                       // workspace for auxiliary tensors (largest kernel, then the shared ones)
     int n_shared = 0;                           // auxiliary kernels that several gradients have in common
     mutable void *side = nullptr;               // second stream and its events (independent memory-bound passes run beside a contraction)

@@ -167,6 +167,7 @@ struct TadpPointers {
     float *out;
     float *part;                       // zsplit > 1: zsplit planes of part_limit partial sums, then one plane of
                                        // flags (non-zero: some share of that output accumulated a term)
+    uint64_t part_bytes;               // room behind part: a contraction takes as many shares as fit (read on the host only)
     unsigned char *image;              // a contraction's column operand split ahead (contract.h); NULL: gather it as usual
     int32_t *debug;                    // NULL unless the plan was compiled with debug_bounds
 };

@@ -157,6 +157,17 @@ struct Side {
     }
 };
 
+// Divides the summation of a contraction among as many blocks as it was planned for, or as there is room for planes of partial
+// sums: fewer shares take longer and give the same sums in another order.
+void fit_shares(TadcProgram &P, uint64_t room)
+{
+    const uint64_t plane = (uint64_t)P.M.extent * (uint64_t)P.N.extent * (uint64_t)P.Z.extent * 4;
+    if (P.ksplit <= 1 || (uint64_t)P.ksplit * plane <= room) return;
+    const int64_t fit = std::max<int64_t>(1, (int64_t)(room / plane)), chunk = ((P.K.extent + fit - 1) / fit + TADC_KS - 1) / TADC_KS * TADC_KS;
+    P.kchunk = (int32_t)chunk;
+    P.ksplit = (int32_t)((P.K.extent + chunk - 1) / chunk);
+}
+
 // contraction kernels: one launch of the tile kernel per program
 tad_status launch_contractions(const tad::Kernel &k, const TadpPointers &ptrs, cudaStream_t stream, Side *side)
 {
@@ -164,7 +175,7 @@ tad_status launch_contractions(const tad::Kernel &k, const TadpPointers &ptrs, c
     for (size_t i = 0; i < k.contract.size(); ++i) {
         TadcProgram P = k.contract[i];
         if (!ptrs.image) P.image = 0;
-        if (P.ksplit > 1 && !ptrs.part) { tad::set_error("internal: partial-sum buffer missing"); return TAD_ERR_WORKSPACE; }
+        fit_shares(P, ptrs.part ? ptrs.part_bytes : 0);
         // 16-byte copies and stores need 16-byte aligned tensors: fall back to 4-byte accesses otherwise
         auto misaligned = [](const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) != 0; };
         if (P.shape == 7) {
@@ -175,7 +186,6 @@ tad_status launch_contractions(const tad::Kernel &k, const TadpPointers &ptrs, c
         else if (P.modeA == TG_ROW16 && misaligned(ptrs.in[P.ptrA])) P.modeA = TG_ROW;
         if (P.shape != 7 && P.ptrB >= 0 && P.modeB == TG_ROW16 && misaligned(ptrs.in[P.ptrB])) P.modeB = TG_ROW;
         if (P.out_vec4 && misaligned(ptrs.out)) P.out_vec4 = 0;
-        // the streaming kernel copies B in 16-byte pieces
         // single-column passes beside the tile kernel: no planes of partial sums, outputs of their own
         const bool beside = side && k.contract.size() > 1 && i > 0 && P.ksplit == 1 && !P.accumulate && (P.shape == 4 || P.shape == 6);
         cudaStream_t on = stream;
@@ -416,14 +426,30 @@ size_t stage_offset(const tad_plan *plan, int s)
     return (plan->opt.debug_bounds ? 256 : 0) + size_t(s) * pad256(size_t(plan->out_elems) * 4);
 }
 
-// workspace layout: ... [planes of partial sums][auxiliary tensors][image of a column operand]
-size_t aux_offset(const tad_plan *plan)
+thread_local bool t_built_in = false;             // set while tad_backward_noalloc runs
+
+// what a plan needs with `partial` bytes for planes of partial sums; contractions whose operand image does not fit behind it
+// gather as usual
+size_t bytes_with(const tad_plan *plan, size_t partial)
 {
-    return stage_offset(plan, (int)plan->stages.size()) + pad256(plan->partial_bytes);
+    return stage_offset(plan, (int)plan->stages.size()) + pad256(partial) + pad256(plan->aux_bytes);
+}
+size_t required_bytes(const tad_plan *plan) { return bytes_with(plan, plan->partial_bytes); }
+
+// Room for the planes in a workspace of this size: all of them, or, in the built-in scratch of tad_backward_noalloc, what the
+// rest leaves over (never less than the summations need that cannot run in fewer shares).
+size_t partial_room(const tad_plan *plan, size_t workspace_bytes)
+{
+    if (workspace_bytes >= required_bytes(plan)) return plan->partial_bytes;
+    const size_t rest = bytes_with(plan, 0);
+    return std::max(plan->partial_least, workspace_bytes > rest ? (workspace_bytes - rest) & ~size_t(255) : 0);
 }
 
-// what a plan cannot do without; contractions whose operand image does not fit behind it gather as usual
-size_t required_bytes(const tad_plan *plan) { return aux_offset(plan) + pad256(plan->aux_bytes); }
+// workspace layout: ... [planes of partial sums][auxiliary tensors][image of a column operand]
+size_t aux_offset(const tad_plan *plan, size_t workspace_bytes)
+{
+    return stage_offset(plan, (int)plan->stages.size()) + pad256(partial_room(plan, workspace_bytes));
+}
 
 unsigned char *image_of(const tad_plan *plan, void *workspace, size_t workspace_bytes)
 {
@@ -431,10 +457,9 @@ unsigned char *image_of(const tad_plan *plan, void *workspace, size_t workspace_
         ? static_cast<unsigned char *>(workspace) + required_bytes(plan) : nullptr;
 }
 
-// some kernel of the forward pass divides a summation among blocks (planes of partial sums in the workspace)
+// some kernel of the forward pass divides a summation among blocks and cannot do otherwise (planes in the workspace)
 bool forward_splits(const tad::Kernel &k)
 {
-    for (const TadcProgram &cp : k.contract) if (cp.ksplit > 1) return true;
     if (k.ew.empty() && k.contract.empty() && k.prog.zsplit > 1) return true;
     for (const tad::Kernel &pk : k.pre) if (forward_splits(pk)) return true;
     return false;
@@ -442,7 +467,7 @@ bool forward_splits(const tad::Kernel &k)
 
 bool check_workspace(const tad_plan *plan, void *workspace, size_t workspace_bytes)
 {
-    const size_t need = required_bytes(plan);
+    const size_t need = t_built_in ? bytes_with(plan, plan->partial_least) : required_bytes(plan);
     if (need && (!workspace || workspace_bytes < need || (reinterpret_cast<uintptr_t>(workspace) & 255u))) {
         tad::set_error("workspace missing, smaller than tad_workspace_bytes() or not 256-byte aligned");
         return false;
@@ -465,7 +490,8 @@ bool fill_inputs(const tad_plan *plan, const float *const *args, const float *df
     for (int s = 0; s < (int)plan->stages.size(); ++s)
         ptrs.in[plan->n_args + 1 + s] = reinterpret_cast<const float *>(static_cast<char *>(workspace) + stage_offset(plan, s));
     ptrs.debug = plan->opt.debug_bounds ? static_cast<int32_t *>(workspace) : nullptr;
-    ptrs.part = plan->partial_bytes
+    ptrs.part_bytes = partial_room(plan, workspace_bytes);
+    ptrs.part = ptrs.part_bytes && workspace
         ? reinterpret_cast<float *>(static_cast<char *>(workspace) + stage_offset(plan, (int)plan->stages.size())) : nullptr;
     return true;
 }
@@ -474,14 +500,13 @@ bool fill_inputs(const tad_plan *plan, const float *const *args, const float *df
 
 namespace {
 std::mutex g_side_mutex;
-thread_local bool t_create_nothing = false;       // set while tad_backward_noalloc runs
 
 // the plan's second stream, created by the first call that can use it (nullptr: run everything on the caller's stream)
 Side *side_of(const tad_plan *plan)
 {
     std::lock_guard<std::mutex> lock(g_side_mutex);
     if (plan->side) return static_cast<Side *>(plan->side);
-    if (t_create_nothing) return nullptr;
+    if (t_built_in) return nullptr;                   // (tad_backward_noalloc creates nothing)
     Side *sd = new (std::nothrow) Side();
     if (!sd) return nullptr;
     bool ok = cudaStreamCreateWithFlags(&sd->s, cudaStreamNonBlocking) == cudaSuccess;
@@ -523,6 +548,8 @@ tad_status tad_forward(const tad_plan *plan, const float *const *args, float *f,
     if (!plan || !f || (plan->n_args && !args)) { tad::set_error("NULL argument"); return TAD_ERR_INVALID_ARG; }
     const bool needs_ws = !plan->forward.aux.empty() || forward_splits(plan->forward);
     if (needs_ws && !check_workspace(plan, workspace, workspace_bytes)) return TAD_ERR_WORKSPACE;
+    // (a contraction's shares do without: they become one)
+    const bool has_ws = workspace && workspace_bytes >= required_bytes(plan) && (reinterpret_cast<uintptr_t>(workspace) & 255u) == 0;
     TadpPointers ptrs{};
     for (int a = 0; a < plan->n_args; ++a) {
         if (!args[a]) { tad::set_error("NULL argument tensor"); return TAD_ERR_INVALID_ARG; }
@@ -532,10 +559,11 @@ tad_status tad_forward(const tad_plan *plan, const float *const *args, float *f,
     ptrs.debug = nullptr;
     char *aux_base = nullptr;
     ptrs.image = image_of(plan, workspace, workspace_bytes);
-    if (needs_ws) {
+    if (has_ws) {
+        ptrs.part_bytes = plan->partial_bytes;
         ptrs.part = plan->partial_bytes
             ? reinterpret_cast<float *>(static_cast<char *>(workspace) + stage_offset(plan, (int)plan->stages.size())) : nullptr;
-        aux_base = static_cast<char *>(workspace) + aux_offset(plan);
+        aux_base = static_cast<char *>(workspace) + aux_offset(plan, workspace_bytes);
     }
     return launch(plan->forward, ptrs, false, (cudaStream_t)cuda_stream, aux_base, side_of(plan));
 }
@@ -550,7 +578,7 @@ tad_status tad_backward_stage(const tad_plan *plan, const float *const *args, co
     for (int s = 0; s < (int)plan->stages.size(); ++s) {
         ptrs.out = reinterpret_cast<float *>(static_cast<char *>(workspace) + stage_offset(plan, s));
         tad_status st = launch(plan->stages[s], ptrs, plan->opt.debug_bounds != 0, (cudaStream_t)cuda_stream,
-                               workspace ? static_cast<char *>(workspace) + aux_offset(plan) : nullptr, side_of(plan));
+                               workspace ? static_cast<char *>(workspace) + aux_offset(plan, workspace_bytes) : nullptr, side_of(plan));
         if (st != TAD_OK) return st;
     }
     return TAD_OK;
@@ -591,7 +619,7 @@ static tad_status backward_arg(const tad_plan *plan, const float *const *args, c
     }
     for (int ki : plan->arg_kernels[arg]) {
         tad_status st = launch(plan->backward[ki], ptrs, plan->opt.debug_bounds != 0, stream,
-                               workspace ? static_cast<char *>(workspace) + aux_offset(plan) : nullptr, side, pending, done);
+                               workspace ? static_cast<char *>(workspace) + aux_offset(plan, workspace_bytes) : nullptr, side, pending, done);
         pending = nullptr;
         if (st != TAD_OK) return st;
     }
@@ -806,7 +834,7 @@ tad_status tad_backward_noalloc(const tad_plan *plan, const float *const *args, 
                                 float *const *dargs, void *cuda_stream)
 {
     if (!plan) { tad::set_error("NULL plan"); return TAD_ERR_INVALID_ARG; }
-    const size_t need = required_bytes(plan);
+    const size_t need = bytes_with(plan, plan->partial_least);
     if (need > TAD_NOALLOC_SCRATCH_BYTES) {
         char msg[160];
         snprintf(msg, sizeof msg, "this plan needs %zu bytes of scratch, tad_backward_noalloc holds at most %zu; "
@@ -842,9 +870,9 @@ tad_status tad_backward_noalloc(const tad_plan *plan, const float *const *args, 
         if (e != cudaSuccess) { tad::set_error(std::string("clearing the debug word: ") + cudaGetErrorString(e)); return TAD_ERR_CUDA; }
     }
     // (this entry point creates nothing: the second stream is used only if an earlier call of another entry point made it)
-    t_create_nothing = true;
+    t_built_in = true;
     const tad_status st = tad_backward(plan, args, df, dargs, scratch, TAD_NOALLOC_SCRATCH_BYTES, cuda_stream);
-    t_create_nothing = false;
+    t_built_in = false;
     return st;
 }
 
