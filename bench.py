@@ -256,7 +256,7 @@ def line_elements(expr, p):
         step = [s + stride * r for s, r in zip(step, row)]
         stride *= extent
     moving = [v for v, s in enumerate(step) if s]
-    if len(moving) != 1 or moving[0] >= len(expr.out_shape) or abs(step[moving[0]]) < 64:
+    if len(moving) != 1 or moving[0] >= len(expr.out_shape) or abs(step[moving[0]]) < 64 or stride < 32768:
         return 0
     return expr.out_shape[moving[0]]
 

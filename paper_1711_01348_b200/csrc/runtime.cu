@@ -672,8 +672,10 @@ tad_status tad_backward(const tad_plan *plan, const float *const *args, const fl
 }
 
 // Elements of an argument that lie on one line  base + step i, 0 <= i < n,  and are the only ones that the expression reads
-// (a diagonal, a strided vector), when they are few enough that a copy of single elements beats a copy of the tensor:
-// 2048 elements of a 2048 x 2048 matrix 12 us instead of 308 us over PCIe, 8192 of 8192 x 8192 68 us instead of 4.8 ms.
+// (a diagonal, a strided vector), when a copy of single elements beats a copy of the tensor.  Such a copy takes 11 us and 1.7 to 3
+// ns an element, whatever the step; a copy of the tensor 9 to 11 us and 4.7 ns per 64 elements.  Measured, pinned, up, line / tensor
+// in us: step 64, 512 elements 12 / 13, 2048 15 / 22, 16384 33 / 88; step 128, 64 elements 11 / 11, 2048 15 / 30; step 2049, 2048
+// 20 / 314; two elements 12 / 9.  Below 128 KB there is nothing to gain, and the gradient's line is a copy more.
 static bool read_line(const tad_plan *plan, int arg, int64_t &base, int64_t &step, int64_t &n)
 {
     bool found = false;
@@ -696,7 +698,7 @@ static bool read_line(const tad_plan *plan, int arg, int64_t &base, int64_t &ste
         if (!s || (found && (b != base || s != step || len != n))) return false;
         base = b; step = s; n = len; found = true;
     }
-    return found && step >= 64 && n >= 2 && step * 4 < (int64_t(1) << 31);
+    return found && step >= 64 && n >= 2 && plan->arg_elems[arg] >= 32768 && step * 4 < (int64_t(1) << 31);
 }
 
 size_t tad_staging_bytes(const tad_plan *plan)

@@ -23,7 +23,7 @@ def _lines(n, k):
 
 
 @pytest.mark.parametrize("saved", [False, True])
-@pytest.mark.parametrize("make", [lambda: W.intro(131, 97, 5), lambda: _lines(200, 7), lambda: W.ex_matmul(65, 70, 33)])
+@pytest.mark.parametrize("make", [lambda: W.intro(131, 97, 5), lambda: W.intro(201, 97, 5), lambda: _lines(200, 7), lambda: W.ex_matmul(65, 70, 33)])
 def test_step_host(make, saved):
     e = make()
     args, df = W.make_inputs(e, ("uniform", -0.5, 0.5), seed=4)
