@@ -779,12 +779,6 @@ bool try_points(Gen &g, Kernel &k, int root, int scale, bool allow_split, const 
         zv.push_back(v);
     }
     // ---- the program: once per output, per term, on the sum ----
-    bool unrolled_sum = false;                               // would the interpreter keep several summands of a sum in flight?
-    {
-        Gen other = g;
-        choose_element_variable(other, true, 0u);
-        unrolled_sum = other.unroll_var >= 0 && other.vars[other.unroll_var].kind == 2;
-    }
     g.unroll_var = -1;
     const int n_temps = assign_temporaries(g, root, scale);
     Emitter em(g);
@@ -862,7 +856,11 @@ bool try_points(Gen &g, Kernel &k, int root, int scale, bool allow_split, const 
     // summands 64 -> 36, 15755 of 2 x 30 108 -> 57, 2647 of 2 x 16 63 -> 48), or next to nothing (one output of 2818 terms with
     // 10 x 29 summands 1415 -> 299, with eleven blocks of points 680).  With terms to spread it loses (274 outputs of 115 terms
     // with 30 summands 2183, here 301), and behind three kernel coordinates (2299 terms with 180 summands 694, here 333).
-    if (unrolled_sum && inner_sum < 0 && inner >= 16 && points * terms < 148.0 * 256 && (terms == 1 || (points <= 4 && g.kappa <= 2))) return false;
+    if (inner_sum < 0 && inner >= 16 && points * terms < 148.0 * 256 && (terms == 1 || (points <= 4 && g.kappa <= 2))) {
+        Gen other = g;
+        choose_element_variable(other, true, 0u);
+        if (other.unroll_var >= 0 && other.vars[other.unroll_var].kind == 2) return false;
+    }
     // plain element-wise programs have a kernel of their own, which a few thousand outputs do not fill
     if (g.kappa == 0 && zv.empty() && sv.empty() && n_temps == 0 && points > POINT_PLAIN) return false;
     // every offset the kernel can form must lie inside its tensor

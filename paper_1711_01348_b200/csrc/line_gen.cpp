@@ -37,7 +37,7 @@ Walks sample_walks(const TadlProgram &P)
         for (int r = 0; r < P.n_lower[l]; ++r) lo = std::max(lo, -floor_div(-row_num(P.lower[l][r], var, z0), P.lower[l][r].den));
         for (int r = 0; r < P.n_upper[l]; ++r) hi = std::min(hi, floor_div(row_num(P.upper[l][r], var, z0), P.upper[l][r].den));
     };
-    constexpr int WARPS = 64;
+    constexpr int WARPS = 64, LANES = 4, LANE[LANES] = {0, 10, 21, 31};      // (four lanes stand for the warp)
     const int in = P.n_loops - 1;
     const int64_t along = (P.outer_ext[P.lane_var] + P.lane_stride - 1) / P.lane_stride;
     int64_t rows = P.lane_stride;
@@ -49,15 +49,15 @@ Walks sample_walks(const TadlProgram &P)
     for (int i = 0; i < WARPS; ++i) {
         const int64_t at = (int64_t)(((double)i + 0.5) / WARPS * (double)total) % total;
         const int64_t row = at / groups, l0 = at % groups * 32;
-        int64_t var[32][TADP_MAX_VARS] = {}, first = INT64_MAX, last = INT64_MIN;
-        bool live[32] = {};
-        int64_t lo0[32], hi0[32];
-        for (int l = 0; l < 32 && l0 + l < along; ++l) {
+        int64_t var[LANES][TADP_MAX_VARS] = {}, first = INT64_MAX, last = INT64_MIN;
+        bool live[LANES] = {};
+        int64_t lo0[LANES], hi0[LANES];
+        for (int l = 0; l < LANES && l0 + LANE[l] < along; ++l) {
             int64_t rem = row;
             const int64_t r = rem % P.lane_stride; rem /= P.lane_stride;
             for (int v = P.n_outer - 1; v >= 0; --v) {
                 const int64_t e = std::max(1, P.outer_ext[v]);
-                if (v == P.lane_var) { var[l][v] = P.outer_lo[v] + P.lane_stride * (l0 + l) + r; continue; }
+                if (v == P.lane_var) { var[l][v] = P.outer_lo[v] + P.lane_stride * (l0 + LANE[l]) + r; continue; }
                 var[l][v] = P.outer_lo[v] + rem % e; rem /= e;
             }
             if (var[l][P.lane_var] >= P.outer_lo[P.lane_var] + (int64_t)P.outer_ext[P.lane_var]) continue;
@@ -74,12 +74,12 @@ Walks sample_walks(const TadlProgram &P)
         const double runs = in ? (double)(last - first + 1) : 1.0;
         const int64_t z0 = first + (last - first) * (2 * (i % 4) + 1) / 8;
         int64_t own = 0, a = INT64_MAX, b = INT64_MIN;
-        for (int l = 0; l < 32; ++l) {
+        for (int l = 0; l < LANES; ++l) {
             if (!live[l]) continue;
             int64_t lo = lo0[l], hi = hi0[l];
             if (in) { if (z0 < lo0[l] || z0 > hi0[l]) continue; range(1, var[l], z0, lo, hi); }
             if (lo > hi) continue;
-            const int64_t skew = P.lane_skew * (l0 + l);
+            const int64_t skew = P.lane_skew * (l0 + LANE[l]);
             own = std::max(own, hi - lo + 1); a = std::min(a, lo - skew); b = std::max(b, hi - skew);
         }
         alive += 1; w.runs += runs;
