@@ -36,9 +36,9 @@ enum TadcGather : int {
     TG_ROW16       // rows contiguous and 16-byte aligned: 16 bytes per copy along the row index
 };
 
-// the same for the tensor-core kernel (shape 7; see mma.cu): which index the lanes run along, or 32-byte vectors
 constexpr int TADC_IMAGE_COLS = 128;    // columns of a tile whose operand is split ahead
 
+// gather of the tensor-core kernel (shape 7; see mma.cu): which index the lanes run along, or 32-byte vectors
 enum TadcMmaGather : int { TM_ROW = 0, TM_KVEC, TM_K, TM_RVEC, TM_IMAGE };     // TM_IMAGE: column operand split ahead (see image)
 
 // steps applied to every finished sum before it is stored (in this order)

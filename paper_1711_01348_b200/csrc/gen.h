@@ -333,8 +333,6 @@ struct System {
     bool loose_box = false;     // the outer box is a bounding box of the live elements, not the set itself
 };
 
-// builds one contraction program from a system whose loops all have fixed ranges; an operand with ptr < 0 is
-// a tensor of ones (a plain summation of the other operand).  strict_fill: refuse mostly empty tiles
 // bytes of the column operand's image (contract.h: image): three bf16 parts of every tile and stage
 inline size_t image_bytes(const TadcProgram &P)
 {
@@ -342,6 +340,8 @@ inline size_t image_bytes(const TadcProgram &P)
     return tiles * stages * size_t(P.Z.extent) * (3 * TADC_IMAGE_COLS * TADC_KS * 2);
 }
 
+// builds one contraction program from a system whose loops all have fixed ranges; an operand with ptr < 0 is
+// a tensor of ones (a plain summation of the other operand).  strict_fill: refuse mostly empty tiles
 bool emit_program(const System &s, float scale, int accumulate, bool allow_split, bool strict_fill, TadcProgram &P, std::string &text);
 
 // contract_gen.cpp: recognises a kernel whose term is a product of two index expressions summed over

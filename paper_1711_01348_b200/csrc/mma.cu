@@ -23,10 +23,10 @@
 // s - 1 is added to the registers.
 //
 // What bounds it: the six bf16 products of a 128 x 128 x 64 stage take 1536 clocks of the tensor core, gathering,
-// splitting and adding up about 2900 clocks of the sixteen warps (4096 x 4096 x 4096: 775 us, 712 us without the
-// MMAs, 543 us without the loads).  Measured against the fp32 multiply-add tiles of contract.cu: strided
-// convolution 64 x 256 x 2048 with 1280 terms 1930 -> 535 us (160 TFLOP/s), its gradients 2110 -> 755 and
-// 1984 -> 534 us; 1500 x 1100 x 1333 product 153 -> 48 us; 37 x 4907 x 159 convolution 26.6 -> 10.2 us.
+// splitting and adding up about 2900 clocks of the sixteen warps where both operands are gathered (4096 x 4096 x 4096: 775 us,
+// 712 us without the MMAs, 543 us without the loads; 705 with the column operand split ahead by tad_mma_image_kernel).
+// Measured against the fp32 multiply-add tiles of contract.cu: strided convolution 64 x 256 x 2048 with 1280 terms 1930 -> 455 us
+// (190 TFLOP/s), 4096 x 2048 x 4096 product 1490 -> 346 us, 37 x 4907 x 159 convolution 26.6 -> 9.3 us.
 #include <cuda_runtime.h>
 
 #include <algorithm>

@@ -243,7 +243,6 @@ bool streams_only(const tad::Kernel &k)
            (k.contract[0].shape == 4 || k.contract[0].shape == 6);
 }
 
-// pending: an event the kernel that writes the output must wait for (the zero fill of its tensor on the second stream)
 // point programs that wait to be launched together: none reads what another of them writes
 struct PointBatch {
     const TadqProgram *prog[TADQ_BATCH];
@@ -269,6 +268,7 @@ struct PointBatch {
     }
 };
 
+// pending: an event the kernel that writes the output must wait for (the zero fill of its tensor on the second stream)
 // done: shared auxiliary tensors that this call of the library has computed already
 tad_status launch(const tad::Kernel &k, TadpPointers ptrs, bool debug, cudaStream_t stream, char *aux_base = nullptr,
                   Side *side = nullptr, cudaEvent_t pending = nullptr, std::vector<char> *done = nullptr)
@@ -285,8 +285,8 @@ tad_status launch(const tad::Kernel &k, TadpPointers ptrs, bool debug, cudaStrea
             return cudaEventRecord(side->join, side->s) == cudaSuccess && cudaStreamWaitEvent(stream, side->join, 0) == cudaSuccess;
         };
         // Launch order: the streaming passes move up to right behind the last kernel whose result they read, so that
-        // they are issued before the long kernels they run beside (every tensor has one writer: moving a kernel up
-        // past kernels that neither feed it nor read it changes nothing)
+        // they are issued before the long kernels they run beside (a tensor has one writer, or writers of columns of
+        // their own: moving a kernel up past kernels that neither feed it nor read it changes nothing)
         const bool use_side = side && k.pre.size() > 1;
         std::vector<int> order;
         for (int i = 0; i < (int)k.pre.size(); ++i) {
