@@ -160,20 +160,27 @@ def test_non_finite_operands_do_not_stall(ni, nk, nj):
     e = W.ex_matmul(ni, nk, nj)
     args, df = W.make_inputs(e, ("normal", 0, 1), seed=1)
 
-    def time(value, full):
-        run = GpuRun(e, args, df)
-        run.args[0].fill_(value) if full else run.args[0].view(-1)[77:78].fill_(value)
-        start, stop = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-        run.forward()
-        start.record()
-        run.forward()
-        stop.record()
-        torch.cuda.synchronize()
-        return start.elapsed_time(stop)
-    ordinary = min(time(1.0, False) for _ in range(3))
-    # (the copy of the result to the host is in all of them; NaNs took 20 to 100 times as long when every output was summed by itself)
-    assert time(math.nan, True) <= 4 * ordinary
-    assert time(math.inf, False) <= 8 * ordinary
+    run = GpuRun(e, args, df)
+    ordinary_x = run.args[0].clone()
+
+    def time():
+        best = math.inf
+        for _ in range(4):
+            start, stop = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            start.record()
+            run.plan.forward([x.data_ptr() for x in run.args], run.f.data_ptr(), torch.cuda.current_stream().cuda_stream,
+                             run.ws.data_ptr(), run.ws.numel())
+            stop.record()
+            torch.cuda.synchronize()
+            best = min(best, start.elapsed_time(stop))
+        return best
+    ordinary = time()
+    # (measured: 4 to 5 times; 60 to 300 times when every output was summed from its own terms)
+    run.args[0].fill_(math.nan)
+    assert time() <= 15 * ordinary
+    run.args[0].copy_(ordinary_x)
+    run.args[0].view(-1)[77:78].fill_(math.inf)
+    assert time() <= 15 * ordinary
 
 
 @pytest.mark.parametrize("nk,nj", [(70, 140), (33, 76000)])
