@@ -235,7 +235,7 @@ tad_status tad_backward_noalloc(const tad_plan *plan, const float *const *args, 
 /*
  * tad_step_host: one forward and one backward pass with HOST buffers (same meaning as
  * tad_forward followed by tad_backward).  Inputs are copied to the device staging area (of an
- * argument that is read along one line only, a diagonal say, just that line), results copied back.  The kernels run on the given stream, after whatever it already
+ * argument of 128 KB or more that is read along one line only, a diagonal say, just that line), results copied back.  The kernels run on the given stream, after whatever it already
  * holds; the copies run on two streams of the plan's own (created by the first call, released
  * by tad_destroy; calls on one plan must not run concurrently), ordered by events so
  * that df goes up during the forward pass and f and each gradient come down while the next
