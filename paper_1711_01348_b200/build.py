@@ -15,8 +15,8 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libtad.so")
-SOURCES = ["intalg.cpp", "plan.cpp", "codegen.cpp", "contract_gen.cpp", "factor.cpp", "line_gen.cpp", "print.cpp", "api.cpp", "runtime.cu", "contract.cu", "mma.cu", "ew.cu", "line.cu", "point.cu"]
-HEADERS = ["intalg.h", "plan.h", "gen.h", "program.h", "contract.h", "contract.cuh", "launch.h", "ew.h", "line.h", "point.h", "vm.cuh", "vm_shapes.h", "vm_inst.cu",
+SOURCES = ["intalg.cpp", "plan.cpp", "codegen.cpp", "contract_gen.cpp", "factor.cpp", "line_gen.cpp", "tile_gen.cpp", "print.cpp", "api.cpp", "runtime.cu", "contract.cu", "mma.cu", "ew.cu", "line.cu", "point.cu", "tile.cu"]
+HEADERS = ["intalg.h", "plan.h", "gen.h", "program.h", "contract.h", "contract.cuh", "launch.h", "ew.h", "line.h", "point.h", "tile.h", "vm.cuh", "vm_shapes.h", "vm_inst.cu",
            os.path.join("..", "..", "include", "tad.h")]
 ARCH = ["-gencode", "arch=compute_100a,code=sm_100a"]
 

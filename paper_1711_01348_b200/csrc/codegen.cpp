@@ -564,12 +564,16 @@ int body_fetch_kind(const TadpLoad &L, int ta, int ub)
 // evaluated first (so that a * (b * c + d) needs no more than X and Y whatever the order it was written in).
 // need(i): value registers the evaluation of i occupies; a binary operation whose operands are both compound puts the
 // first into Y, which the second must then leave alone (need 1).
-bool elementwise_steps_of(const Gen &g, int root, std::vector<TadeStep> &steps)
+}  // namespace
+
+bool elementwise_steps_of(const Gen &g, int root, std::vector<TadeStep> &steps, int leaf)
 {
     auto push_step = [&](int op, int a = 0, int b = 0, float imm = 0.f) { TadeStep s{}; s.op = (uint8_t)op; s.a = (int16_t)a; s.b = (uint8_t)b; s.imm = imm; steps.push_back(s); };
-    auto is_load = [&](int i) { return g.inst[i].op == I_LOAD; };
+    auto is_load = [&](int i) { return g.inst[i].op == I_LOAD || i == leaf; };
+    auto load_of = [&](int i) { return i == leaf ? -1 : g.inst[i].load; };
     std::function<int(int)> need = [&](int i) -> int {
         const Inst &in = g.inst[i];
+        if (i == leaf) return 1;
         switch (in.op) {
         case I_CONST: case I_LOAD: return 1;
         case I_SUM: return 99;
@@ -583,6 +587,7 @@ bool elementwise_steps_of(const Gen &g, int root, std::vector<TadeStep> &steps)
     };
     std::function<bool(int)> emit = [&](int i) -> bool {
         const Inst &in = g.inst[i];
+        if (i == leaf) { push_step(E_LD, -1, 0); return true; }
         if (in.temp >= 0) return false;
         auto fn = [&](int f, int e = 0) { if (!emit(in.a)) return false; push_step(E_FN, e, f); return true; };
         switch (in.op) {
@@ -604,8 +609,8 @@ bool elementwise_steps_of(const Gen &g, int root, std::vector<TadeStep> &steps)
         case I_COSH: return fn(F_COSH);
         case I_ADD: case I_MUL: {
             const int mode = in.op == I_ADD ? 1 : 2;
-            if (is_load(in.b) && !(is_load(in.a) && need(in.b) < need(in.a))) { if (!emit(in.a)) return false; push_step(E_LD, g.inst[in.b].load, mode); return true; }
-            if (is_load(in.a)) { if (!emit(in.b)) return false; push_step(E_LD, g.inst[in.a].load, mode); return true; }
+            if (is_load(in.b) && !(is_load(in.a) && need(in.b) < need(in.a))) { if (!emit(in.a)) return false; push_step(E_LD, load_of(in.b), mode); return true; }
+            if (is_load(in.a)) { if (!emit(in.b)) return false; push_step(E_LD, load_of(in.a), mode); return true; }
             const int first = need(in.a) >= need(in.b) ? in.a : in.b, second = first == in.a ? in.b : in.a;
             if (need(first) > 2 || need(second) != 1) return false;
             if (!emit(first)) return false;
@@ -627,6 +632,8 @@ bool elementwise_steps_of(const Gen &g, int root, std::vector<TadeStep> &steps)
     if (need(root) > 2) return false;
     return emit(root) && (int)steps.size() <= TADE_MAX_STEPS;
 }
+
+namespace {
 
 bool try_elementwise(Gen &g, Kernel &k, const Emitter &em, const std::vector<TadpRow> &guards, int root)
 {
@@ -994,6 +1001,12 @@ bool try_points(Gen &g, Kernel &k, int root, int scale, bool allow_split, const 
     return true;
 }
 
+// Sums whose term couples two variables run as tile programs from 2^18.6 points on, where they are as fast as point programs, which
+// share launches (a step of the intro expression, us: 162 x 95 x 11 48 -> 51, 70 x 675 x 16 91 -> 56, 3978 x 73 x 20 563 -> 79,
+// 2992 x 162 x 31 999 -> 95), up to 5e7, where the sums pushed inside and contracted are (2564 x 2507 x 5 462 -> 214, 7263 x 352 x 21
+// 194 -> 183, 1868 x 2663 x 11 165 -> 177, 1655 x 2679 x 23 163 -> 215).
+constexpr double TILE_LEAST = double(3 << 17), TILE_MOST = 5e7;
+
 // shared tail: choose temps, emit, fill the program
 void emit_kernel(Gen &g, Kernel &k, int root, const std::vector<std::vector<TadpRow>> &lower,
                  const std::vector<std::vector<TadpRow>> &upper, const std::vector<TadpRow> &guards, bool allow_split = false,
@@ -1037,6 +1050,8 @@ void emit_kernel(Gen &g, Kernel &k, int root, const std::vector<std::vector<Tadp
     }
     // a product of two index expressions under summations runs on the tile kernel, not in the interpreter
     if (try_contraction(g, k, root, scale, allow_split, lower, upper, guards)) return;
+    // sums of a term that couples two variables, as written, by tiles of both
+    if (try_tile(g, k, root, scale, lower, upper, guards, TILE_LEAST, TILE_MOST)) return;
     // sums that can be pushed inside the term (Sec. 6's missing clean-up step): auxiliary kernels + a smaller kernel
     if (may_factor && try_factoring(g, k, root, scale, allow_split, lower, upper, guards)) return;
     // short sums ahead of a kernel: as point programs they share a launch with the others
@@ -1710,6 +1725,7 @@ bool reads_inputs_only(const tad_plan &p, const Kernel &k)
         return true;
     }
     if (!k.ew.empty()) { for (int i = 0; i < k.ew[0].n_loads; ++i) if (!input(k.ew[0].loads[i].ptr)) return false; return true; }
+    if (!k.tile.empty()) { for (int i = 0; i < k.tile[0].n_loads; ++i) if (!input(k.tile[0].loads[i].ptr)) return false; return true; }
     if (!k.point.empty()) { for (const TadqLoad &L : k.point[0].loads) if (!input(L.ptr)) return false; return true; }
     if (!k.line.empty()) {
         for (int i = 0; i < k.line[0].n_loads; ++i) if (!input(k.line[0].loads[i].ptr)) return false;
@@ -1723,8 +1739,8 @@ bool reads_inputs_only(const tad_plan &p, const Kernel &k)
 bool same_kernel(const Kernel &a, const Kernel &b)
 {
     if (a.vec != b.vec || a.vec_u != b.vec_u || a.rich != b.rich) return false;
-    if (!same_bytes(a.contract, b.contract) || !same_bytes(a.ew, b.ew) || !same_bytes(a.point, b.point) || !same_bytes(a.line, b.line)) return false;
-    return !a.contract.empty() || !a.ew.empty() || !std::memcmp(&a.prog, &b.prog, sizeof a.prog);
+    if (!same_bytes(a.contract, b.contract) || !same_bytes(a.ew, b.ew) || !same_bytes(a.point, b.point) || !same_bytes(a.tile, b.tile) || !same_bytes(a.line, b.line)) return false;
+    return !a.contract.empty() || !a.ew.empty() || !a.tile.empty() || !std::memcmp(&a.prog, &b.prog, sizeof a.prog);
 }
 
 }  // namespace

@@ -350,6 +350,11 @@ bool emit_program(const System &s, float scale, int accumulate, bool allow_split
 bool try_contraction(Gen &g, Kernel &k, int root, int scale, bool allow_split, const std::vector<std::vector<TadpRow>> &lower,
                      const std::vector<std::vector<TadpRow>> &upper, const std::vector<TadpRow> &guards);
 
+// tile_gen.cpp: a sum whose term couples two variables becomes a tile program, if its number of points lies in the given range
+bool try_tile(Gen &g, Kernel &k, int root, int scale, const std::vector<std::vector<TadpRow>> &lower, const std::vector<std::vector<TadpRow>> &upper,
+              const std::vector<TadpRow> &guards, double min_space, double max_space);
+// codegen.cpp: steps of an element-wise program (ew.h) for an instance; the instance `leaf` is read as load -1
+bool elementwise_steps_of(const Gen &g, int root, std::vector<TadeStep> &steps, int leaf = -1);
 // line_gen.cpp: a gradient kernel whose term is a product of index expressions becomes a line-sum program
 bool try_line(Gen &g, Kernel &k, int root, int scale, bool allow_split, const std::vector<std::vector<TadpRow>> &lower,
               const std::vector<std::vector<TadpRow>> &upper, const std::vector<TadpRow> &guards);

@@ -12,6 +12,7 @@
 #include "ew.h"
 #include "line.h"
 #include "point.h"
+#include "tile.h"
 
 namespace tad {
 
@@ -75,6 +76,7 @@ struct Kernel {
                                          // program) instead of the interpreter
     std::vector<TadeProgram> ew;         // non-empty: a kernel without loops, run by the element-wise kernel
     std::vector<TadqProgram> point;      // non-empty: a general term over a small index space, run by the point kernel
+    std::vector<TadtProgram> tile;       // non-empty: sums of a term that couples two variables, run by the tile-sum kernel
     std::vector<TadlProgram> line;       // non-empty: sums of products of index expressions, run by the line-sum kernel
     // Expression optimisation: tensors in the auxiliary area of the workspace and the kernels that fill them
     // (launched in this order before the kernel itself, each writing the tensor out_aux)

@@ -28,6 +28,7 @@ cudaError_t tad_launch_contract(const TadcProgram &P, const TadpPointers &ptrs, 
 cudaError_t tad_launch_ew(const TadeProgram &P, const TadpPointers &ptrs, unsigned sms, cudaStream_t stream);
 cudaError_t tad_launch_points(const TadqProgram &P, const TadpPointers &ptrs, cudaStream_t stream);
 cudaError_t tad_launch_point_batch(const TadqProgram *const *progs, float *const *out, int n, const TadpPointers &ptrs, cudaStream_t stream);
+cudaError_t tad_launch_tiles(const TadtProgram *const *progs, float *const *out, int n, const TadpPointers &ptrs, cudaStream_t stream);
 cudaError_t tad_launch_line(const TadlProgram &P, const TadpPointers &ptrs, unsigned sms, cudaStream_t stream);
 
 namespace {
@@ -222,6 +223,10 @@ bool reads_slot(const tad::Kernel &k, int slot)
         for (int i = 0; i < k.ew[0].n_loads; ++i) if (k.ew[0].loads[i].ptr == slot) return true;
         return false;
     }
+    if (!k.tile.empty()) {
+        for (int i = 0; i < k.tile[0].n_loads; ++i) if (k.tile[0].loads[i].ptr == slot) return true;
+        return false;
+    }
     if (!k.point.empty()) {
         for (const TadqStep *st = k.point[0].steps; st < k.point[0].steps + k.point[0].n_steps; ++st)
             if ((st->op == Q_LOAD || st->op == Q_LDADD || st->op == Q_LDMUL || st->op == Q_LDADDSQ) && k.point[0].loads[st->a].ptr == slot) return true;
@@ -336,6 +341,12 @@ tad_status launch(const tad::Kernel &k, TadpPointers ptrs, bool debug, cudaStrea
     if (!k.ew.empty()) {
         const cudaError_t e = tad_launch_ew(k.ew[0], ptrs, (unsigned)sm_count(), stream);
         if (e != cudaSuccess) { tad::set_error(std::string("element-wise launch failed: ") + cudaGetErrorString(e)); return TAD_ERR_CUDA; }
+        return TAD_OK;
+    }
+    if (!k.tile.empty()) {
+        const TadtProgram *const prog = &k.tile[0];
+        const cudaError_t e = tad_launch_tiles(&prog, &ptrs.out, 1, ptrs, stream);
+        if (e != cudaSuccess) { tad::set_error(std::string("tile-sum launch failed: ") + cudaGetErrorString(e)); return TAD_ERR_CUDA; }
         return TAD_OK;
     }
     if (!k.line.empty() || !k.point.empty()) {
