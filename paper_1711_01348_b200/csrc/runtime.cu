@@ -273,6 +273,31 @@ struct PointBatch {
     }
 };
 
+// tile programs of gradients that wait to be launched together: they read inputs and staged adjoints only
+struct TileBatch {
+    const TadtProgram *prog[TADT_BATCH];
+    float *out[TADT_BATCH];
+    int n = 0;
+    TadpPointers ptrs{};
+    tad_status flush(cudaStream_t stream)
+    {
+        if (n == 0) return TAD_OK;
+        const cudaError_t e = tad_launch_tiles(prog, out, n, ptrs, stream);
+        n = 0;
+        if (e != cudaSuccess) { tad::set_error(std::string("tile-sum launch failed: ") + cudaGetErrorString(e)); return TAD_ERR_CUDA; }
+        return TAD_OK;
+    }
+    tad_status add(const TadtProgram &P, const TadpPointers &p, float *o, cudaStream_t stream)
+    {
+        if (n == TADT_BATCH || (n > 0 && prog[0]->tm != P.tm)) { const tad_status st = flush(stream); if (st != TAD_OK) return st; }
+        ptrs = p; ptrs.out = o; prog[n] = &P; out[n] = o; ++n;
+        return TAD_OK;
+    }
+};
+
+// programs of a call to tad_backward that are launched at its end
+struct Later { PointBatch points; TileBatch tiles; };
+
 // pending: an event the kernel that writes the output must wait for (the zero fill of its tensor on the second stream)
 // done: shared auxiliary tensors that this call of the library has computed already
 tad_status launch(const tad::Kernel &k, TadpPointers ptrs, bool debug, cudaStream_t stream, char *aux_base = nullptr,
@@ -597,7 +622,7 @@ tad_status tad_backward_stage(const tad_plan *plan, const float *const *args, co
 
 static tad_status backward_arg(const tad_plan *plan, const float *const *args, const float *df, int32_t arg, float *darg,
                                void *workspace, size_t workspace_bytes, void *cuda_stream, std::vector<char> *done,
-                               PointBatch *later = nullptr, bool filled = false)
+                               Later *later = nullptr, bool filled = false)
 {
     if (!plan || !df || !darg || (plan->n_args && !args)) { tad::set_error("NULL argument"); return TAD_ERR_INVALID_ARG; }
     if (arg < 0 || arg >= plan->n_args) { tad::set_error("no such argument"); return TAD_ERR_INVALID_ARG; }
@@ -623,10 +648,11 @@ static tad_status backward_arg(const tad_plan *plan, const float *const *args, c
         }
     }
     ptrs.out = darg;
-    // a gradient that is one point program reads inputs and staged adjoints only: it may share a launch with others
+    // a gradient that is one point or tile program reads inputs and staged adjoints only: it may share a launch with others
     if (later && plan->arg_kernels[arg].size() == 1) {
         const tad::Kernel &k = plan->backward[plan->arg_kernels[arg][0]];
-        if (!k.point.empty() && k.point[0].zsplit <= 1 && k.pre.empty()) return later->add(k.point[0], ptrs, darg, stream);
+        if (!k.point.empty() && k.point[0].zsplit <= 1 && k.pre.empty()) return later->points.add(k.point[0], ptrs, darg, stream);
+        if (!k.tile.empty() && k.pre.empty()) return later->tiles.add(k.tile[0], ptrs, darg, stream);
     }
     for (int ki : plan->arg_kernels[arg]) {
         tad_status st = launch(plan->backward[ki], ptrs, plan->opt.debug_bounds != 0, stream,
@@ -673,13 +699,14 @@ tad_status tad_backward(const tad_plan *plan, const float *const *args, const fl
         const cudaError_t e = tad_launch(tad_fill_zero_many, std::max(1u, blocks), 256, 0, (cudaStream_t)cuda_stream, fill);
         if (e != cudaSuccess) { tad::set_error(std::string("zero fill launch failed: ") + cudaGetErrorString(e)); return TAD_ERR_CUDA; }
     }
-    PointBatch later;
+    Later later;
     for (int a = 0; a < plan->n_args; ++a) {
         if (!dargs[a]) continue;
         tad_status st = backward_arg(plan, args, df, a, dargs[a], workspace, workspace_bytes, cuda_stream, &done, &later, filled[a]);
         if (st != TAD_OK) return st;
     }
-    return later.flush((cudaStream_t)cuda_stream);
+    const tad_status st = later.tiles.flush((cudaStream_t)cuda_stream);
+    return st != TAD_OK ? st : later.points.flush((cudaStream_t)cuda_stream);
 }
 
 // Elements of an argument that lie on one line  base + step i, 0 <= i < n,  and are the only ones that the expression reads
