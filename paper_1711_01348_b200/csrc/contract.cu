@@ -403,66 +403,80 @@ tad_contract_reduce(const __grid_constant__ TadcProgram P, const __grid_constant
     }
 }
 
-// Plain summation of one operand (contraction with a tensor of ones and a single output column):
-//     out[m] (+)= scale * sum_k A[row(m) + k * stride]
-// One warp per output; its lanes walk the summation index (128-bit loads when that index is contiguous
-// and aligned), then a fixed-order shuffle tree.  Bound by HBM: every element of A is read once.
+// Plain or weighted sums of the rows of one operand (a contraction with a single output column):
+//     out[m] (+)= scale * sum_k A[row(m) + k * stride] (* B[k])
+// Bound by HBM: every element of A is read once, in pieces of 16 bytes from the first aligned one on where the row is consecutive
+// (and its weights lie alike), four in flight per lane.  A warp per output, or, where that would leave the GPU idle, a block of
+// eight (WARPS): 264 rows of 6523 elements.  Sums are added in a fixed order.
+template <int WARPS>
 __global__ void __launch_bounds__(256)
 tad_rowsum_kernel(const __grid_constant__ TadcProgram P, const __grid_constant__ TadpPointers ptrs)
 {
     tad_wait_previous();
-    const unsigned lane = threadIdx.x & 31u;
-    const unsigned warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, n_warps = (gridDim.x * blockDim.x) >> 5;
+    constexpr unsigned N = 32 * WARPS;                    // threads of a row
+    __shared__ float parts[8];
+    const unsigned lane = threadIdx.x % N;
+    const unsigned first = WARPS == 1 ? (blockIdx.x * blockDim.x + threadIdx.x) >> 5 : blockIdx.x, step = WARPS == 1 ? (gridDim.x * blockDim.x) >> 5 : gridDim.x;
     const float *__restrict__ A = ptrs.in[P.ptrA];
     const bool weighted = P.ptrB >= 0;                   // B[k]: one weight per summation index
-    const float *__restrict__ B = weighted ? ptrs.in[P.ptrB] : A;
+    const float *__restrict__ B = (weighted ? ptrs.in[P.ptrB] : A) + (weighted ? P.baseB : 0);
     const int kb = P.K.n_digits ? P.K.sB[0] : 0;
     const unsigned K = (unsigned)P.K.extent;
     const int ks = P.K.n_digits ? P.K.sA[0] : 0;
-    for (unsigned m = warp; m < (unsigned)P.M.extent; m += n_warps) {
+    for (unsigned m = first; m < (unsigned)P.M.extent; m += step) {
         const Parts p = decode(P.M, m);
-        const int base = P.baseA + p.a;
+        const float *row = A + (P.baseA + p.a);
         float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-        if (weighted && ks == 1 && kb == 1 && ((base & 3) == 0) && ((P.baseB & 3) == 0) &&
-            (((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B)) & 15u) == 0)) {
-            const float4 *row = reinterpret_cast<const float4 *>(A + (unsigned)base);
-            const float4 *wts = reinterpret_cast<const float4 *>(B + (unsigned)P.baseB);
-            const unsigned K4 = K / 4;
+        const unsigned off_a = (unsigned)(reinterpret_cast<uintptr_t>(row) >> 2) & 3u, off_b = (unsigned)(reinterpret_cast<uintptr_t>(B) >> 2) & 3u;
+        if (ks == 1 && (!weighted || kb == 1)) {
+            const unsigned head = min((4u - off_a) & 3u, K), K4 = (K - head) / 4u, tail = head + 4u * K4;
+            const float4 *row4 = reinterpret_cast<const float4 *>(row + head), *wts4 = reinterpret_cast<const float4 *>(B + head);
             unsigned k = lane;
-            for (; k + 96 < K4; k += 128) {
-                const float4 a = __ldg(row + k), b = __ldg(row + k + 32), c = __ldg(row + k + 64), d = __ldg(row + k + 96);
-                const float4 wa = __ldg(wts + k), wb = __ldg(wts + k + 32), wc = __ldg(wts + k + 64), wd = __ldg(wts + k + 96);
-                s0 += (a.x * wa.x + a.y * wa.y) + (a.z * wa.z + a.w * wa.w); s1 += (b.x * wb.x + b.y * wb.y) + (b.z * wb.z + b.w * wb.w);
-                s2 += (c.x * wc.x + c.y * wc.y) + (c.z * wc.z + c.w * wc.w); s3 += (d.x * wd.x + d.y * wd.y) + (d.z * wd.z + d.w * wd.w);
+            if (weighted && off_a != off_b) {
+                // (the weights are the same for every row: their lines are in the L1 cache)
+                const float *w = B + head;
+                auto four = [&](unsigned i) { const float4 a = __ldg(row4 + i); const float *q = w + 4 * i; return (a.x * __ldg(q) + a.y * __ldg(q + 1)) + (a.z * __ldg(q + 2) + a.w * __ldg(q + 3)); };
+                for (; k + N < K4; k += 2 * N) { const float a = four(k), b = four(k + N); s0 += a; s1 += b; }
+                for (; k < K4; k += N) s0 += four(k);
+            } else if (weighted) {
+                for (; k + 3 * N < K4; k += 4 * N) {
+                    const float4 a = __ldg(row4 + k), b = __ldg(row4 + k + N), c = __ldg(row4 + k + 2 * N), d = __ldg(row4 + k + 3 * N);
+                    const float4 wa = __ldg(wts4 + k), wb = __ldg(wts4 + k + N), wc = __ldg(wts4 + k + 2 * N), wd = __ldg(wts4 + k + 3 * N);
+                    s0 += (a.x * wa.x + a.y * wa.y) + (a.z * wa.z + a.w * wa.w); s1 += (b.x * wb.x + b.y * wb.y) + (b.z * wb.z + b.w * wb.w);
+                    s2 += (c.x * wc.x + c.y * wc.y) + (c.z * wc.z + c.w * wc.w); s3 += (d.x * wd.x + d.y * wd.y) + (d.z * wd.z + d.w * wd.w);
+                }
+                for (; k < K4; k += N) { const float4 a = __ldg(row4 + k), wa = __ldg(wts4 + k); s0 += (a.x * wa.x + a.y * wa.y) + (a.z * wa.z + a.w * wa.w); }
+            } else {
+                for (; k + 3 * N < K4; k += 4 * N) {
+                    const float4 a = __ldg(row4 + k), b = __ldg(row4 + k + N), c = __ldg(row4 + k + 2 * N), d = __ldg(row4 + k + 3 * N);
+                    s0 += (a.x + a.y) + (a.z + a.w); s1 += (b.x + b.y) + (b.z + b.w);
+                    s2 += (c.x + c.y) + (c.z + c.w); s3 += (d.x + d.y) + (d.z + d.w);
+                }
+                for (; k < K4; k += N) { const float4 a = __ldg(row4 + k); s0 += (a.x + a.y) + (a.z + a.w); }
             }
-            for (; k < K4; k += 32) { const float4 a = __ldg(row + k), wa = __ldg(wts + k); s0 += (a.x * wa.x + a.y * wa.y) + (a.z * wa.z + a.w * wa.w); }
-            for (unsigned t = K4 * 4 + lane; t < K; t += 32) s1 = fmaf(__ldg(A + (unsigned)(base + (int)t)), __ldg(B + (unsigned)(P.baseB + (int)t)), s1);
-        } else if (weighted) {
-            unsigned k = lane;
-            for (; k + 96 < K; k += 128) {
-                s0 = fmaf(__ldg(A + (unsigned)(base + (int)k * ks)), __ldg(B + (unsigned)(P.baseB + (int)k * kb)), s0);
-                s1 = fmaf(__ldg(A + (unsigned)(base + (int)(k + 32) * ks)), __ldg(B + (unsigned)(P.baseB + (int)(k + 32) * kb)), s1);
-                s2 = fmaf(__ldg(A + (unsigned)(base + (int)(k + 64) * ks)), __ldg(B + (unsigned)(P.baseB + (int)(k + 64) * kb)), s2);
-                s3 = fmaf(__ldg(A + (unsigned)(base + (int)(k + 96) * ks)), __ldg(B + (unsigned)(P.baseB + (int)(k + 96) * kb)), s3);
-            }
-            for (; k < K; k += 32) s0 = fmaf(__ldg(A + (unsigned)(base + (int)k * ks)), __ldg(B + (unsigned)(P.baseB + (int)k * kb)), s0);
-        } else if (ks == 1 && ((base & 3) == 0) && ((reinterpret_cast<uintptr_t>(A) & 15u) == 0)) {
-            const float4 *row = reinterpret_cast<const float4 *>(A + (unsigned)base);
-            const unsigned K4 = K / 4;
-            unsigned k = lane;
-            for (; k + 96 < K4; k += 128) {
-                const float4 a = __ldg(row + k), b = __ldg(row + k + 32), c = __ldg(row + k + 64), d = __ldg(row + k + 96);
-                s0 += (a.x + a.y) + (a.z + a.w); s1 += (b.x + b.y) + (b.z + b.w);
-                s2 += (c.x + c.y) + (c.z + c.w); s3 += (d.x + d.y) + (d.z + d.w);
-            }
-            for (; k < K4; k += 32) { const float4 a = __ldg(row + k); s0 += (a.x + a.y) + (a.z + a.w); }
-            for (unsigned t = K4 * 4 + lane; t < K; t += 32) s1 += __ldg(A + (unsigned)(base + (int)t));
+            if (lane < head) s1 = weighted ? fmaf(__ldg(row + lane), __ldg(B + lane), s1) : s1 + __ldg(row + lane);
+            if (tail + lane < K) s2 = weighted ? fmaf(__ldg(row + tail + lane), __ldg(B + tail + lane), s2) : s2 + __ldg(row + tail + lane);
         } else {
-            for (unsigned k = lane; k < K; k += 32) s0 += __ldg(A + (unsigned)(base + (int)k * ks));
+            unsigned k = lane;
+            auto at = [&](unsigned i) { return __ldg(row + (int)i * ks); };
+            auto wt = [&](unsigned i) { return __ldg(B + (int)i * kb); };
+            if (weighted) {
+                for (; k + 3 * N < K; k += 4 * N) { s0 = fmaf(at(k), wt(k), s0); s1 = fmaf(at(k + N), wt(k + N), s1); s2 = fmaf(at(k + 2 * N), wt(k + 2 * N), s2); s3 = fmaf(at(k + 3 * N), wt(k + 3 * N), s3); }
+                for (; k < K; k += N) s0 = fmaf(at(k), wt(k), s0);
+            } else {
+                for (; k + 3 * N < K; k += 4 * N) { const float a = at(k), b = at(k + N), c = at(k + 2 * N), d = at(k + 3 * N); s0 += a; s1 += b; s2 += c; s3 += d; }
+                for (; k < K; k += N) s0 += at(k);
+            }
         }
         float s = (s0 + s1) + (s2 + s3);
 #pragma unroll
         for (int d = 16; d >= 1; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
+        if constexpr (WARPS > 1) {
+            if ((threadIdx.x & 31u) == 0) parts[threadIdx.x >> 5] = s;
+            __syncthreads();
+            s = ((parts[0] + parts[1]) + (parts[2] + parts[3])) + ((parts[4] + parts[5]) + (parts[6] + parts[7]));
+            __syncthreads();
+        }
         if (lane == 0) {
             const unsigned off = (unsigned)(P.baseO + p.o);
             float v = s * P.scale;
@@ -555,9 +569,10 @@ cudaError_t tad_launch_contract(const TadcProgram &P, const TadpPointers &ptrs, 
         return e;
     }
     if (P.shape == 4) {
-        const unsigned warps = (unsigned)P.M.extent;
-        const unsigned blocks = std::min((warps + 7u) / 8u, sms * 16u);
-        tad_launch(tad_rowsum_kernel, blocks, 256, 0, stream, P, ptrs);
+        // (a warp to each of 1200 rows is eight warps to an SM)
+        const unsigned rows = (unsigned)P.M.extent;
+        if (rows < sms * 8u && P.K.extent >= 512) tad_launch(tad_rowsum_kernel<8>, rows, 256, 0, stream, P, ptrs);
+        else tad_launch(tad_rowsum_kernel<1>, std::min((rows + 7u) / 8u, sms * 16u), 256, 0, stream, P, ptrs);
         return cudaGetLastError();
     }
     cudaError_t e = P.shape == 1 ? launch_shape<128, 32, 8, 4>(P, ptrs, stream)
