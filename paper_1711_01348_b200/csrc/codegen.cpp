@@ -1001,11 +1001,11 @@ bool try_points(Gen &g, Kernel &k, int root, int scale, bool allow_split, const 
     return true;
 }
 
-// Sums whose term couples two variables run as tile programs from 2^18.6 points on, where they are as fast as point programs, which
-// share launches (a step of the intro expression, us: 162 x 95 x 11 48 -> 51, 70 x 675 x 16 91 -> 56, 3978 x 73 x 20 563 -> 79,
-// 2992 x 162 x 31 999 -> 95), up to 5e7, where the sums pushed inside and contracted are (2564 x 2507 x 5 462 -> 214, 7263 x 352 x 21
-// 194 -> 183, 1868 x 2663 x 11 165 -> 177, 1655 x 2679 x 23 163 -> 215).
-constexpr double TILE_LEAST = double(3 << 17), TILE_MOST = 5e7;
+// Sums whose term couples two variables run as tile programs from 2^16 points on, where they are faster than point programs (a step of
+// the intro expression, us: 64 x 64 x 5 27 -> 34, 66 x 85 x 19 42 -> 37, 203 x 157 x 7 48 -> 37, 90 x 400 x 10 65 -> 39,
+// 3978 x 73 x 20 563 -> 79), up to 5e7, where the sums pushed inside and contracted are (2564 x 2507 x 5 462 -> 184, 7263 x 352 x 21
+// 194 -> 188, 1868 x 2663 x 11 165 -> 177, 1655 x 2679 x 23 163 -> 215).
+constexpr double TILE_LEAST = double(1 << 16), TILE_MOST = 5e7;
 
 // shared tail: choose temps, emit, fill the program
 void emit_kernel(Gen &g, Kernel &k, int root, const std::vector<std::vector<TadpRow>> &lower,

@@ -522,13 +522,15 @@ template <int N, int KIND, int TM>
 __global__ void __launch_bounds__(NT, 2)
 tad_tile_kernel(const __grid_constant__ TadtBatch<N> B, const __grid_constant__ TadpPointers ptrs)
 {
-    tad_wait_previous();
     extern __shared__ __align__(16) float sm[];
-    if constexpr (KIND >= 0) run_block<TM, KIND / 2, KIND % 2 != 0>(B.p[0], ptrs, B.out[0], sm, blockIdx.x);
-    else {
+    if constexpr (KIND >= 0) {
+        tad_wait_previous();
+        run_block<TM, KIND / 2, KIND % 2 != 0>(B.p[0], ptrs, B.out[0], sm, blockIdx.x);
+    } else {
         int i = 0;
         while (i + 1 < B.n && blockIdx.x >= B.first[i + 1]) ++i;
         const TadtProgram &P = B.p[i];
+        tad_wait_previous();
         const unsigned bx = blockIdx.x - B.first[i];
         switch (2 * P.path + P.q_sum) {
         case 2: run_block<TM, 1, false>(P, ptrs, B.out[i], sm, bx); break;
