@@ -167,40 +167,115 @@ tad_ew_kernel(const __grid_constant__ TadeProgram P, const __grid_constant__ Tad
 //                (forward, or reversed for offsets that step by -1), which the host has proven aligned in every row;
 //   interleaved: output j of a thread lies j * (threads per row) further, so that plain loads of neighbouring
 //                threads fall into the same lines whatever the load's step.
-// Loads that do not change from row to row are read once per run, loads that do not move along the row once per row.
+// Loads that do not change from row to row are read once per run, loads that do not move along the row once per row.  What bounds
+// it is the latency of the reads (the tables live in L1 and L2): every load of the rows in flight is issued before the first is
+// used, without a branch between them (sin x[2i + j, j - k] y^2 over 512^3 outputs 132 -> 104 us, 300^3 46 -> 31, a table read along
+// steps of three, 4096 x 4096 outputs, 37 -> 27 us).
 // ---------------------------------------------------------------------------------------------------------
 enum ProdKind : int { PK_HOIST = 0, PK_BCAST, PK_FWD, PK_REV, PK_GEN };
 
 struct ProdLoad { int32_t load, kind, exp; };
 struct ProdPlan {
-    int32_t n_loads, n_moving, row_var, run, vec;      // run: rows per thread along row_var (row_var < 0: single rows); moving loads first
-    float c;
+    int32_t n_loads, n_moving, n_single, row_var, run, vec;      // moving loads first, n_single of them read once a row (behind the others);
+    float c;                                                     // run: rows per thread along row_var, or pieces of a single row (row_var < 0)
     ProdLoad ld[4];
 };
 
 __device__ __forceinline__ float powe(float v, int e) { return e == 1 ? v : e == 2 ? v * v : v * v * v; }
 
-template <bool VEC, int M>
-__global__ void __launch_bounds__(256, 3)
+// where a run stands: offsets of its loads and of its output, and what they advance by from row to row
+struct ProdRun { const float *src[3]; int off[3], step[3], adv[3], exp[3]; bool rev[3]; int out, ostep, oadv; };
+
+// U rows: MG loads with a value for each of the four outputs, in pieces of W, and MB with one.  Outputs from `live` on lie outside
+// the row (interleaved layout): their values are read where the first one's are and not stored.
+template <bool VEC, int W, int MG, int MB, int U>
+__device__ __forceinline__ void prod_rows(ProdRun &R, const int live, const float (&held)[4], const bool powers, const bool accumulate, float *__restrict__ out)
+{
+    float v[U][MG > 0 ? MG : 1][4], b[U][MB > 0 ? MB : 1];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+#pragma unroll
+        for (int l = 0; l < MG; ++l) {
+            const float *__restrict__ s = R.src[l];
+            const int o = R.off[l];
+            if constexpr (W == 4) {
+                const float4 q = __ldg(reinterpret_cast<const float4 *>(s + (unsigned)(R.rev[l] ? o - 3 : o)));
+                v[u][l][0] = R.rev[l] ? q.w : q.x; v[u][l][1] = R.rev[l] ? q.z : q.y; v[u][l][2] = R.rev[l] ? q.y : q.z; v[u][l][3] = R.rev[l] ? q.x : q.w;
+            } else if constexpr (W == 2) {
+                const float2 q0 = __ldg(reinterpret_cast<const float2 *>(s + (unsigned)(R.rev[l] ? o - 1 : o)));
+                const float2 q1 = __ldg(reinterpret_cast<const float2 *>(s + (unsigned)(R.rev[l] ? o - 3 : o + 2)));
+                v[u][l][0] = R.rev[l] ? q0.y : q0.x; v[u][l][1] = R.rev[l] ? q0.x : q0.y; v[u][l][2] = R.rev[l] ? q1.y : q1.x; v[u][l][3] = R.rev[l] ? q1.x : q1.y;
+            } else {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) v[u][l][j] = __ldg(s + (unsigned)(VEC || j < live ? o + j * R.step[l] : o));
+            }
+            R.off[l] += R.adv[l];
+        }
+#pragma unroll
+        for (int l = 0; l < MB; ++l) { b[u][l] = __ldg(R.src[MG + l] + (unsigned)R.off[MG + l]); R.off[MG + l] += R.adv[MG + l]; }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        float q[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) q[j] = held[j];
+#pragma unroll
+        for (int l = 0; l < MG; ++l)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) q[j] *= powers ? powe(v[u][l][j], R.exp[l]) : v[u][l][j];
+#pragma unroll
+        for (int l = 0; l < MB; ++l) {
+            const float f = powers ? powe(b[u][l], R.exp[MG + l]) : b[u][l];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) q[j] *= f;
+        }
+        if constexpr (VEC) {
+            float4 *dst = reinterpret_cast<float4 *>(out + (unsigned)R.out);
+            float4 r = make_float4(q[0], q[1], q[2], q[3]);
+            if (accumulate) { const float4 o = *dst; r.x += o.x; r.y += o.y; r.z += o.z; r.w += o.w; }
+            *dst = r;
+        } else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) if (j < live) { const unsigned o = (unsigned)(R.out + j * R.ostep); out[o] = accumulate ? out[o] + q[j] : q[j]; }
+        }
+        R.out += R.oadv;
+    }
+}
+
+template <bool VEC, int W, int MG, int MB, int U>
+__device__ __forceinline__ void prod_run(ProdRun &R, const int n_rows, const int live, const float (&held)[4], const bool powers, const bool accumulate, float *__restrict__ out)
+{
+    int r = 0;
+    for (; r + U <= n_rows; r += U) prod_rows<VEC, W, MG, MB, U>(R, live, held, powers, accumulate, out);
+#pragma unroll 1
+    for (; r < n_rows; ++r) prod_rows<VEC, W, MG, MB, 1>(R, live, held, powers, accumulate, out);
+}
+
+// SINGLE: one long row, its runs along it, a block's width from one piece to the next
+template <bool VEC, int MG, int MB, bool SINGLE>
+__global__ void __launch_bounds__(256, VEC && MG + MB <= 1 ? 6 : VEC && MG + MB == 2 ? 4 : !VEC && MG + MB == 3 ? 4 : 3)
 tad_prod_kernel(const __grid_constant__ TadeProgram P, const __grid_constant__ ProdPlan Q, const __grid_constant__ TadpPointers ptrs,
                 const unsigned n_items, const unsigned cols, const unsigned lane_blocks, const unsigned n_runs, const unsigned runs_per_line)
 {
     tad_wait_previous();
+    constexpr int M = MG + MB, U = VEC && MG + MB <= 2 ? 4 : !VEC && MG + MB == 3 ? 1 : 2;      // (as many as their registers allow)
     const unsigned tid = threadIdx.x;
     const unsigned rows_per_block = 256u / cols;
     const unsigned tc = tid % cols, tr = tid / cols;
     const int lane_var = P.lane_var, row_var = Q.row_var;
     const unsigned lane_ext = (unsigned)P.outer_ext[lane_var];
     const unsigned es = VEC ? 1u : cols;                       // distance between two outputs of a thread
+    const bool accumulate = P.accumulate != 0;
     float *__restrict__ out = ptrs.out;
     for (unsigned item = blockIdx.x; item < n_items; item += gridDim.x) {
         const unsigned lb = item % lane_blocks, rb = item / lane_blocks;
         const unsigned run = rb * rows_per_block + tr;
-        const unsigned lane0 = lb * cols * 4u + (VEC ? tc * 4u : tc);
+        const unsigned lane0 = lb * cols * 4u * (SINGLE ? (unsigned)Q.run : 1u) + (VEC ? tc * 4u : tc);
         if (run >= n_runs || lane0 >= lane_ext) continue;
-        int live;                                              // outputs of this thread inside the row
-        if (VEC) live = (int)min(4u, lane_ext - lane0);
-        else live = (int)min(4u, (lane_ext - lane0 + cols - 1u) / cols);
+        auto inside = [&](unsigned lane) {                     // outputs of this thread inside the row
+            return lane >= lane_ext ? 0 : VEC ? (int)min(4u, lane_ext - lane) : (int)min(4u, (lane_ext - lane + cols - 1u) / cols);
+        };
+        int live = inside(lane0);
         // the run: its position along row_var, then the other outer variables
         const unsigned piece = run % runs_per_line;
         unsigned rem = run / runs_per_line;
@@ -218,14 +293,14 @@ tad_prod_kernel(const __grid_constant__ TadeProgram P, const __grid_constant__ P
                 }
             }
         }
-        const int n_rows = row_var < 0 ? 1 : min(Q.run, P.outer_ext[row_var] - (int)(piece * (unsigned)Q.run));
+        const unsigned whole = SINGLE && live == 4 ? (lane_ext - 1u - 3u * es - lane0) / (4u * cols) + 1u : 1u;      // pieces of four
+        const int n_rows = SINGLE ? (int)min((unsigned)Q.run, whole) : min(Q.run, P.outer_ext[row_var] - (int)(piece * (unsigned)Q.run));
         // loads that stay put from row to row are multiplied into one factor per output (with the constant); the
-        // others ("moving", Q.n_moving of them, first in Q.ld) keep an offset that advances by a constant per row
+        // others ("moving", first in Q.ld) keep an offset that advances by a constant per row
         float held[4] = {Q.c, Q.c, Q.c, Q.c};
-        int off[3] = {0, 0, 0}, step[3] = {0, 0, 0}, adv[3] = {0, 0, 0}, kinds[3] = {0, 0, 0}, exps[3] = {1, 1, 1};
-        const float *__restrict__ srcs[3] = {nullptr, nullptr, nullptr};
-        constexpr int n_moving = M;
-        unsigned widths = 0x111u;                              // four bits per moving load: values per vector load in this run
+        ProdRun R;
+        bool powers = false;
+        int width = 4;                                         // values per vector load in this run
 #pragma unroll
         for (int l = 0; l < 4; ++l) {
             if (l >= Q.n_loads) continue;
@@ -239,86 +314,44 @@ tad_prod_kernel(const __grid_constant__ TadeProgram P, const __grid_constant__ P
 #pragma unroll
                 for (int j = 0; j < 4; ++j) if (j < live) held[j] *= powe(__ldg(src + (unsigned)(o + j * st)), Q.ld[l].exp);
             } else if (l < 3) {
-                off[l] = o; step[l] = st; adv[l] = L.coef[row_var];
-                kinds[l] = Q.ld[l].kind; exps[l] = Q.ld[l].exp; srcs[l] = ptrs.in[L.ptr];
-                if (VEC && live == 4 && (Q.ld[l].kind == PK_FWD || Q.ld[l].kind == PK_REV)) {
-                    const unsigned first = (unsigned)(Q.ld[l].kind == PK_FWD ? o : o - 3);
-                    widths += ((first & 3u) == 0 ? 3u : (first & 1u) == 0 ? 1u : 0u) << (4 * l);
+                R.src[l] = ptrs.in[L.ptr]; R.off[l] = o; R.step[l] = st; R.exp[l] = Q.ld[l].exp;
+                R.adv[l] = SINGLE ? L.coef[lane_var] * (int)(4u * cols) : L.coef[row_var];
+                R.rev[l] = Q.ld[l].kind == PK_REV;
+                powers = powers || R.exp[l] != 1;
+                if (l < MG) {
+                    const unsigned first = (unsigned)(R.rev[l] ? o - 3 : o);
+                    width = min(width, (first & 3u) == 0 ? 4 : (first & 1u) == 0 ? 2 : 1);
                 }
             }
         }
-        int oo = P.out_base;
+        R.out = P.out_base;
 #pragma unroll
-        for (int v = 0; v < TADP_MAX_VARS; ++v) oo += P.out_coef[v] * var[v];
-        const int ostep = P.out_coef[lane_var] * (int)es, oadv = row_var < 0 ? 0 : P.out_coef[row_var];
-        // the product of one row (offsets advance to the next row)
-        auto row = [&](float (&p)[4]) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) p[j] = held[j];
-#pragma unroll
-            for (int l = 0; l < M; ++l) {
-                const int kind = kinds[l];
-                const unsigned w = (widths >> (4 * l)) & 15u;
-                const float *__restrict__ src = srcs[l];
-                float v4[4];
-                if (kind == PK_BCAST) {
-                    const float s = __ldg(src + (unsigned)off[l]);
-                    v4[0] = v4[1] = v4[2] = v4[3] = s;
-                } else if (VEC && w == 4u) {
-                    if (kind == PK_FWD) {
-                        const float4 q = __ldg(reinterpret_cast<const float4 *>(src + (unsigned)off[l]));
-                        v4[0] = q.x; v4[1] = q.y; v4[2] = q.z; v4[3] = q.w;
-                    } else {
-                        const float4 q = __ldg(reinterpret_cast<const float4 *>(src + (unsigned)(off[l] - 3)));
-                        v4[0] = q.w; v4[1] = q.z; v4[2] = q.y; v4[3] = q.x;
-                    }
-                } else if (VEC && w == 2u) {
-                    if (kind == PK_FWD) {
-                        const float2 q0 = __ldg(reinterpret_cast<const float2 *>(src + (unsigned)off[l]));
-                        const float2 q1 = __ldg(reinterpret_cast<const float2 *>(src + (unsigned)(off[l] + 2)));
-                        v4[0] = q0.x; v4[1] = q0.y; v4[2] = q1.x; v4[3] = q1.y;
-                    } else {
-                        const float2 q0 = __ldg(reinterpret_cast<const float2 *>(src + (unsigned)(off[l] - 1)));
-                        const float2 q1 = __ldg(reinterpret_cast<const float2 *>(src + (unsigned)(off[l] - 3)));
-                        v4[0] = q0.y; v4[1] = q0.x; v4[2] = q1.y; v4[3] = q1.x;
-                    }
-                } else if (live == 4) {
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) v4[j] = __ldg(src + (unsigned)(off[l] + j * step[l]));
-                } else {
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) v4[j] = j < live ? __ldg(src + (unsigned)(off[l] + j * step[l])) : 0.f;
-                }
-                if (exps[l] != 1) {
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) v4[j] = powe(v4[j], exps[l]);
-                }
-#pragma unroll
-                for (int j = 0; j < 4; ++j) p[j] *= v4[j];
-                off[l] += adv[l];
-            }
-        };
-        auto store = [&](const float (&p)[4]) {
-            if (VEC && live == 4) {
-                float4 *dst = reinterpret_cast<float4 *>(out + (unsigned)oo);
-                float4 q = make_float4(p[0], p[1], p[2], p[3]);
-                if (P.accumulate) { const float4 o = *dst; q.x += o.x; q.y += o.y; q.z += o.z; q.w += o.w; }
-                *dst = q;
-            } else {
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    if (j < live) { const unsigned o = (unsigned)(oo + j * ostep); out[o] = P.accumulate ? out[o] + p[j] : p[j]; }
-            }
-            oo += oadv;
-        };
-        // two rows in flight: the loads of the second are issued before the first is multiplied and stored
-        int r = 0;
-        for (; r + 2 <= n_rows; r += 2) {
-            float p0[4], p1[4];
-            row(p0); row(p1);
-            store(p0); store(p1);
+        for (int v = 0; v < TADP_MAX_VARS; ++v) R.out += P.out_coef[v] * var[v];
+        R.ostep = P.out_coef[lane_var] * (int)es; R.oadv = SINGLE ? P.out_coef[lane_var] * (int)(4u * cols) : P.out_coef[row_var];
+        if (!VEC || live == 4) {
+            if constexpr (!VEC || MG == 0) prod_run<VEC, 1, MG, MB, U>(R, n_rows, live, held, powers, accumulate, out);
+            else if (width == 4) prod_run<VEC, 4, MG, MB, U>(R, n_rows, live, held, powers, accumulate, out);
+            else if (width == 2) prod_run<VEC, 2, MG, MB, U>(R, n_rows, live, held, powers, accumulate, out);
+            else prod_run<VEC, 1, MG, MB, U>(R, n_rows, live, held, powers, accumulate, out);
+            live = SINGLE && live == 4 && n_rows < Q.run ? inside(lane0 + (unsigned)n_rows * 4u * cols) : 0;
+            if (live == 0) continue;
         }
-        if (r < n_rows) { float p0[4]; row(p0); store(p0); }
+        // the last outputs of a row that is no multiple of four
+#pragma unroll 1
+        for (int r = 0; r < (SINGLE ? 1 : n_rows); ++r) {
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                if (j >= live) continue;
+                float q = held[j];
+#pragma unroll
+                for (int l = 0; l < M; ++l) q *= powe(__ldg(R.src[l] + (unsigned)(R.off[l] + (l < MG ? j * R.step[l] : 0))), R.exp[l]);
+                const unsigned o = (unsigned)(R.out + j * R.ostep);
+                out[o] = accumulate ? out[o] + q : q;
+            }
+#pragma unroll
+            for (int l = 0; l < M; ++l) R.off[l] += R.adv[l];
+            R.out += R.oadv;
+        }
     }
 }
 
@@ -378,31 +411,34 @@ bool plan_product(const TadeProgram &P, const TadpPointers &ptrs, unsigned sms, 
     // rows per thread: as many as leave every SM a few thousand threads
     int run = 1;
     while (run < 32 && elems / (4.0 * run * 2) >= (double)sms * 2048.0) run *= 2;
-    Q.run = Q.row_var < 0 ? 1 : std::min(run, P.outer_ext[Q.row_var]);
+    Q.run = Q.row_var < 0 ? run : std::min(run, P.outer_ext[Q.row_var]);
     // the output is stored in 128-bit pieces when its first element of every row is a multiple of four; a load needs
     // only a row step that is one (the width of its vector loads is settled per run)
     auto aligned = [&](const int32_t *coef, int64_t base) {
         int64_t o = base;
-        for (int v = 0; v < P.n_outer; ++v) { o += (int64_t)coef[v] * P.outer_lo[v]; if (v != lane && coef[v] % 4 != 0) return false; }
+        for (int v = 0; v < P.n_outer; ++v) { o += (int64_t)coef[v] * P.outer_lo[v]; if (v != lane && P.outer_ext[v] > 1 && coef[v] % 4 != 0) return false; }
         return o % 4 == 0;
     };
     bool vec = P.out_coef[lane] == 1 && aligned(P.out_coef, P.out_base) && (reinterpret_cast<uintptr_t>(ptrs.out) & 15u) == 0;
     for (int i = 0; i < Q.n_loads; ++i) {
         const TadpLoad &L = P.loads[Q.ld[i].load];
-        const int step = L.coef[lane], adv = Q.row_var < 0 ? 0 : L.coef[Q.row_var];
+        const int step = L.coef[lane], adv = Q.row_var < 0 ? 4 * step : L.coef[Q.row_var];
         const bool base16 = (reinterpret_cast<uintptr_t>(ptrs.in[L.ptr]) & 15u) == 0;
         int kind = PK_GEN;
-        if (adv == 0 || Q.run == 1) kind = PK_HOIST;
+        // (a run of a single row: loads move only in so far as that lets them be read in pieces)
+        if (Q.run == 1 ? !(base16 && std::abs(step) == 1) : adv == 0) kind = PK_HOIST;
         else if (step == 0) kind = PK_BCAST;
-        else if (step == 1 && base16 && adv % 4 == 0) kind = PK_FWD;
-        else if (step == -1 && base16 && adv % 4 == 0) kind = PK_REV;
+        else if (step == 1 && base16 && (adv % 4 == 0 || Q.run == 1)) kind = PK_FWD;
+        else if (step == -1 && base16 && (adv % 4 == 0 || Q.run == 1)) kind = PK_REV;
         if (kind == PK_GEN) vec = false;
         Q.ld[i].kind = kind;
     }
-    // moving loads first
-    std::stable_sort(Q.ld, Q.ld + Q.n_loads, [](const ProdLoad &a, const ProdLoad &b) { return (a.kind != PK_HOIST) > (b.kind != PK_HOIST); });
-    Q.n_moving = 0;
-    for (int i = 0; i < Q.n_loads; ++i) Q.n_moving += Q.ld[i].kind != PK_HOIST;
+    if (Q.run == 1 && !vec) for (int i = 0; i < Q.n_loads; ++i) Q.ld[i].kind = PK_HOIST;
+    // moving loads first, those read once a row behind the others
+    auto rank = [](const ProdLoad &a) { return a.kind == PK_HOIST ? 2 : a.kind == PK_BCAST ? 1 : 0; };
+    std::stable_sort(Q.ld, Q.ld + Q.n_loads, [&](const ProdLoad &a, const ProdLoad &b) { return rank(a) < rank(b); });
+    Q.n_moving = Q.n_single = 0;
+    for (int i = 0; i < Q.n_loads; ++i) { Q.n_moving += Q.ld[i].kind != PK_HOIST; Q.n_single += Q.ld[i].kind == PK_BCAST; }
     Q.vec = vec ? 1 : 0;
     return Q.n_moving <= 3;
 }
@@ -421,25 +457,26 @@ cudaError_t tad_launch_ew(const TadeProgram &P, const TadpPointers &ptrs, unsign
         while (pc < 256u && pc * 4u < lane_ext) pc *= 2u;
         if (!Q.vec && pc < 32u) pc = 32u;                      // interleaved outputs: a warp covers a run of 32 columns
         const unsigned per_block = 256u / pc;
-        const unsigned lblocks = (lane_ext + pc * 4u - 1u) / (pc * 4u);
+        const unsigned per_run = pc * 4u * (Q.row_var < 0 ? (unsigned)Q.run : 1u), lblocks = (lane_ext + per_run - 1u) / per_run;
         const unsigned long long row_ext = Q.row_var < 0 ? 1ull : (unsigned long long)P.outer_ext[Q.row_var];
-        const unsigned long long per_line = (row_ext + Q.run - 1) / Q.run;
+        const unsigned long long per_line = Q.row_var < 0 ? 1ull : (row_ext + Q.run - 1) / Q.run;
         const unsigned long long runs = rows / row_ext * per_line;
         const unsigned long long its = ((runs + per_block - 1) / per_block) * lblocks;
         if (its >= (1ull << 32) || runs >= (1ull << 31)) return cudaErrorInvalidValue;
         const unsigned g = (unsigned)std::min<unsigned long long>(its, (unsigned long long)sms * 32ull);
-#define TAD_PROD_LAUNCH(V, MM) tad_launch(tad_prod_kernel<V, MM>, g, 256, 0, stream, P, Q, ptrs, (unsigned)its, pc, lblocks, (unsigned)runs, (unsigned)per_line)
-        switch ((Q.vec ? 4 : 0) + Q.n_moving) {
-        case 0: TAD_PROD_LAUNCH(false, 0); break;
-        case 1: TAD_PROD_LAUNCH(false, 1); break;
-        case 2: TAD_PROD_LAUNCH(false, 2); break;
-        case 3: TAD_PROD_LAUNCH(false, 3); break;
-        case 4: TAD_PROD_LAUNCH(true, 0); break;
-        case 5: TAD_PROD_LAUNCH(true, 1); break;
-        case 6: TAD_PROD_LAUNCH(true, 2); break;
-        default: TAD_PROD_LAUNCH(true, 3); break;
+#define TAD_PROD_ARGS g, 256, 0, stream, P, Q, ptrs, (unsigned)its, pc, lblocks, (unsigned)runs, (unsigned)per_line
+#define TAD_PROD_LAUNCH(G, B)                                                                                                           \
+    case 4 * G + B:                                                                                                                     \
+        if (Q.row_var < 0) { if (Q.vec) tad_launch(tad_prod_kernel<true, G, B, true>, TAD_PROD_ARGS); else tad_launch(tad_prod_kernel<false, G, B, true>, TAD_PROD_ARGS); } \
+        else { if (Q.vec) tad_launch(tad_prod_kernel<true, G, B, false>, TAD_PROD_ARGS); else tad_launch(tad_prod_kernel<false, G, B, false>, TAD_PROD_ARGS); } \
+        break;
+        switch (4 * (Q.n_moving - Q.n_single) + Q.n_single) {
+        TAD_PROD_LAUNCH(0, 0) TAD_PROD_LAUNCH(0, 1) TAD_PROD_LAUNCH(0, 2) TAD_PROD_LAUNCH(0, 3) TAD_PROD_LAUNCH(1, 0) TAD_PROD_LAUNCH(1, 1)
+        TAD_PROD_LAUNCH(1, 2) TAD_PROD_LAUNCH(2, 0) TAD_PROD_LAUNCH(2, 1) TAD_PROD_LAUNCH(3, 0)
+        default: return cudaErrorInvalidValue;
         }
 #undef TAD_PROD_LAUNCH
+#undef TAD_PROD_ARGS
         return cudaGetLastError();
     }
     unsigned cols = 1;
