@@ -433,7 +433,7 @@ bool plan_product(const TadeProgram &P, const TadpPointers &ptrs, unsigned sms, 
         if (kind == PK_GEN) vec = false;
         Q.ld[i].kind = kind;
     }
-    if (Q.run == 1 && !vec) for (int i = 0; i < Q.n_loads; ++i) Q.ld[i].kind = PK_HOIST;
+    if (Q.run == 1 && (!vec || Q.row_var >= 0)) for (int i = 0; i < Q.n_loads; ++i) Q.ld[i].kind = PK_HOIST;
     // moving loads first, those read once a row behind the others
     auto rank = [](const ProdLoad &a) { return a.kind == PK_HOIST ? 2 : a.kind == PK_BCAST ? 1 : 0; };
     std::stable_sort(Q.ld, Q.ld + Q.n_loads, [&](const ProdLoad &a, const ProdLoad &b) { return rank(a) < rank(b); });

@@ -480,6 +480,20 @@ bool try_tile(Gen &g, Kernel &k, int root, int scale, const std::vector<std::vec
               const std::vector<TadpRow> &guards, double min_space, double max_space)
 {
     if (g.p.opt.debug_bounds || root < 0 || !guards.empty()) return false;
+    // the number of points, ahead of any work: the outputs, loops with fixed ranges, one sum inside the term
+    double points = 1;
+    for (int v = 0; v < g.n_outer; ++v) points *= (double)std::max(1, k.prog.outer_ext[v]);
+    for (int c = 0; c < g.kappa; ++c) {
+        int64_t a = INT64_MIN, b = INT64_MAX;
+        for (const TadpRow &r : lower[c]) a = std::max(a, ceil_div(r.c0, r.den));
+        for (const TadpRow &r : upper[c]) b = std::min(b, floor_div(r.c0, r.den));
+        for (const std::vector<TadpRow> *rows : {&lower[c], &upper[c]})
+            for (const TadpRow &r : *rows) for (int v = 0; v < TADP_MAX_VARS; ++v) if (r.coef[v]) return false;
+        if (a == INT64_MIN || b == INT64_MAX || b < a) return false;
+        points *= (double)(b - a + 1);
+    }
+    for (const Inst &in : g.inst) if (in.uses && in.op == I_SUM) points *= (double)std::max<int64_t>(1, in.hi - in.lo + 1);
+    if (points < min_space || points > max_space) return false;
     Tiler all(g, k);
     if (!all.analyse(root, scale, lower, upper)) return false;
     std::unique_ptr<Tiler> found;
@@ -490,8 +504,6 @@ bool try_tile(Gen &g, Kernel &k, int root, int scale, const std::vector<std::vec
     }
     if (!found) return false;
     const Tiler &t = *found;
-    const double space = (double)t.T.p_ext * t.T.q_ext * t.T.l_ext * t.T.z_ext[0] * t.T.z_ext[1];
-    if (space < min_space || space > max_space) return false;
     k.tile = {t.T};
     k.prog.zsplit = 1;
     k.vec = 0; k.vec_u = 0;
