@@ -1070,6 +1070,8 @@ void emit_kernel(Gen &g, Kernel &k, int root, const std::vector<std::vector<Tadp
     if (try_tile(g, k, root, scale, lower, upper, guards, TILE_LEAST, TILE_MOST)) return;
     // sums that can be pushed inside the term (Sec. 6's missing clean-up step): auxiliary kernels + a smaller kernel
     if (may_factor && try_factoring(g, k, root, scale, allow_split, lower, upper, guards)) return;
+    // (sums too short to gain from that)
+    if (try_tile(g, k, root, scale, lower, upper, guards, TILE_MOST, 1e18)) return;
     // short sums ahead of a kernel: as point programs they share a launch with the others
     if (!may_factor && g.kappa == 0 && g.inst[root].op == I_SUM) {
         try {

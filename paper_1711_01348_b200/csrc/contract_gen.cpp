@@ -174,7 +174,7 @@ bool emit_program(const System &s0, float scale, int accumulate, bool allow_spli
     // one output column: plain or weighted sums of A (B is ones or a vector over k), run at memory speed by a warp
     // per row (A along k) or a thread per row (A along m)
     // (fewer than 1024 rows take a block each: 264 rows of 6523 elements, summed for a band of 287 outputs, 80 us as a sum of both loops)
-    const bool long_rows = P.M.extent >= 32 && P.K.n_digits == 1 && P.K.extent >= 512 && P.K.sA[0] == 1;
+    const bool long_rows = P.M.extent >= 32 && P.K.n_digits == 1 && P.K.extent >= 64 && P.K.sA[0] == 1;
     const bool one_column = P.N.extent == 1 && P.Z.extent == 1 && P.K.n_digits <= 1 && !P.guardA && !P.guardB && (P.M.extent >= 1024 || long_rows);
     const bool col_sums = one_column && P.M.n_digits == 1 && P.M.sA[0] == 1 && P.K.n_digits == 1 && std::llabs((int64_t)P.K.sA[0]) != 1;
     const bool row_sums = one_column && !col_sums;

@@ -11,7 +11,7 @@ namespace tad {
 
 namespace {
 
-constexpr double TILE_COPY = 9, TILE_START = 500, TILE_FIXED = 3500;      // issue slots (schedule)
+constexpr double TILE_COPY = 9, TILE_START = 300, TILE_FIXED = 3500;      // issue slots (schedule)
 constexpr int64_t TILE_MIN_SUM = 4;           // fewer terms than this: nothing to share between the values of a tile
 
 struct Tiler {
@@ -463,7 +463,7 @@ void Tiler::schedule()
                 const double arith = pieces * std::ceil((double)c.chunk / lg) * per_value;
                 const double copies = ((double)T.n_rows * bm / (T.q_sum && pieces == 1 ? q_per : 1) + (double)T.n_cols * bn) * l_per / TADT_NT * TILE_COPY;
                 const double tail = T.q_sum ? 4 * slots : (T.n_epi * 2.5 + 6) * slots / (lg * shares);
-                const double per_tile = 2 * (arith + copies + tail) * q_per + 2 * pieces * q_per * (100 + 60 * T.n_ops);
+                const double per_tile = 2 * (arith + copies + tail) * q_per + 2 * pieces * q_per * (100 + 60 * T.n_ops) + (T.q_sum ? 1400.0 * q_per : 0);    // (a tile's factor is waited for)
                 const double fixed = TILE_FIXED + (shares > 1 ? 1500 : 0) + (lg > 1 ? 300 + lg * 12 : 0);
                 // a block alone on its SM issues in about half of its slots, two in three quarters; clusters leave some SMs to one
                 const double total = blocks * shares, room = shares > 1 ? 264 : 296, cost = 2 * TILE_START + per_tile;

@@ -40,6 +40,7 @@ CASES = {
     "long_pieces": lambda: W.intro(33, 31, 1201),
     "aligned": lambda: W.intro(512, 256, 16),
     "two_to_the_24": lambda: W.intro(1024, 512, 32),
+    "short_and_large": lambda: W.intro(4500, 2700, 5),
     "functions": lambda: _functions(411, 253, 9),
     "planes": lambda: _planes(3, 290, 77, 11),
 }
@@ -50,7 +51,7 @@ def test_taken(name):
     e = CASES[name]()
     plan = Plan(e)
     text = "".join(plan.disassemble(w) for w in [-1] + [-2 - s for s in range(plan.num_stages())] + list(range(len(e.accesses))))
-    assert text.count("; tile program") >= (1 if name in ("functions", "planes") else 3)
+    assert text.count("; tile program") >= (1 if name in ("functions", "planes") else 2 if name == "short_and_large" else 3)
 
 
 @pytest.mark.gpu
