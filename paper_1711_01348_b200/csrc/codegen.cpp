@@ -558,33 +558,30 @@ int body_fetch_kind(const TadpLoad &L, int ta, int ub)
     return BF_EACH;
 }
 
-// A program without loops and temporaries whose pending values never exceed two becomes an element-wise program
-// (ew.h); a thread owns four consecutive values of the lane variable.
-// Steps of an element-wise program read off the expression itself, the operand that needs the second value register
-// evaluated first (so that a * (b * c + d) needs no more than X and Y whatever the order it was written in).
-// need(i): value registers the evaluation of i occupies; a binary operation whose operands are both compound puts the
-// first into Y, which the second must then leave alone (need 1).
 }  // namespace
 
+int values_held(const Gen &g, int i, const std::function<bool(int)> &in_place, bool subtracts)
+{
+    const Inst &in = g.inst[i];
+    if (in_place(i)) return 1;
+    if (in.op == I_SUM) return 99;
+    if (in.a < 0) return 1;
+    const int a = values_held(g, in.a, in_place, subtracts);
+    if (in.b < 0) return a;
+    const int b = values_held(g, in.b, in_place, subtracts);
+    const bool commutes = in.op == I_ADD || in.op == I_MUL;
+    if ((commutes || (in.op == I_SUB && subtracts)) && (in_place(in.a) || in_place(in.b))) return std::max(a, b);
+    return commutes ? std::max(std::max(a, b), std::min(a, b) + 1) : std::max(a, b + 1);
+}
+
+// Steps of an element-wise program read off the expression itself, the operand that needs the second value register
+// evaluated first (so that a * (b * c + d) needs no more than X and Y whatever the order it was written in).
 bool elementwise_steps_of(const Gen &g, int root, std::vector<TadeStep> &steps, int leaf)
 {
     auto push_step = [&](int op, int a = 0, int b = 0, float imm = 0.f) { TadeStep s{}; s.op = (uint8_t)op; s.a = (int16_t)a; s.b = (uint8_t)b; s.imm = imm; steps.push_back(s); };
     auto is_load = [&](int i) { return g.inst[i].op == I_LOAD || i == leaf; };
     auto load_of = [&](int i) { return i == leaf ? -1 : g.inst[i].load; };
-    std::function<int(int)> need = [&](int i) -> int {
-        const Inst &in = g.inst[i];
-        if (i == leaf) return 1;
-        switch (in.op) {
-        case I_CONST: case I_LOAD: return 1;
-        case I_SUM: return 99;
-        case I_ADD: case I_MUL:
-            if (is_load(in.a)) return need(in.b);
-            if (is_load(in.b)) return need(in.a);
-            return std::max(std::max(need(in.a), need(in.b)), std::min(need(in.a), need(in.b)) + 1);
-        case I_SUB: case I_DIV: return std::max(need(in.a), need(in.b) + 1);
-        default: return need(in.a);
-        }
-    };
+    auto need = [&](int i) { return values_held(g, i, is_load, false); };
     std::function<bool(int)> emit = [&](int i) -> bool {
         const Inst &in = g.inst[i];
         if (i == leaf) { push_step(E_LD, -1, 0); return true; }
@@ -635,6 +632,8 @@ bool elementwise_steps_of(const Gen &g, int root, std::vector<TadeStep> &steps, 
 
 namespace {
 
+// A program without loops and temporaries whose pending values never exceed two becomes an element-wise program
+// (ew.h); a thread owns four consecutive values of the lane variable.
 bool try_elementwise(Gen &g, Kernel &k, const Emitter &em, const std::vector<TadpRow> &guards, int root)
 {
     const TadpProgram &prog = k.prog;

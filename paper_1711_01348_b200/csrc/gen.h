@@ -6,6 +6,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <functional>
 #include <map>
 #include <tuple>
 
@@ -353,6 +354,10 @@ bool try_contraction(Gen &g, Kernel &k, int root, int scale, bool allow_split, c
 // tile_gen.cpp: a sum whose term couples two variables becomes a tile program, if its number of points lies in the given range
 bool try_tile(Gen &g, Kernel &k, int root, int scale, const std::vector<std::vector<TadpRow>> &lower, const std::vector<std::vector<TadpRow>> &upper,
               const std::vector<TadpRow> &guards, double min_space, double max_space);
+// codegen.cpp: values that an accumulator program over X and Y holds at once while it evaluates instance i.  Instances for which in_place
+// holds are read in one step, also as the second operand of a sum, a product and (subtracts) a difference; every other binary operation
+// puts its first operand into Y, which the second must then leave alone (hold one value).
+int values_held(const Gen &g, int i, const std::function<bool(int)> &in_place, bool subtracts);
 // codegen.cpp: steps of an element-wise program (ew.h) for an instance; the instance `leaf` is read as load -1
 bool elementwise_steps_of(const Gen &g, int root, std::vector<TadeStep> &steps, int leaf = -1);
 // line_gen.cpp: a gradient kernel whose term is a product of index expressions becomes a line-sum program

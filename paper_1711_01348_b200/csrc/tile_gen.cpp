@@ -173,17 +173,8 @@ struct Tiler {
         T.imm[n_imm] = v;
         return code(op, n_imm++);
     }
-    // values that the evaluation of i holds at once: 0 an operand, else 1 or 2
-    int need(int i) const
-    {
-        if (is_operand(i)) return 0;
-        const Inst &in = g.inst[i];
-        if (in.a < 0) return 1;
-        if (in.b < 0) return std::max(1, need(in.a));
-        const int a = need(in.a), b = need(in.b);
-        if (a == 0 || b == 0) return std::max(1, std::max(a, b));
-        return std::max(std::max(a, b), std::min(a, b) + 1);
-    }
+    // values that the evaluation of i holds at once: operands are read in one step, also where they are subtracted
+    int need(int i) const { return values_held(g, i, [this](int j) { return is_operand(j); }, true); }
     // the operand that comes first when both are: what stays in registers, rows, columns
     bool before(int a, int b) const
     {
@@ -239,7 +230,7 @@ struct Tiler {
             if (is_operand(in.a)) return emit(in.b) && code(T_RSUB, operand(in.a));
             return need(in.a) <= 2 && need(in.b) == 1 && emit(in.a) && code(T_PUSH) && emit(in.b) && code(T_BINY, 1);
         case I_DIV:
-            return need(in.a) <= 2 && need(in.b) <= 1 && emit(in.a) && code(T_PUSH) && emit(in.b) && code(T_BINY, 3);
+            return need(in.a) <= 2 && need(in.b) == 1 && emit(in.a) && code(T_PUSH) && emit(in.b) && code(T_BINY, 3);
         default: return false;
         }
     }
@@ -363,7 +354,7 @@ bool Tiler::build(int root, int scale, const Choice &choice)
     const bool outside = q_sum && !post.empty();              // a constant factor goes where it costs nothing
     if (last >= 0 && !outside) last = g.mulc(last, cfac);
     grow();
-    if (need(body) == 0 || !emit(body)) return false;
+    if (is_operand(body) || need(body) > 2 || !emit(body)) return false;
     if (cfac != 1.f && !outside && last < 0 && !imm_step(T_MULC, cfac)) return false;
     if (last >= 0 ? !code(T_ACC, operand(last), 1) : !code(T_ACC)) return false;
     if (outside && !program(g.mulc(product(post), cfac), -1, T.post0, T.n_post)) return false;
