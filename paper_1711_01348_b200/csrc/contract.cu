@@ -407,9 +407,11 @@ tad_contract_reduce(const __grid_constant__ TadcProgram P, const __grid_constant
 //     out[m] (+)= scale * sum_k A[row(m) + k * stride] (* B[k])
 // Bound by HBM: every element of A is read once, in pieces of 16 bytes from the first aligned one on where the row is consecutive
 // (and its weights lie alike), four in flight per lane.  A warp per output, or, where that would leave the GPU idle, a block of
-// eight (WARPS): 264 rows of 6523 elements.  Sums are added in a fixed order.
+// eight (WARPS): 264 rows of 6523 elements.  Sums are added in a fixed order.  Four blocks to an SM: short rows wait for one load after
+// another and live on the warps beside them (with two, weighted 500000 x 64 197 us, 30000 x 100 13.4, strided 500000 x 9 184; with four
+// 113, 7.9, 74).
 template <int WARPS>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 4)
 tad_rowsum_kernel(const __grid_constant__ TadcProgram P, const __grid_constant__ TadpPointers ptrs)
 {
     tad_wait_previous();
@@ -423,12 +425,14 @@ tad_rowsum_kernel(const __grid_constant__ TadcProgram P, const __grid_constant__
     const int kb = P.K.n_digits ? P.K.sB[0] : 0;
     const unsigned K = (unsigned)P.K.extent;
     const int ks = P.K.n_digits ? P.K.sA[0] : 0;
+    const bool pieces = ks == 1 && (!weighted || kb == 1) && K > 32u;      // (an element a lane is not worth the alignment)
     for (unsigned m = first; m < (unsigned)P.M.extent; m += step) {
         const Parts p = decode(P.M, m);
-        const float *row = A + (P.baseA + p.a);
+        const int base = P.baseA + p.a;
         float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
-        const unsigned off_a = (unsigned)(reinterpret_cast<uintptr_t>(row) >> 2) & 3u, off_b = (unsigned)(reinterpret_cast<uintptr_t>(B) >> 2) & 3u;
-        if (ks == 1 && (!weighted || kb == 1)) {
+        if (pieces) {
+            const float *row = A + base;
+            const unsigned off_a = (unsigned)(reinterpret_cast<uintptr_t>(row) >> 2) & 3u, off_b = (unsigned)(reinterpret_cast<uintptr_t>(B) >> 2) & 3u;
             const unsigned head = min((4u - off_a) & 3u, K), K4 = (K - head) / 4u, tail = head + 4u * K4;
             const float4 *row4 = reinterpret_cast<const float4 *>(row + head), *wts4 = reinterpret_cast<const float4 *>(B + head);
             unsigned k = lane;
@@ -458,8 +462,8 @@ tad_rowsum_kernel(const __grid_constant__ TadcProgram P, const __grid_constant__
             if (tail + lane < K) s2 = weighted ? fmaf(__ldg(row + tail + lane), __ldg(B + tail + lane), s2) : s2 + __ldg(row + tail + lane);
         } else {
             unsigned k = lane;
-            auto at = [&](unsigned i) { return __ldg(row + (int)i * ks); };
-            auto wt = [&](unsigned i) { return __ldg(B + (int)i * kb); };
+            auto at = [&](unsigned i) { return __ldg(A + (unsigned)(base + (int)i * ks)); };
+            auto wt = [&](unsigned i) { return __ldg(ptrs.in[P.ptrB] + (unsigned)(P.baseB + (int)i * kb)); };
             if (weighted) {
                 for (; k + 3 * N < K; k += 4 * N) { s0 = fmaf(at(k), wt(k), s0); s1 = fmaf(at(k + N), wt(k + N), s1); s2 = fmaf(at(k + 2 * N), wt(k + 2 * N), s2); s3 = fmaf(at(k + 3 * N), wt(k + 3 * N), s3); }
                 for (; k < K; k += N) s0 = fmaf(at(k), wt(k), s0);
@@ -569,9 +573,10 @@ cudaError_t tad_launch_contract(const TadcProgram &P, const TadpPointers &ptrs, 
         return e;
     }
     if (P.shape == 4) {
-        // (a warp to each of 1200 rows is eight warps to an SM)
+        // (weighted rows, warp / block a row, us: 264 of 512 2.1 / 2.3, of 1024 2.5 / 2.4, of 8192 7.5 / 3.0; 592 of 1024 2.5 / 2.8, of 4096
+        // 4.7 / 3.0; 1100 of 1024 2.6 / 4.0, of 4096 4.9 / 4.5; 1200 rows are eight warps to an SM)
         const unsigned rows = (unsigned)P.M.extent;
-        if (rows < sms * 8u && P.K.extent >= 512) tad_launch(tad_rowsum_kernel<8>, rows, 256, 0, stream, P, ptrs);
+        if (rows < sms * 8u && (unsigned)P.K.extent >= std::max(512u, 4u * rows)) tad_launch(tad_rowsum_kernel<8>, rows, 256, 0, stream, P, ptrs);
         else tad_launch(tad_rowsum_kernel<1>, std::min((rows + 7u) / 8u, sms * 16u), 256, 0, stream, P, ptrs);
         return cudaGetLastError();
     }

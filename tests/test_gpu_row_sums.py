@@ -17,13 +17,17 @@ def _weighted(n, k, step):
     return b.done()
 
 
+# an element a lane or pieces, a warp or a block a row: either side of each line
+EDGES = [(2001, 32, 1), (2001, 33, 1), (1500, 32, 2), (1500, 33, 2), (1200, 65, 1), (250, 999, 1), (250, 1000, 1), (1183, 4731, 1), (1183, 4732, 1), (1184, 4736, 1)]
+
+
 @pytest.mark.parametrize("n,k,step", CASES)
 def test_taken(n, k, step):
     assert "row sums" in Plan(_weighted(n, k, step)).disassemble(-1)
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("n,k,step", CASES)
+@pytest.mark.parametrize("n,k,step", CASES + EDGES)
 def test_weighted_rows(n, k, step):
     from tests.gpu_util import check_against_oracle
     e = _weighted(n, k, step)
