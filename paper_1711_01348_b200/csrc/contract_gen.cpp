@@ -174,7 +174,11 @@ bool emit_program(const System &s0, float scale, int accumulate, bool allow_spli
     // one output column: plain or weighted sums of A (B is ones or a vector over k), run at memory speed by a warp
     // per row (A along k) or a thread per row (A along m)
     // (fewer than 1024 rows take a block each: 264 rows of 6523 elements, summed for a band of 287 outputs, 80 us as a sum of both loops)
-    const bool long_rows = P.M.extent >= 32 && P.K.n_digits == 1 && P.K.extent >= 64 && P.K.sA[0] == 1;
+    // A block streams about 50 GB/s: where rows are fewer than the SMs, long ones are split instead (weighted, read from HBM, row sums /
+    // split, us: 32 x 60000 17 / 17, 32 x 100000 24 / 17, 36 x 300000 56 / 26, 64 x 50000 15 / 17, 64 x 200000 42 / 30, 100 x 60000 19 / 24,
+    // 100 x 200000 46 / 38, 128 x 100000 28 / 30, 128 x 200000 48 / 44, 148 x 500000 101 / 101, 200 x 300000 73 / 83).
+    const bool long_rows = P.M.extent >= 32 && P.K.n_digits == 1 && P.K.extent >= 64 && P.K.sA[0] == 1 &&
+                           (P.M.extent >= 148 || P.K.extent <= 30000 + 800 * (int64_t)P.M.extent);
     const bool one_column = P.N.extent == 1 && P.Z.extent == 1 && P.K.n_digits <= 1 && !P.guardA && !P.guardB && (P.M.extent >= 1024 || long_rows);
     const bool col_sums = one_column && P.M.n_digits == 1 && P.M.sA[0] == 1 && P.K.n_digits == 1 && std::llabs((int64_t)P.K.sA[0]) != 1;
     const bool row_sums = one_column && !col_sums;

@@ -26,8 +26,14 @@ def test_taken(n, k, step):
     assert "row sums" in Plan(_weighted(n, k, step)).disassemble(-1)
 
 
+# fewer rows than SMs, too long for a block each: (30000 + 800 n) elements are the last
+@pytest.mark.parametrize("n,k,rows", [(40, 62000, True), (40, 62001, False), (147, 147600, True), (147, 147601, False), (148, 200000, True), (32, 1000000, False)])
+def test_long_rows_are_split(n, k, rows):
+    assert ("row sums" in Plan(_weighted(n, k, 1)).disassemble(-1)) == rows
+
+
 @pytest.mark.gpu
-@pytest.mark.parametrize("n,k,step", CASES + EDGES)
+@pytest.mark.parametrize("n,k,step", CASES + EDGES + [(40, 62000, 1), (40, 62001, 1)])
 def test_weighted_rows(n, k, step):
     from tests.gpu_util import check_against_oracle
     e = _weighted(n, k, step)
