@@ -170,7 +170,8 @@ tad_ew_kernel(const __grid_constant__ TadeProgram P, const __grid_constant__ Tad
 // Loads that do not change from row to row are read once per run, loads that do not move along the row once per row.  What bounds
 // it is the latency of the reads (the tables live in L1 and L2): every load of the rows in flight is issued before the first is
 // used, without a branch between them (sin x[2i + j, j - k] y^2 over 512^3 outputs 132 -> 104 us, 300^3 46 -> 31, a table read along
-// steps of three, 4096 x 4096 outputs, 37 -> 27 us).
+// steps of three, 4096 x 4096 outputs, 37 -> 27 us).  Where a thread has one piece only there is nothing to keep in flight, and the
+// registers for it cost warps (x y w over 10^6 outputs 7.8 us with them, 5.5 without; x y over 2 10^6 9.3, 7.8): builds of their own.
 // ---------------------------------------------------------------------------------------------------------
 enum ProdKind : int { PK_HOIST = 0, PK_BCAST, PK_FWD, PK_REV, PK_GEN };
 
@@ -251,14 +252,14 @@ __device__ __forceinline__ void prod_run(ProdRun &R, const int n_rows, const int
     for (; r < n_rows; ++r) prod_rows<VEC, W, MG, MB, 1>(R, live, held, powers, accumulate, out);
 }
 
-// SINGLE: one long row, its runs along it, a block's width from one piece to the next
-template <bool VEC, int MG, int MB, bool SINGLE>
-__global__ void __launch_bounds__(256, VEC && MG + MB <= 1 ? 6 : VEC && MG + MB == 2 ? 4 : !VEC && MG + MB == 3 ? 4 : 3)
+// SINGLE: one long row, its runs along it, a block's width from one piece to the next; ONE: runs of one piece
+template <bool VEC, int MG, int MB, bool SINGLE, bool ONE>
+__global__ void __launch_bounds__(256, ONE ? 6 - (MG + 1) / 2 : VEC && MG + MB <= 1 ? 6 : VEC && MG + MB == 2 ? 4 : !VEC && MG + MB == 3 ? 4 : 3)
 tad_prod_kernel(const __grid_constant__ TadeProgram P, const __grid_constant__ ProdPlan Q, const __grid_constant__ TadpPointers ptrs,
                 const unsigned n_items, const unsigned cols, const unsigned lane_blocks, const unsigned n_runs, const unsigned runs_per_line)
 {
     tad_wait_previous();
-    constexpr int M = MG + MB, U = VEC && MG + MB <= 2 ? 4 : !VEC && MG + MB == 3 ? 1 : 2;      // (as many as their registers allow)
+    constexpr int M = MG + MB, U = ONE ? 1 : VEC && MG + MB <= 2 ? 4 : !VEC && MG + MB == 3 ? 1 : 2;      // (as many as their registers allow)
     const unsigned tid = threadIdx.x;
     const unsigned rows_per_block = 256u / cols;
     const unsigned tc = tid % cols, tr = tid / cols;
@@ -328,8 +329,33 @@ tad_prod_kernel(const __grid_constant__ TadeProgram P, const __grid_constant__ P
 #pragma unroll
         for (int v = 0; v < TADP_MAX_VARS; ++v) R.out += P.out_coef[v] * var[v];
         R.ostep = P.out_coef[lane_var] * (int)es; R.oadv = SINGLE ? P.out_coef[lane_var] * (int)(4u * cols) : P.out_coef[row_var];
-        if (!VEC || live == 4) {
-            if constexpr (!VEC || MG == 0) prod_run<VEC, 1, MG, MB, U>(R, n_rows, live, held, powers, accumulate, out);
+        if constexpr (M == 0 && (ONE || !SINGLE)) {
+#pragma unroll 1
+            for (int r = 0; r < (ONE ? 1 : n_rows); ++r) {
+                if (VEC && live == 4) {
+                    float4 *dst = reinterpret_cast<float4 *>(out + (unsigned)R.out);
+                    float4 q = make_float4(held[0], held[1], held[2], held[3]);
+                    if (accumulate) { const float4 o = *dst; q.x += o.x; q.y += o.y; q.z += o.z; q.w += o.w; }
+                    *dst = q;
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) if (j < live) { const unsigned o = (unsigned)(R.out + j * R.ostep); out[o] = accumulate ? out[o] + held[j] : held[j]; }
+                }
+                R.out += R.oadv;
+            }
+            continue;
+        }
+        if (ONE && live == 4) {
+            if constexpr (ONE && M > 0) {                      // (one piece: no loop, no remainder behind it)
+                if (width == 4) prod_rows<VEC, 4, MG, MB, 1>(R, live, held, powers, accumulate, out);
+                else if (width == 2) prod_rows<VEC, 2, MG, MB, 1>(R, live, held, powers, accumulate, out);
+                else prod_rows<VEC, 1, MG, MB, 1>(R, live, held, powers, accumulate, out);
+            }
+            continue;
+        }
+        if (!ONE && (!VEC || live == 4)) {
+            if constexpr (ONE) {}
+            else if constexpr (!VEC || MG == 0) prod_run<VEC, 1, MG, MB, U>(R, n_rows, live, held, powers, accumulate, out);
             else if (width == 4) prod_run<VEC, 4, MG, MB, U>(R, n_rows, live, held, powers, accumulate, out);
             else if (width == 2) prod_run<VEC, 2, MG, MB, U>(R, n_rows, live, held, powers, accumulate, out);
             else prod_run<VEC, 1, MG, MB, U>(R, n_rows, live, held, powers, accumulate, out);
@@ -467,14 +493,22 @@ cudaError_t tad_launch_ew(const TadeProgram &P, const TadpPointers &ptrs, unsign
 #define TAD_PROD_ARGS g, 256, 0, stream, P, Q, ptrs, (unsigned)its, pc, lblocks, (unsigned)runs, (unsigned)per_line
 #define TAD_PROD_LAUNCH(G, B)                                                                                                           \
     case 4 * G + B:                                                                                                                     \
-        if (Q.row_var < 0) { if (Q.vec) tad_launch(tad_prod_kernel<true, G, B, true>, TAD_PROD_ARGS); else tad_launch(tad_prod_kernel<false, G, B, true>, TAD_PROD_ARGS); } \
-        else { if (Q.vec) tad_launch(tad_prod_kernel<true, G, B, false>, TAD_PROD_ARGS); else tad_launch(tad_prod_kernel<false, G, B, false>, TAD_PROD_ARGS); } \
+        if (Q.row_var < 0) { if (Q.vec) tad_launch(tad_prod_kernel<true, G, B, true, false>, TAD_PROD_ARGS); else tad_launch(tad_prod_kernel<false, G, B, true, false>, TAD_PROD_ARGS); } \
+        else { if (Q.vec) tad_launch(tad_prod_kernel<true, G, B, false, false>, TAD_PROD_ARGS); else tad_launch(tad_prod_kernel<false, G, B, false, false>, TAD_PROD_ARGS); } \
         break;
-        switch (4 * (Q.n_moving - Q.n_single) + Q.n_single) {
+#define TAD_PROD_LAUNCH_ONE(G) case G: tad_launch(tad_prod_kernel<true, G, 0, true, true>, TAD_PROD_ARGS); break;
+        if (Q.row_var < 0 && Q.run == 1) {
+            if (!Q.vec) tad_launch(tad_prod_kernel<false, 0, 0, true, true>, TAD_PROD_ARGS);      // (nothing moves then)
+            else switch (Q.n_moving) {
+            TAD_PROD_LAUNCH_ONE(0) TAD_PROD_LAUNCH_ONE(1) TAD_PROD_LAUNCH_ONE(2) TAD_PROD_LAUNCH_ONE(3)
+            default: return cudaErrorInvalidValue;
+            }
+        } else switch (4 * (Q.n_moving - Q.n_single) + Q.n_single) {
         TAD_PROD_LAUNCH(0, 0) TAD_PROD_LAUNCH(0, 1) TAD_PROD_LAUNCH(0, 2) TAD_PROD_LAUNCH(0, 3) TAD_PROD_LAUNCH(1, 0) TAD_PROD_LAUNCH(1, 1)
         TAD_PROD_LAUNCH(1, 2) TAD_PROD_LAUNCH(2, 0) TAD_PROD_LAUNCH(2, 1) TAD_PROD_LAUNCH(3, 0)
         default: return cudaErrorInvalidValue;
         }
+#undef TAD_PROD_LAUNCH_ONE
 #undef TAD_PROD_LAUNCH
 #undef TAD_PROD_ARGS
         return cudaGetLastError();

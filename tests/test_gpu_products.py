@@ -36,6 +36,16 @@ def _cube(n, m):
     return b.done()
 
 
+def _line(n, off, loads):
+    """f_i = x_i y_{n-1-i} w_{i+off}, the first `loads` of them: one row, a piece or several a thread"""
+    b = Builder("line", [n], 0, ["x", "y", "w"][:loads], [[n], [n], [n + off]][:loads])
+    r = b.load("x", [unit(1, (0, 1))])
+    if loads > 1:
+        r = b.bin("mul", r, b.load("y", [unit(1, (0, -1))], [n - 1]))
+    b.bin("mul", r, b.load("w", [unit(1, (0, 1))], [off])) if loads > 2 else b.bin("mul", r, b.const(2.0))
+    return b.done()
+
+
 CASES = {
     "flat_1": lambda: _flat(3, 1), "flat_7": lambda: _flat(1, 7), "flat_small": lambda: _flat(33, 31), "flat_odd": lambda: _flat(1301, 2477),
     "flat_run": lambda: _flat(2048, 2049), "flat_remainder": lambda: _flat(1025, 4099), "flat_aligned": lambda: _flat(1024, 4096),
@@ -67,6 +77,13 @@ def _check(e, shift=0):
 @pytest.mark.parametrize("name", sorted(CASES))
 def test_products(name):
     _check(CASES[name]())
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("loads", [1, 2, 3])
+@pytest.mark.parametrize("n,off", [(3, 1), (1024, 4), (1027, 2), (100001, 1), (600000, 4), (2424831, 2), (2424836, 4)])
+def test_one_row(n, off, loads):
+    _check(_line(n, off, loads))
 
 
 @pytest.mark.gpu
