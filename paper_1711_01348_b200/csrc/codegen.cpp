@@ -811,10 +811,14 @@ bool try_points(Gen &g, Kernel &k, int root, int scale, bool allow_split, const 
         double outs = 1;
         for (int v = 0; v < g.n_outer; ++v) outs *= (double)ext[v];
         // (two or three summands each, without sums of their own, while four lanes to an output are no more than the GPU's: the serial
-        // steps of a sum of three terms of four functions 18.2 -> 13.0 us for 18000 outputs, 18.9 -> 16.9 for 50000, 20.0 -> 21.9 for 75000)
+        // steps of a sum of three terms of four functions 18.2 -> 13.0 us for 18000 outputs, 18.9 -> 16.9 for 50000, 20.0 -> 21.9 for 75000.
+        // Three terms of next to nothing gain while they are one wave: a product 5.6 -> 5.3 us for 37800 outputs, 5.7 -> 7.3 for 38000; with
+        // a sinh 9.8 -> 9.3 for 38000, 9.9 -> 10.2 for 50000)
         const int64_t last = inner_sum < 0 ? 0 : g.inst[inner_sum].hi - g.inst[inner_sum].lo;
-        const auto n_sums = std::count_if(g.inst.begin(), g.inst.end(), [](const Inst &in) { return in.uses && in.op == I_SUM; });
-        if (n_outer_sums != 1 || outs > POINT_CHAIN || last < 1 || (last < 3 && (n_sums > 1 || outs > POINT_CHAIN * 2 / 3))) inner_sum = -1;
+        int n_sums = 0, n_fns = 0;
+        for (const Inst &in : g.inst) if (in.uses) { n_sums += in.op == I_SUM; n_fns += inner_sum >= 0 && (in.deps >> g.inst[inner_sum].var & 1u) && in.op >= I_EXP && in.op <= I_COSH; }
+        const double most = last >= 3 ? POINT_CHAIN : last == 1 || n_fns >= 1 ? POINT_CHAIN * 2 / 3 : POINT_CHAIN / 2;
+        if (n_outer_sums != 1 || last < 1 || outs > most || (last < 3 && n_sums > 1)) inner_sum = -1;
     }
     if (inner_sum >= 0) {
         on_sum[inner_sum] = 1;

@@ -26,6 +26,30 @@ def test_taken(n, nk):
     assert ("%d outputs x %d terms" % (n, nk if spread else 1)) in text
 
 
+def _cheap(n, nk):
+    """f_i = exp(sum_k u_ik v_k): summands without functions"""
+    b = Builder("cheap", [n], 1, ["u", "v"], [[n, nk], [nk]])
+    b.un("exp", b.sum(1, 0, nk - 1, b.bin("mul", b.load("u", [unit(2, (0, 1)), unit(2, (1, 1))]), b.load("v", [unit(2, (1, 1))]))))
+    return b.done()
+
+
+# three terms without functions are spread up to 37888 outputs, two up to 50517, four and more up to 75776
+CHEAP = [(37888, 3, True), (37889, 3, False), (50517, 2, True), (50518, 2, False), (75776, 4, True)]
+
+
+@pytest.mark.parametrize("n,nk,spread", CHEAP)
+def test_cheap_taken(n, nk, spread):
+    assert ("%d outputs x %d terms" % (n, nk if spread else 1)) in Plan(_cheap(n, nk)).disassemble(-1)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,nk,spread", CHEAP)
+def test_cheap_sums(n, nk, spread):
+    from tests.gpu_util import check_against_oracle
+    e = _cheap(n, nk)
+    check_against_oracle(e, *W.make_inputs(e, ("uniform", -0.9, 0.9), seed=n), nthreads=max_threads())
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("n,nk", SIZES)
 def test_short_sums(n, nk):
