@@ -14,10 +14,46 @@ namespace {
 constexpr double TILE_COPY = 9, TILE_START = 300, TILE_FIXED = 3500;      // issue slots (schedule)
 constexpr int64_t TILE_MIN_SUM = 4;           // fewer terms than this: nothing to share between the values of a tile
 
+// How often a term is written out as a tree, and whether a sum lies at or below an instance
+struct Trees {
+    std::vector<char> sum_in;
+    std::vector<double> nodes;                // (an expression may share a lot)
+    void grow(const Gen &g)
+    {
+        for (int i = (int)nodes.size(); i < (int)g.inst.size(); ++i) {
+            const Inst &in = g.inst[i];
+            sum_in.push_back(in.op == I_SUM || (in.a >= 0 && sum_in[in.a]) || (in.b >= 0 && sum_in[in.b]));
+            nodes.push_back(1 + (in.a >= 0 ? nodes[in.a] : 0) + (in.b >= 0 ? nodes[in.b] : 0));
+        }
+    }
+};
+
+struct Choice { int p, q, l; bool q_sum; double worth; };
+
+// What a kernel sums and over which variables, read off its instances without a change to them
+struct Analysis {
+    const Gen &g;
+    const TadpProgram &prog;
+    std::vector<int64_t> lo, ext;
+    Trees trees;
+    int leaf = -1, term = -1;
+    std::vector<int> outer, factors;
+    float cfac = 1.f;
+    std::vector<Choice> choices;
+
+    Analysis(const Gen &gen, const Kernel &kern) : g(gen), prog(kern.prog), lo(TADP_MAX_VARS, 0), ext(TADP_MAX_VARS, 1) {}
+    bool run(int root, int scale, const std::vector<std::vector<TadpRow>> &lower, const std::vector<std::vector<TadpRow>> &upper);
+    int least_steps(const Choice &c) const;
+};
+
 struct Tiler {
     Gen g;                                    // (a copy: combined factors become instances of it)
     const TadpProgram &prog;
-    std::vector<int64_t> lo, ext;
+    const std::vector<int64_t> &lo, &ext;
+    const std::vector<int> &outer, &factors;
+    const int leaf;
+    const float cfac;
+    Trees trees;
     int p = -1, q = -1, l = -1;
     bool q_sum = false;
     std::vector<int> z;
@@ -27,7 +63,7 @@ struct Tiler {
     int n_loads = 0, n_code = 0, n_imm = 0;
     std::vector<int> op_inst;
 
-    Tiler(const Gen &gen, const Kernel &kern) : g(gen), prog(kern.prog), lo(TADP_MAX_VARS, 0), ext(TADP_MAX_VARS, 1) {}
+    Tiler(const Analysis &a) : g(a.g), prog(a.prog), lo(a.lo), ext(a.ext), outer(a.outer), factors(a.factors), leaf(a.leaf), cfac(a.cfac), trees(a.trees) {}
 
     // which of p, q, l an instance varies with
     int cls(int i) const
@@ -35,17 +71,6 @@ struct Tiler {
         const uint32_t d = g.inst[i].deps;
         auto bit = [&](int v) { return v >= 0 && ((d >> v) & 1u) && ext[v] > 1; };
         return (bit(p) ? 1 : 0) | (bit(q) ? 2 : 0) | (bit(l) ? 4 : 0);
-    }
-    // per instance: a sum at or below it; nodes of it written out as a tree (an expression may share a lot)
-    std::vector<char> sum_in;
-    std::vector<double> tree;
-    void grow()
-    {
-        for (int i = (int)tree.size(); i < (int)g.inst.size(); ++i) {
-            const Inst &in = g.inst[i];
-            sum_in.push_back(in.op == I_SUM || (in.a >= 0 && sum_in[in.a]) || (in.b >= 0 && sum_in[in.b]));
-            tree.push_back(1 + (in.a >= 0 ? tree[in.a] : 0) + (in.b >= 0 ? tree[in.b] : 0));
-        }
     }
     bool add_load(int id)
     {
@@ -81,8 +106,8 @@ struct Tiler {
     bool program(int i, int sum, int32_t &at, int32_t &n)
     {
         std::vector<TadeStep> st;
-        grow();
-        if (tree[i] > 4 * TADT_STEPS || !elementwise_steps_of(g, i, st, sum)) return false;
+        trees.grow(g);
+        if (trees.nodes[i] > 4 * TADT_STEPS || !elementwise_steps_of(g, i, st, sum)) return false;
         at = (int32_t)steps.size();
         for (TadeStep &s : st) {
             if (s.op == E_LD && s.a >= 0) { if (!add_load(s.a)) return false; s.a = (int16_t)load_at[s.a]; }
@@ -99,7 +124,7 @@ struct Tiler {
         if (c == 2 && q_sum) return TK_COL;                   // (another one for every tile)
         return c == 4 || c == 5 ? TK_ROW : c == 6 ? TK_COL : c == 2 ? TK_COLC : c == 3 ? TK_MAT : TK_ROWC;
     }
-    bool is_operand(int i) const { return cls(i) != 7 && !sum_in[i]; }
+    bool is_operand(int i) const { return cls(i) != 7 && !trees.sum_in[i]; }
     // c times powers of loads
     bool monomial(int i, int e, double &c, std::vector<std::pair<int, int>> &powers) const
     {
@@ -128,7 +153,7 @@ struct Tiler {
         O.load1 = -1; O.e = 1; O.c = 1.f;
         std::vector<std::pair<int, int>> powers;                 // (load, exponent)
         double cf = 1;
-        if (O.kind != TK_MAT && tree[i] < 16 && monomial(i, 1, cf, powers) && (powers.size() == 1 || (powers.size() == 2 && powers[1].second == 1))) {
+        if (O.kind != TK_MAT && trees.nodes[i] < 16 && monomial(i, 1, cf, powers) && (powers.size() == 1 || (powers.size() == 2 && powers[1].second == 1))) {
             for (auto &pw : powers) if (!add_load(pw.first)) return -1;
             O.load0 = (int16_t)load_at[powers[0].first]; O.e = (int16_t)powers[0].second; O.c = (float)cf;
             if (powers.size() == 2) O.load1 = (int16_t)load_at[powers[1].first];
@@ -223,7 +248,7 @@ struct Tiler {
                 // a - b as a + (-b), -b staged: the same sum, and the cores that are built cover differences too
                 if (std::find(op_inst.begin(), op_inst.end(), in.b) != op_inst.end()) return emit(in.a) && code(T_SUB, operand(in.b));
                 const int minus = g.neg(in.b);
-                grow();
+                trees.grow(g);
                 if (is_operand(in.a) && before(minus, in.a) && !before(in.a, minus)) return code(T_LD, operand(minus)) && code(T_ADD, operand(in.a));
                 return emit(in.a) && code(T_ADD, operand(minus));
             }
@@ -235,20 +260,14 @@ struct Tiler {
         }
     }
 
-    struct Choice { int p, q, l; bool q_sum; double worth; };
-    int leaf = -1, term = -1;
-    std::vector<int> outer, factors;
-    float cfac = 1.f;
-    std::vector<Choice> choices;
-    bool analyse(int root, int scale, const std::vector<std::vector<TadpRow>> &lower, const std::vector<std::vector<TadpRow>> &upper);
     bool build(int root, int scale, const Choice &c);
     void schedule();
 };
 
 // the sum, its factors, and which variables can be p, q and l, the most promising choice first
-bool Tiler::analyse(int root, int scale, const std::vector<std::vector<TadpRow>> &lower, const std::vector<std::vector<TadpRow>> &upper)
+bool Analysis::run(int root, int scale, const std::vector<std::vector<TadpRow>> &lower, const std::vector<std::vector<TadpRow>> &upper)
 {
-    grow();
+    trees.grow(g);
     for (int v = 0; v < g.n_outer; ++v) { lo[v] = prog.outer_lo[v]; ext[v] = prog.outer_ext[v]; if (ext[v] < 1) return false; }
     std::vector<int> sums;
     for (int c = 0; c < g.kappa; ++c) {
@@ -266,7 +285,7 @@ bool Tiler::analyse(int root, int scale, const std::vector<std::vector<TadpRow>>
     // ---- the sum: the loops around the term, or the one sum inside an element-wise expression ----
     term = root;
     if (g.kappa == 0) {
-        if (scale >= 0 || tree[root] > 1000) return false;
+        if (scale >= 0 || trees.nodes[root] > 1000) return false;
         bool several = false;
         std::function<void(int)> outermost = [&](int i) {
             const Inst &in = g.inst[i];
@@ -284,7 +303,7 @@ bool Tiler::analyse(int root, int scale, const std::vector<std::vector<TadpRow>>
         sums.push_back(in.var);
         term = in.a;
     }
-    if (sum_in[term] || tree[term] > 1000) return false;
+    if (trees.sum_in[term] || trees.nodes[term] > 1000) return false;
     for (int v = 0; v < g.n_outer; ++v) if (ext[v] > 1) outer.push_back(v);
     sums.erase(std::remove_if(sums.begin(), sums.end(), [&](int v) { return ext[v] == 1; }), sums.end());
     for (int v : sums) if (!(g.inst[term].deps & (1u << v))) return false;
@@ -302,7 +321,7 @@ bool Tiler::analyse(int root, int scale, const std::vector<std::vector<TadpRow>>
     }
     auto out_step = [&](int v) { return prog.out_coef[v] ? std::abs((int64_t)prog.out_coef[v]) : INT64_MAX; };
     auto couples = [&](int a, int b, int c) { for (int f : factors) { const uint32_t d = g.inst[f].deps; if ((d >> a & 1u) && (d >> b & 1u) && (d >> c & 1u)) return true; } return false; };
-    if (sums.size() == 1) {
+    if (sums.size() == 1 && ext[sums[0]] >= TILE_MIN_SUM && (int)outer.size() <= 2 + TADT_Z) {
         // two output variables, the larger ones first; the output is written along q
         for (size_t i = 0; i < outer.size(); ++i)
             for (size_t j = i + 1; j < outer.size(); ++j) {
@@ -310,11 +329,11 @@ bool Tiler::analyse(int root, int scale, const std::vector<std::vector<TadpRow>>
                 const bool flip = out_step(a) < out_step(b);
                 if (couples(a, b, sums[0])) choices.push_back({flip ? b : a, flip ? a : b, sums[0], false, (double)ext[a] * (double)ext[b]});
             }
-    } else if (sums.size() == 2) {
+    } else if (sums.size() == 2 && (int)outer.size() <= 1 + TADT_Z) {
         // one output variable; l is the sum that leaves most of the factors outside (the largest tensor is then read once)
         for (int i = 0; i < 2; ++i)
             for (int a : outer) {
-                if (!couples(a, sums[0], sums[1])) continue;
+                if (ext[sums[i]] < TILE_MIN_SUM || !couples(a, sums[0], sums[1])) continue;
                 double outside = 0;
                 for (int f : factors) {
                     const uint32_t d = g.inst[f].deps;
@@ -326,15 +345,37 @@ bool Tiler::analyse(int root, int scale, const std::vector<std::vector<TadpRow>>
                 choices.push_back({a, sums[1 - i], sums[i], true, outside * 1e9 + (double)ext[a]});
             }
     }
+    choices.erase(std::remove_if(choices.begin(), choices.end(), [&](const Choice &c) { return least_steps(c) > 8; }), choices.end());
     std::stable_sort(choices.begin(), choices.end(), [](const Choice &a, const Choice &b) { return a.worth > b.worth; });
     return !choices.empty();
+}
+
+// Steps that the core takes at least: one for what couples the three variables, but for a sum behind a product; the first load, the sum
+int Analysis::least_steps(const Choice &c) const
+{
+    const uint32_t all = 1u << c.p | 1u << c.q | 1u << c.l;
+    auto coupled = [&](int i) { return (g.inst[i].deps & all) == all; };
+    std::function<int(int)> steps = [&](int i) -> int {
+        if (!coupled(i)) return 0;
+        const Inst &in = g.inst[i];
+        if (in.a < 0 || (in.op == I_POWI && in.ipow != 3)) return 99;
+        if (in.b < 0) return 1 + steps(in.a);
+        int own = in.op == I_DIV ? 2 : 1;
+        if (in.op == I_ADD && coupled(in.a) != coupled(in.b)) {
+            const Inst &m = g.inst[coupled(in.a) ? in.a : in.b];
+            if (m.op == I_MUL && coupled(m.a) != coupled(m.b)) own = 0;
+        }
+        return own + steps(in.a) + steps(in.b);
+    };
+    int n = 2;
+    for (int f : factors) n += steps(f);
+    return n;
 }
 
 bool Tiler::build(int root, int scale, const Choice &choice)
 {
     p = choice.p; q = choice.q; l = choice.l; q_sum = choice.q_sum;
     for (int v : outer) if (v != p && v != q) z.push_back(v);
-    if (z.size() > TADT_Z || ext[l] < TILE_MIN_SUM) return false;
     // ---- factors: outside the sum over l (q summed), rows, columns, the core ----
     std::vector<int> post, rows, cols, core;
     bool coupled = false;
@@ -353,7 +394,7 @@ bool Tiler::build(int root, int scale, const Choice &choice)
     int last = !rows.empty() ? product(rows) : !cols.empty() ? product(cols) : -1;
     const bool outside = q_sum && !post.empty();              // a constant factor goes where it costs nothing
     if (last >= 0 && !outside) last = g.mulc(last, cfac);
-    grow();
+    trees.grow(g);
     if (is_operand(body) || need(body) > 2 || !emit(body)) return false;
     if (cfac != 1.f && !outside && last < 0 && !imm_step(T_MULC, cfac)) return false;
     if (last >= 0 ? !code(T_ACC, operand(last), 1) : !code(T_ACC)) return false;
@@ -485,10 +526,10 @@ bool try_tile(Gen &g, Kernel &k, int root, int scale, const std::vector<std::vec
     }
     for (const Inst &in : g.inst) if (in.uses && in.op == I_SUM) points *= (double)std::max<int64_t>(1, in.hi - in.lo + 1);
     if (points < min_space || points > max_space) return false;
-    Tiler all(g, k);
-    if (!all.analyse(root, scale, lower, upper)) return false;
+    Analysis all(g, k);
+    if (!all.run(root, scale, lower, upper)) return false;
     std::unique_ptr<Tiler> found;
-    for (const Tiler::Choice &c : all.choices) {
+    for (const Choice &c : all.choices) {
         found.reset(new Tiler(all));
         if (found->build(root, scale, c)) break;
         found.reset();
