@@ -775,6 +775,25 @@ int assign_temporaries(Gen &g, int root, int scale)
 // Plain element-wise programs (no sums, no temporaries) have the element-wise kernel, which is as fast from 2^16 outputs on.
 constexpr double POINT_SPACE = double(1 << 22), POINT_PLAIN = double(1 << 16), POINT_CHAIN = 148.0 * 512, POINT_AHEAD = double(1 << 17);
 
+}  // namespace
+
+// The schedule of try_points below, and a fit to 320 kernels (of the estimate / measured 90 % lie between 0.55 and 1.24): what a launch takes,
+// the dependent steps of a thread, the steps of all threads on the SMs, and the sum of the shares' planes where there are some.
+double point_time(double points, double terms, double steps, bool chain, bool loops, bool along)
+{
+    if (points * terms > POINT_SPACE || (chain && points > POINT_CHAIN)) return 1e9;
+    const double unroll = terms >= 4 && !chain ? 4 : 1;
+    double lanes = 1;
+    if (along && (terms >= 32 || points < 148.0 * 512.0)) while (lanes < 32 && lanes < terms) lanes *= 2;
+    while (lanes < 256 && points * lanes < 148.0 * 512.0 && lanes * unroll < terms) lanes *= 2;
+    const double blocks = std::ceil(points * lanes / 256), rounds = terms / (lanes * unroll);
+    const double shares = loops && blocks < 148 && rounds >= 8 ? std::max(1.0, std::min({128.0, std::floor(740 / blocks), std::floor(rounds / 1.5)})) : 1;
+    const double turns = std::ceil(rounds / shares);
+    return 3.7 + (shares > 1 ? 4 : 0) + 0.045 * steps + turns * (0.053 * steps + 0.23 * unroll) + 0.023 / 148 * blocks * shares * turns * steps * unroll;
+}
+
+namespace {
+
 bool try_points(Gen &g, Kernel &k, int root, int scale, bool allow_split, const std::vector<std::vector<TadpRow>> &lower,
                 const std::vector<std::vector<TadpRow>> &upper, const std::vector<TadpRow> &guards, double limit = POINT_SPACE)
 {
@@ -1020,10 +1039,12 @@ bool try_points(Gen &g, Kernel &k, int root, int scale, bool allow_split, const 
     return true;
 }
 
-// Sums whose term couples two variables run as tile programs from 2^16 points on, where they are faster than point programs (a step of
-// the intro expression, us: 64 x 64 x 5 27 -> 34, 66 x 85 x 19 42 -> 37, 203 x 157 x 7 48 -> 37, 90 x 400 x 10 65 -> 39,
-// 3978 x 73 x 20 563 -> 79), up to 5e7, where the sums pushed inside and contracted are (2564 x 2507 x 5 462 -> 184, 7263 x 352 x 21
-// 194 -> 188, 1868 x 2663 x 11 165 -> 177, 1655 x 2679 x 23 163 -> 215).
+// Sums whose term couples two variables run as tile programs from 2^16 points on, unless a point program is estimated to be faster (try_tile;
+// a step of the intro expression, us: 64 x 64 x 5 27 -> 34, 66 x 85 x 19 42 -> 37, 203 x 157 x 7 48 -> 37, 90 x 400 x 10 65 -> 39, 3978 x 73 x
+// 20 563 -> 79), up to 5e7, where the sums pushed inside and contracted are (2564 x 2507 x 5 462 -> 184, 7263 x 352 x 21 194 -> 188,
+// 1868 x 2663 x 11 165 -> 177, 1655 x 2679 x 23 163 -> 215); beyond, only what is not pushed inside.  Above 2^24 a core that is read step by
+// step costs more than the parts (gradients of (x - y)^3, us: 2000 x 2000 x 10 66 -> 180, 340 x 340 x 340 63 -> 161, forward 560 -> 79) and
+// keeps the digits that they lose (Analysis::apart).
 constexpr double TILE_LEAST = double(1 << 16), TILE_MOST = 5e7;
 
 // shared tail: choose temps, emit, fill the program
@@ -1070,11 +1091,18 @@ void emit_kernel(Gen &g, Kernel &k, int root, const std::vector<std::vector<Tadp
     // a product of two index expressions under summations runs on the tile kernel, not in the interpreter
     if (try_contraction(g, k, root, scale, allow_split, lower, upper, guards)) return;
     // sums of a term that couples two variables, as written, by tiles of both
-    if (try_tile(g, k, root, scale, lower, upper, guards, TILE_LEAST, TILE_MOST)) return;
+    TileElse other = TILE_NO_OTHER;
+    if (try_tile(g, k, root, scale, lower, upper, guards, TILE_LEAST, TILE_MOST, may_factor, other)) return;
+    if (other == TILE_POINTS) {
+        try {
+            if (try_points(g, k, root, scale, allow_split, lower, upper, guards)) return;
+        } catch (const Unsupported &) {                       // too deep or too many temporaries for it
+        }
+    }
     // sums that can be pushed inside the term (Sec. 6's missing clean-up step): auxiliary kernels + a smaller kernel
     if (may_factor && try_factoring(g, k, root, scale, allow_split, lower, upper, guards)) return;
-    // (sums too short to gain from that)
-    if (try_tile(g, k, root, scale, lower, upper, guards, TILE_MOST, 1e18)) return;
+    // (sums that do not gain from that)
+    if (try_tile(g, k, root, scale, lower, upper, guards, other == TILE_APART ? TILE_LEAST : TILE_MOST, 1e18, false, other)) return;
     // short sums ahead of a kernel: as point programs they share a launch with the others
     if (!may_factor && g.kappa == 0 && g.inst[root].op == I_SUM) {
         try {

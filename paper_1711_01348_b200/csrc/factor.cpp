@@ -23,8 +23,8 @@ namespace tad {
 
 namespace {
 
-// Index spaces up to this size are summed by one kernel of their own, as written (what couples two variables never gets here up to
-// 5e7 points: tile programs take it).  Smaller ones were faster as contractions than on the interpreter
+// Index spaces up to this size are summed by one kernel of their own, as written (of what couples two variables, only sums of products
+// get here up to 5e7 points: tile programs take the rest).  Smaller ones were faster as contractions than on the interpreter
 // (the intro expression with a line at 2^24 / 2^22, forward and all gradients in us: 1000 x 1500 x 6 56 + 475 / 22 + 158,
 // 1000 x 1000 x 16 116 + 595 / 19 + 148), but a sum of squares (a + b)^2 with a near -b loses digits when it is expanded
 // (a about 10, b about -10: 1.6 times the tolerance of 1e-4; about 30: 12 times), so the line stays where the size demands it.

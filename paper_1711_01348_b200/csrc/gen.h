@@ -351,9 +351,14 @@ bool emit_program(const System &s, float scale, int accumulate, bool allow_split
 bool try_contraction(Gen &g, Kernel &k, int root, int scale, bool allow_split, const std::vector<std::vector<TadpRow>> &lower,
                      const std::vector<std::vector<TadpRow>> &upper, const std::vector<TadpRow> &guards);
 
-// tile_gen.cpp: a sum whose term couples two variables becomes a tile program, if its number of points lies in the given range
+// tile_gen.cpp: a sum whose term couples two variables becomes a tile program, if its number of points lies in the given range.
+// declined: ... and what else is faster: a point program, or (may_factor) the summation pushed inside with nothing to multiply out
+enum TileElse { TILE_NO_OTHER = 0, TILE_POINTS, TILE_APART };
 bool try_tile(Gen &g, Kernel &k, int root, int scale, const std::vector<std::vector<TadpRow>> &lower, const std::vector<std::vector<TadpRow>> &upper,
-              const std::vector<TadpRow> &guards, double min_space, double max_space);
+              const std::vector<TadpRow> &guards, double min_space, double max_space, bool may_factor, TileElse &other);
+// codegen.cpp: estimated microseconds of a point program of so many outputs, terms each and steps a term (chain: what is computed from
+// the sum follows it in the same thread; loops: the sum may be shared out; along: lanes lie along the terms)
+double point_time(double points, double terms, double steps, bool chain, bool loops, bool along);
 // codegen.cpp: values that an accumulator program over X and Y holds at once while it evaluates instance i.  Instances for which in_place
 // holds are read in one step, also as the second operand of a sum, a product and (subtracts) a difference; every other binary operation
 // puts its first operand into Y, which the second must then leave alone (hold one value).

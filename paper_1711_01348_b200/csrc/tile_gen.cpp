@@ -12,6 +12,9 @@ namespace tad {
 namespace {
 
 constexpr double TILE_COPY = 9, TILE_START = 300, TILE_FIXED = 3500;      // issue slots (schedule)
+// Sums of products are pushed inside from here on (us, tile / contractions: sum_k x_ik y_jk + u_ik v_jk, 340 x 340 x 340 128 / 25, 1000 x 1000 x 40
+// 105 / 18; below, 300 x 200 x 9 and 64 x 64 x 64, a tile 8.3 and 7.3, a point program 38 and 7.4)
+constexpr double TILE_APART_LEAST = double(1 << 22);
 constexpr int64_t TILE_MIN_SUM = 4;           // fewer terms than this: nothing to share between the values of a tile
 
 // How often a term is written out as a tree, and whether a sum lies at or below an instance
@@ -44,6 +47,7 @@ struct Analysis {
     Analysis(const Gen &gen, const Kernel &kern) : g(gen), prog(kern.prog), lo(TADP_MAX_VARS, 0), ext(TADP_MAX_VARS, 1) {}
     bool run(int root, int scale, const std::vector<std::vector<TadpRow>> &lower, const std::vector<std::vector<TadpRow>> &upper);
     int least_steps(const Choice &c) const;
+    bool apart() const;
 };
 
 struct Tiler {
@@ -262,6 +266,7 @@ struct Tiler {
 
     bool build(int root, int scale, const Choice &c);
     void schedule();
+    double slots = 0;                         // estimate of schedule()
 };
 
 // the sum, its factors, and which variables can be p, q and l, the most promising choice first
@@ -372,6 +377,30 @@ int Analysis::least_steps(const Choice &c) const
     return n;
 }
 
+// A sum of rounded values (products of loads, functions) and at most one exact one (a load, a constant): nothing would be multiplied out
+// to push the summation inside, and each part's sum carries the rounding errors that the term has.  Exact values that nearly cancel
+// leave none in the term but all of theirs in the parts (a + 10 and b - 10, 300 x 300 x 300, error against 64 bits: (a + b)^2 as written 4e-8, in
+// parts 5e-5; the gradients of (a - b)^3 1e-7 and 7e-5).
+bool Analysis::apart() const
+{
+    std::function<bool(int)> product = [&](int i) -> bool {
+        const Inst &in = g.inst[i];
+        if (in.op == I_MUL) return product(in.a) && product(in.b);
+        if (in.op == I_MULC || in.op == I_NEG || in.op == I_SQR || in.op == I_POWI) return product(in.a);
+        return in.op != I_ADD && in.op != I_SUB && in.op != I_ADDC && in.op != I_SUM;
+    };
+    int exact = 0;
+    std::function<bool(int)> sum = [&](int i) -> bool {
+        const Inst &in = g.inst[i];
+        if (in.op == I_ADD || in.op == I_SUB) return sum(in.a) && sum(in.b);
+        if (in.op == I_ADDC) ++exact;
+        if (in.op == I_ADDC || in.op == I_MULC || in.op == I_NEG) return sum(in.a);
+        exact += in.op == I_LOAD || in.op == I_CONST;
+        return product(i);
+    };
+    return sum(term) && exact <= 1;
+}
+
 bool Tiler::build(int root, int scale, const Choice &choice)
 {
     p = choice.p; q = choice.q; l = choice.l; q_sum = choice.q_sum;
@@ -451,7 +480,7 @@ bool Tiler::build(int root, int scale, const Choice &choice)
 }
 
 // Tile, groups and shares with the least estimated time.  A thread's values cost their multiply-adds (about thirty issue slots
-// a step where the core is read step by step), the staging about eight issue slots an element of every operand, both shared by
+// a step where the core is read step by step), the staging about nine issue slots an element of every operand, both shared by
 // the blocks that are resident; a block by itself is bound by its start, its copies and the sums of groups and shares.
 void Tiler::schedule()
 {
@@ -504,17 +533,20 @@ void Tiler::schedule()
             }
         }
     T = pick;
+    slots = best;
 }
 
 }  // namespace
 
 bool try_tile(Gen &g, Kernel &k, int root, int scale, const std::vector<std::vector<TadpRow>> &lower, const std::vector<std::vector<TadpRow>> &upper,
-              const std::vector<TadpRow> &guards, double min_space, double max_space)
+              const std::vector<TadpRow> &guards, double min_space, double max_space, bool may_factor, TileElse &other)
 {
+    other = TILE_NO_OTHER;
     if (g.p.opt.debug_bounds || root < 0 || !guards.empty()) return false;
     // the number of points, ahead of any work: the outputs, loops with fixed ranges, one sum inside the term
-    double points = 1;
-    for (int v = 0; v < g.n_outer; ++v) points *= (double)std::max(1, k.prog.outer_ext[v]);
+    double points = 1, outs = 1;
+    for (int v = 0; v < g.n_outer; ++v) outs *= (double)std::max(1, k.prog.outer_ext[v]);
+    points = outs;
     for (int c = 0; c < g.kappa; ++c) {
         int64_t a = INT64_MIN, b = INT64_MAX;
         for (const TadpRow &r : lower[c]) a = std::max(a, ceil_div(r.c0, r.den));
@@ -528,6 +560,7 @@ bool try_tile(Gen &g, Kernel &k, int root, int scale, const std::vector<std::vec
     if (points < min_space || points > max_space) return false;
     Analysis all(g, k);
     if (!all.run(root, scale, lower, upper)) return false;
+    if (may_factor && points > TILE_APART_LEAST && all.apart()) { other = TILE_APART; return false; }
     std::unique_ptr<Tiler> found;
     for (const Choice &c : all.choices) {
         found.reset(new Tiler(all));
@@ -536,6 +569,22 @@ bool try_tile(Gen &g, Kernel &k, int root, int scale, const std::vector<std::vec
     }
     if (!found) return false;
     const Tiler &t = *found;
+    // Taken where it is estimated to be faster than what else would run it.  Microseconds of a tile program, fitted to 840 kernels of 2 to
+    // 5000 rows, columns and terms (of the estimate / measured 90 % lie between 0.63 and 1.36); of a point program, see point_time.  A
+    // built core is given twice that, the others 15 % more: gradients that are tile programs share a launch.
+    // (us, tile / point: 2000 batches of 4 x 4 sums of 8 squares 31 / 9.5, of tanh 42 / 10; tanh, 64 x 64 x 17 7.1 / 6.3 and its gradients 14 / 7.3;
+    // tanh, 64 x 1000 x 17 10 / 65.)  Beyond 2^21 outputs the interpreter is at its best, 0.001 ns a point and step, and a tile of which short
+    // sums or few rows leave little is not (5 x 3655 x 4 in 149 batches, a sum: 80 / 32).
+    const double us = t.T.path ? 1.1 + t.slots / 1275 : std::max(1.0, 0.29 * t.n_code - 4 + t.slots / 700);
+    const double steps = 2 + all.trees.nodes[all.term] + (scale >= 0 ? all.trees.nodes[scale] : 0);
+    const bool chain = g.kappa == 0 && g.inst[root].op != I_SUM;
+    const TadpLoad *big = nullptr;
+    for (const TadpLoad &L : g.loads) if (!big || L.limit > big->limit) big = &L;
+    bool along = false, across = false;
+    for (int v = 0; v < (int)g.vars.size(); ++v) if (std::abs(big->coef[v]) == 1 && all.ext[v] > 1) (v < g.n_outer ? across : along) = true;
+    const bool serial = chain && t.T.q_sum && g.inst[all.leaf].hi - g.inst[all.leaf].lo < 3;      // (a short sum of sums stays in its thread)
+    if (!serial && us > (t.T.path ? 2.0 : 1.15) * point_time(outs, points / outs, steps, chain, g.kappa >= 1, along && !across)) { other = TILE_POINTS; return false; }
+    if (outs >= double(1 << 21) && us > 4 + 1.2e-6 * t.n_code * points) return false;
     k.tile = {t.T};
     k.prog.zsplit = 1;
     k.vec = 0; k.vec_u = 0;
