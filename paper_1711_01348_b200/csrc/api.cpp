@@ -140,12 +140,13 @@ size_t tad_plan_disassemble(const tad_plan *plan, int32_t which, char *buf, size
     if (!plan) return 0;
     const Kernel *k = pick_kernel(plan, which);
     if (!k) return 0;
+    const std::string text = k->tile.empty() ? k->listing : k->listing + tile_listing(k->tile[0]);
     if (buf && cap) {
-        size_t n = std::min(cap - 1, k->listing.size());
-        std::memcpy(buf, k->listing.data(), n);
+        size_t n = std::min(cap - 1, text.size());
+        std::memcpy(buf, text.data(), n);
         buf[n] = 0;
     }
-    return k->listing.size() + 1;
+    return text.size() + 1;
 }
 
 size_t tad_plan_print(const tad_plan *plan, int32_t which, const char *const *arg_names, const char *const *idx_names,

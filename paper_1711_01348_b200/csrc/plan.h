@@ -148,4 +148,6 @@ void share_auxiliaries(tad_plan &p);
 // print.cpp: the expression (which = -1) or the derivative through index expression `which` in the notation of Sec. 6
 std::string print_expression(const tad_plan &p, int which, const char *const *arg_names, const char *const *idx_names);
 
+std::string tile_listing(const TadtProgram &T);      // tile_gen.cpp: loads, operands, steps, core and output of a tile program
+
 }  // namespace tad

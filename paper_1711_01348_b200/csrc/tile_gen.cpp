@@ -538,6 +538,32 @@ void Tiler::schedule()
 
 }  // namespace
 
+std::string tile_listing(const TadtProgram &T)
+{
+    static const char *const core[] = {"END", "LD", "ADD", "SUB", "RSUB", "MUL", "FMA", "SQR", "CUBE", "NEG", "MULC", "ADDC", "PUSH", "BINY", "FN", "ACC"};
+    static const char *const steps[] = {"END", "LD", "PUSH", "CONST", "NEG", "SQR", "CUBE", "MULC", "ADDC", "ADDY", "SUBY", "MULY", "DIVY", "FN"};
+    static const char *const kinds[] = {"ROW", "COL", "ROWC", "COLC", "MAT"};
+    std::string text;
+    char line[160];
+    auto add = [&](auto... v) { std::snprintf(line, sizeof line, v...); text += line; };
+    for (int i = 0; i < T.n_loads; ++i)
+        add(";   load %d ptr=%d base=%d p=%d q=%d l=%d z=%d,%d\n", i, T.loads[i].ptr, T.loads[i].base, T.loads[i].cp, T.loads[i].cq, T.loads[i].cl, T.loads[i].cz[0], T.loads[i].cz[1]);
+    for (int i = 0; i < T.n_ops; ++i) {
+        const TadtOperand &o = T.op[i];
+        if (o.n_steps) add(";   operand %d %s steps=%d+%d\n", i, kinds[o.kind], o.step0, o.n_steps);
+        else add(";   operand %d %s %.9g load %d ^ %d load %d\n", i, kinds[o.kind], o.c, o.load0, o.e, o.load1);
+    }
+    for (uint64_t c = T.core; c; c >>= 8) {
+        const int op = (int)c & 15, o = (int)(c >> 4) & 3;
+        add(";   core %s %d %d %.9g\n", core[op], o, (int)(c >> 6) & 3, op == T_MULC || op == T_ADDC ? T.imm[o] : 0.f);
+    }
+    const int last = std::max({T.epi0 + T.n_epi, T.post0 + T.n_post, [&] { int n = 0; for (int i = 0; i < T.n_ops; ++i) n = std::max(n, T.op[i].step0 + T.op[i].n_steps); return n; }()});
+    for (int i = 0; i < last; ++i) add(";   step %d %s %d %d %.9g\n", i, steps[T.steps[i].op], T.steps[i].a, T.steps[i].b, T.steps[i].imm);
+    add(";   post=%d+%d tail=%d+%d out base=%d p=%d q=%d z=%d,%d of %d,%d accumulate=%d\n", T.post0, T.n_post, T.epi0, T.n_epi, T.out_base, T.out_cp, T.out_cq,
+        T.out_cz[0], T.out_cz[1], T.z_ext[0], T.z_ext[1], T.accumulate);
+    return text;
+}
+
 bool try_tile(Gen &g, Kernel &k, int root, int scale, const std::vector<std::vector<TadpRow>> &lower, const std::vector<std::vector<TadpRow>> &upper,
               const std::vector<TadpRow> &guards, double min_space, double max_space, bool may_factor, TileElse &other)
 {

@@ -1,6 +1,6 @@
 """Tile programs (sums of a term that couples two variables, as written) against the oracle: edges of tiles in every direction,
-groups of threads and blocks that share a sum, summed columns, further output variables, operands that are expressions, every step of
-a core, strides and reversed reads, inputs that are not 16-byte aligned."""
+groups of threads and blocks that share a sum, summed columns, further output variables, operands that are expressions, a core that is
+read step by step (all of its steps: test_gpu_tile_cores.py), strides and reversed reads, inputs that are not 16-byte aligned."""
 import pytest
 import torch
 
