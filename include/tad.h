@@ -164,8 +164,9 @@ size_t tad_workspace_bytes(const tad_plan *plan);
  *   f          DEVICE pointer, prod(out_shape) floats, fully overwritten
  *   workspace  DEVICE pointer, tad_workspace_bytes() bytes, 256-byte aligned, caller-owned.  Only plans
  *              whose forward pass uses auxiliary tensors or a split summation other than a contraction's need
- *              it; every other plan accepts NULL / 0 (a contraction is faster with it).  TAD_ERR_WORKSPACE when it
- *              is needed and missing or too small.
+ *              it, and not where a kernel without them does as well (sums of products by tiles, long rows by a block
+ *              each); every other plan accepts NULL / 0 (these and contractions are faster with it).  TAD_ERR_WORKSPACE when
+ *              it is needed and missing or too small.
  */
 tad_status tad_forward(const tad_plan *plan, const float *const *args, float *f,
                        void *workspace, size_t workspace_bytes, void *cuda_stream);
@@ -215,8 +216,8 @@ tad_status tad_backward_arg(const tad_plan *plan, const float *const *args, cons
  *
  * The scratch is a fixed array of TAD_NOALLOC_SCRATCH_BYTES inside the library image; every
  * GPU that loads the library holds that much memory until the process exits.  A plan whose
- * workspace is larger even without what a contraction can do without (an operand laid out for the
- * tensor cores, planes of a split sum) is rejected with TAD_ERR_WORKSPACE and a message; nothing
+ * workspace is larger even without what its kernels can do without (an operand laid out for the
+ * tensor cores, planes of a split contraction, tensors of sums that tiles can run as well) is rejected with TAD_ERR_WORKSPACE and a message; nothing
  * is launched in that case.  The call allocates nothing (no cudaMalloc / cudaFree, no
  * allocating library routine); inputs and outputs are still the caller's buffers, with the
  * same meaning as in tad_backward.

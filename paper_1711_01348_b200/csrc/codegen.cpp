@@ -1047,10 +1047,10 @@ bool try_points(Gen &g, Kernel &k, int root, int scale, bool allow_split, const 
 // keeps the digits that they lose (Analysis::apart).
 constexpr double TILE_LEAST = double(1 << 16), TILE_MOST = 5e7;
 
-// shared tail: choose temps, emit, fill the program
-void emit_kernel(Gen &g, Kernel &k, int root, const std::vector<std::vector<TadpRow>> &lower,
-                 const std::vector<std::vector<TadpRow>> &upper, const std::vector<TadpRow> &guards, bool allow_split = false,
-                 bool may_factor = true)
+// shared tail: choose temps, emit, fill the program; spare: what needs no workspace, where something faster was taken
+void emit_chosen(Gen &g, Kernel &k, int root, const std::vector<std::vector<TadpRow>> &lower,
+                 const std::vector<std::vector<TadpRow>> &upper, const std::vector<TadpRow> &guards, bool allow_split,
+                 bool may_factor, std::vector<Kernel> &spare)
 {
     TadpProgram &prog = k.prog;
     place(g);
@@ -1089,10 +1089,10 @@ void emit_kernel(Gen &g, Kernel &k, int root, const std::vector<std::vector<Tadp
         }
     }
     // a product of two index expressions under summations runs on the tile kernel, not in the interpreter
-    if (try_contraction(g, k, root, scale, allow_split, lower, upper, guards)) return;
+    if (try_contraction(g, k, root, scale, allow_split, lower, upper, guards, spare)) return;
     // sums of a term that couples two variables, as written, by tiles of both
     TileElse other = TILE_NO_OTHER;
-    if (try_tile(g, k, root, scale, lower, upper, guards, TILE_LEAST, TILE_MOST, may_factor, other)) return;
+    if (try_tile(g, k, root, scale, lower, upper, guards, TILE_LEAST, TILE_MOST, may_factor, other, spare)) return;
     if (other == TILE_POINTS) {
         try {
             if (try_points(g, k, root, scale, allow_split, lower, upper, guards)) return;
@@ -1102,7 +1102,7 @@ void emit_kernel(Gen &g, Kernel &k, int root, const std::vector<std::vector<Tadp
     // sums that can be pushed inside the term (Sec. 6's missing clean-up step): auxiliary kernels + a smaller kernel
     if (may_factor && try_factoring(g, k, root, scale, allow_split, lower, upper, guards)) return;
     // (sums that do not gain from that)
-    if (try_tile(g, k, root, scale, lower, upper, guards, other == TILE_APART ? TILE_LEAST : TILE_MOST, 1e18, false, other)) return;
+    if (try_tile(g, k, root, scale, lower, upper, guards, other == TILE_APART ? TILE_LEAST : TILE_MOST, 1e18, false, other, spare)) return;
     // short sums ahead of a kernel: as point programs they share a launch with the others
     if (!may_factor && g.kappa == 0 && g.inst[root].op == I_SUM) {
         try {
@@ -1402,6 +1402,24 @@ void emit_kernel(Gen &g, Kernel &k, int root, const std::vector<std::vector<Tadp
     }
 }
 
+// planes that cannot be done without, of a kernel or one of its auxiliary kernels
+size_t planes_of(const Kernel &k)
+{
+    size_t most = 0;
+    if (k.ew.empty() && k.contract.empty() && k.prog.zsplit > 1) most = (size_t(k.prog.zsplit) + 1) * size_t(k.prog.part_limit) * 4;      // (line sums too)
+    for (const Kernel &y : k.pre) most = std::max(most, planes_of(y));
+    return most;
+}
+
+void emit_kernel(Gen &g, Kernel &k, int root, const std::vector<std::vector<TadpRow>> &lower,
+                 const std::vector<std::vector<TadpRow>> &upper, const std::vector<TadpRow> &guards, bool allow_split = false,
+                 bool may_factor = true)
+{
+    std::vector<Kernel> spare;
+    emit_chosen(g, k, root, lower, upper, guards, allow_split, may_factor, spare);
+    if (may_factor && (!k.aux.empty() || planes_of(k))) k.spare = std::move(spare);
+}
+
 }  // namespace
 
 void emit_plain_kernel(Gen &g, Kernel &k, int root, const std::vector<std::vector<TadpRow>> &lower,
@@ -1432,8 +1450,6 @@ static void account(tad_plan &p, Kernel &k)
 {
     batch_auxiliaries(k);
     std::function<void(const Kernel &)> walk = [&](const Kernel &x) {
-        if (x.ew.empty() && x.contract.empty() && x.prog.zsplit > 1)   // (line-sum kernels keep their shares in prog too)
-            p.partial_least = std::max(p.partial_least, (size_t(x.prog.zsplit) + 1) * size_t(x.prog.part_limit) * 4);
         for (const TadcProgram &cp : x.contract) {
             if (cp.ksplit > 1)
                 p.partial_bytes = std::max(p.partial_bytes, size_t(cp.ksplit) * size_t(cp.M.extent) * size_t(cp.N.extent) * size_t(cp.Z.extent) * 4);
@@ -1442,6 +1458,8 @@ static void account(tad_plan &p, Kernel &k)
         for (const Kernel &y : x.pre) walk(y);
     };
     walk(k);
+    p.partial_least = std::max(p.partial_least, planes_of(k));
+    if (k.spare.empty()) p.partial_lean = std::max(p.partial_lean, planes_of(k));
     p.partial_bytes = std::max(p.partial_bytes, p.partial_least);
     p.aux_bytes = std::max(p.aux_bytes, k.aux_bytes);
     std::function<int(const Kernel &)> launches = [&](const Kernel &x) {
@@ -1817,6 +1835,11 @@ void share_auxiliaries(tad_plan &p)
         ++p.n_shared;
     }
     if (p.n_shared) p.aux_bytes = cursor;
+    // what is left where spare kernels run
+    auto lean = [&](const Kernel &k) { if (k.spare.empty()) for (const Kernel::Aux &a : k.aux) p.aux_lean = std::max(p.aux_lean, (a.offset + a.bytes + 255) & ~size_t(255)); };
+    lean(p.forward);
+    for (const Kernel &k : p.stages) lean(k);
+    for (const Kernel &k : p.backward) lean(k);
 }
 
 }  // namespace tad

@@ -66,8 +66,9 @@ bool mma_pays(int64_t a, int64_t b, int64_t k)
 }  // namespace
 
 // builds one contraction program from a system whose loops all have fixed ranges
-bool emit_program(const System &s0, float scale, int accumulate, bool allow_split, bool strict_fill, TadcProgram &P, std::string &text)
+bool emit_program(const System &s0, float scale, int accumulate, bool allow_split, bool strict_fill, TadcProgram &P, std::string &text, bool *long_rows)
 {
+    if (long_rows) *long_rows = false;
     System s = s0;
     const int nv = (int)s.vars.size();
     if (s.A.ptr < 0) std::swap(s.A, s.B);                  // an operand of ones plays B
@@ -174,12 +175,12 @@ bool emit_program(const System &s0, float scale, int accumulate, bool allow_spli
     // one output column: plain or weighted sums of A (B is ones or a vector over k), run at memory speed by a warp
     // per row (A along k) or a thread per row (A along m)
     // (fewer than 1024 rows take a block each: 264 rows of 6523 elements, summed for a band of 287 outputs, 80 us as a sum of both loops)
-    // A block streams about 50 GB/s: where rows are fewer than the SMs, long ones are split instead (weighted, read from HBM, row sums /
-    // split, us: 32 x 60000 17 / 17, 32 x 100000 24 / 17, 36 x 300000 56 / 26, 64 x 50000 15 / 17, 64 x 200000 42 / 30, 100 x 60000 19 / 24,
-    // 100 x 200000 46 / 38, 128 x 100000 28 / 30, 128 x 200000 48 / 44, 148 x 500000 101 / 101, 200 x 300000 73 / 83).
-    const bool long_rows = P.M.extent >= 32 && P.K.n_digits == 1 && P.K.extent >= 64 && P.K.sA[0] == 1 &&
-                           (P.M.extent >= 148 || P.K.extent <= 30000 + 800 * (int64_t)P.M.extent);
-    const bool one_column = P.N.extent == 1 && P.Z.extent == 1 && P.K.n_digits <= 1 && !P.guardA && !P.guardB && (P.M.extent >= 1024 || long_rows);
+    // A block streams about 50 GB/s: where rows are fewer than the SMs, a kernel that is one sum of long ones is better split over blocks
+    // (weighted, read from HBM, row sums / split, us: 32 x 60000 17 / 17, 32 x 100000 24 / 17, 36 x 300000 56 / 26, 64 x 50000 15 / 17,
+    // 64 x 200000 42 / 30, 100 x 60000 19 / 24, 100 x 200000 46 / 38, 128 x 100000 28 / 30, 128 x 200000 48 / 44, 148 x 500000 101 / 101).
+    const bool block_rows = P.M.extent >= 32 && P.K.n_digits == 1 && P.K.extent >= 64 && P.K.sA[0] == 1;
+    const bool too_long = long_rows && P.M.extent < 148 && P.K.extent > 30000 + 800 * (int64_t)P.M.extent;
+    const bool one_column = P.N.extent == 1 && P.Z.extent == 1 && P.K.n_digits <= 1 && !P.guardA && !P.guardB && (P.M.extent >= 1024 || block_rows);
     const bool col_sums = one_column && P.M.n_digits == 1 && P.M.sA[0] == 1 && P.K.n_digits == 1 && std::llabs((int64_t)P.K.sA[0]) != 1;
     const bool row_sums = one_column && !col_sums;
     if (!one_column && !mma && fill < (strict_fill ? 0.15 : 0.05)) return false;    // mostly empty tiles: the interpreter's schedules do better
@@ -337,11 +338,12 @@ bool emit_program(const System &s0, float scale, int accumulate, bool allow_spli
     if (P.image) std::snprintf(line + std::strlen(line) - 1, sizeof line - std::strlen(line), ", columns split ahead\n");
     text += line;
     text += group_text("m", P.M) + group_text("n", P.N) + group_text("k", P.K) + group_text("z", P.Z);
+    if (row_sums && too_long) { *long_rows = true; return false; }
     return true;
 }
 
 bool try_contraction(Gen &g, Kernel &k, int root, int scale, bool allow_split, const std::vector<std::vector<TadpRow>> &lower,
-                     const std::vector<std::vector<TadpRow>> &upper, const std::vector<TadpRow> &guards)
+                     const std::vector<std::vector<TadpRow>> &upper, const std::vector<TadpRow> &guards, std::vector<Kernel> &spare)
 {
     if (g.p.opt.debug_bounds || !guards.empty() || root < 0) return false;
     const TadpProgram &prog = k.prog;
@@ -492,8 +494,15 @@ bool try_contraction(Gen &g, Kernel &k, int root, int scale, bool allow_split, c
         for (int v = 0; v < nv; ++v) if (!s.vars[v].reduce && s.vars[v].ext <= 0) empty_out = true;
         if (empty_out) continue;
         TadcProgram P;
-        if (!emit_program(s, cfac, prog.accumulate, allow_split, true, P, text)) return false;
+        bool long_rows;
+        const bool taken = emit_program(s, cfac, prog.accumulate, allow_split, true, P, text, &long_rows);
+        if (!taken && !(long_rows && systems.size() == 1)) return false;
         progs.push_back(P);
+        if (taken) continue;
+        spare = {k};
+        spare[0].contract = progs;
+        spare[0].vec = 0; spare[0].vec_u = 0;
+        return false;
     }
     if (progs.empty()) return false;
     k.contract = progs;

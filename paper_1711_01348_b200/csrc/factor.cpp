@@ -1043,7 +1043,8 @@ static bool factor_kernel(Gen &g, Kernel &k, int root, int scale, bool allow_spl
                 }
             }
             TadcProgram cp;
-            if (!emit_program(s, 1.f, 0, true, false, cp, text)) return false;
+            bool long_rows;                                // (nothing but that sum: it goes on to what splits it)
+            if (!emit_program(s, 1.f, 0, true, false, cp, text, F.nodes.size() == 1 ? &long_rows : nullptr)) return false;
             ak.contract.push_back(cp);
             ak.listing = "; contraction -> tensor " + std::to_string(N.tensor) + "\n";
             ak.vec = 0; ak.vec_u = 0;

@@ -343,19 +343,22 @@ inline size_t image_bytes(const TadcProgram &P)
 
 // builds one contraction program from a system whose loops all have fixed ranges; an operand with ptr < 0 is
 // a tensor of ones (a plain summation of the other operand).  strict_fill: refuse mostly empty tiles
-bool emit_program(const System &s, float scale, int accumulate, bool allow_split, bool strict_fill, TadcProgram &P, std::string &text);
+// (long_rows, not null: a sum of few long rows is declined, to be split over blocks; P is built all the same and *long_rows set)
+bool emit_program(const System &s, float scale, int accumulate, bool allow_split, bool strict_fill, TadcProgram &P, std::string &text, bool *long_rows = nullptr);
 
 // contract_gen.cpp: recognises a kernel whose term is a product of two index expressions summed over
 // loops with fixed ranges and fills k.contract; returns false (and leaves k alone) otherwise.
 // allow_split: the caller has a workspace for partial sums of a split summation
+// (spare: what it would be without that)
 bool try_contraction(Gen &g, Kernel &k, int root, int scale, bool allow_split, const std::vector<std::vector<TadpRow>> &lower,
-                     const std::vector<std::vector<TadpRow>> &upper, const std::vector<TadpRow> &guards);
+                     const std::vector<std::vector<TadpRow>> &upper, const std::vector<TadpRow> &guards, std::vector<Kernel> &spare);
 
 // tile_gen.cpp: a sum whose term couples two variables becomes a tile program, if its number of points lies in the given range.
-// declined: ... and what else is faster: a point program, or (may_factor) the summation pushed inside with nothing to multiply out
+// other: declined, because a point program is faster or (may_factor) the summation is pushed inside with nothing to multiply out; spare:
+// the tile program all the same
 enum TileElse { TILE_NO_OTHER = 0, TILE_POINTS, TILE_APART };
 bool try_tile(Gen &g, Kernel &k, int root, int scale, const std::vector<std::vector<TadpRow>> &lower, const std::vector<std::vector<TadpRow>> &upper,
-              const std::vector<TadpRow> &guards, double min_space, double max_space, bool may_factor, TileElse &other);
+              const std::vector<TadpRow> &guards, double min_space, double max_space, bool may_factor, TileElse &other, std::vector<Kernel> &spare);
 // codegen.cpp: estimated microseconds of a point program of so many outputs, terms each and steps a term (chain: what is computed from
 // the sum follows it in the same thread; loops: the sum may be shared out; along: lanes lie along the terms)
 double point_time(double points, double terms, double steps, bool chain, bool loops, bool along);

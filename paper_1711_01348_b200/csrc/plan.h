@@ -88,6 +88,7 @@ struct Kernel {
     int batch = -1;            // an auxiliary kernel that runs in one launch with the others of the same number
     int shared = -1;           // an auxiliary kernel whose result other gradients need too: its number in the plan (its tensor then
                                // lies behind the kernels' own areas)
+    std::vector<Kernel> spare; // what runs instead where there is no room for the auxiliary tensors or planes of this one (needs neither)
     KernelStats stats;
     std::string listing;
 };
@@ -120,6 +121,7 @@ struct tad_plan {
     size_t partial_bytes = 0;                   // workspace for the partial sums of split summations (largest kernel)
     size_t partial_least = 0;                   // ... of the summations that cannot do without (a contraction can run in fewer shares)
     size_t aux_bytes = 0;                       // workspace for auxiliary tensors (largest kernel, then the shared ones)
+    size_t partial_lean = 0, aux_lean = 0;      // partial_least and aux_bytes where spare kernels run
     int n_shared = 0;                           // auxiliary kernels that several gradients have in common
     mutable void *side = nullptr;               // second stream and its events (independent memory-bound passes run beside a contraction)
     mutable void *host_step = nullptr;          // streams and events of tad_step_host, created by its first call

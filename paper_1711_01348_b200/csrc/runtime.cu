@@ -463,12 +463,16 @@ size_t stage_offset(const tad_plan *plan, int s)
 }
 
 thread_local bool t_built_in = false;             // set while tad_backward_noalloc runs
+thread_local bool t_lean = false;                 // set while it runs with spare kernels, because the others' tensors do not fit
+
+const tad::Kernel &fitting(const tad::Kernel &k) { return t_lean && !k.spare.empty() ? k.spare[0] : k; }
+size_t least_planes(const tad_plan *plan) { return t_lean ? plan->partial_lean : plan->partial_least; }
 
 // what a plan needs with `partial` bytes for planes of partial sums; contractions whose operand image does not fit behind it
 // gather as usual
 size_t bytes_with(const tad_plan *plan, size_t partial)
 {
-    return stage_offset(plan, (int)plan->stages.size()) + pad256(partial) + pad256(plan->aux_bytes);
+    return stage_offset(plan, (int)plan->stages.size()) + pad256(partial) + pad256(t_lean ? plan->aux_lean : plan->aux_bytes);
 }
 size_t required_bytes(const tad_plan *plan) { return bytes_with(plan, plan->partial_bytes); }
 
@@ -478,7 +482,7 @@ size_t partial_room(const tad_plan *plan, size_t workspace_bytes)
 {
     if (workspace_bytes >= required_bytes(plan)) return plan->partial_bytes;
     const size_t rest = bytes_with(plan, 0);
-    return std::max(plan->partial_least, workspace_bytes > rest ? (workspace_bytes - rest) & ~size_t(255) : 0);
+    return std::max(least_planes(plan), workspace_bytes > rest ? (workspace_bytes - rest) & ~size_t(255) : 0);
 }
 
 // workspace layout: ... [planes of partial sums][auxiliary tensors][image of a column operand]
@@ -501,10 +505,15 @@ bool forward_splits(const tad::Kernel &k)
     return false;
 }
 
+bool has_room(const tad_plan *plan, const void *workspace, size_t workspace_bytes)
+{
+    const size_t need = t_built_in ? bytes_with(plan, least_planes(plan)) : required_bytes(plan);
+    return !need || (workspace && workspace_bytes >= need && !(reinterpret_cast<uintptr_t>(workspace) & 255u));
+}
+
 bool check_workspace(const tad_plan *plan, void *workspace, size_t workspace_bytes)
 {
-    const size_t need = t_built_in ? bytes_with(plan, plan->partial_least) : required_bytes(plan);
-    if (need && (!workspace || workspace_bytes < need || (reinterpret_cast<uintptr_t>(workspace) & 255u))) {
+    if (!has_room(plan, workspace, workspace_bytes)) {
         tad::set_error("workspace missing, smaller than tad_workspace_bytes() or not 256-byte aligned");
         return false;
     }
@@ -583,7 +592,8 @@ tad_status tad_forward(const tad_plan *plan, const float *const *args, float *f,
 {
     if (!plan || !f || (plan->n_args && !args)) { tad::set_error("NULL argument"); return TAD_ERR_INVALID_ARG; }
     const bool needs_ws = !plan->forward.aux.empty() || forward_splits(plan->forward);
-    if (needs_ws && !check_workspace(plan, workspace, workspace_bytes)) return TAD_ERR_WORKSPACE;
+    const bool spare = needs_ws && !plan->forward.spare.empty() && !has_room(plan, workspace, workspace_bytes);
+    if (needs_ws && !spare && !check_workspace(plan, workspace, workspace_bytes)) return TAD_ERR_WORKSPACE;
     // (a contraction's shares do without: they become one)
     const bool has_ws = workspace && workspace_bytes >= required_bytes(plan) && (reinterpret_cast<uintptr_t>(workspace) & 255u) == 0;
     TadpPointers ptrs{};
@@ -601,7 +611,7 @@ tad_status tad_forward(const tad_plan *plan, const float *const *args, float *f,
             ? reinterpret_cast<float *>(static_cast<char *>(workspace) + stage_offset(plan, (int)plan->stages.size())) : nullptr;
         aux_base = static_cast<char *>(workspace) + aux_offset(plan, workspace_bytes);
     }
-    return launch(plan->forward, ptrs, false, (cudaStream_t)cuda_stream, aux_base, side_of(plan));
+    return launch(spare ? plan->forward.spare[0] : plan->forward, ptrs, false, (cudaStream_t)cuda_stream, aux_base, side_of(plan));
 }
 
 tad_status tad_backward_stage(const tad_plan *plan, const float *const *args, const float *df,
@@ -613,7 +623,7 @@ tad_status tad_backward_stage(const tad_plan *plan, const float *const *args, co
     if (!fill_inputs(plan, args, df, workspace, workspace_bytes, ptrs)) return TAD_ERR_INVALID_ARG;
     for (int s = 0; s < (int)plan->stages.size(); ++s) {
         ptrs.out = reinterpret_cast<float *>(static_cast<char *>(workspace) + stage_offset(plan, s));
-        tad_status st = launch(plan->stages[s], ptrs, plan->opt.debug_bounds != 0, (cudaStream_t)cuda_stream,
+        tad_status st = launch(fitting(plan->stages[s]), ptrs, plan->opt.debug_bounds != 0, (cudaStream_t)cuda_stream,
                                workspace ? static_cast<char *>(workspace) + aux_offset(plan, workspace_bytes) : nullptr, side_of(plan));
         if (st != TAD_OK) return st;
     }
@@ -655,7 +665,7 @@ static tad_status backward_arg(const tad_plan *plan, const float *const *args, c
         if (!k.tile.empty() && k.pre.empty()) return later->tiles.add(k.tile[0], ptrs, darg, stream);
     }
     for (int ki : plan->arg_kernels[arg]) {
-        tad_status st = launch(plan->backward[ki], ptrs, plan->opt.debug_bounds != 0, stream,
+        tad_status st = launch(fitting(plan->backward[ki]), ptrs, plan->opt.debug_bounds != 0, stream,
                                workspace ? static_cast<char *>(workspace) + aux_offset(plan, workspace_bytes) : nullptr, side, pending, done);
         pending = nullptr;
         if (st != TAD_OK) return st;
@@ -874,7 +884,9 @@ tad_status tad_backward_noalloc(const tad_plan *plan, const float *const *args, 
                                 float *const *dargs, void *cuda_stream)
 {
     if (!plan) { tad::set_error("NULL plan"); return TAD_ERR_INVALID_ARG; }
-    const size_t need = bytes_with(plan, plan->partial_least);
+    size_t need = bytes_with(plan, plan->partial_least);
+    struct Lean { ~Lean() { t_lean = false; } } lean_ends;
+    if (need > TAD_NOALLOC_SCRATCH_BYTES) { t_lean = true; need = bytes_with(plan, plan->partial_lean); }
     if (need > TAD_NOALLOC_SCRATCH_BYTES) {
         char msg[160];
         snprintf(msg, sizeof msg, "this plan needs %zu bytes of scratch, tad_backward_noalloc holds at most %zu; "

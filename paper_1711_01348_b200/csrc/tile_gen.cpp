@@ -565,7 +565,7 @@ std::string tile_listing(const TadtProgram &T)
 }
 
 bool try_tile(Gen &g, Kernel &k, int root, int scale, const std::vector<std::vector<TadpRow>> &lower, const std::vector<std::vector<TadpRow>> &upper,
-              const std::vector<TadpRow> &guards, double min_space, double max_space, bool may_factor, TileElse &other)
+              const std::vector<TadpRow> &guards, double min_space, double max_space, bool may_factor, TileElse &other, std::vector<Kernel> &spare)
 {
     other = TILE_NO_OTHER;
     if (g.p.opt.debug_bounds || root < 0 || !guards.empty()) return false;
@@ -586,14 +586,14 @@ bool try_tile(Gen &g, Kernel &k, int root, int scale, const std::vector<std::vec
     if (points < min_space || points > max_space) return false;
     Analysis all(g, k);
     if (!all.run(root, scale, lower, upper)) return false;
-    if (may_factor && points > TILE_APART_LEAST && all.apart()) { other = TILE_APART; return false; }
+    if (may_factor && points > TILE_APART_LEAST && all.apart()) other = TILE_APART;
     std::unique_ptr<Tiler> found;
     for (const Choice &c : all.choices) {
         found.reset(new Tiler(all));
         if (found->build(root, scale, c)) break;
         found.reset();
     }
-    if (!found) return false;
+    if (!found) { other = TILE_NO_OTHER; return false; }
     const Tiler &t = *found;
     // Taken where it is estimated to be faster than what else would run it.  Microseconds of a tile program, fitted to 840 kernels of 2 to
     // 5000 rows, columns and terms (of the estimate / measured 90 % lie between 0.63 and 1.36); of a point program, see point_time.  A
@@ -609,8 +609,14 @@ bool try_tile(Gen &g, Kernel &k, int root, int scale, const std::vector<std::vec
     bool along = false, across = false;
     for (int v = 0; v < (int)g.vars.size(); ++v) if (std::abs(big->coef[v]) == 1 && all.ext[v] > 1) (v < g.n_outer ? across : along) = true;
     const bool serial = chain && t.T.q_sum && g.inst[all.leaf].hi - g.inst[all.leaf].lo < 3;      // (a short sum of sums stays in its thread)
-    if (!serial && us > (t.T.path ? 2.0 : 1.15) * point_time(outs, points / outs, steps, chain, g.kappa >= 1, along && !across)) { other = TILE_POINTS; return false; }
-    if (outs >= double(1 << 21) && us > 4 + 1.2e-6 * t.n_code * points) return false;
+    if (other == TILE_NO_OTHER && !serial && us > (t.T.path ? 2.0 : 1.15) * point_time(outs, points / outs, steps, chain, g.kappa >= 1, along && !across)) other = TILE_POINTS;
+    const bool streams = outs >= double(1 << 21) && us > 4 + 1.2e-6 * t.n_code * points;
+    if (other != TILE_NO_OTHER || streams) {
+        spare = {k};
+        spare[0].tile = {t.T};
+        spare[0].prog.zsplit = 1;
+        return false;
+    }
     k.tile = {t.T};
     k.prog.zsplit = 1;
     k.vec = 0; k.vec_u = 0;
