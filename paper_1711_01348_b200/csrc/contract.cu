@@ -407,11 +407,12 @@ tad_contract_reduce(const __grid_constant__ TadcProgram P, const __grid_constant
 //     out[m] (+)= scale * sum_k A[row(m) + k * stride] (* B[k])
 // Bound by HBM: every element of A is read once, in pieces of 16 bytes from the first aligned one on where the row is consecutive
 // (and its weights lie alike), four in flight per lane.  A warp per output, or, where that would leave the GPU idle, a block of
-// eight (WARPS): 264 rows of 6523 elements.  Sums are added in a fixed order.  Four blocks to an SM: short rows wait for one load after
-// another and live on the warps beside them (with two, weighted 500000 x 64 197 us, 30000 x 100 13.4, strided 500000 x 9 184; with four
-// 113, 7.9, 74).
-template <int WARPS>
-__global__ void __launch_bounds__(256, 4)
+// eight (WARPS): 264 rows of 6523 elements.  Sums are added in a fixed order.  Four blocks to an SM (BLOCKS): short rows wait for one load
+// after another and live on the warps beside them (with two, weighted 500000 x 64 197 us, 30000 x 100 13.4, strided 500000 x 9 184; with
+// four 113, 7.9, 74).  Two where weighted rows are no more than that many: eight pieces in flight per lane take the registers of four blocks
+// (1500 x 60000 77 and 122 us, 200 x 500000 90 and 140).
+template <int WARPS, int BLOCKS>
+__global__ void __launch_bounds__(256, BLOCKS)
 tad_rowsum_kernel(const __grid_constant__ TadcProgram P, const __grid_constant__ TadpPointers ptrs)
 {
     tad_wait_previous();
@@ -576,8 +577,11 @@ cudaError_t tad_launch_contract(const TadcProgram &P, const TadpPointers &ptrs, 
         // (weighted rows, warp / block a row, us: 264 of 512 2.1 / 2.3, of 1024 2.5 / 2.4, of 8192 7.5 / 3.0; 592 of 1024 2.5 / 2.8, of 4096
         // 4.7 / 3.0; 1100 of 1024 2.6 / 4.0, of 4096 4.9 / 4.5; 1200 rows are eight warps to an SM)
         const unsigned rows = (unsigned)P.M.extent;
-        if (rows < sms * 8u && (unsigned)P.K.extent >= std::max(512u, 4u * rows)) tad_launch(tad_rowsum_kernel<8>, rows, 256, 0, stream, P, ptrs);
-        else tad_launch(tad_rowsum_kernel<1>, std::min((rows + 7u) / 8u, sms * 16u), 256, 0, stream, P, ptrs);
+        const bool by_block = rows < sms * 8u && (unsigned)P.K.extent >= std::max(512u, 4u * rows);
+        const unsigned blocks = by_block ? rows : (rows + 7u) / 8u;
+        const bool few = P.ptrB >= 0 && blocks <= sms * 2u;
+        auto kernel = by_block ? (few ? tad_rowsum_kernel<8, 2> : tad_rowsum_kernel<8, 4>) : (few ? tad_rowsum_kernel<1, 2> : tad_rowsum_kernel<1, 4>);
+        tad_launch(kernel, std::min(blocks, by_block ? blocks : sms * 16u), 256, 0, stream, P, ptrs);
         return cudaGetLastError();
     }
     cudaError_t e = P.shape == 1 ? launch_shape<128, 32, 8, 4>(P, ptrs, stream)

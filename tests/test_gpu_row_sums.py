@@ -18,7 +18,7 @@ def _weighted(n, k, step):
 
 
 # an element a lane or pieces, a warp or a block a row: either side of each line
-EDGES = [(2001, 32, 1), (2001, 33, 1), (1500, 32, 2), (1500, 33, 2), (1200, 65, 1), (250, 999, 1), (250, 1000, 1), (1183, 4731, 1), (1183, 4732, 1), (1184, 4736, 1)]
+EDGES = [(2001, 32, 1), (2001, 33, 1), (1500, 32, 2), (1500, 33, 2), (1200, 65, 1), (250, 999, 1), (250, 1000, 1), (1183, 4731, 1), (1183, 4732, 1), (1184, 4736, 1), (296, 1185, 1), (297, 1189, 1), (2368, 601, 1), (2369, 601, 1)]
 
 
 @pytest.mark.parametrize("n,k,step", CASES)
