@@ -329,19 +329,15 @@ tad_prod_kernel(const __grid_constant__ TadeProgram P, const __grid_constant__ P
 #pragma unroll
         for (int v = 0; v < TADP_MAX_VARS; ++v) R.out += P.out_coef[v] * var[v];
         R.ostep = P.out_coef[lane_var] * (int)es; R.oadv = SINGLE ? P.out_coef[lane_var] * (int)(4u * cols) : P.out_coef[row_var];
-        if constexpr (M == 0 && (ONE || !SINGLE)) {
-#pragma unroll 1
-            for (int r = 0; r < (ONE ? 1 : n_rows); ++r) {
-                if (VEC && live == 4) {
-                    float4 *dst = reinterpret_cast<float4 *>(out + (unsigned)R.out);
-                    float4 q = make_float4(held[0], held[1], held[2], held[3]);
-                    if (accumulate) { const float4 o = *dst; q.x += o.x; q.y += o.y; q.z += o.z; q.w += o.w; }
-                    *dst = q;
-                } else {
+        if constexpr (M == 0 && ONE) {
+            if (VEC && live == 4) {
+                float4 *dst = reinterpret_cast<float4 *>(out + (unsigned)R.out);
+                float4 q = make_float4(held[0], held[1], held[2], held[3]);
+                if (accumulate) { const float4 o = *dst; q.x += o.x; q.y += o.y; q.z += o.z; q.w += o.w; }
+                *dst = q;
+            } else {
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) if (j < live) { const unsigned o = (unsigned)(R.out + j * R.ostep); out[o] = accumulate ? out[o] + held[j] : held[j]; }
-                }
-                R.out += R.oadv;
+                for (int j = 0; j < 4; ++j) if (j < live) { const unsigned o = (unsigned)(R.out + j * R.ostep); out[o] = accumulate ? out[o] + held[j] : held[j]; }
             }
             continue;
         }
@@ -497,8 +493,10 @@ cudaError_t tad_launch_ew(const TadeProgram &P, const TadpPointers &ptrs, unsign
         else { if (Q.vec) tad_launch(tad_prod_kernel<true, G, B, false, false>, TAD_PROD_ARGS); else tad_launch(tad_prod_kernel<false, G, B, false, false>, TAD_PROD_ARGS); } \
         break;
 #define TAD_PROD_LAUNCH_ONE(G) case G: tad_launch(tad_prod_kernel<true, G, 0, true, true>, TAD_PROD_ARGS); break;
-        if (Q.row_var < 0 && Q.run == 1) {
-            if (!Q.vec) tad_launch(tad_prod_kernel<false, 0, 0, true, true>, TAD_PROD_ARGS);      // (nothing moves then)
+        if (Q.run == 1) {                                      // (nothing moves but in a single row that is read in pieces)
+            if (Q.row_var >= 0 && Q.vec) tad_launch(tad_prod_kernel<true, 0, 0, false, true>, TAD_PROD_ARGS);
+            else if (Q.row_var >= 0) tad_launch(tad_prod_kernel<false, 0, 0, false, true>, TAD_PROD_ARGS);
+            else if (!Q.vec) tad_launch(tad_prod_kernel<false, 0, 0, true, true>, TAD_PROD_ARGS);
             else switch (Q.n_moving) {
             TAD_PROD_LAUNCH_ONE(0) TAD_PROD_LAUNCH_ONE(1) TAD_PROD_LAUNCH_ONE(2) TAD_PROD_LAUNCH_ONE(3)
             default: return cudaErrorInvalidValue;

@@ -93,5 +93,17 @@ def test_off_a_boundary(name, shift):
     _check(CASES[name](), shift)
 
 
+@pytest.mark.gpu
+@pytest.mark.parametrize("ni,nj", [(70, 5001), (600, 1000), (1000, 4003)])
+def test_repeated(ni, nj):
+    """the gradient of x in f_i = sum_j w_i x_ij repeats w_i df_i (w inside the sum: f, which nearly cancels, is then measured by its
+    terms; of 4003 of them it is off by some 4003^(1/2) 2^-24 60, 1.4e-5 where |f| may be 0.02)"""
+    b = Builder("repeated", [ni], 1, ["x", "w"], [[ni, nj], [ni]])
+    b.sum(1, 0, nj - 1, b.bin("mul", b.load("w", [unit(2, (0, 1))]), b.load("x", [unit(2, (0, 1)), unit(2, (1, 1))])))
+    e = b.done()
+    assert "element-wise" in Plan(e).disassemble(0) or "element-wise" in Plan(e).disassemble(1)
+    _check(e)
+
+
 def test_rows_are_joined():
     assert "rows of %d along" % (1301 * 2477) in Plan(_flat(1301, 2477)).disassemble(-1)
